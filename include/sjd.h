@@ -162,7 +162,8 @@ size_t sjd_workspace_bytes(const sjd_params* params);
  * looked at).  Decided from the shape alone: it assumes the driver offers the tensor-map encoder the range
  * kernel needs, which every driver that runs this library's kernels does.  Launches nothing.
  */
-#define SJD_ROWS_GENERIC 0 /* any shape: radix select over global memory, several passes                   */
+#define SJD_ROWS_GENERIC 0 /* any shape: sifted by a sampled threshold in one pass where V >= 2,048 and K is a modest
+                              share of it, else a radix select over global memory in several passes         */
 #define SJD_ROWS_TILES 1   /* V a multiple of 2,048: one pass, tiles dealt to the filter warps             */
 #define SJD_ROWS_RANGES 2  /* V a multiple of 256, kcap <= 2,048: one pass, one id range per filter thread */
 int sjd_row_kernel(const sjd_params* params);

@@ -1,0 +1,1063 @@
+// Row kernels that sift a row by a sampled threshold: the sampling head (guidance merge, temperature, top-K,
+// softmax, the row's own draw) in one pass over the logits.
+//
+// A row is cut into segments of consecutive ids, one per warp.  Its phases:
+//
+//   sample    256 pieces spread evenly over the row (64 bytes each, 16 where the row is short) give a threshold
+//             tau0 that a little more than K of the row's entries reach.
+//   sift      every warp takes its segment through shared memory in units of 4 KB per logits array: all entries
+//             are merged and compared with tau0, which leaves one bit per entry in a register of the lane; the
+//             set bits become a dense list of ids by one scan; the listed entries are merged once more from
+//             shared memory and kept with their ids.  Comparing costs ~5 instructions per entry whatever comes of it,
+//             keeping is paid for the few per cent that are kept, at full lanes.
+//   finish    exact K-th largest among the candidates by a histogram and a ranking inside one bin (ties to the
+//             lower id), softmax, output, inverse-CDF draw.  Every warp works on its own candidates, which are in
+//             ascending id order already; what the warps exchange is a histogram and a few sums.
+//
+// A row whose candidates cannot contain its top-K for sure (fewer than K), do not fit the lists, or have no finite
+// maximum is redone by row_generic() from global memory: results are exact for any input.
+//
+// Two kernels share the phases:
+//
+//   rows_stream_kernel   many rows: one persistent CTA per SM of up to three teams of eight warps.  A team takes a row
+//                        through all phases; the teams take the CTA's rows in turn.  The rows' units come through one
+//                        ring of shared-memory slots per segment, in row order, so that one team sifts at the
+//                        memory's pace while the others finish their row and sample their next one.
+//   rows_cluster_kernel  few rows: one cluster of up to eight CTAs of sixteen warps per row, the whole row in shared
+//                        memory at once.  The candidates go straight into the first CTA's lists (distributed shared
+//                        memory), which finishes the row.
+//
+// Measured against what took these shapes before: 231 rows of 50,264 bf16 entries, K=500: 32.2 us a step, any-shape
+// kernel 100.6 (four radix passes and a compaction over the row in the L2); 1,024 rows of 65,536, K=8,192: 254, 524;
+// 16 rows of 4,096 fp32 entries, K=64: 12.5, tile kernel 16.3.
+//
+// Every wait on an mbarrier is bounded; a wait that gives up marks the row (and the CTA's unfinished rows) with
+// kRowStatusTimeout, and the CTA waits (bounded) for its copies in flight before it exits.
+#pragma once
+
+#include "rows_pipeline.cuh"
+
+namespace sjd {
+
+constexpr int kSiftPieces = 256;          // sample pieces per row
+constexpr int kSiftBins = 1024;           // bins of a row's histogram (the sample's, then the candidates')
+constexpr int kBinsLow = 768;             // candidates' bins 1 .. kBinsLow cover the stretch that holds the threshold
+constexpr int kSiftKeyShift = 22;         // key bits dropped by the sample's first pass: sign, exponent, one mantissa bit stay
+constexpr int kMemberCap = 512;           // members of the threshold bin ranked by brute force
+constexpr int kUnitBytes = 4096;          // bytes of one logits array per unit: 128 for each lane
+constexpr int kTeamWarps = 8;             // stream kernel: warps per team
+constexpr int kTeamThreads = kTeamWarps * 32;
+constexpr int kMaxTeams = 3;
+constexpr int kMaxSlots = 4;              // ring slots per warp
+constexpr int kStreamRows = 64;           // live rows a CTA takes in one launch (the host splits larger problems)
+constexpr int kClusterWarps = 16;
+constexpr int kMaxCluster = 8;
+
+struct SiftCfg {
+  int piece_stride;  // elements between the starts of two sample pieces (a multiple of 8)
+  int piece_vecs;    // 16-byte vectors per piece: 4 or 1
+  int by_vectors;    // 1: ranks among the vectors' maxima; 0: among all sampled elements
+  int rank;          // rank (from the top) of tau0
+  int rank_high;     // rank of a value that the threshold hardly ever exceeds
+  int seg_len;       // ids per segment, a multiple of 8
+  int seg_cap;       // candidates a segment's list holds (a multiple of 8)
+  int teams, slots;  // stream kernel: teams per CTA, ring slots per warp
+  int row_begin, row_end;  // stream kernel: this launch covers rows [row_begin, row_end)
+};
+
+struct SiftMember {  // member of the threshold bin: value and id
+  float y;
+  int32_t id;
+};
+
+// what the warps that work on one row share
+struct alignas(16) SiftShared {
+  union {
+    uint32_t hist[kSiftBins];        // zero whenever it is not in use
+    SiftMember member[kMemberCap];   // the threshold bin's members, after the histogram's last search
+  };
+  uint64_t wtot[kClusterWarps];
+  uint32_t wcnt[kClusterWarps];
+  float wz[kClusterWarps];
+  uint32_t top_key;   // largest sample value
+  uint32_t max_key;   // largest candidate
+  uint32_t over;      // a list ran over, or a wait gave up
+  int members;
+  uint32_t rank_bin, rank_above, rank_count, rank_bin2;  // results of a rank search
+  float thr_y;
+  int thr_id;
+  float ptok;
+  uint32_t rnd_lo, rnd_hi;
+};
+
+// barrier of the warps that work on one row
+template <int NT>
+__device__ __forceinline__ void row_sync(int bar) {
+  asm volatile("bar.sync %0, %1;" ::"r"(bar), "n"(NT) : "memory");
+}
+
+// ---------------------------------------------------------------------------------------------------
+// logits: sixteen bytes of each array at a time
+// ---------------------------------------------------------------------------------------------------
+template <int DTYPE>
+struct SiftTraits {
+  static constexpr int kElem = DTYPE == 0 ? 4 : 2;           // bytes
+  static constexpr int kVec = 16 / kElem;                    // elements per 16-byte vector
+  static constexpr int kUnit = kUnitBytes / kElem;           // elements per unit
+  static constexpr int kPiece = 64 / kElem;                  // elements of 64 bytes; a lane has two such pieces of a unit
+};
+
+// Merged logits of one vector, packed in pairs: d = c - u; g = fma(s, d, u); y = g * inv_T, one rounding per
+// operation (a 16-bit c goes into the subtraction as it is).
+template <int DTYPE, bool HAS_U, bool HAS_T>
+__device__ __forceinline__ void merge_vec(const uint4& cv, const uint4& uv, uint64_t s2, uint64_t t2,
+                                          uint64_t (&y)[SiftTraits<DTYPE>::kVec / 2]) {
+  const uint32_t cw[4] = {cv.x, cv.y, cv.z, cv.w}, uw[4] = {uv.x, uv.y, uv.z, uv.w};
+#pragma unroll
+  for (int k = 0; k < SiftTraits<DTYPE>::kVec / 2; ++k) {
+    uint64_t g;
+    if (DTYPE == 0) {
+      g = (uint64_t)cw[2 * k & 3] | ((uint64_t)cw[(2 * k + 1) & 3] << 32);
+      if (HAS_U) {
+        const uint64_t u = (uint64_t)uw[2 * k & 3] | ((uint64_t)uw[(2 * k + 1) & 3] << 32);
+        g = fma2(s2, sub2(g, u), u);
+      }
+    } else if (HAS_U) {
+      uint64_t u;
+      if (DTYPE == 1) {
+        u = pack2(bf16_lo(uw[k]), bf16_hi(uw[k]));
+      } else {
+        const float2 f = f16_pair(uw[k]);
+        u = pack2(f.x, f.y);
+      }
+      g = fma2(s2, sub2_narrow<DTYPE>(cw[k], u), u);
+    } else if (DTYPE == 1) {
+      g = pack2(bf16_lo(cw[k]), bf16_hi(cw[k]));
+    } else {
+      const float2 f = f16_pair(cw[k]);
+      g = pack2(f.x, f.y);
+    }
+    if (HAS_T) g = mul2(g, t2);
+    y[k] = g;
+  }
+}
+
+__device__ __forceinline__ uint32_t lds32(uint32_t at) {
+  uint32_t v;
+  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(at));
+  return v;
+}
+__device__ __forceinline__ uint32_t lds16(uint32_t at) {
+  uint16_t v;
+  asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(at));
+  return v;
+}
+
+// y of one staged entry; a NaN ranks with -inf.
+template <int DTYPE, bool HAS_U, bool HAS_T>
+__device__ __forceinline__ float merge_entry(uint32_t c_at, uint32_t u_at, float s, float inv_T) {
+  float c, u = 0.0f;
+  if (DTYPE == 0) {
+    c = __uint_as_float(lds32(c_at));
+    if (HAS_U) u = __uint_as_float(lds32(u_at));
+  } else if (DTYPE == 1) {
+    c = __uint_as_float(lds16(c_at) << 16);
+    if (HAS_U) u = __uint_as_float(lds16(u_at) << 16);
+  } else {
+    c = f16_pair(lds16(c_at)).x;
+    if (HAS_U) u = f16_pair(lds16(u_at)).x;
+  }
+  float g = HAS_U ? __fmaf_rn(s, __fsub_rn(c, u), u) : c;
+  if (HAS_T) g = __fmul_rn(g, inv_T);
+  return fmaxf(g, __int_as_float(0xff800000));
+}
+
+__device__ __forceinline__ uint32_t scan_incl(uint32_t v, int lane) {
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const uint32_t n = __shfl_up_sync(0xffffffffu, v, d);
+    if (lane >= d) v += n;
+  }
+  return v;
+}
+
+// ---------------------------------------------------------------------------------------------------
+// rank search: the bin b with (entries above b) < target <= (entries in b and above), for one or two targets, by one
+// warp, which also leaves the histogram zero.  A bin is 0 when there are fewer than `target` entries in bins 1 and
+// above.  A call of its own: all searches of a row run the same few instructions, which matters where every
+// instruction is fetched for the first time.
+// ---------------------------------------------------------------------------------------------------
+static __device__ __noinline__ void rank_search(SiftShared* sm, uint32_t* hist, uint32_t target, uint32_t target2) {
+  const int lane = threadIdx.x & 31;
+  // lane l: bins 32 l .. 32 l + 31; the eight lanes served together start at different 16-byte pieces
+  uint4* const mine = reinterpret_cast<uint4*>(hist + 32 * lane);
+  uint32_t sum = 0;
+#pragma unroll
+  for (int x = 0; x < 8; ++x) {
+    const uint4 w = mine[(x + lane) & 7];
+    sum += w.x + w.y + w.z + w.w;
+  }
+  // entries above this lane's bins
+  uint32_t above = sum;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const uint32_t n = __shfl_down_sync(0xffffffffu, above, d);
+    if (lane + d < 32) above += n;
+  }
+  above -= sum;
+#pragma unroll 1
+  for (int pass = 0; pass < 2; ++pass) {
+    const uint32_t t = pass == 0 ? target : target2;
+    const uint32_t votes = __ballot_sync(0xffffffffu, above < t && t <= above + sum);
+    uint32_t bin = 0, before = 0, count = 0;
+    if (votes != 0u) {
+      const int l1 = __ffs((int)votes) - 1;
+      const uint32_t above1 = __shfl_sync(0xffffffffu, above, l1);
+      const uint32_t f = hist[32 * l1 + 31 - lane];  // lane 0 takes the topmost
+      const uint32_t a2 = above1 + scan_incl(f, lane) - f;
+      const int l2 = __ffs((int)__ballot_sync(0xffffffffu, a2 < t && t <= a2 + f)) - 1;
+      bin = (uint32_t)(32 * l1 + 31 - l2);
+      before = __shfl_sync(0xffffffffu, a2, l2);
+      count = __shfl_sync(0xffffffffu, f, l2);
+    }
+    if (lane == 0) {
+      if (pass == 0) {
+        sm->rank_bin = bin;
+        sm->rank_above = before;
+        sm->rank_count = count;
+      } else {
+        sm->rank_bin2 = bin;
+      }
+    }
+    if (target2 == 0u) break;
+  }
+  __syncwarp();
+#pragma unroll
+  for (int x = 0; x < 8; ++x) mine[(x + lane) & 7] = make_uint4(0u, 0u, 0u, 0u);
+}
+
+// ---------------------------------------------------------------------------------------------------
+// sample phase: tau0 and the candidates' bins, by the NT threads that work on the row.  hist is zero on entry and after.
+// ---------------------------------------------------------------------------------------------------
+// First the maxima of the vectors (or, by_vectors == 0, all sampled elements) are binned by the top bits of their
+// order-preserving key, which gives a floor with enough of them above it; a second, linear histogram over
+// [floor, largest] resolves the wanted rank.  With exchangeable entries a vector of G elements has its maximum above t
+// with probability 1 - (1 - p(t))^G, which is how the host translates the wanted share of entries into a rank
+// among maxima: an eighth of the work for nearly the same sharpness while few entries lie above the threshold.
+// tau0 only steers how many candidates there are; the result is exact whatever it is.
+//
+// The candidates' bins are 1 .. kSiftBins - 1; bin 0 takes what is no candidate.  bin(y) is the smaller of two rising lines
+// over y - tau0, the first of which spends kBinsLow bins on the stretch up to a value that the K-th largest hardly
+// ever exceeds (the same sample says where that is): the threshold's bin then holds two or three members.  Any
+// rising function would do: a higher bin never holds a smaller value.
+struct SiftBinning {
+  float tau0, s1, s2, c2;
+  __device__ __forceinline__ float at(float y) const {
+    const float d = __fsub_rn(y, tau0);
+    return fminf(__fmaf_rn(d, s1, 1.0f), __fmaf_rn(d, s2, c2));
+  }
+};
+
+__device__ __forceinline__ int sample_element(const SiftCfg& cfg, int vec, int ev, int V) {
+  const int piece = cfg.piece_vecs == 4 ? vec >> 2 : vec, k = cfg.piece_vecs == 4 ? vec & 3 : 0;
+  const int at = piece * cfg.piece_stride + k * ev;
+  return piece < kSiftPieces && k * ev < cfg.piece_stride && at < V ? at : -1;
+}
+
+template <int DTYPE, bool HAS_U, bool HAS_T, int NT>
+__device__ __forceinline__ SiftBinning sift_sample(const RowArgs& a, const SiftCfg& cfg, SiftShared& sm, uint32_t* hist,
+                                                   const char* c_row, const char* u_row, int tid, int bar) {
+  constexpr int EV = SiftTraits<DTYPE>::kVec, ES = SiftTraits<DTYPE>::kElem;
+  constexpr int NV = 4 * kSiftPieces / NT;  // vectors per thread
+  const int lane = tid & 31, warp = tid >> 5;
+  const float neg_inf = __int_as_float(0xff800000), lowest = -3.402823466e38f;
+  const uint64_t s2 = pack2(a.s, a.s), t2 = pack2(a.inv_T, a.inv_T);
+  float v[NV][EV];  // v[j][0]: the vector's maximum (by_vectors), or the vector's elements
+  uint32_t have = 0;
+  uint4 c[NV], u[NV];
+#pragma unroll
+  for (int j = 0; j < NV; ++j) {
+    const int e = sample_element(cfg, tid + j * NT, EV, a.V);
+    c[j] = u[j] = make_uint4(0u, 0u, 0u, 0u);
+    if (e >= 0) {
+      have |= 1u << j;
+      c[j] = __ldg(reinterpret_cast<const uint4*>(c_row + (size_t)e * ES));
+      if (HAS_U) u[j] = __ldg(reinterpret_cast<const uint4*>(u_row + (size_t)e * ES));
+    }
+  }
+  float top = neg_inf;
+  const bool by_vectors = cfg.by_vectors != 0;
+#pragma unroll
+  for (int j = 0; j < NV; ++j) {
+    uint64_t y[EV / 2];
+    merge_vec<DTYPE, HAS_U, HAS_T>(c[j], u[j], s2, t2, y);
+    float m = neg_inf;
+#pragma unroll
+    for (int k = 0; k < EV / 2; ++k) {
+      unpack2(y[k], v[j][2 * k], v[j][2 * k + 1]);
+      m = max3(m, v[j][2 * k], v[j][2 * k + 1]);
+    }
+    const bool in = (have >> j) & 1u;
+    m = in ? canonical(m) : neg_inf;
+    top = fmaxf(top, m);
+    // an atomic with part of its lanes off runs several times slower than one with all lanes on: what is not there
+    // counts as -inf, below every threshold
+    if (by_vectors) {
+      v[j][0] = m;
+      atomicAdd(&hist[float_key(m) >> kSiftKeyShift], 1u);
+    } else {
+#pragma unroll
+      for (int k = 0; k < EV; ++k) {
+        v[j][k] = in ? canonical(v[j][k]) : neg_inf;
+        atomicAdd(&hist[float_key(v[j][k]) >> kSiftKeyShift], 1u);
+      }
+    }
+  }
+  const uint32_t warp_top = __reduce_max_sync(0xffffffffu, float_key(top));
+  if (lane == 0) atomicMax(&sm.top_key, warp_top);
+  row_sync<NT>(bar);
+  if (warp == 0) rank_search(&sm, hist, (uint32_t)cfg.rank, 0u);
+  row_sync<NT>(bar);
+  float floor_y = key_float(sm.rank_bin << kSiftKeyShift);
+  if (!(floor_y >= lowest)) floor_y = lowest;  // the edge fell on -inf or into the NaN patterns
+  const float top_y = key_float(sm.top_key);
+  const bool refine = floor_y > lowest && top_y >= floor_y && top_y <= 3.402823466e38f;
+  const float range = __fsub_rn(top_y, floor_y);
+  const float scale = (refine && range > 0.0f) ? __fdiv_rn((float)kSiftBins - 1.5f, range) : 0.0f;
+  SiftBinning bins{lowest, 0.0f, 0.0f, (float)kSiftBins};
+  if (refine) {
+    // bins 1 .. kSiftBins - 1; what lies below the floor counts in bin 0 (a negative argument converts to 0)
+#pragma unroll
+    for (int j = 0; j < NV; ++j) {
+#pragma unroll
+      for (int k = 0; k < EV; ++k) {
+        if (k > 0 && by_vectors) break;
+        const float x = v[j][k];
+        const uint32_t bin = x >= floor_y ? __float2uint_rz(__fmaf_rn(__fsub_rn(x, floor_y), scale, 1.0f)) : 0u;
+        atomicAdd(&hist[min(bin, (uint32_t)kSiftBins - 1u)], 1u);
+      }
+    }
+    row_sync<NT>(bar);
+    if (warp == 0) rank_search(&sm, hist, (uint32_t)cfg.rank, (uint32_t)cfg.rank_high);
+    row_sync<NT>(bar);
+    const float tbin = (float)sm.rank_bin, hbin = (float)sm.rank_bin2;
+    bins.tau0 = floor_y;
+    if (scale > 0.0f) {
+      const float width = __fdiv_rn(1.0f, scale);
+      // a little below the lower edge of the bin, so that rounding cannot exclude one of its members
+      if (tbin > 1.0f) bins.tau0 = __fmaf_rd(__fmul_rd(tbin - 1.0f, 0.9999f), width, floor_y);
+      const float high = __fsub_rn(__fmaf_rn(hbin, width, floor_y), bins.tau0);
+      const float rest = __fsub_rn(__fsub_rn(top_y, bins.tau0), high);
+      bins.s1 = __fdiv_rn((float)kBinsLow, fmaxf(high, width));
+      // (never the steeper line: it would undercut the first one below their crossing)
+      bins.s2 = rest > 0.0f ? fminf(__fdiv_rn((float)(kSiftBins - 2 - kBinsLow), rest), bins.s1) : 0.0f;
+      bins.c2 = __fmaf_rn(-high, bins.s2, (float)(kBinsLow + 1));
+    }
+  }
+  return bins;
+}
+
+// ---------------------------------------------------------------------------------------------------
+// sift phase
+// ---------------------------------------------------------------------------------------------------
+// Hit bits of 64 bytes per array of a lane: bit k is set when element k reaches tau0 (or is a NaN, sorted out when the
+// candidate is merged).  The sign of y - tau0 is exact (a difference rounds to zero only when it is zero) and is
+// moved in with one funnel shift per element.  Lanes start at different 16-byte pieces (`rot`), so that the eight lanes
+// served together touch different banks; the word is rotated back afterwards.
+template <int DTYPE, bool HAS_U, bool HAS_T>
+__device__ __forceinline__ uint32_t piece_hits(uint32_t c_at, uint32_t u_at, int rot, uint64_t s2, uint64_t t2, uint64_t neg_tau2) {
+  constexpr int EV = SiftTraits<DTYPE>::kVec;
+  uint32_t miss = 0;
+#pragma unroll
+  for (int j = 3; j >= 0; --j) {
+    const uint32_t off = (uint32_t)(((j + rot) & 3) << 4);
+    const uint4 c = lds128(c_at + off);
+    uint4 u = make_uint4(0u, 0u, 0u, 0u);
+    if (HAS_U) u = lds128(u_at + off);
+    uint64_t y[EV / 2];
+    merge_vec<DTYPE, HAS_U, HAS_T>(c, u, s2, t2, y);
+#pragma unroll
+    for (int k = EV / 2 - 1; k >= 0; --k) {
+      uint64_t t;
+      asm("add.rn.f32x2 %0, %1, %2;" : "=l"(t) : "l"(y[k]), "l"(neg_tau2));
+      miss = __funnelshift_l((uint32_t)(t >> 32), miss, 1);
+      miss = __funnelshift_l((uint32_t)t, miss, 1);
+    }
+  }
+  if (DTYPE != 0) return __funnelshift_l(~miss, ~miss, 8 * rot);
+  const uint32_t x = (~miss & 0xffffu) * 0x10001u;
+  return (x >> (16 - 4 * rot)) & 0xffffu;
+}
+
+// ids of the set bits of x (bit 0: id `first`), from the highest down, to the halfwords below `put`
+__device__ __forceinline__ uint32_t put_ids(uint32_t x, uint32_t first, uint32_t put) {
+  while (x != 0u) {
+    uint32_t b;
+    asm("bfind.u32 %0, %1;" : "=r"(b) : "r"(x));
+    x ^= 1u << b;
+    put -= 2u;
+    asm volatile("st.shared.u16 [%0], %1;" ::"r"(put), "h"((uint16_t)(first + b)) : "memory");
+  }
+  return put;
+}
+
+// where a warp's candidates go
+struct SiftTarget {
+  uint32_t y_at, id_at;    // shared-memory addresses of the segment's lists (of the cluster's first CTA when REMOTE)
+  uint32_t hist_at;        // of the candidates' histogram
+  uint32_t scratch_at;     // local id list (the same as id_at unless REMOTE)
+};
+
+template <bool REMOTE>
+__device__ __forceinline__ void put_f32(uint32_t at, float v) {
+  if (REMOTE) asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(at), "f"(v) : "memory");
+  else asm volatile("st.shared.f32 [%0], %1;" ::"r"(at), "f"(v) : "memory");
+}
+template <bool REMOTE>
+__device__ __forceinline__ void put_u16(uint32_t at, uint32_t v) {
+  if (REMOTE) asm volatile("st.shared::cluster.u16 [%0], %1;" ::"r"(at), "h"((uint16_t)v) : "memory");
+  else asm volatile("st.shared.u16 [%0], %1;" ::"r"(at), "h"((uint16_t)v) : "memory");
+}
+template <bool REMOTE>
+__device__ __forceinline__ void count_at(uint32_t at) {
+  if (REMOTE) asm volatile("red.relaxed.cluster.shared::cluster.add.u32 [%0], 1;" ::"r"(at) : "memory");
+  else asm volatile("red.relaxed.cta.shared::cta.add.u32 [%0], 1;" ::"r"(at) : "memory");
+}
+
+// One unit: `valid` elements of it belong to the segment; element 0 has id `rel` in the segment's numbering, which is
+// what the list keeps plus `bias`.  n: candidates so far (cap + 1 or more: the list has run over).
+template <int DTYPE, bool HAS_U, bool HAS_T, bool REMOTE>
+__device__ __forceinline__ void sift_unit(const RowArgs& a, uint32_t c_unit, uint32_t u_unit, int valid, uint32_t rel, uint32_t bias,
+                                          uint64_t s2, uint64_t t2, const SiftBinning& bins, const SiftTarget& to, uint32_t cap,
+                                          int lane, uint32_t& n, float& vmax) {
+  constexpr int ES = SiftTraits<DTYPE>::kElem, EP = SiftTraits<DTYPE>::kPiece, EU = SiftTraits<DTYPE>::kUnit;
+  const uint64_t neg_tau2 = pack2(-bins.tau0, -bins.tau0);
+  uint32_t x0, x1 = 0;    // hits of the lane's first and second piece
+  uint32_t run = 2 * EP;  // consecutive elements of a lane
+  if (valid > EU / 2) {
+    const uint32_t at = 128u * (uint32_t)lane, swap = ((uint32_t)lane & 4u) << 4;
+    x0 = piece_hits<DTYPE, HAS_U, HAS_T>(c_unit + (at ^ swap), u_unit + (at ^ swap), lane & 3, s2, t2, neg_tau2);
+    x1 = piece_hits<DTYPE, HAS_U, HAS_T>(c_unit + (at ^ swap ^ 64u), u_unit + (at ^ swap ^ 64u), lane & 3, s2, t2, neg_tau2);
+    if (swap) {
+      const uint32_t x = x0;
+      x0 = x1;
+      x1 = x;
+    }
+  } else {
+    run = EP;
+    x0 = piece_hits<DTYPE, HAS_U, HAS_T>(c_unit + 64u * (uint32_t)lane, u_unit + 64u * (uint32_t)lane, (lane >> 1) & 3, s2, t2, neg_tau2);
+  }
+  if (DTYPE == 0) {
+    x0 |= x1 << 16;
+    x1 = 0;
+  }
+  if (valid < EU) {
+    const int left = valid - lane * (int)run;
+    x0 = left >= 32 ? x0 : left > 0 ? x0 & ((1u << left) - 1u) : 0u;
+    x1 = left >= 64 ? x1 : left > 32 ? x1 & ((1u << (left - 32)) - 1u) : 0u;
+  }
+  const uint32_t inc = scan_incl((uint32_t)(__popc(x0) + __popc(x1)), lane);
+  const uint32_t total = __shfl_sync(0xffffffffu, inc, 31);
+  if (n + total > cap) {
+    n = cap + 1u;
+    return;
+  }
+  // ids, from the lane's highest one down
+  {
+    const uint32_t first = rel + (uint32_t)lane * run;
+    uint32_t put = to.scratch_at + 2u * (n + inc);
+    if (DTYPE != 0) put = put_ids(x1, first + 32u, put);
+    put_ids(x0, first, put);
+  }
+  __syncwarp();
+  // candidates: merged, binned and kept
+  const uint32_t c_rel = c_unit - rel * (uint32_t)ES, u_rel = u_unit - rel * (uint32_t)ES;
+  for (uint32_t i = (uint32_t)lane; i < ((total + 31u) & ~31u); i += 32u) {
+    const bool in = i < total;
+    const uint32_t k = n + min(i, total - 1u);
+    const uint32_t id = lds16(to.scratch_at + 2u * k);
+    const float y = merge_entry<DTYPE, HAS_U, HAS_T>(c_rel + id * (uint32_t)ES, u_rel + id * (uint32_t)ES, a.s, a.inv_T);
+    const uint32_t bin = in ? min(__float2uint_rz(bins.at(y)), (uint32_t)kSiftBins - 1u) : 0u;
+    count_at<REMOTE>(to.hist_at + 4u * bin);
+    vmax = fmaxf(vmax, y);
+    if (in) {
+      put_f32<REMOTE>(to.y_at + 4u * k, y);
+      if (REMOTE) put_u16<true>(to.id_at + 2u * k, id + bias);
+    }
+  }
+  n += total;
+}
+
+// exp(y - m) with the rounding of the difference compensated (exp_diff without its case for y = -inf)
+__device__ __forceinline__ float exp_diff_finite(float y, float m) {
+  const float t = __fsub_rn(y, m);
+  const float bb = __fsub_rn(t, y);                                                // ~ -m
+  const float err = __fadd_rn(__fsub_rn(y, __fsub_rn(t, bb)), __fsub_rn(-m, bb));  // (y - m) - t, exact
+  const float e = expf(t);
+  return __fmaf_rn(e, err, e);
+}
+
+// ---------------------------------------------------------------------------------------------------
+// finish phase, by the NW warps that work on the row
+// ---------------------------------------------------------------------------------------------------
+// Warp w holds the candidates of `per_warp` consecutive segments in lists of seg_cap entries each, ids relative to
+// the warp's first id.  Starts with a barrier.  Returns false when the row has to be redone; the histogram is zero
+// again and the counters are reset either way.
+template <int NW>
+__device__ __forceinline__ bool finish_row(const RowArgs& a, const SiftCfg& cfg, SiftShared& sm, float* list_y, uint16_t* list_id,
+                                           const uint32_t* seg_n, int per_warp, const SiftBinning& bins, int row, int pos, int iter,
+                                           int draft, int tid, int bar) {
+  constexpr int NT = NW * 32;
+  const int lane = tid & 31, warp = tid >> 5;
+  const uint32_t kcap = (uint32_t)a.kcap;
+  const uint32_t below = (1u << lane) - 1u;
+  row_sync<NT>(bar);
+  if (warp == 0) rank_search(&sm, sm.hist, kcap, 0u);
+  if (tid == NT - 1) {
+    // the row's own random number, needed at the end
+    const Philox4 r = philox4x32_10((uint32_t)pos, (uint32_t)(a.seq_base + row / a.W), (uint32_t)iter, (uint32_t)a.purpose, a.seed_lo,
+                                    a.seed_hi);
+    sm.rnd_lo = r.x0;
+    sm.rnd_hi = r.x1;
+    sm.ptok = 0.0f;
+  }
+  const float vmax = key_float(sm.max_key);
+  const bool over = sm.over != 0u;
+  row_sync<NT>(bar);
+  const uint32_t tbin = sm.rank_bin, need = kcap - sm.rank_above, nbin = sm.rank_count;
+  if (tid == 0) {
+    sm.max_key = 0u;
+    sm.top_key = 0u;
+    sm.over = 0u;
+  }
+  // fewer than kcap candidates, a threshold bin too crowded for the ranking, or no finite maximum
+  if (over || tbin == 0u || nbin > (uint32_t)kMemberCap || !(vmax <= 3.402823466e38f)) {
+    row_sync<NT>(bar);
+    return false;
+  }
+  const size_t first_seg = (size_t)warp * per_warp;
+  float* const my_y = list_y + first_seg * cfg.seg_cap;
+  uint16_t* const my_id = list_id + first_seg * cfg.seg_cap;
+  const int id0 = warp * per_warp * cfg.seg_len;
+  // ---- the threshold bin's members
+  {
+    const float lo = (float)tbin, hi = tbin == (uint32_t)kSiftBins - 1u ? __int_as_float(0x7f800000) : (float)(tbin + 1u);
+    for (int g = 0; g < per_warp; ++g) {
+      const uint32_t n = seg_n[first_seg + g];
+      const float* const y_g = my_y + g * cfg.seg_cap;
+#pragma unroll 2
+      for (uint32_t i = (uint32_t)lane; i < n; i += 32u) {
+        const float y = y_g[i], x = bins.at(y);
+        if (x >= lo && x < hi) sm.member[atomicAdd(&sm.members, 1)] = SiftMember{y, id0 + (int32_t)my_id[g * cfg.seg_cap + i]};
+      }
+    }
+  }
+  row_sync<NT>(bar);
+  // the `need`-th of them by (y descending, id ascending) is the last survivor
+  float thr_y;
+  int thr_id;
+  if (nbin <= 32u) {
+    // every warp ranks them for itself, a lane per member
+    SiftMember me{0.0f, 0};
+    if (lane < (int)nbin) me = sm.member[lane];
+    uint32_t ahead = 0;
+    for (int x = 0; x < (int)nbin; ++x) {
+      const float oy = __shfl_sync(0xffffffffu, me.y, x);
+      const int oid = __shfl_sync(0xffffffffu, me.id, x);
+      ahead += (oy > me.y || (oy == me.y && oid < me.id)) ? 1u : 0u;
+    }
+    const int who = __ffs((int)__ballot_sync(0xffffffffu, lane < (int)nbin && ahead == need - 1u)) - 1;
+    thr_y = __shfl_sync(0xffffffffu, me.y, who);
+    thr_id = __shfl_sync(0xffffffffu, me.id, who);
+  } else {
+    // a warp per member, a lane per rival
+    for (uint32_t x = (uint32_t)warp; x < nbin; x += NW) {
+      const SiftMember me = sm.member[x];
+      uint32_t ahead = 0;
+      for (uint32_t z = (uint32_t)lane; z < nbin; z += 32u) {
+        const SiftMember o = sm.member[z];
+        ahead += (o.y > me.y || (o.y == me.y && o.id < me.id)) ? 1u : 0u;
+      }
+      ahead = __reduce_add_sync(0xffffffffu, ahead);
+      if (lane == 0 && ahead == need - 1u) {
+        sm.thr_y = me.y;
+        sm.thr_id = me.id;
+      }
+    }
+    row_sync<NT>(bar);
+    thr_y = sm.thr_y;
+    thr_id = sm.thr_id;
+  }
+  // ---- survivors: exponentials and ids to the front of the warp's lists, their number and sum
+  const int thr_rel = thr_id - id0;
+  uint32_t cnt = 0;
+  float z = 0.0f;
+  for (int g = 0; g < per_warp; ++g) {
+    const uint32_t n = seg_n[first_seg + g];
+    const float* const y_g = my_y + g * cfg.seg_cap;
+    const uint16_t* const id_g = my_id + g * cfg.seg_cap;
+#pragma unroll 2
+    for (uint32_t i0 = 0; i0 < n; i0 += 32u) {
+      const uint32_t i = i0 + (uint32_t)lane;
+      float y = __int_as_float(0xff800000);
+      int id = 0x7fffffff;
+      if (i < n) {
+        y = y_g[i];
+        id = (int)id_g[i];
+      }
+      const bool alive = y > thr_y || (y == thr_y && id <= thr_rel);
+      const float e = exp_diff_finite(y, vmax);
+      const uint32_t votes = __ballot_sync(0xffffffffu, alive);
+      __syncwarp();  // every lane has read its entry: what follows overwrites entries up to this group's
+      if (alive) {
+        const uint32_t at = cnt + (uint32_t)__popc(votes & below);
+        my_y[at] = e;
+        my_id[at] = (uint16_t)id;
+        z += e;
+      }
+      cnt += (uint32_t)__popc(votes);
+    }
+  }
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1) z += __shfl_xor_sync(0xffffffffu, z, d);
+  if (lane == 0) {
+    sm.wcnt[warp] = cnt;
+    sm.wz[warp] = z;
+  }
+  row_sync<NT>(bar);
+  for (uint32_t x = (uint32_t)tid; x < nbin; x += NT) sm.member[x] = SiftMember{0.0f, 0};  // the histogram's words again
+  if (tid == 0) sm.members = 0;
+  const uint32_t cw = lane < NW ? sm.wcnt[lane] : 0u;
+  const uint32_t before = __reduce_add_sync(0xffffffffu, lane < warp ? cw : 0u);
+  if (__reduce_add_sync(0xffffffffu, cw) != kcap) return false;  // cannot happen; the result stays exact anyway
+  float Z = sm.wz[lane & (NW - 1)];
+#pragma unroll
+  for (int d = NW / 2; d > 0; d >>= 1) Z += __shfl_xor_sync(0xffffffffu, Z, d);
+  const float inv_Z = __fdiv_rn(1.0f, Z);  // p = e / Z within 1.5 ulp
+  // ---- output and fixed-point weights
+  int32_t* const out_ids = a.out_ids + (size_t)row * kcap + before;
+  float* const out_vals = a.out_vals + (size_t)row * kcap + before;
+  uint64_t wsum = 0;
+#pragma unroll 2
+  for (uint32_t i = (uint32_t)lane; i < cnt; i += 32u) {
+    const float p = __fmul_rn(my_y[i], inv_Z);
+    const int id = id0 + (int)my_id[i];
+    out_ids[i] = id;
+    out_vals[i] = p;
+    wsum += fixed_weight(p);
+    if (id == draft) sm.ptok = p;
+  }
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1) {
+    const uint32_t lo = __shfl_xor_sync(0xffffffffu, (uint32_t)wsum, d), hi = __shfl_xor_sync(0xffffffffu, (uint32_t)(wsum >> 32), d);
+    wsum += (uint64_t)lo | ((uint64_t)hi << 32);
+  }
+  if (lane == 0) sm.wtot[warp] = wsum;
+  row_sync<NT>(bar);
+  // ---- the row's own draw: fixed-point inverse CDF in ascending id order.  Every warp finds out whether the draw
+  // falls to it; the one that holds it gives each lane a run of its survivors.
+  const uint64_t x = lane < NW ? sm.wtot[lane] : 0ull;
+  uint64_t xi = x;
+#pragma unroll
+  for (int d = 1; d < NW; d <<= 1) {
+    const uint64_t o = shfl_up_u64(xi, d);
+    if (lane >= d) xi += o;
+  }
+  const uint64_t total = shfl_u64(xi, NW - 1);
+  const uint64_t t = __umul64hi((uint64_t)sm.rnd_lo | ((uint64_t)sm.rnd_hi << 32), total);
+  uint64_t lo = shfl_u64(xi - x, warp);
+  const uint64_t hi = shfl_u64(xi, warp);
+  if (total == 0ull) {  // all weights rounded to zero: the first survivor
+    if (lane == 0 && before == 0u && cnt > 0u) {
+      a.out_cnt[row] = (int)kcap;
+      a.scratch[row] = RowScratch{sm.ptok, id0 + (int32_t)my_id[0], __fmul_rn(my_y[0], inv_Z), 0};
+    }
+  } else if (t >= lo && t < hi) {
+    const uint32_t run = (cnt + 31u) / 32u;
+    const uint32_t beg = min((uint32_t)lane * run, cnt), end = min(beg + run, cnt);
+    uint64_t own = 0;
+    for (uint32_t i = beg; i < end; ++i) own += fixed_weight(__fmul_rn(my_y[i], inv_Z));
+    uint64_t inc = own;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const uint64_t o = shfl_up_u64(inc, d);
+      if (lane >= d) inc += o;
+    }
+    lo += inc - own;
+    if (t >= lo && t < lo + own) {
+      uint32_t i = beg;
+      float p;
+      for (;; ++i) {  // ends before `end`: the run's weights sum to more than t - lo
+        p = __fmul_rn(my_y[i], inv_Z);
+        lo += fixed_weight(p);
+        if (t < lo || i + 1u >= end) break;
+      }
+      a.out_cnt[row] = (int)kcap;
+      a.scratch[row] = RowScratch{sm.ptok, id0 + (int32_t)my_id[i], p, 0};
+    }
+  }
+  return true;
+}
+
+// row_generic as a call of its own: it is rarely needed and its registers and code stay out of the hot loops.
+template <int DTYPE, int NT>
+__device__ __noinline__ void sift_redo(const RowArgs& a, int row, int tid, GenericSmem& sm) {
+  row_generic<DTYPE, NT, 0>(a, row, tid, sm, kRowStatusRedone);
+}
+
+__device__ __forceinline__ void init_shared(SiftShared& sm, int tid, int nt) {
+  for (int k = tid; k < kSiftBins / 4; k += nt) reinterpret_cast<uint4*>(sm.hist)[k] = make_uint4(0u, 0u, 0u, 0u);
+  if (tid == 0) {
+    sm.top_key = 0u;
+    sm.max_key = 0u;
+    sm.over = 0u;
+    sm.members = 0;
+  }
+}
+
+// a row and what there is to know about it
+struct SiftRow {
+  int64_t off;    // of its first logit, in elements
+  int32_t row;    // b * W + i
+  int32_t pos;    // absolute position: pos_base[b] + i
+  int32_t iter;   // iteration counter of its sequence
+  int32_t draft;  // its draft token, -1 when every row is drafted
+  bool live;      // inside its sequence's window
+};
+__device__ __forceinline__ SiftRow sift_row(const RowArgs& a, int row) {
+  SiftRow r;
+  const int b = row / a.W, i = row - b * a.W;
+  r.row = row;
+  r.off = (int64_t)b * a.stride_b + (int64_t)i * a.stride_w;
+  r.live = a.win_len == nullptr || i < a.win_len[b];
+  r.pos = (a.pos_base ? a.pos_base[b] : 0) + i;
+  r.iter = a.iteration ? a.iteration[b] : a.iteration0;
+  r.draft = a.drafts ? a.drafts[row] : -1;
+  return r;
+}
+
+// ---------------------------------------------------------------------------------------------------
+// many rows
+// ---------------------------------------------------------------------------------------------------
+struct alignas(16) StreamShared {
+  SiftRow tab[kStreamRows];                    // the CTA's live rows
+  // A unit of one of team t's rows has landed in the slot: [warp][team][slot].  A barrier of its own for every team: a
+  // parity wait tells a phase from its neighbours only, so each barrier is waited on by one warp, phase after phase.
+  uint64_t full[kTeamWarps * kMaxTeams * kMaxSlots];
+  uint32_t used[kTeamWarps * kMaxTeams * kMaxSlots];  // copies issued for that barrier so far
+  uint32_t seg_n[kMaxTeams * kTeamWarps];      // candidates per segment
+  int32_t redo[kStreamRows];                   // rows the single pass could not finish (redone at the end)
+  int n_live, n_redo, abort;
+};
+// shared memory: StreamShared | SiftShared x teams | list values | list ids | rings
+__host__ __device__ inline size_t sift_stream_rings(int teams, int seg_cap) {
+  const size_t b = sizeof(StreamShared) + teams * (sizeof(SiftShared) + (size_t)kTeamWarps * seg_cap * 6);
+  return (b + 127) & ~(size_t)127;
+}
+__host__ __device__ inline size_t sift_stream_smem(int teams, int seg_cap, int slots, bool has_u) {
+  return sift_stream_rings(teams, seg_cap) + (size_t)kTeamWarps * slots * kUnitBytes * (has_u ? 2 : 1);
+}
+
+// bounded wait that also ends when another warp of the CTA has given up.  The wait stays suspended in hardware for up to
+// a few microseconds at a time: a waiting warp spends next to no issue slots.
+__device__ __forceinline__ bool sift_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
+  if (mbar_try_wait(bar, parity)) return true;
+  const long long t0 = clock64();
+  for (uint32_t i = 0; i < kSpinLimit; ++i) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(smem_u32(bar)), "r"(parity), "r"(4000u)
+        : "memory");
+    if (ok) return true;
+    if (*abort_flag != 0 || clock64() - t0 > kSpinCycles) break;
+  }
+  return false;
+}
+
+template <int DTYPE, bool HAS_U, bool HAS_T>
+__global__ void __launch_bounds__(kTeamThreads * kMaxTeams, 1)
+rows_stream_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ SiftCfg cfg) {
+  constexpr int ES = SiftTraits<DTYPE>::kElem, EU = SiftTraits<DTYPE>::kUnit;
+  constexpr uint32_t kSlot = kUnitBytes * (HAS_U ? 2u : 1u);
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  StreamShared& st = *reinterpret_cast<StreamShared*>(smem_raw);
+  const int teams = cfg.teams, slots = cfg.slots;
+  const int team = (int)threadIdx.x / kTeamThreads;
+  const int tid = (int)threadIdx.x % kTeamThreads, lane = tid & 31, warp = tid >> 5, bar = 1 + team;
+  SiftShared* const team_sm = reinterpret_cast<SiftShared*>(smem_raw + sizeof(StreamShared));
+  SiftShared& sm = team_sm[team];
+  float* const lists = reinterpret_cast<float*>(team_sm + teams);
+  float* const list_y = lists + (size_t)team * kTeamWarps * cfg.seg_cap;
+  uint16_t* const list_id = reinterpret_cast<uint16_t*>(lists + (size_t)teams * kTeamWarps * cfg.seg_cap) + (size_t)team * kTeamWarps * cfg.seg_cap;
+  unsigned char* const ring = smem_raw + sift_stream_rings(teams, cfg.seg_cap) + (size_t)warp * slots * kSlot;
+  init_shared(sm, tid, kTeamThreads);
+  if (threadIdx.x < kTeamWarps * kMaxTeams * kMaxSlots) {
+    mbar_init(&st.full[threadIdx.x], 1);
+    st.used[threadIdx.x] = 0;
+  }
+  if (threadIdx.x == 0) {
+    st.n_redo = 0;
+    st.abort = 0;
+  }
+  fence_barrier_init();
+  grid_dependency_wait();  // shared memory only up to here; a launch that overlaps the previous kernel waits for its end
+  // ---- the CTA's rows: row_begin + blockIdx.x, + gridDim.x, ... (at most kStreamRows).  Rows beyond their sequence's window
+  // length get their empty result; the others go into a table, so that no warp reads global memory for them later.
+  if (threadIdx.x < 32) {
+    int n = 0;
+    for (int k0 = 0; k0 < kStreamRows; k0 += 32) {
+      const int64_t row = (int64_t)cfg.row_begin + blockIdx.x + (int64_t)(k0 + lane) * gridDim.x;
+      SiftRow r;
+      r.live = false;
+      if (row < cfg.row_end) {
+        r = sift_row(a, (int)row);
+        if (!r.live) {
+          a.out_cnt[row] = 0;
+          a.scratch[row] = RowScratch{0.0f, -1, 0.0f, 0};
+        }
+      }
+      const uint32_t votes = __ballot_sync(0xffffffffu, r.live);
+      if (r.live) st.tab[n + __popc(votes & ((1u << lane) - 1u))] = r;
+      n += __popc(votes);
+    }
+    if (lane == 0) st.n_live = n;
+  }
+  __syncthreads();
+  const int n_live = st.n_live;
+  const int seg0 = warp * cfg.seg_len;
+  const int seg_n = min(max(a.V - seg0, 0), cfg.seg_len);  // ids of this warp's segment
+  const int units = (seg_n + EU - 1) / EU;
+  // Copies go through the ring of the warp's segment in order: the units of the segment for row 0, row 1, ...; team t takes
+  // rows t, t + teams, ...  Whoever has worked a unit through asks for the copy that goes into its slot next.
+  auto issue = [&](int k, int unit, int slot) {
+    if (unit >= units) {
+      k += unit / units;
+      unit = unit % units;
+    }
+    if (k >= n_live) return;
+    const uint32_t bytes = (uint32_t)min(seg_n - unit * EU, EU) * ES;
+    const int64_t off = st.tab[k].off + seg0 + (int64_t)unit * EU;
+    unsigned char* const dst = ring + (size_t)slot * kSlot;
+    const int x = (warp * kMaxTeams + k % teams) * kMaxSlots + slot;
+    ++st.used[x];
+    mbar_arrive_expect_tx(&st.full[x], bytes * (HAS_U ? 2u : 1u));
+    bulk_g2s(dst, row_ptr(a.cond, DTYPE, off), bytes, &st.full[x]);
+    if (HAS_U) bulk_g2s(dst + kUnitBytes, row_ptr(a.uncond, DTYPE, off), bytes, &st.full[x]);
+  };
+  if (team == 0 && lane == 0 && units > 0) {
+    for (int k = 0; k < slots; ++k) issue(0, k, k);
+  }
+  const uint64_t s2 = pack2(a.s, a.s), t2 = pack2(a.inv_T, a.inv_T);
+  SiftTarget to;
+  to.y_at = smem_u32(list_y + warp * cfg.seg_cap);
+  to.id_at = to.scratch_at = smem_u32(list_id + warp * cfg.seg_cap);
+  to.hist_at = smem_u32(sm.hist);
+  const uint32_t ring_at = smem_u32(ring), cap = (uint32_t)cfg.seg_cap;
+  volatile int* const abort_flag = &st.abort;
+  uint64_t* const full = st.full + (warp * kMaxTeams + team) * kMaxSlots;
+  uint32_t phase = 0;  // bit s: parity of the next phase of full[s]
+  for (int k = team; k < n_live; k += teams) {
+    // from the CTA's last row on, the verification grid may be scheduled (it waits for this grid's end)
+    if (k == n_live - 1) allow_dependent_launch();
+    const int64_t off = st.tab[k].off;
+    const SiftBinning bins = sift_sample<DTYPE, HAS_U, HAS_T, kTeamThreads>(
+        a, cfg, sm, sm.hist, static_cast<const char*>(row_ptr(a.cond, DTYPE, off)),
+        HAS_U ? static_cast<const char*>(row_ptr(a.uncond, DTYPE, off)) : nullptr, tid, bar);
+    uint32_t n = 0;
+    float vmax = __int_as_float(0xff800000);
+    bool ok = *abort_flag == 0;
+    int slot = (k * units) % slots;
+    for (int unit = 0; unit < units; ++unit) {
+      if (ok) ok = sift_wait(&full[slot], (phase >> slot) & 1u, abort_flag);
+      if (!ok) break;
+      phase ^= 1u << slot;
+      const uint32_t c_unit = ring_at + (uint32_t)slot * kSlot;
+      sift_unit<DTYPE, HAS_U, HAS_T, false>(a, c_unit, c_unit + kUnitBytes, seg_n - unit * EU, (uint32_t)(unit * EU), 0u, s2, t2, bins,
+                                            to, cap, lane, n, vmax);
+      __syncwarp();
+      if (lane == 0) issue(k, unit + slots, slot);
+      if (++slot == slots) slot = 0;
+    }
+    const uint32_t wmax = __reduce_max_sync(0xffffffffu, float_key(vmax));
+    if (lane == 0) {
+      st.seg_n[team * kTeamWarps + warp] = n;
+      atomicMax(&sm.max_key, wmax);
+      if (n > cap || !ok) sm.over = 1u;
+      if (!ok) *abort_flag = 1;
+    }
+    const SiftRow& r = st.tab[k];
+    if (!finish_row<kTeamWarps>(a, cfg, sm, list_y, list_id, st.seg_n + team * kTeamWarps, 1, bins, r.row, r.pos, r.iter, r.draft, tid, bar) &&
+        tid == 0) {
+      if (*abort_flag != 0) {
+        a.out_cnt[r.row] = 0;
+        a.scratch[r.row] = RowScratch{0.0f, -1, 0.0f, kRowStatusTimeout};
+      } else {
+        st.redo[atomicAdd(&st.n_redo, 1)] = r.row;
+      }
+    }
+  }
+  __syncthreads();
+  if (st.abort != 0 && lane == 0) {
+    // a wait gave up: the copies in flight have to land (the wait is bounded) before the CTA may go
+    for (int s = 0; s < slots; ++s) {
+      const uint32_t u = st.used[(warp * kMaxTeams + team) * kMaxSlots + s];
+      if (u > 0) mbar_wait(&full[s], (u - 1u) & 1u);
+    }
+  }
+  // ---- rows the single pass could not finish: the exact any-shape path from global memory (rare)
+  const int n_redo = st.n_redo;
+  for (int x = 0; x < n_redo; ++x) {
+    GenericSmem& gs = *reinterpret_cast<GenericSmem*>(team_sm);
+    if (teams == 3) sift_redo<DTYPE, 3 * kTeamThreads>(a, st.redo[x], (int)threadIdx.x, gs);
+    else if (teams == 2) sift_redo<DTYPE, 2 * kTeamThreads>(a, st.redo[x], (int)threadIdx.x, gs);
+    else sift_redo<DTYPE, kTeamThreads>(a, st.redo[x], (int)threadIdx.x, gs);
+  }
+}
+
+// ---------------------------------------------------------------------------------------------------
+// few rows
+// ---------------------------------------------------------------------------------------------------
+struct alignas(16) ClusterShared {
+  SiftShared row;                                // the first CTA's: histogram of the candidates, finish phase
+  uint32_t hist_s[kSiftBins];                    // the sample's histogram
+  uint64_t full[kClusterWarps];                  // a warp's segment has landed
+  uint32_t seg_n[kClusterWarps * kMaxCluster];   // candidates per segment (the first CTA's)
+  uint32_t lost;                                 // a bounded wait of the cluster gave up (the first CTA's)
+};
+// shared memory: ClusterShared | list values | list ids | local ids | cond | uncond.  Only the cluster's first CTA uses the
+// lists (one per segment of the row).
+__host__ __device__ inline size_t sift_cluster_lists(const SiftCfg& cfg, int n_cta) {
+  const size_t segs = (size_t)kClusterWarps * n_cta;
+  const size_t b = sizeof(ClusterShared) + segs * cfg.seg_cap * 6 + (n_cta > 1 ? (size_t)kClusterWarps * cfg.seg_cap * 2 : 0);
+  return (b + 127) & ~(size_t)127;
+}
+__host__ __device__ inline size_t sift_cluster_stage(const SiftCfg& cfg, int elem_bytes) {  // one array of one segment
+  return ((size_t)cfg.seg_len * elem_bytes + kUnitBytes / 2 - 1) & ~(size_t)(kUnitBytes / 2 - 1);
+}
+__host__ __device__ inline size_t sift_cluster_smem(const SiftCfg& cfg, int n_cta, int elem_bytes, bool has_u) {
+  return sift_cluster_lists(cfg, n_cta) + kClusterWarps * sift_cluster_stage(cfg, elem_bytes) * (has_u ? 2 : 1);
+}
+
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ uint32_t cluster_size() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+// the shared-memory address of `p` in the cluster's first CTA
+__device__ __forceinline__ uint32_t in_first_cta(const void* p) {
+  uint32_t at;
+  asm("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(at) : "r"(smem_u32(p)));
+  return at;
+}
+
+template <int DTYPE, bool HAS_U, bool HAS_T>
+__global__ void __launch_bounds__(kClusterWarps * 32, 1)
+rows_cluster_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ SiftCfg cfg) {
+  constexpr int NT = kClusterWarps * 32;
+  constexpr int ES = SiftTraits<DTYPE>::kElem, EU = SiftTraits<DTYPE>::kUnit;
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  ClusterShared& sm = *reinterpret_cast<ClusterShared*>(smem_raw);
+  const uint32_t crank = cluster_rank(), csize = cluster_size();
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  float* const list_y = reinterpret_cast<float*>(smem_raw + sizeof(ClusterShared));
+  uint16_t* const list_id = reinterpret_cast<uint16_t*>(list_y + kClusterWarps * csize * cfg.seg_cap);
+  uint16_t* const local_id = list_id + kClusterWarps * csize * cfg.seg_cap;
+  const size_t stage_bytes = sift_cluster_stage(cfg, ES);
+  unsigned char* const stage = smem_raw + sift_cluster_lists(cfg, (int)csize) + (size_t)warp * stage_bytes * (HAS_U ? 2 : 1);
+  const int row = (int)(blockIdx.x / csize);
+  const uint64_t s2 = pack2(a.s, a.s), t2 = pack2(a.inv_T, a.inv_T);
+  init_shared(sm.row, tid, NT);
+  for (int k = tid; k < kSiftBins / 4; k += NT) reinterpret_cast<uint4*>(sm.hist_s)[k] = make_uint4(0u, 0u, 0u, 0u);
+  if (tid < kClusterWarps) mbar_init(&sm.full[tid], 1);
+  if (tid == 0) sm.lost = 0u;
+  fence_barrier_init();
+  __syncthreads();
+  cluster_arrive();        // from here on the first CTA's histogram and lists are ready for the others
+  grid_dependency_wait();  // shared memory only up to here
+  allow_dependent_launch();
+  const SiftRow r = sift_row(a, row);
+  if (!r.live) {  // the whole cluster
+    if (crank == 0 && tid == 0) {
+      a.out_cnt[row] = 0;
+      a.scratch[row] = RowScratch{0.0f, -1, 0.0f, 0};
+    }
+    __syncwarp();
+    cluster_wait();
+    return;
+  }
+  const char* const c_row = static_cast<const char*>(row_ptr(a.cond, DTYPE, r.off));
+  const char* const u_row = HAS_U ? static_cast<const char*>(row_ptr(a.uncond, DTYPE, r.off)) : nullptr;
+  const int seg = (int)crank * kClusterWarps + warp;
+  const int seg0 = seg * cfg.seg_len;
+  const int seg_n = min(max(a.V - seg0, 0), cfg.seg_len);
+  const int units = (seg_n + EU - 1) / EU;
+  unsigned char* const u_stage = stage + stage_bytes;
+  bool copied = seg_n > 0;
+#ifdef SJD_TEST_DROP_COPY
+  // test builds only: one warp's copies are never issued, so that the wait for them runs out and the time-out path
+  // (status instead of a hang) can be watched
+  if (warp == SJD_TEST_DROP_COPY) copied = false;
+#endif
+  if (copied && lane == 0) {
+    const uint32_t bytes = (uint32_t)seg_n * ES;
+    mbar_arrive_expect_tx(&sm.full[warp], bytes * (HAS_U ? 2u : 1u));
+    bulk_g2s(stage, c_row + (size_t)seg0 * ES, bytes, &sm.full[warp]);
+    if (HAS_U) bulk_g2s(u_stage, u_row + (size_t)seg0 * ES, bytes, &sm.full[warp]);
+  }
+  __syncwarp();
+  // every CTA of the cluster finds the threshold for itself: the sample is small, an exchange would cost more
+  const SiftBinning bins = sift_sample<DTYPE, HAS_U, HAS_T, NT>(a, cfg, sm.row, sm.hist_s, c_row, u_row, tid, 0);
+  SiftTarget to;
+  to.y_at = in_first_cta(list_y + (size_t)seg * cfg.seg_cap);
+  to.id_at = in_first_cta(list_id + (size_t)seg * cfg.seg_cap);
+  to.hist_at = in_first_cta(sm.row.hist);
+  to.scratch_at = smem_u32(csize > 1 ? local_id + (size_t)warp * cfg.seg_cap : list_id + (size_t)seg * cfg.seg_cap);
+  const uint32_t cap = (uint32_t)cfg.seg_cap;
+  const uint32_t bias = (uint32_t)((seg % (int)csize) * cfg.seg_len);  // ids are kept relative to the finishing warp's first one
+  uint32_t n = 0;
+  float vmax = __int_as_float(0xff800000);
+  cluster_wait();  // every CTA of the cluster has begun
+  const bool ok = seg_n == 0 || mbar_wait(&sm.full[warp], 0u);
+  if (ok) {
+    const uint32_t c_at = smem_u32(stage), u_at = smem_u32(u_stage);
+    for (int k = 0; k < units; ++k)
+      sift_unit<DTYPE, HAS_U, HAS_T, true>(a, c_at + (uint32_t)k * kUnitBytes, u_at + (uint32_t)k * kUnitBytes, seg_n - k * EU,
+                                           (uint32_t)(k * EU), bias, s2, t2, bins, to, cap, lane, n, vmax);
+  }
+  __syncwarp();
+  const uint32_t wmax = __reduce_max_sync(0xffffffffu, float_key(vmax));
+  if (lane == 0) {
+    const uint32_t n_at = in_first_cta(&sm.seg_n[seg]), max_at = in_first_cta(&sm.row.max_key);
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(n_at), "r"(n) : "memory");
+    asm volatile("red.relaxed.cluster.shared::cluster.max.u32 [%0], %1;" ::"r"(max_at), "r"(wmax) : "memory");
+    if (n > cap) asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(in_first_cta(&sm.row.over)), "r"(1u) : "memory");
+    if (!ok) asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(in_first_cta(&sm.lost)), "r"(1u) : "memory");
+  }
+  if (!ok && copied) mbar_wait(&sm.full[warp], 0u);  // bounded: no copy of this CTA outlives it
+  __syncwarp();
+  cluster_arrive();
+  cluster_wait();
+  if (crank != 0) return;
+  if (sm.lost != 0u) {
+    if (tid == 0) {
+      a.out_cnt[row] = 0;
+      a.scratch[row] = RowScratch{0.0f, -1, 0.0f, kRowStatusTimeout};
+    }
+    return;
+  }
+  if (!finish_row<kClusterWarps>(a, cfg, sm.row, list_y, list_id, sm.seg_n, (int)csize, bins, row, r.pos, r.iter, r.draft, tid, 0))
+    sift_redo<DTYPE, NT>(a, row, tid, *reinterpret_cast<GenericSmem*>(sm.hist_s));
+}
+
+}  // namespace sjd

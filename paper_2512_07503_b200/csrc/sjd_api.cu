@@ -14,6 +14,7 @@
 #include "row_kernels.cuh"
 #include "rows_pipeline.cuh"
 #include "rows_ranges.cuh"
+#include "rows_sift.cuh"
 #include "verify_kernel.cuh"
 #include "advance_kernel.cuh"
 
@@ -222,17 +223,24 @@ bool make_range_map(CUtensorMap* map, const void* base, const sjd_params* P, con
 // an event or a copy this is an ordinary launch.
 template <typename... KArgs, typename... Args>
 cudaError_t launch_after(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, bool dependent,
-                         Args&&... args) {
+                         int cluster, Args&&... args) {
   cudaLaunchConfig_t lc = {};
   lc.gridDim = grid;
   lc.blockDim = block;
   lc.dynamicSmemBytes = smem;
   lc.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchAttribute attr[2];
   lc.attrs = attr;
-  lc.numAttrs = dependent ? 1 : 0;
+  if (dependent) {
+    attr[lc.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[lc.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (cluster > 1) {
+    attr[lc.numAttrs].id = cudaLaunchAttributeClusterDimension;
+    attr[lc.numAttrs].val.clusterDim.x = (unsigned)cluster;
+    attr[lc.numAttrs].val.clusterDim.y = 1;
+    attr[lc.numAttrs++].val.clusterDim.z = 1;
+  }
   return cudaLaunchKernelEx(&lc, kern, std::forward<Args>(args)...);
 }
 
@@ -249,7 +257,7 @@ cudaError_t launch_ranges_as(const sjd::RowArgs& ra, const sjd::RangeCfg& cfg, c
   static sjd::DeviceOnce configured;  // per instantiation
   const cudaError_t e = allow_large_smem(kern, configured, (int)kSmemLimit);
   if (e != cudaSuccess) return e;
-  return launch_after(kern, dim3((unsigned)grid), dim3((8 + kRangeFinisherWarps + kSamplerWarps + 1) * 32), smem, st, true, ra,
+  return launch_after(kern, dim3((unsigned)grid), dim3((8 + kRangeFinisherWarps + kSamplerWarps + 1) * 32), smem, st, true, 1, ra,
                       cfg, mc, mu);
 }
 
@@ -275,7 +283,122 @@ cudaError_t launch_pipeline(const sjd::RowArgs& ra, const sjd::PipeCfg& cfg, siz
   static sjd::DeviceOnce configured;  // per instantiation
   const cudaError_t e = allow_large_smem(kern, configured, (int)kSmemLimit);
   if (e != cudaSuccess) return e;
-  return launch_after(kern, dim3((unsigned)grid), dim3((kFilterWarps + kFinisherWarps + 1) * 32), smem, st, true, ra, cfg);
+  return launch_after(kern, dim3((unsigned)grid), dim3((kFilterWarps + kFinisherWarps + 1) * 32), smem, st, true, 1, ra, cfg);
+}
+
+// ---- the kernels that sift a row by a sampled threshold (rows_sift.cuh) ----
+// Share p of a row's entries to aim the threshold at, such that a row with exchangeable entries still has its
+// kcap candidates when the estimate is off by 4.5 standard deviations (probability below 4e-6): p - 4.5 sd(p) =
+// kcap / V.  From the n sampled elements themselves sd(p) = sqrt(p (1 - p) / n); from the maxima of N vectors of G
+// elements, of which the share q = 1 - (1 - p)^G lies above the threshold, sd(p) = sqrt(q (1 - q) / N) / (dq/dp).
+double aimed_share(double want, double N, int G, double* sd) {
+  double p = want;
+  for (int it = 0; it < 40; ++it) {
+    const double q = 1.0 - std::pow(1.0 - p, G);
+    *sd = std::sqrt(q * (1.0 - q) / N) / (G * std::pow(1.0 - p, G - 1));
+    p = want + 4.5 * *sd;
+    if (!(p < 0.9)) return 1.0;
+  }
+  return p;
+}
+
+struct SiftPlan {
+  sjd::SiftCfg cfg;
+  int cluster;  // CTAs per row; 0: the stream kernel
+  size_t smem;
+};
+
+// Segments of equal length, each with a list that holds its share of the candidates with four standard deviations of
+// the threshold's estimate and 4.5 of the segment's own count to spare.
+void cut_segments(sjd::SiftCfg* c, int V, int segs, double p, double sd) {
+  c->seg_len = (((V + segs - 1) / segs) + 7) & ~7;
+  const double mean = c->seg_len * (p + 4.0 * sd);
+  int cap = (int)(mean + 4.5 * std::sqrt(mean) + 8.0);
+  if (cap > c->seg_len) cap = c->seg_len;
+  c->seg_cap = (cap + 7) & ~7;
+}
+
+bool plan_sift(const sjd_params* P, int kcap, bool has_u, SiftPlan* plan) {
+  const int V = P->V, es = P->logits_dtype == SJD_F32 ? 4 : 2, ev = 16 / es, unit = sjd::kUnitBytes / es;
+  if (V < 2048 || V > 65536 * sjd::kTeamWarps) return false;
+  sjd::SiftCfg& c = plan->cfg;
+  std::memset(&c, 0, sizeof(c));
+  c.piece_stride = (((V + sjd::kSiftPieces - 1) / sjd::kSiftPieces) + 7) & ~7;
+  c.piece_vecs = c.piece_stride * es >= 128 ? 4 : 1;
+  int vecs = 0;
+  for (int j = 0; j < sjd::kSiftPieces; ++j)
+    for (int k = 0; k < c.piece_vecs; ++k)
+      if (k * ev < c.piece_stride && j * c.piece_stride + k * ev < V) ++vecs;
+  const double want = (double)kcap / V;
+  double sd_e, sd_v;
+  const double p_e = aimed_share(want, (double)vecs * ev, 1, &sd_e), p_v = aimed_share(want, vecs, ev, &sd_v);
+  c.by_vectors = p_v <= 1.1 * p_e ? 1 : 0;
+  const double p = c.by_vectors ? p_v : p_e, sd = c.by_vectors ? sd_v : sd_e;
+  if (p > 0.6) return false;
+  auto rank_of = [&](double share) {
+    return (int)std::ceil(c.by_vectors ? vecs * (1.0 - std::pow(1.0 - share, ev)) : share * vecs * ev);
+  };
+  c.rank = rank_of(p);
+  const double p_high = want - 3.0 * sd;
+  c.rank_high = p_high > 0 ? rank_of(p_high) : 1;
+  if (c.rank_high < 1) c.rank_high = 1;
+  const int sms = sm_count();
+  const int64_t rows = (int64_t)P->B * P->W;
+  // few rows: as many CTAs per row as there are SMs for, as long as a warp has half a unit of its own
+  for (int n_cta = sjd::kMaxCluster; n_cta >= 1; n_cta >>= 1) {
+    if (rows * n_cta > sms) continue;
+    if (n_cta > 1 && (int64_t)V < (int64_t)unit * sjd::kClusterWarps * n_cta / 4) continue;
+    cut_segments(&c, V, sjd::kClusterWarps * n_cta, p, sd);
+    plan->cluster = n_cta;
+    plan->smem = sjd::sift_cluster_smem(c, n_cta, es, has_u);
+    if (plan->smem <= kSmemLimit && (int64_t)n_cta * c.seg_len <= 65536) return true;
+    break;
+  }
+  cut_segments(&c, V, sjd::kTeamWarps, p, sd);
+  plan->cluster = 0;
+  static const int choices[][2] = {{3, 4}, {3, 3}, {3, 2}, {2, 2}, {2, 1}, {1, 2}, {1, 1}};
+  for (const auto& ch : choices) {
+    c.teams = ch[0];
+    c.slots = ch[1];
+    plan->smem = sjd::sift_stream_smem(c.teams, c.seg_cap, c.slots, has_u);
+    if (plan->smem <= kSmemLimit) return true;
+  }
+  return false;
+}
+
+template <int DTYPE, bool HAS_U, bool HAS_T>
+cudaError_t launch_sift_as(const sjd::RowArgs& ra, const SiftPlan& plan, cudaStream_t st) {
+  const int rows = ra.B * ra.W;
+  if (plan.cluster > 0) {
+    auto kern = sjd::rows_cluster_kernel<DTYPE, HAS_U, HAS_T>;
+    static sjd::DeviceOnce configured;
+    const cudaError_t e = allow_large_smem(kern, configured, (int)kSmemLimit);
+    if (e != cudaSuccess) return e;
+    return launch_after(kern, dim3((unsigned)(rows * plan.cluster)), dim3(sjd::kClusterWarps * 32), plan.smem, st, true, plan.cluster, ra,
+                        plan.cfg);
+  }
+  auto kern = sjd::rows_stream_kernel<DTYPE, HAS_U, HAS_T>;
+  static sjd::DeviceOnce configured;
+  cudaError_t e = allow_large_smem(kern, configured, (int)kSmemLimit);
+  // a CTA takes at most kStreamRows rows per launch: larger problems go in several launches
+  const int64_t per_launch = (int64_t)sjd::kStreamRows * sm_count();
+  sjd::SiftCfg cfg = plan.cfg;
+  for (int64_t r0 = 0; r0 < rows && e == cudaSuccess; r0 += per_launch) {
+    cfg.row_begin = (int)r0;
+    cfg.row_end = (int)(r0 + per_launch < rows ? r0 + per_launch : rows);
+    const int n = cfg.row_end - cfg.row_begin;
+    e = launch_after(kern, dim3((unsigned)(n < sm_count() ? n : sm_count())), dim3((unsigned)(cfg.teams * sjd::kTeamThreads)), plan.smem, st,
+                     true, 1, ra, cfg);
+    if (e == cudaSuccess && r0 > 0) ++g_launches;
+  }
+  return e;
+}
+
+template <int DTYPE>
+cudaError_t launch_sift(const sjd::RowArgs& ra, const SiftPlan& plan, cudaStream_t st) {
+  const bool t = ra.inv_T != 1.0f;
+  if (ra.uncond != nullptr) return t ? launch_sift_as<DTYPE, true, true>(ra, plan, st) : launch_sift_as<DTYPE, true, false>(ra, plan, st);
+  return t ? launch_sift_as<DTYPE, false, true>(ra, plan, st) : launch_sift_as<DTYPE, false, false>(ra, plan, st);
 }
 
 // Scratch of sjd_step_static(): lives in the library's device image, so every GPU that loads the library
@@ -412,6 +535,7 @@ int sjd_step(const void* logits_cond, const void* logits_uncond, const int32_t* 
   {
     sjd::PipeCfg cfg;
     sjd::RangeCfg rcfg;
+    SiftPlan splan;
     size_t smem = 0;
     cudaError_t e;
     CUtensorMap map_c, map_u;
@@ -431,6 +555,10 @@ int sjd_step(const void* logits_cond, const void* logits_uncond, const int32_t* 
                                          : launch_ranges<0>(ra, rcfg, map_c, map_u, smem, grid, stream);
         if (e == cudaSuccess && r0 > 0) ++g_launches;
       }
+    } else if (fast && plan_sift(P, kcap, logits_uncond != nullptr, &splan)) {
+      e = P->logits_dtype == SJD_BF16  ? launch_sift<1>(ra, splan, stream)
+          : P->logits_dtype == SJD_F16 ? launch_sift<2>(ra, splan, stream)
+                                       : launch_sift<0>(ra, splan, stream);
     } else if (!(P->flags & SJD_FLAG_FORCE_GENERIC) && plan_pipeline(P, kcap, &cfg, &smem)) {
       const int grid = rows < sm_count() ? rows : sm_count();
       e = P->logits_dtype == SJD_BF16  ? launch_pipeline<1>(ra, cfg, smem, grid, stream)
@@ -439,10 +567,10 @@ int sjd_step(const void* logits_cond, const void* logits_uncond, const int32_t* 
     } else {
       const int grid = rows < 4 * sm_count() ? rows : 4 * sm_count();
       e = P->logits_dtype == SJD_BF16
-              ? launch_after(sjd::rows_generic_kernel<1, kGenericThreads>, dim3((unsigned)grid), dim3(kGenericThreads), 0, stream, true, ra)
+              ? launch_after(sjd::rows_generic_kernel<1, kGenericThreads>, dim3((unsigned)grid), dim3(kGenericThreads), 0, stream, true, 1, ra)
           : P->logits_dtype == SJD_F16
-              ? launch_after(sjd::rows_generic_kernel<2, kGenericThreads>, dim3((unsigned)grid), dim3(kGenericThreads), 0, stream, true, ra)
-              : launch_after(sjd::rows_generic_kernel<0, kGenericThreads>, dim3((unsigned)grid), dim3(kGenericThreads), 0, stream, true, ra);
+              ? launch_after(sjd::rows_generic_kernel<2, kGenericThreads>, dim3((unsigned)grid), dim3(kGenericThreads), 0, stream, true, 1, ra)
+              : launch_after(sjd::rows_generic_kernel<0, kGenericThreads>, dim3((unsigned)grid), dim3(kGenericThreads), 0, stream, true, 1, ra);
     }
     if (e != cudaSuccess) return cuda_fail(e, "row kernel launch");
     ++g_launches;
@@ -481,7 +609,7 @@ int sjd_step(const void* logits_cond, const void* logits_uncond, const int32_t* 
     // blocks are placed as the row kernel's last blocks retire and wait inside the kernel for its completion.
     // An event recorded in between makes it an ordinary launch.
     const cudaError_t e = launch_after(sjd::verify_kernel<kVerifyThreads>, dim3((unsigned)P->B), dim3(kVerifyThreads), 0, stream,
-                                       P->ev_rows_end == nullptr, va);
+                                       P->ev_rows_end == nullptr, 1, va);
     if (e != cudaSuccess) return cuda_fail(e, "verify kernel launch");
     ++g_launches;
   }
@@ -548,7 +676,9 @@ int sjd_row_kernel(const sjd_params* P) {
   sjd::RangeCfg rcfg;
   size_t smem = 0;
   const bool fast = !(P->flags & (SJD_FLAG_FORCE_GENERIC | SJD_FLAG_FORCE_TILES));
+  SiftPlan splan;
   if (fast && plan_ranges(P, kcap, &rcfg, &smem, false)) return SJD_ROWS_RANGES;
+  if (fast && plan_sift(P, kcap, true, &splan)) return SJD_ROWS_GENERIC;
   if (!(P->flags & SJD_FLAG_FORCE_GENERIC) && plan_pipeline(P, kcap, &cfg, &smem)) return SJD_ROWS_TILES;
   return SJD_ROWS_GENERIC;
 }
@@ -583,10 +713,10 @@ int sjd_window_advance(const sjd_params* P, int32_t n_total, uint64_t philox_see
   a.committed = committed;
   a.n_committed = n_committed;
   cudaStream_t st = static_cast<cudaStream_t>(P->stream);
-  cudaError_t e = launch_after(sjd::advance_rows_kernel<256>, dim3((unsigned)(P->B * P->W)), dim3(256), 0, st, true, a);
+  cudaError_t e = launch_after(sjd::advance_rows_kernel<256>, dim3((unsigned)(P->B * P->W)), dim3(256), 0, st, true, 1, a);
   if (e != cudaSuccess) return cuda_fail(e, "window advance launch");
   ++g_launches;
-  e = launch_after(sjd::advance_state_kernel, dim3((unsigned)((P->B + 127) / 128)), dim3(128), 0, st, true, a);
+  e = launch_after(sjd::advance_state_kernel, dim3((unsigned)((P->B + 127) / 128)), dim3(128), 0, st, true, 1, a);
   if (e != cudaSuccess) return cuda_fail(e, "window state launch");
   ++g_launches;
   return SJD_OK;
