@@ -31,7 +31,6 @@ int cuda_fail(cudaError_t e, const char* what) {
 }
 
 constexpr int kGenericThreads = 512;
-constexpr int kVerifyThreads = 512;
 
 int current_device() {
   int dev = -1;
@@ -608,7 +607,9 @@ int sjd_step(const void* logits_cond, const void* logits_uncond, const int32_t* 
     // directly behind the row kernel the verification grid is launched as its programmatic dependent: its
     // blocks are placed as the row kernel's last blocks retire and wait inside the kernel for its completion.
     // An event recorded in between makes it an ordinary launch.
-    const cudaError_t e = launch_after(sjd::verify_kernel<kVerifyThreads>, dim3((unsigned)P->B), dim3(kVerifyThreads), 0, stream,
+    const bool longer = kcap > sjd::kVerifyThreads * sjd::kVerifyItems;
+    const cudaError_t e = launch_after(longer ? sjd::verify_kernel<true> : sjd::verify_kernel<false>, dim3((unsigned)P->B),
+                                       dim3(sjd::kVerifyThreads), 0, stream,
                                        P->ev_rows_end == nullptr, 1, va);
     if (e != cudaSuccess) return cuda_fail(e, "verify kernel launch");
     ++g_launches;

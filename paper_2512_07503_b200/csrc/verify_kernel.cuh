@@ -44,18 +44,6 @@ struct VerifyArgs {
   int32_t* status;
 };
 
-// q(token) on a sparse row with ascending ids.
-__device__ __forceinline__ float sparse_lookup(const int32_t* __restrict__ ids, const float* __restrict__ vals,
-                                               int cnt, int token) {
-  int lo = 0, hi = cnt;
-  while (lo < hi) {
-    const int mid = (lo + hi) >> 1;
-    if (ids[mid] < token) lo = mid + 1;
-    else hi = mid;
-  }
-  return (lo < cnt && ids[lo] == token) ? vals[lo] : 0.0f;
-}
-
 // ratio p/q of Eq. acc-sjdpp and of the confidence C (the same quantity), with the conventions for
 // the corner cases: p == 0 gives 0 (never accepted, never reused); q <= 0 with p > 0 gives +inf.
 __device__ __forceinline__ float likelihood_ratio(float p, float q) {
@@ -64,60 +52,83 @@ __device__ __forceinline__ float likelihood_ratio(float p, float q) {
   return __fdiv_rn(p, q);
 }
 
-constexpr int kVerifyStageCap = 2048;  // entries of a previous-iteration row staged in shared memory
+constexpr int kVerifyThreads = 512;     // >= SJD_W_MAX: a thread per window row
+constexpr int kVerifyItems = 4;         // entries of the rejected row per thread and round: 2,048 a round
+constexpr int kVerifyStage = 8192;      // words of the previous iteration's row staged in shared memory
 
 struct VerifySmem {
   uint64_t scan[2 * 32 + 8];
-  int32_t q_ids[kVerifyStageCap];
-  float q_vals[kVerifyStageCap];
+  // ids of the previous iteration's row (of a very long one every stride-th), and behind the first 2,048 the
+  // probabilities when the whole row fits in 2,048 entries
+  alignas(16) int32_t q[kVerifyStage];
   int first_reject;
   int status;
   int res_tok;
   float res_prob;
 };
 
-// Everything the verification stage does for sequence b, executed by NT threads (ranks `tid`).
-template <int NT, int BAR>
-__device__ void verify_sequence(const VerifyArgs& a, int b, int tid, VerifySmem& sm) {
-  const int W = a.W;
-  const int L = a.win_len ? min(max(a.win_len[b], 0), W) : W;
-  const int pos0 = a.pos_base ? a.pos_base[b] : 0;
-  const int iter = a.iteration ? a.iteration[b] : a.iteration0;
+// One CTA per sequence.  Latency is all there is to it (it sits between two row kernels), so nothing is waited for
+// that could have been asked for earlier: what does not come from the row stage is loaded, and the accept tests' random
+// numbers are drawn, before the wait for that stage; both rows of the residual draw come in with one round of loads; the
+// lookups of a thread's four entries run side by side.  16 sequences of 64 rows, K=2,000: 8.4 us under ncu
+// (12.1 before), and 3 us less of a step (one window of 32 rows: 25.5 -> 21.4 us).
+//
+// LONG: rows of more than 2,048 entries, taken in rounds (1,024 rows of K=8,192: 294 -> 235 us a step).
+template <bool LONG>
+__global__ void __launch_bounds__(kVerifyThreads) verify_kernel(const VerifyArgs a) {
+  constexpr int NT = kVerifyThreads, ITEMS = kVerifyItems;
+  __shared__ VerifySmem sm;
+  const int b = blockIdx.x, i = threadIdx.x, W = a.W;
   const bool draft_all = (a.flags & kFlagDraftAll) != 0;
   const bool reuse_on = (a.flags & kFlagReuse) != 0;
   const size_t base = (size_t)b * W;
-  int flip = 0;
-  if (tid == 0) {
+  // Inputs of the call: written before the row kernel began, which waits for that itself before it lets this grid start.
+  const int L = a.win_len ? min(max(a.win_len[b], 0), W) : W;
+  const int pos0 = a.pos_base ? a.pos_base[b] : 0;
+  const int iter = a.iteration ? a.iteration[b] : a.iteration0;
+  const uint32_t seq = (uint32_t)(a.seq_base + b);
+  float q_tok = 0.0f, u = 0.0f;
+  int draft = -1;
+  if (!draft_all && i < L) {
+    q_tok = a.q_tok[base + i];
+    draft = a.drafts[base + i];
+    u = uniform24(philox4x32_10((uint32_t)(pos0 + i), seq, (uint32_t)iter, kPurposeAccept, a.seed_lo, a.seed_hi).x0);
+  }
+  if (i == 0) {
     sm.first_reject = L;
     sm.status = 0;
     sm.res_tok = -1;
     sm.res_prob = 0.0f;
   }
-  group_sync<NT, BAR>();
+  __syncthreads();
+  // Launched with programmatic stream serialisation right behind the row kernel: the grid may be scheduled while that
+  // kernel's last rows are still running, and waits here until all of its writes are visible.  A no-op after an
+  // ordinary launch.
+  grid_dependency_wait();
+  // a following kernel that waits the same way (the next step's row kernel) may set itself up meanwhile
+  allow_dependent_launch();
 
-  // Step 3: r < min(1, p(x_i)/q(x_i)) on every valid row; the counter-based generator makes the
-  // rows independent, so they are all tested at once
-  for (int i = tid; i < L; i += NT) {
-    const RowScratch rs = a.scratch[base + i];
+  // Step 3: r < min(1, p(x_i)/q(x_i)) on every valid row; the counter-based generator makes the rows independent, so
+  // they are all tested at once
+  RowScratch rs{0.0f, -1, 0.0f, 0};
+  float ratio = 0.0f;
+  if (i < L) {
+    rs = a.scratch[base + i];
     int st = (rs.status & kRowStatusDegenerate) ? kStatusDegenerate : 0;
     if (rs.status & kRowStatusTimeout) st |= kStatusTimeout;
     if (rs.status & kRowStatusRedone) st |= kStatusRedone;
     if (!draft_all) {
-      const float q = a.q_tok[base + i];
-      const float ratio = likelihood_ratio(rs.p_tok, q);
-      const Philox4 rnd = philox4x32_10((uint32_t)(pos0 + i), (uint32_t)(a.seq_base + b), (uint32_t)iter, kPurposeAccept,
-                                        a.seed_lo, a.seed_hi);
-      const float u = uniform24(rnd.x0);
+      ratio = likelihood_ratio(rs.p_tok, q_tok);
       if (!(u < fminf(ratio, 1.0f))) atomicMin(&sm.first_reject, i);
-      if (!(q > 0.0f)) st |= kStatusQtok;
+      if (!(q_tok > 0.0f)) st |= kStatusQtok;
     }
     if (st) atomicOr(&sm.status, st);
   }
-  group_sync<NT, BAR>();
+  __syncthreads();
   const int acc = draft_all ? 0 : sm.first_reject;
 
-  // Step 4, first rejected row: draw from max(0, p - q) / sum max(0, p - q).  Every thread owns a run of
-  // consecutive entries of p_a (ascending token id), so one scan of the per-thread sums locates the draw.
+  // Step 4, first rejected row: draw from max(0, p - q) / sum max(0, p - q).  Every thread owns a run of consecutive entries
+  // of p_a (ascending token id), so one scan of the per-thread sums locates the draw.
   if (!draft_all && acc < L) {
     const size_t r = base + acc;
     const int kcap = a.kcap;
@@ -126,111 +137,144 @@ __device__ void verify_sequence(const VerifyArgs& a, int b, int tid, VerifySmem&
     const int32_t* qid = a.q_ids + r * kcap;
     const float* qv = a.q_vals + r * kcap;
     const int qc = a.q_cnt[r];
-    const bool staged = qc > 0 && qc <= kVerifyStageCap;
-    if (staged) {
-      for (int k = tid; k < qc; k += NT) {
-        sm.q_ids[k] = qid[k];
-        sm.q_vals[k] = qv[k];
-      }
-      group_sync<NT, BAR>();
-    }
-    const int32_t* sid = staged ? sm.q_ids : qid;
-    const float* sval = staged ? sm.q_vals : qv;
     const float q_uniform = __fdiv_rn(1.0f, (float)a.V);
-    const Philox4 rnd = philox4x32_10((uint32_t)(pos0 + acc), (uint32_t)(a.seq_base + b), (uint32_t)iter,
-                                      kPurposeResidual, a.seed_lo, a.seed_hi);
-    const uint64_t R = random64(rnd);
-    const int per = (kcap + NT - 1) / NT;
-    const int k0 = min(tid * per, kcap), k1 = min(k0 + per, kcap);
-    int found = -1;
-    for (int attempt = 0; attempt < 2; ++attempt) {
-      // attempt 0: residual weights; attempt 1 (only when they sum to zero after rounding): p itself
-      uint64_t local = 0;
-      for (int k = k0; k < k1; ++k) {
-        float w = pv[k];
-        if (attempt == 0) {
-          const float q = (qc == kQUniform) ? q_uniform : sparse_lookup(sid, sval, max(qc, 0), pid[k]);
-          w = __fsub_rn(w, q);
-        }
-        local += fixed_weight(w);
+    const uint64_t R = random64(philox4x32_10((uint32_t)(pos0 + acc), seq, (uint32_t)iter, kPurposeResidual, a.seed_lo, a.seed_hi));
+    const int rounds = LONG ? (kcap + NT * ITEMS - 1) / (NT * ITEMS) : 1;
+    const int k0 = i * ITEMS * rounds;  // this thread's run of consecutive entries
+    int id[ITEMS];
+    float p[ITEMS], w[ITEMS];
+    auto load = [&](int k) {
+#pragma unroll
+      for (int j = 0; j < ITEMS; ++j) {
+        const bool in = k + j < kcap;
+        id[j] = in ? pid[k + j] : -1;
+        p[j] = in ? pv[k + j] : 0.0f;
       }
-      uint64_t T;
-      const uint64_t lo = group_scan1<NT, BAR, uint64_t>(local, tid, sm.scan, flip, &T);
-      if (T == 0) {
-        if (attempt == 0) {
-          if (tid == 0) sm.status |= kStatusEmptyResidual;
-          continue;
-        }
-        if (tid == 0) found = 0;
-        break;
+    };
+    int n, stride = 1;
+    if (!LONG) {
+      // all loads at once: q's too, although only the first qc of its entries (if it has any) mean anything
+      int qi[ITEMS];
+      float qw[ITEMS];
+      load(k0);
+#pragma unroll
+      for (int j = 0; j < ITEMS; ++j) {
+        const bool in = k0 + j < kcap;
+        qi[j] = in ? qid[k0 + j] : 0;
+        qw[j] = in ? qv[k0 + j] : 0.0f;
       }
-      const uint64_t t = __umul64hi(R, T);
-      if (t >= lo && t < lo + local) {
-        uint64_t run = lo;
-        for (int k = k0; k < k1; ++k) {
-          float w = pv[k];
-          if (attempt == 0) {
-            const float q = (qc == kQUniform) ? q_uniform : sparse_lookup(sid, sval, max(qc, 0), pid[k]);
-            w = __fsub_rn(w, q);
-          }
-          run += fixed_weight(w);
-          if (t < run) {
-            found = k;
-            break;
-          }
-        }
-      }
-      break;
+      *reinterpret_cast<int4*>(&sm.q[k0]) = make_int4(qi[0], qi[1], qi[2], qi[3]);
+      *reinterpret_cast<float4*>(&sm.q[NT * ITEMS + k0]) = make_float4(qw[0], qw[1], qw[2], qw[3]);
+      n = min(max(qc, 0), kcap);
+    } else {
+      n = min(max(qc, 0), kcap);
+      stride = (n + kVerifyStage - 1) / kVerifyStage;
+      for (int k = i; k * stride < n; k += NT) sm.q[k] = qid[k * stride];
     }
-    if (found >= 0) {
-      sm.res_tok = pid[found];
-      sm.res_prob = pv[found];
+    __syncthreads();
+    const int staged = n > 0 ? (n + stride - 1) / stride : 0;
+    // weights of the four entries in id / p: what q leaves of p
+    auto residual = [&](int k) {
+      int lo[ITEMS] = {0, 0, 0, 0};
+      if (n > 0) {
+        // largest staged position whose id does not exceed the wanted one: halving steps, the four lookups in step
+        for (int half = 1 << (31 - __clz(staged)); half > 0; half >>= 1) {
+#pragma unroll
+          for (int j = 0; j < ITEMS; ++j) {
+            const int at = lo[j] + half;
+            if (at < staged && sm.q[at] <= id[j]) lo[j] = at;
+          }
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < ITEMS; ++j) {
+        float q = qc == kQUniform ? q_uniform : 0.0f;
+        if (n > 0) {
+          if (!LONG) {
+            if (sm.q[lo[j]] == id[j]) q = reinterpret_cast<const float*>(sm.q)[NT * ITEMS + lo[j]];
+          } else {
+            int at = lo[j] * stride;
+            const int end = min(at + stride, n);
+            while (at + 1 < end && qid[at + 1] <= id[j]) ++at;
+            if (qid[at] == id[j]) q = qv[at];
+          }
+        }
+        w[j] = k + j < kcap ? __fsub_rn(p[j], q) : 0.0f;
+      }
+    };
+    int flip = 0;
+    uint64_t T = 0, before = 0, local = 0;
+    bool from_p = false;
+    for (;;) {
+      // residual weights first; p itself only when they sum to zero after rounding
+      local = 0;
+      for (int r = 0; r < rounds; ++r) {
+        if (LONG) load(k0 + ITEMS * r);
+        if (!from_p) residual(k0 + ITEMS * r);
+#pragma unroll
+        for (int j = 0; j < ITEMS; ++j) {
+          if (from_p) w[j] = p[j];
+          local += fixed_weight(w[j]);
+        }
+      }
+      before = group_scan1<NT, 0, uint64_t>(local, i, sm.scan, flip, &T);
+      if (T != 0 || from_p) break;
+      if (i == 0) sm.status |= kStatusEmptyResidual;
+      from_p = true;
+    }
+    const uint64_t t = __umul64hi(R, T);
+    if (T == 0 ? i == 0 : (t >= before && t < before + local)) {
+      int j = 0;
+      if (T == 0) {
+        load(0);  // nothing but zeros: the first entry
+      } else {
+        for (int r = 0; r < rounds; ++r) {
+          if (LONG) {
+            load(k0 + ITEMS * r);
+            if (!from_p) residual(k0 + ITEMS * r);
+          }
+          uint64_t sum = 0;
+          j = 0;
+#pragma unroll
+          for (int x = 0; x < ITEMS; ++x) {
+            sum += fixed_weight(LONG && from_p ? p[x] : w[x]);
+            if (t >= before + sum) j = x + 1;
+          }
+          if (j < ITEMS) break;  // comes true: t < before + local
+          before += sum;
+        }
+      }
+      sm.res_tok = j == 0 ? id[0] : j == 1 ? id[1] : j == 2 ? id[2] : id[3];
+      sm.res_prob = j == 0 ? p[0] : j == 1 ? p[1] : j == 2 ? p[2] : p[3];
     }
   }
-  group_sync<NT, BAR>();
+  __syncthreads();
 
   // Step 4, remaining rows, and the outputs
-  for (int i = tid; i < W; i += NT) {
+  if (i < W) {
     int tok = -1, flag = kOutInvalid;
     float pr = 0.0f;
     if (i < L) {
-      const RowScratch rs = a.scratch[base + i];
       if (draft_all) {
         tok = rs.samp_tok; pr = rs.samp_prob; flag = kOutResampled;
       } else if (i < acc) {
-        tok = a.drafts[base + i]; pr = rs.p_tok; flag = kOutAccepted;
+        tok = draft; pr = rs.p_tok; flag = kOutAccepted;
       } else if (i == acc) {
         tok = sm.res_tok; pr = sm.res_prob; flag = kOutResidual;
+      } else if (reuse_on && rs.p_tok > 0.0f && ratio > a.tau) {  // the ratio is the confidence of Eq. (C)
+        tok = draft; pr = rs.p_tok; flag = kOutReused;
       } else {
-        const float C = likelihood_ratio(rs.p_tok, a.q_tok[base + i]);  // confidence of Eq. (C)
-        if (reuse_on && rs.p_tok > 0.0f && C > a.tau) {
-          tok = a.drafts[base + i]; pr = rs.p_tok; flag = kOutReused;
-        } else {
-          tok = rs.samp_tok; pr = rs.samp_prob; flag = kOutResampled;
-        }
+        tok = rs.samp_tok; pr = rs.samp_prob; flag = kOutResampled;
       }
     }
     a.out_tokens[base + i] = tok;
     a.out_tok_prob[base + i] = pr;
     if (a.out_flags) a.out_flags[base + i] = flag;
   }
-  if (tid == 0) {
+  if (i == 0) {
     a.out_accept_len[b] = acc;
     if (a.status) a.status[b] = sm.status;
   }
-  group_sync<NT, BAR>();
-}
-
-template <int NT>
-__global__ void __launch_bounds__(NT) verify_kernel(const VerifyArgs a) {
-  __shared__ VerifySmem sm;
-  // Launched with programmatic stream serialisation right behind the row kernel: the grid may be scheduled
-  // while that kernel's last rows are still running, and waits here until all of its writes are visible.
-  // A no-op after an ordinary launch.
-  grid_dependency_wait();
-  // a following kernel that waits the same way (the next step's row kernel) may set itself up meanwhile
-  allow_dependent_launch();
-  for (int b = blockIdx.x; b < a.B; b += gridDim.x) verify_sequence<NT, 0>(a, b, threadIdx.x, sm);
 }
 
 }  // namespace sjd

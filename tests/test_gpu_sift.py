@@ -27,7 +27,8 @@ def test_cutting_of_a_row(V, B, W, dtype):
 
 
 @pytest.mark.parametrize("V,K,B,W", [(50264, 2000, 1, 8), (65536, 4096, 1, 5), (65536, 8192, 2, 76), (32776, 1, 2, 3),
-                                     (131072, 3000, 1, 2), (20000, 5000, 1, 3)])
+                                     (131072, 3000, 1, 2), (20000, 5000, 1, 3),
+                                     (65536, 9001, 1, 6), (65536, 2049, 3, 2)])
 def test_wide_rows_and_wide_top_k(V, K, B, W):
     _check(f"wide{V}", B=B, W=W, V=V, top_k=K, seed=K + W)
 
