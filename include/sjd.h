@@ -62,8 +62,8 @@ extern "C" {
 
 #define SJD_FLAG_FORCE_GENERIC 4 /* diagnostics: use the any-shape multi-pass row kernel even where a
                                    single-pass kernel applies (results are identical)                    */
-#define SJD_FLAG_FORCE_TILES 8   /* diagnostics: skip the single-pass kernel that cuts a row into one id
-                                   range per thread; the tile-dealing one is used where it applies        */
+#define SJD_FLAG_FORCE_TILES 8   /* diagnostics: skip the single-pass kernels that cut a row into one id
+                                   range per warp; the tile-dealing one is used where it applies          */
 
 /* cnt value of a row of sjd_probs that stands for the uniform distribution over V (1/V each); used for
  * window slots that were initialised at random and have no previous-iteration distribution. */
@@ -159,13 +159,12 @@ size_t sjd_workspace_bytes(const sjd_params* params);
  * Which row kernel sjd_step() selects for this shape and these flags (Section 3.1's sampling head has three
  * implementations that give identical results): SJD_ROWS_RANGES, SJD_ROWS_TILES or SJD_ROWS_GENERIC, or a
  * negative SJD_ERR_* for a shape, dtype or strides sjd_step() would refuse (pointers and the workspace are not
- * looked at).  Decided from the shape alone: it assumes the driver offers the tensor-map encoder the range
- * kernel needs, which every driver that runs this library's kernels does.  Launches nothing.
+ * looked at).  Decided from the shape alone.  Launches nothing.
  */
-#define SJD_ROWS_GENERIC 0 /* any shape: sifted by a sampled threshold in one pass where V >= 2,048 and K is a modest
-                              share of it, else a radix select over global memory in several passes         */
-#define SJD_ROWS_TILES 1   /* V a multiple of 2,048: one pass, tiles dealt to the filter warps             */
-#define SJD_ROWS_RANGES 2  /* V a multiple of 256, kcap <= 2,048: one pass, one id range per filter thread */
+#define SJD_ROWS_GENERIC 0 /* any shape: several passes over a row in global memory (kcap > 2,048: one pass where V and
+                              K allow it)                                                                    */
+#define SJD_ROWS_TILES 1   /* V a multiple of 2,048: one pass, tiles dealt to the filter warps               */
+#define SJD_ROWS_RANGES 2  /* V >= 2,048, kcap <= 2,048 and a modest share of V: one pass, one id range per warp */
 int sjd_row_kernel(const sjd_params* params);
 
 /*
@@ -187,7 +186,7 @@ int sjd_row_kernel(const sjd_params* params);
  * Asynchronous on params->stream.  Returns SJD_OK once the kernels are enqueued.  A negative SJD_ERR_* for a
  * bad argument means that nothing was enqueued; SJD_ERR_CUDA (a launch or an event record refused by the
  * runtime) may leave the work enqueued before the failing call on the stream.  Conditions found on the
- * device (status bits) never abort the kernels.  A problem of more than 32 rows per SM takes several launches
+ * device (status bits) never abort the kernels.  A problem of more than 64 rows per SM takes several launches
  * of the row kernel.
  */
 int sjd_step(const void* logits_cond, const void* logits_uncond, const int32_t* drafts,

@@ -19,17 +19,22 @@
 //
 // Two kernels share the phases:
 //
-//   rows_stream_kernel   many rows: one persistent CTA per SM of up to three teams of eight warps.  A team takes a row
-//                        through all phases; the teams take the CTA's rows in turn.  The rows' units come through one
-//                        ring of shared-memory slots per segment, in row order, so that one team sifts at the
-//                        memory's pace while the others finish their row and sample their next one.
+//   rows_stream_kernel   many rows: one persistent CTA per SM of up to three teams of eight warps and one sampler warp for
+//                        each team.  A team sifts and finishes a row; the teams take the CTA's rows in turn, so that one
+//                        sifts while others finish.  The rows' units come through one ring of shared-memory slots per
+//                        segment, in row order.  The samplers find the thresholds of rows to come: a team's own sample
+//                        phase (its first row's) is 9-14 K cycles of barriers and short searches that would hold up
+//                        eight warps (with every row sampled by its team: 94 us where this takes 82).
 //   rows_cluster_kernel  few rows: one cluster of up to eight CTAs of sixteen warps per row, the whole row in shared
 //                        memory at once.  The candidates go straight into the first CTA's lists (distributed shared
 //                        memory), which finishes the row.
 //
-// Measured against what took these shapes before: 231 rows of 50,264 bf16 entries, K=500: 32.2 us a step, any-shape
-// kernel 100.6 (four radix passes and a compaction over the row in the L2); 1,024 rows of 65,536, K=8,192: 254, 524;
-// 16 rows of 4,096 fp32 entries, K=64: 12.5, tile kernel 16.3.
+// What bounds it: at V=65,536 and K=2,000 a row is about 35 K warp instructions at 60 % of the issue slots; a row of the
+// memory stream alone would be 12.3 K cycles.  us a step against the kernels that took these shapes before: 1,024 rows of
+// 65,536 bf16, K=2,000: 82.4 (85.4 with a kernel of one id range per filter thread); of 16,384: 53.0 (65.0); 1,024 ragged
+// rows of 16,384 fp32, K=1,000: 51.8 (58.5); 1,024 rows of 32,768 bf16 without guidance: 50.2 (63.4); 231 rows of
+// 50,264, K=500: 31.6 (100.6, four radix passes and a compaction over the row in the L2); 1,024 rows of 65,536, K=8,192:
+// 215 (524); 16 rows of 4,096 fp32, K=64: 11.7 (16.3, tiles dealt to filter warps).
 //
 // Every wait on an mbarrier is bounded; a wait that gives up marks the row (and the CTA's unfinished rows) with
 // kRowStatusTimeout, and the CTA waits (bounded) for its copies in flight before it exits.
@@ -41,7 +46,8 @@ namespace sjd {
 
 constexpr int kSiftPieces = 256;          // sample pieces per row
 constexpr int kSiftBins = 1024;           // bins of a row's histogram (the sample's, then the candidates')
-constexpr int kBinsLow = 768;             // candidates' bins 1 .. kBinsLow cover the stretch that holds the threshold
+constexpr int kBinsLow = 768;             // candidates' bins 1 .. kBinsLow cover the lowest eighth of their values
+constexpr float kBinsCross = (8.0f * (kBinsLow + 1) - (kSiftBins - 2)) / 7.0f;  // where the upper bins' line starts
 constexpr int kSiftKeyShift = 22;         // key bits dropped by the sample's first pass: sign, exponent, one mantissa bit stay
 constexpr int kMemberCap = 512;           // members of the threshold bin ranked by brute force
 constexpr int kUnitBytes = 4096;          // bytes of one logits array per unit: 128 for each lane
@@ -58,7 +64,6 @@ struct SiftCfg {
   int piece_vecs;    // 16-byte vectors per piece: 4 or 1
   int by_vectors;    // 1: ranks among the vectors' maxima; 0: among all sampled elements
   int rank;          // rank (from the top) of tau0
-  int rank_high;     // rank of a value that the threshold hardly ever exceeds
   int seg_len;       // ids per segment, a multiple of 8
   int seg_cap;       // candidates a segment's list holds (a multiple of 8)
   int teams, slots;  // stream kernel: teams per CTA, ring slots per warp
@@ -70,12 +75,23 @@ struct SiftMember {  // member of the threshold bin: value and id
   int32_t id;
 };
 
-// what the warps that work on one row share
-struct alignas(16) SiftShared {
+// Fine bins and one coarse bin per 32 of them: whoever counts in a fine bin counts in its coarse bin as well, which costs
+// next to nothing and makes the search for a rank two scans of 32 words, done while everybody waits.
+struct alignas(16) SiftHist {
   union {
-    uint32_t hist[kSiftBins];        // zero whenever it is not in use
+    uint32_t fine[kSiftBins];        // zero whenever it is not in use
     SiftMember member[kMemberCap];   // the threshold bin's members, after the histogram's last search
   };
+  uint32_t coarse[kSiftBins / 32];
+  __device__ __forceinline__ void count(uint32_t bin) {
+    atomicAdd(&fine[bin], 1u);
+    atomicAdd(&coarse[bin >> 5], 1u);
+  }
+};
+
+// what the warps that work on one row share
+struct alignas(16) SiftShared {
+  SiftHist hist;
   uint64_t wtot[kClusterWarps];
   uint32_t wcnt[kClusterWarps];
   float wz[kClusterWarps];
@@ -83,7 +99,7 @@ struct alignas(16) SiftShared {
   uint32_t max_key;   // largest candidate
   uint32_t over;      // a list ran over, or a wait gave up
   int members;
-  uint32_t rank_bin, rank_above, rank_count, rank_bin2;  // results of a rank search
+  uint32_t rank_bin, rank_above, rank_count;  // results of a rank search
   float thr_y;
   int thr_id;
   float ptok;
@@ -182,58 +198,36 @@ __device__ __forceinline__ uint32_t scan_incl(uint32_t v, int lane) {
 }
 
 // ---------------------------------------------------------------------------------------------------
-// rank search: the bin b with (entries above b) < target <= (entries in b and above), for one or two targets, by one
+// rank search: the bin b with (entries above b) < target <= (entries in b and above), by one
 // warp, which also leaves the histogram zero.  A bin is 0 when there are fewer than `target` entries in bins 1 and
 // above.  A call of its own: all searches of a row run the same few instructions, which matters where every
 // instruction is fetched for the first time.
 // ---------------------------------------------------------------------------------------------------
-static __device__ __noinline__ void rank_search(SiftShared* sm, uint32_t* hist, uint32_t target, uint32_t target2) {
+static __device__ __noinline__ void rank_search(SiftShared* sm, SiftHist* h, uint32_t t) {
   const int lane = threadIdx.x & 31;
-  // lane l: bins 32 l .. 32 l + 31; the eight lanes served together start at different 16-byte pieces
-  uint4* const mine = reinterpret_cast<uint4*>(hist + 32 * lane);
-  uint32_t sum = 0;
-#pragma unroll
-  for (int x = 0; x < 8; ++x) {
-    const uint4 w = mine[(x + lane) & 7];
-    sum += w.x + w.y + w.z + w.w;
+  const uint32_t sum = h->coarse[31 - lane];  // lane 0 takes the topmost
+  const uint32_t upto = scan_incl(sum, lane);
+  const uint32_t votes = __ballot_sync(0xffffffffu, upto - sum < t && t <= upto);
+  uint32_t bin = 0, before = 0, count = 0;
+  if (votes != 0u) {
+    const int l1 = __ffs((int)votes) - 1;
+    const uint32_t above1 = __shfl_sync(0xffffffffu, upto - sum, l1);
+    const uint32_t f = h->fine[32 * (31 - l1) + 31 - lane];
+    const uint32_t a2 = above1 + scan_incl(f, lane) - f;
+    const int l2 = __ffs((int)__ballot_sync(0xffffffffu, a2 < t && t <= a2 + f)) - 1;
+    bin = (uint32_t)(32 * (31 - l1) + 31 - l2);
+    before = __shfl_sync(0xffffffffu, a2, l2);
+    count = __shfl_sync(0xffffffffu, f, l2);
   }
-  // entries above this lane's bins
-  uint32_t above = sum;
-#pragma unroll
-  for (int d = 1; d < 32; d <<= 1) {
-    const uint32_t n = __shfl_down_sync(0xffffffffu, above, d);
-    if (lane + d < 32) above += n;
-  }
-  above -= sum;
-#pragma unroll 1
-  for (int pass = 0; pass < 2; ++pass) {
-    const uint32_t t = pass == 0 ? target : target2;
-    const uint32_t votes = __ballot_sync(0xffffffffu, above < t && t <= above + sum);
-    uint32_t bin = 0, before = 0, count = 0;
-    if (votes != 0u) {
-      const int l1 = __ffs((int)votes) - 1;
-      const uint32_t above1 = __shfl_sync(0xffffffffu, above, l1);
-      const uint32_t f = hist[32 * l1 + 31 - lane];  // lane 0 takes the topmost
-      const uint32_t a2 = above1 + scan_incl(f, lane) - f;
-      const int l2 = __ffs((int)__ballot_sync(0xffffffffu, a2 < t && t <= a2 + f)) - 1;
-      bin = (uint32_t)(32 * l1 + 31 - l2);
-      before = __shfl_sync(0xffffffffu, a2, l2);
-      count = __shfl_sync(0xffffffffu, f, l2);
-    }
-    if (lane == 0) {
-      if (pass == 0) {
-        sm->rank_bin = bin;
-        sm->rank_above = before;
-        sm->rank_count = count;
-      } else {
-        sm->rank_bin2 = bin;
-      }
-    }
-    if (target2 == 0u) break;
+  if (lane == 0) {
+    sm->rank_bin = bin;
+    sm->rank_above = before;
+    sm->rank_count = count;
   }
   __syncwarp();
 #pragma unroll
-  for (int x = 0; x < 8; ++x) mine[(x + lane) & 7] = make_uint4(0u, 0u, 0u, 0u);
+  for (int x = 0; x < kSiftBins / 128; ++x) reinterpret_cast<uint4*>(h->fine)[lane + 32 * x] = make_uint4(0u, 0u, 0u, 0u);
+  h->coarse[lane] = 0u;
 }
 
 // ---------------------------------------------------------------------------------------------------
@@ -247,16 +241,27 @@ static __device__ __noinline__ void rank_search(SiftShared* sm, uint32_t* hist, 
 // tau0 only steers how many candidates there are; the result is exact whatever it is.
 //
 // The candidates' bins are 1 .. kSiftBins - 1; bin 0 takes what is no candidate.  bin(y) is the smaller of two rising lines
-// over y - tau0, the first of which spends kBinsLow bins on the stretch up to a value that the K-th largest hardly
-// ever exceeds (the same sample says where that is): the threshold's bin then holds two or three members.  Any
-// rising function would do: a higher bin never holds a smaller value.
+// over y - tau0, the first of which spends kBinsLow bins on the lowest eighth of [tau0, largest sample value], where
+// the candidates crowd: the threshold's bin then holds a handful of members.  Any rising function would do: a
+// higher bin never holds a smaller value.
 struct SiftBinning {
-  float tau0, s1, s2, c2;
+  float tau0, s1, s2;
   __device__ __forceinline__ float at(float y) const {
     const float d = __fsub_rn(y, tau0);
-    return fminf(__fmaf_rn(d, s1, 1.0f), __fmaf_rn(d, s2, c2));
+    return fminf(__fmaf_rn(d, s1, 1.0f), __fmaf_rn(d, s2, kBinsCross));
   }
 };
+__device__ __forceinline__ SiftBinning sift_bins(float tau0, float top) {
+  const float range = __fsub_rn(top, tau0);
+  const float per = range > 0.0f ? __fdiv_rn(1.0f, range) : 0.0f;
+  return SiftBinning{tau0, __fmul_rn(8.0f * kBinsLow, per), __fmul_rn((kSiftBins - 2) - kBinsCross, per)};
+}
+
+__device__ __forceinline__ uint4 ldg_now(const void* p) {  // issued where it stands: the values are wanted much later
+  uint4 v;
+  asm volatile("ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+  return v;
+}
 
 __device__ __forceinline__ int sample_element(const SiftCfg& cfg, int vec, int ev, int V) {
   const int piece = cfg.piece_vecs == 4 ? vec >> 2 : vec, k = cfg.piece_vecs == 4 ? vec & 3 : 0;
@@ -264,59 +269,63 @@ __device__ __forceinline__ int sample_element(const SiftCfg& cfg, int vec, int e
   return piece < kSiftPieces && k * ev < cfg.piece_stride && at < V ? at : -1;
 }
 
+// the sampled vectors of one thread
+template <int DTYPE, bool HAS_U, int NT>
+struct SampleLoad {
+  static constexpr int NV = 4 * kSiftPieces / NT;
+  uint4 c[NV], u[HAS_U ? NV : 1];
+  __device__ __forceinline__ void load(const SiftCfg& cfg, int V, const char* c_row, const char* u_row, int tid) {
+    constexpr int EV = SiftTraits<DTYPE>::kVec, ES = SiftTraits<DTYPE>::kElem;
+#pragma unroll
+    for (int j = 0; j < NV; ++j) {
+      const int e = max(sample_element(cfg, tid + j * NT, EV, V), 0);  // a vector that is not there: the row's first, not counted
+      c[j] = ldg_now(c_row + (size_t)e * ES);
+      if (HAS_U) u[HAS_U ? j : 0] = ldg_now(u_row + (size_t)e * ES);
+    }
+  }
+};
+
 template <int DTYPE, bool HAS_U, bool HAS_T, int NT>
-__device__ __forceinline__ SiftBinning sift_sample(const RowArgs& a, const SiftCfg& cfg, SiftShared& sm, uint32_t* hist,
-                                                   const char* c_row, const char* u_row, int tid, int bar) {
-  constexpr int EV = SiftTraits<DTYPE>::kVec, ES = SiftTraits<DTYPE>::kElem;
+__device__ __forceinline__ SiftBinning sift_sample(const RowArgs& a, const SiftCfg& cfg, SiftShared& sm, SiftHist& hist,
+                                                   const SampleLoad<DTYPE, HAS_U, NT>& in, int tid, int bar) {
+  constexpr int EV = SiftTraits<DTYPE>::kVec;
   constexpr int NV = 4 * kSiftPieces / NT;  // vectors per thread
   const int lane = tid & 31, warp = tid >> 5;
   const float neg_inf = __int_as_float(0xff800000), lowest = -3.402823466e38f;
   const uint64_t s2 = pack2(a.s, a.s), t2 = pack2(a.inv_T, a.inv_T);
   float v[NV][EV];  // v[j][0]: the vector's maximum (by_vectors), or the vector's elements
-  uint32_t have = 0;
-  uint4 c[NV], u[NV];
-#pragma unroll
-  for (int j = 0; j < NV; ++j) {
-    const int e = sample_element(cfg, tid + j * NT, EV, a.V);
-    c[j] = u[j] = make_uint4(0u, 0u, 0u, 0u);
-    if (e >= 0) {
-      have |= 1u << j;
-      c[j] = __ldg(reinterpret_cast<const uint4*>(c_row + (size_t)e * ES));
-      if (HAS_U) u[j] = __ldg(reinterpret_cast<const uint4*>(u_row + (size_t)e * ES));
-    }
-  }
   float top = neg_inf;
   const bool by_vectors = cfg.by_vectors != 0;
 #pragma unroll
   for (int j = 0; j < NV; ++j) {
     uint64_t y[EV / 2];
-    merge_vec<DTYPE, HAS_U, HAS_T>(c[j], u[j], s2, t2, y);
+    merge_vec<DTYPE, HAS_U, HAS_T>(in.c[j], in.u[HAS_U ? j : 0], s2, t2, y);
     float m = neg_inf;
 #pragma unroll
     for (int k = 0; k < EV / 2; ++k) {
       unpack2(y[k], v[j][2 * k], v[j][2 * k + 1]);
       m = max3(m, v[j][2 * k], v[j][2 * k + 1]);
     }
-    const bool in = (have >> j) & 1u;
-    m = in ? canonical(m) : neg_inf;
+    const bool there = sample_element(cfg, tid + j * NT, EV, a.V) >= 0;
+    m = there ? canonical(m) : neg_inf;
     top = fmaxf(top, m);
     // an atomic with part of its lanes off runs several times slower than one with all lanes on: what is not there
     // counts as -inf, below every threshold
     if (by_vectors) {
       v[j][0] = m;
-      atomicAdd(&hist[float_key(m) >> kSiftKeyShift], 1u);
+      hist.count(float_key(m) >> kSiftKeyShift);
     } else {
 #pragma unroll
       for (int k = 0; k < EV; ++k) {
-        v[j][k] = in ? canonical(v[j][k]) : neg_inf;
-        atomicAdd(&hist[float_key(v[j][k]) >> kSiftKeyShift], 1u);
+        v[j][k] = there ? canonical(v[j][k]) : neg_inf;
+        hist.count(float_key(v[j][k]) >> kSiftKeyShift);
       }
     }
   }
   const uint32_t warp_top = __reduce_max_sync(0xffffffffu, float_key(top));
   if (lane == 0) atomicMax(&sm.top_key, warp_top);
   row_sync<NT>(bar);
-  if (warp == 0) rank_search(&sm, hist, (uint32_t)cfg.rank, 0u);
+  if (warp == 0) rank_search(&sm, &hist, (uint32_t)cfg.rank);
   row_sync<NT>(bar);
   float floor_y = key_float(sm.rank_bin << kSiftKeyShift);
   if (!(floor_y >= lowest)) floor_y = lowest;  // the edge fell on -inf or into the NaN patterns
@@ -324,7 +333,7 @@ __device__ __forceinline__ SiftBinning sift_sample(const RowArgs& a, const SiftC
   const bool refine = floor_y > lowest && top_y >= floor_y && top_y <= 3.402823466e38f;
   const float range = __fsub_rn(top_y, floor_y);
   const float scale = (refine && range > 0.0f) ? __fdiv_rn((float)kSiftBins - 1.5f, range) : 0.0f;
-  SiftBinning bins{lowest, 0.0f, 0.0f, (float)kSiftBins};
+  float tau0 = lowest;
   if (refine) {
     // bins 1 .. kSiftBins - 1; what lies below the floor counts in bin 0 (a negative argument converts to 0)
 #pragma unroll
@@ -334,27 +343,87 @@ __device__ __forceinline__ SiftBinning sift_sample(const RowArgs& a, const SiftC
         if (k > 0 && by_vectors) break;
         const float x = v[j][k];
         const uint32_t bin = x >= floor_y ? __float2uint_rz(__fmaf_rn(__fsub_rn(x, floor_y), scale, 1.0f)) : 0u;
-        atomicAdd(&hist[min(bin, (uint32_t)kSiftBins - 1u)], 1u);
+        hist.count(min(bin, (uint32_t)kSiftBins - 1u));
       }
     }
     row_sync<NT>(bar);
-    if (warp == 0) rank_search(&sm, hist, (uint32_t)cfg.rank, (uint32_t)cfg.rank_high);
+    if (warp == 0) rank_search(&sm, &hist, (uint32_t)cfg.rank);
     row_sync<NT>(bar);
-    const float tbin = (float)sm.rank_bin, hbin = (float)sm.rank_bin2;
-    bins.tau0 = floor_y;
-    if (scale > 0.0f) {
-      const float width = __fdiv_rn(1.0f, scale);
-      // a little below the lower edge of the bin, so that rounding cannot exclude one of its members
-      if (tbin > 1.0f) bins.tau0 = __fmaf_rd(__fmul_rd(tbin - 1.0f, 0.9999f), width, floor_y);
-      const float high = __fsub_rn(__fmaf_rn(hbin, width, floor_y), bins.tau0);
-      const float rest = __fsub_rn(__fsub_rn(top_y, bins.tau0), high);
-      bins.s1 = __fdiv_rn((float)kBinsLow, fmaxf(high, width));
-      // (never the steeper line: it would undercut the first one below their crossing)
-      bins.s2 = rest > 0.0f ? fminf(__fdiv_rn((float)(kSiftBins - 2 - kBinsLow), rest), bins.s1) : 0.0f;
-      bins.c2 = __fmaf_rn(-high, bins.s2, (float)(kBinsLow + 1));
+    const float tbin = (float)sm.rank_bin;
+    tau0 = floor_y;
+    // a little below the lower edge of the bin, so that rounding cannot exclude one of its members
+    if (tbin > 1.0f && scale > 0.0f) tau0 = __fmaf_rd(__fmul_rd(tbin - 1.0f, 0.9999f), __fdiv_rn(1.0f, scale), floor_y);
+  }
+  return sift_bins(tau0, top_y);
+}
+
+// The same by ONE warp, for a row that is not wanted yet: no barriers, and the vectors' maxima stay in registers, rounded
+// to bf16 pairs, through a binary search for the rank (sixteen packed comparisons and additions a step).  A few
+// thousand cycles that nobody waits for; the whole team would be held up by its barriers for as long.
+template <int DTYPE, bool HAS_U, bool HAS_T>
+__device__ __forceinline__ float2 sift_sample_ahead(const RowArgs& a, const SiftCfg& cfg, const char* c_row, const char* u_row, int lane) {
+  constexpr int EV = SiftTraits<DTYPE>::kVec, ES = SiftTraits<DTYPE>::kElem;
+  constexpr int NV = 4 * kSiftPieces / 32, BATCH = 4;
+  const uint64_t s2 = pack2(a.s, a.s), t2 = pack2(a.inv_T, a.inv_T);
+  uint32_t m2[NV / 2];  // maxima as bf16 pairs
+  float top = __int_as_float(0xff800000);
+#pragma unroll
+  for (int j0 = 0; j0 < NV; j0 += BATCH) {
+    uint4 c[BATCH], u[BATCH];
+    int e[BATCH];
+#pragma unroll
+    for (int j = 0; j < BATCH; ++j) {
+      e[j] = sample_element(cfg, lane + 32 * (j0 + j), EV, a.V);
+      const size_t at = (size_t)max(e[j], 0) * ES;
+      c[j] = ldg_now(c_row + at);
+      u[j] = HAS_U ? ldg_now(u_row + at) : c[j];
+    }
+    float m[BATCH];
+#pragma unroll
+    for (int j = 0; j < BATCH; ++j) {
+      uint64_t y[EV / 2];
+      merge_vec<DTYPE, HAS_U, HAS_T>(c[j], u[j], s2, t2, y);
+      float x = __int_as_float(0xff800000);
+#pragma unroll
+      for (int k = 0; k < EV / 2; ++k) {
+        float y0, y1;
+        unpack2(y[k], y0, y1);
+        x = max3(x, y0, y1);
+      }
+      m[j] = e[j] >= 0 ? x : __int_as_float(0xff800000);
+      top = fmaxf(top, m[j]);
+    }
+#pragma unroll
+    for (int j = 0; j < BATCH; j += 2) {
+      asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(m2[(j0 + j) / 2]) : "f"(m[j + 1]), "f"(m[j]));
     }
   }
-  return bins;
+  // largest 16-bit key whose value at least `rank` of the maxima reach (keys are ordered like the values)
+  uint32_t key = 0;
+#pragma unroll 1
+  for (uint32_t bit = 0x8000u; bit != 0u; bit >>= 1) {
+    const uint32_t k = key | bit;
+    const uint32_t v = (k & 0x8000u) ? k & 0x7fffu : ~k & 0xffffu;  // bf16 pattern of the key
+    const uint32_t t = v | (v << 16);
+    uint32_t acc0 = 0, acc1 = 0;
+#pragma unroll
+    for (int x = 0; x < NV / 2; x += 2) {
+      uint32_t g0, g1;
+      asm("set.ge.bf16x2.bf16x2 %0, %1, %2;" : "=r"(g0) : "r"(m2[x]), "r"(t));
+      asm("set.ge.bf16x2.bf16x2 %0, %1, %2;" : "=r"(g1) : "r"(m2[x + 1]), "r"(t));
+      asm("add.rn.bf16x2 %0, %0, %1;" : "+r"(acc0) : "r"(g0));
+      asm("add.rn.bf16x2 %0, %0, %1;" : "+r"(acc1) : "r"(g1));
+    }
+    asm("add.rn.bf16x2 %0, %0, %1;" : "+r"(acc0) : "r"(acc1));
+    const uint32_t n = __reduce_add_sync(0xffffffffu, (uint32_t)(bf16_lo(acc0) + bf16_hi(acc0)));
+    if (n >= (uint32_t)cfg.rank) key = k;
+  }
+  top = key_float(__reduce_max_sync(0xffffffffu, float_key(canonical(top))));
+  // The maxima were rounded to nearest: the middle between this bf16 value and the one below is what they all reach.
+  const float at = key_float(key << 16), below = key_float((key - 1u) << 16);
+  float tau0 = __fmaf_rd(__fsub_rn(at, below), -0.51f, at);
+  if (key == 0u || !(tau0 >= -3.402823466e38f) || !(top <= 3.402823466e38f)) tau0 = -3.402823466e38f;
+  return make_float2(tau0, top);
 }
 
 // ---------------------------------------------------------------------------------------------------
@@ -404,7 +473,7 @@ __device__ __forceinline__ uint32_t put_ids(uint32_t x, uint32_t first, uint32_t
 // where a warp's candidates go
 struct SiftTarget {
   uint32_t y_at, id_at;    // shared-memory addresses of the segment's lists (of the cluster's first CTA when REMOTE)
-  uint32_t hist_at;        // of the candidates' histogram
+  uint32_t hist_at;        // of the candidates' histogram (a SiftHist)
   uint32_t scratch_at;     // local id list (the same as id_at unless REMOTE)
 };
 
@@ -479,6 +548,7 @@ __device__ __forceinline__ void sift_unit(const RowArgs& a, uint32_t c_unit, uin
     const float y = merge_entry<DTYPE, HAS_U, HAS_T>(c_rel + id * (uint32_t)ES, u_rel + id * (uint32_t)ES, a.s, a.inv_T);
     const uint32_t bin = in ? min(__float2uint_rz(bins.at(y)), (uint32_t)kSiftBins - 1u) : 0u;
     count_at<REMOTE>(to.hist_at + 4u * bin);
+    count_at<REMOTE>(to.hist_at + 4u * (kSiftBins + (bin >> 5)));
     vmax = fmaxf(vmax, y);
     if (in) {
       put_f32<REMOTE>(to.y_at + 4u * k, y);
@@ -512,7 +582,7 @@ __device__ __forceinline__ bool finish_row(const RowArgs& a, const SiftCfg& cfg,
   const uint32_t kcap = (uint32_t)a.kcap;
   const uint32_t below = (1u << lane) - 1u;
   row_sync<NT>(bar);
-  if (warp == 0) rank_search(&sm, sm.hist, kcap, 0u);
+  if (warp == 0) rank_search(&sm, &sm.hist, kcap);
   if (tid == NT - 1) {
     // the row's own random number, needed at the end
     const Philox4 r = philox4x32_10((uint32_t)pos, (uint32_t)(a.seq_base + row / a.W), (uint32_t)iter, (uint32_t)a.purpose, a.seed_lo,
@@ -548,7 +618,7 @@ __device__ __forceinline__ bool finish_row(const RowArgs& a, const SiftCfg& cfg,
 #pragma unroll 2
       for (uint32_t i = (uint32_t)lane; i < n; i += 32u) {
         const float y = y_g[i], x = bins.at(y);
-        if (x >= lo && x < hi) sm.member[atomicAdd(&sm.members, 1)] = SiftMember{y, id0 + (int32_t)my_id[g * cfg.seg_cap + i]};
+        if (x >= lo && x < hi) sm.hist.member[atomicAdd(&sm.members, 1)] = SiftMember{y, id0 + (int32_t)my_id[g * cfg.seg_cap + i]};
       }
     }
   }
@@ -558,13 +628,12 @@ __device__ __forceinline__ bool finish_row(const RowArgs& a, const SiftCfg& cfg,
   int thr_id;
   if (nbin <= 32u) {
     // every warp ranks them for itself, a lane per member
-    SiftMember me{0.0f, 0};
-    if (lane < (int)nbin) me = sm.member[lane];
+    const SiftMember me = sm.hist.member[min(lane, (int)nbin - 1)];
     uint32_t ahead = 0;
+#pragma unroll 4
     for (int x = 0; x < (int)nbin; ++x) {
-      const float oy = __shfl_sync(0xffffffffu, me.y, x);
-      const int oid = __shfl_sync(0xffffffffu, me.id, x);
-      ahead += (oy > me.y || (oy == me.y && oid < me.id)) ? 1u : 0u;
+      const SiftMember o = sm.hist.member[x];
+      ahead += (o.y > me.y || (o.y == me.y && o.id < me.id)) ? 1u : 0u;
     }
     const int who = __ffs((int)__ballot_sync(0xffffffffu, lane < (int)nbin && ahead == need - 1u)) - 1;
     thr_y = __shfl_sync(0xffffffffu, me.y, who);
@@ -572,10 +641,10 @@ __device__ __forceinline__ bool finish_row(const RowArgs& a, const SiftCfg& cfg,
   } else {
     // a warp per member, a lane per rival
     for (uint32_t x = (uint32_t)warp; x < nbin; x += NW) {
-      const SiftMember me = sm.member[x];
+      const SiftMember me = sm.hist.member[x];
       uint32_t ahead = 0;
       for (uint32_t z = (uint32_t)lane; z < nbin; z += 32u) {
-        const SiftMember o = sm.member[z];
+        const SiftMember o = sm.hist.member[z];
         ahead += (o.y > me.y || (o.y == me.y && o.id < me.id)) ? 1u : 0u;
       }
       ahead = __reduce_add_sync(0xffffffffu, ahead);
@@ -625,7 +694,7 @@ __device__ __forceinline__ bool finish_row(const RowArgs& a, const SiftCfg& cfg,
     sm.wz[warp] = z;
   }
   row_sync<NT>(bar);
-  for (uint32_t x = (uint32_t)tid; x < nbin; x += NT) sm.member[x] = SiftMember{0.0f, 0};  // the histogram's words again
+  for (uint32_t x = (uint32_t)tid; x < nbin; x += NT) sm.hist.member[x] = SiftMember{0.0f, 0};  // the histogram's words again
   if (tid == 0) sm.members = 0;
   const uint32_t cw = lane < NW ? sm.wcnt[lane] : 0u;
   const uint32_t before = __reduce_add_sync(0xffffffffu, lane < warp ? cw : 0u);
@@ -700,13 +769,13 @@ __device__ __forceinline__ bool finish_row(const RowArgs& a, const SiftCfg& cfg,
 }
 
 // row_generic as a call of its own: it is rarely needed and its registers and code stay out of the hot loops.
-template <int DTYPE, int NT>
+template <int DTYPE, int NT, int BAR>
 __device__ __noinline__ void sift_redo(const RowArgs& a, int row, int tid, GenericSmem& sm) {
-  row_generic<DTYPE, NT, 0>(a, row, tid, sm, kRowStatusRedone);
+  row_generic<DTYPE, NT, BAR>(a, row, tid, sm, kRowStatusRedone);
 }
 
 __device__ __forceinline__ void init_shared(SiftShared& sm, int tid, int nt) {
-  for (int k = tid; k < kSiftBins / 4; k += nt) reinterpret_cast<uint4*>(sm.hist)[k] = make_uint4(0u, 0u, 0u, 0u);
+  for (int k = tid; k < (int)sizeof(SiftHist) / 16; k += nt) reinterpret_cast<uint4*>(&sm.hist)[k] = make_uint4(0u, 0u, 0u, 0u);
   if (tid == 0) {
     sm.top_key = 0u;
     sm.max_key = 0u;
@@ -745,6 +814,9 @@ struct alignas(16) StreamShared {
   // parity wait tells a phase from its neighbours only, so each barrier is waited on by one warp, phase after phase.
   uint64_t full[kTeamWarps * kMaxTeams * kMaxSlots];
   uint32_t used[kTeamWarps * kMaxTeams * kMaxSlots];  // copies issued for that barrier so far
+  // thresholds of a team's rows after its first: {tau0, largest sample value}, two places used in turn
+  uint64_t tau_full[kMaxTeams * 2], tau_free[kMaxTeams * 2];
+  float2 tau[kMaxTeams * 2];
   uint32_t seg_n[kMaxTeams * kTeamWarps];      // candidates per segment
   int32_t redo[kStreamRows];                   // rows the single pass could not finish (redone at the end)
   int n_live, n_redo, abort;
@@ -779,25 +851,31 @@ __device__ __forceinline__ bool sift_wait(uint64_t* bar, uint32_t parity, volati
 }
 
 template <int DTYPE, bool HAS_U, bool HAS_T>
-__global__ void __launch_bounds__(kTeamThreads * kMaxTeams, 1)
+__global__ void __launch_bounds__((kTeamThreads + 32) * kMaxTeams, 1)
 rows_stream_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ SiftCfg cfg) {
   constexpr int ES = SiftTraits<DTYPE>::kElem, EU = SiftTraits<DTYPE>::kUnit;
   constexpr uint32_t kSlot = kUnitBytes * (HAS_U ? 2u : 1u);
   extern __shared__ __align__(128) unsigned char smem_raw[];
   StreamShared& st = *reinterpret_cast<StreamShared*>(smem_raw);
   const int teams = cfg.teams, slots = cfg.slots;
-  const int team = (int)threadIdx.x / kTeamThreads;
-  const int tid = (int)threadIdx.x % kTeamThreads, lane = tid & 31, warp = tid >> 5, bar = 1 + team;
+  // warps: those of team 0, of team 1, ..., then a sampler for each team
+  const bool sampler = (int)threadIdx.x >= teams * kTeamThreads;
+  const int team = sampler ? ((int)threadIdx.x - teams * kTeamThreads) >> 5 : (int)threadIdx.x / kTeamThreads;
+  const int tid = sampler ? (int)threadIdx.x & 31 : (int)threadIdx.x % kTeamThreads, lane = tid & 31, warp = tid >> 5, bar = 1 + team;
   SiftShared* const team_sm = reinterpret_cast<SiftShared*>(smem_raw + sizeof(StreamShared));
   SiftShared& sm = team_sm[team];
   float* const lists = reinterpret_cast<float*>(team_sm + teams);
   float* const list_y = lists + (size_t)team * kTeamWarps * cfg.seg_cap;
   uint16_t* const list_id = reinterpret_cast<uint16_t*>(lists + (size_t)teams * kTeamWarps * cfg.seg_cap) + (size_t)team * kTeamWarps * cfg.seg_cap;
   unsigned char* const ring = smem_raw + sift_stream_rings(teams, cfg.seg_cap) + (size_t)warp * slots * kSlot;
-  init_shared(sm, tid, kTeamThreads);
+  if (!sampler) init_shared(sm, tid, kTeamThreads);
   if (threadIdx.x < kTeamWarps * kMaxTeams * kMaxSlots) {
     mbar_init(&st.full[threadIdx.x], 1);
     st.used[threadIdx.x] = 0;
+  }
+  if (threadIdx.x < kMaxTeams * 2) {
+    mbar_init(&st.tau_full[threadIdx.x], 1);
+    mbar_init(&st.tau_free[threadIdx.x], kTeamWarps);
   }
   if (threadIdx.x == 0) {
     st.n_redo = 0;
@@ -828,20 +906,46 @@ rows_stream_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ Si
   }
   __syncthreads();
   const int n_live = st.n_live;
+  volatile int* const abort_flag = &st.abort;
+  if (sampler) {
+    // ======================================= samplers =======================================
+    // thresholds of the team's rows after its first, one or two rows ahead
+    int at = 0;
+    uint32_t round = 0;
+    for (int k = team + teams; k < n_live && cfg.by_vectors; k += teams) {
+      const int64_t off = st.tab[k].off;
+      const float2 tau = sift_sample_ahead<DTYPE, HAS_U, HAS_T>(a, cfg, static_cast<const char*>(row_ptr(a.cond, DTYPE, off)),
+                                                                HAS_U ? static_cast<const char*>(row_ptr(a.uncond, DTYPE, off)) : nullptr, lane);
+      const int x = 2 * team + at;
+      if (round > 0 && !sift_wait(&st.tau_free[x], (round - 1u) & 1u, abort_flag)) break;
+      if (lane == 0) {
+        st.tau[x] = tau;
+        mbar_arrive(&st.tau_full[x]);
+      }
+      __syncwarp();
+      round += (uint32_t)at;
+      at ^= 1;
+    }
+    __syncthreads();
+    return;
+  }
   const int seg0 = warp * cfg.seg_len;
   const int seg_n = min(max(a.V - seg0, 0), cfg.seg_len);  // ids of this warp's segment
   const int units = (seg_n + EU - 1) / EU;
   // Copies go through the ring of the warp's segment in order: the units of the segment for row 0, row 1, ...; team t takes
   // rows t, t + teams, ...  Whoever has worked a unit through asks for the copy that goes into its slot next.
   auto issue = [&](int k, int unit, int slot) {
-    if (unit >= units) {
-      k += unit / units;
-      unit = unit % units;
+    while (unit >= units) {
+      ++k;
+      unit -= units;
     }
     if (k >= n_live) return;
     const uint32_t bytes = (uint32_t)min(seg_n - unit * EU, EU) * ES;
     const int64_t off = st.tab[k].off + seg0 + (int64_t)unit * EU;
     unsigned char* const dst = ring + (size_t)slot * kSlot;
+#ifdef SJD_TEST_DROP_COPY
+    if (warp == SJD_TEST_DROP_COPY && k == 1 && unit == 0) return;  // test builds only, see rows_cluster_kernel
+#endif
     const int x = (warp * kMaxTeams + k % teams) * kMaxSlots + slot;
     ++st.used[x];
     mbar_arrive_expect_tx(&st.full[x], bytes * (HAS_U ? 2u : 1u));
@@ -855,21 +959,34 @@ rows_stream_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ Si
   SiftTarget to;
   to.y_at = smem_u32(list_y + warp * cfg.seg_cap);
   to.id_at = to.scratch_at = smem_u32(list_id + warp * cfg.seg_cap);
-  to.hist_at = smem_u32(sm.hist);
+  to.hist_at = smem_u32(&sm.hist);
   const uint32_t ring_at = smem_u32(ring), cap = (uint32_t)cfg.seg_cap;
-  volatile int* const abort_flag = &st.abort;
   uint64_t* const full = st.full + (warp * kMaxTeams + team) * kMaxSlots;
-  uint32_t phase = 0;  // bit s: parity of the next phase of full[s]
+  uint32_t phase = 0;      // bit s: parity of the next phase of full[s]
+  int tau_at = 0;          // thresholds come through two places in turn
+  uint32_t tau_phase = 0;
   for (int k = team; k < n_live; k += teams) {
     // from the CTA's last row on, the verification grid may be scheduled (it waits for this grid's end)
     if (k == n_live - 1) allow_dependent_launch();
-    const int64_t off = st.tab[k].off;
-    const SiftBinning bins = sift_sample<DTYPE, HAS_U, HAS_T, kTeamThreads>(
-        a, cfg, sm, sm.hist, static_cast<const char*>(row_ptr(a.cond, DTYPE, off)),
-        HAS_U ? static_cast<const char*>(row_ptr(a.uncond, DTYPE, off)) : nullptr, tid, bar);
+    bool ok = *abort_flag == 0;
+    SiftBinning bins;
+    if (k == team || !cfg.by_vectors) {
+      SampleLoad<DTYPE, HAS_U, kTeamThreads> sample;
+      const int64_t off = st.tab[k].off;
+      sample.load(cfg, a.V, static_cast<const char*>(row_ptr(a.cond, DTYPE, off)),
+                  HAS_U ? static_cast<const char*>(row_ptr(a.uncond, DTYPE, off)) : nullptr, tid);
+      bins = sift_sample<DTYPE, HAS_U, HAS_T, kTeamThreads>(a, cfg, sm, sm.hist, sample, tid, bar);
+    } else {
+      const int x = 2 * team + tau_at;
+      if (ok) ok = sift_wait(&st.tau_full[x], tau_phase, abort_flag);
+      bins = sift_bins(st.tau[x].x, st.tau[x].y);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&st.tau_free[x]);
+      tau_phase ^= (uint32_t)tau_at;
+      tau_at ^= 1;
+    }
     uint32_t n = 0;
     float vmax = __int_as_float(0xff800000);
-    bool ok = *abort_flag == 0;
     int slot = (k * units) % slots;
     for (int unit = 0; unit < units; ++unit) {
       if (ok) ok = sift_wait(&full[slot], (phase >> slot) & 1u, abort_flag);
@@ -912,9 +1029,9 @@ rows_stream_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ Si
   const int n_redo = st.n_redo;
   for (int x = 0; x < n_redo; ++x) {
     GenericSmem& gs = *reinterpret_cast<GenericSmem*>(team_sm);
-    if (teams == 3) sift_redo<DTYPE, 3 * kTeamThreads>(a, st.redo[x], (int)threadIdx.x, gs);
-    else if (teams == 2) sift_redo<DTYPE, 2 * kTeamThreads>(a, st.redo[x], (int)threadIdx.x, gs);
-    else sift_redo<DTYPE, kTeamThreads>(a, st.redo[x], (int)threadIdx.x, gs);
+    if (teams == 3) sift_redo<DTYPE, 3 * kTeamThreads, 1>(a, st.redo[x], (int)threadIdx.x, gs);
+    else if (teams == 2) sift_redo<DTYPE, 2 * kTeamThreads, 1>(a, st.redo[x], (int)threadIdx.x, gs);
+    else sift_redo<DTYPE, kTeamThreads, 1>(a, st.redo[x], (int)threadIdx.x, gs);
   }
 }
 
@@ -923,7 +1040,7 @@ rows_stream_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ Si
 // ---------------------------------------------------------------------------------------------------
 struct alignas(16) ClusterShared {
   SiftShared row;                                // the first CTA's: histogram of the candidates, finish phase
-  uint32_t hist_s[kSiftBins];                    // the sample's histogram
+  SiftHist hist_s;                               // the sample's histogram
   uint64_t full[kClusterWarps];                  // a warp's segment has landed
   uint32_t seg_n[kClusterWarps * kMaxCluster];   // candidates per segment (the first CTA's)
   uint32_t lost;                                 // a bounded wait of the cluster gave up (the first CTA's)
@@ -978,7 +1095,7 @@ rows_cluster_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ S
   const int row = (int)(blockIdx.x / csize);
   const uint64_t s2 = pack2(a.s, a.s), t2 = pack2(a.inv_T, a.inv_T);
   init_shared(sm.row, tid, NT);
-  for (int k = tid; k < kSiftBins / 4; k += NT) reinterpret_cast<uint4*>(sm.hist_s)[k] = make_uint4(0u, 0u, 0u, 0u);
+  for (int k = tid; k < (int)sizeof(SiftHist) / 16; k += NT) reinterpret_cast<uint4*>(&sm.hist_s)[k] = make_uint4(0u, 0u, 0u, 0u);
   if (tid < kClusterWarps) mbar_init(&sm.full[tid], 1);
   if (tid == 0) sm.lost = 0u;
   fence_barrier_init();
@@ -1017,11 +1134,13 @@ rows_cluster_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ S
   }
   __syncwarp();
   // every CTA of the cluster finds the threshold for itself: the sample is small, an exchange would cost more
-  const SiftBinning bins = sift_sample<DTYPE, HAS_U, HAS_T, NT>(a, cfg, sm.row, sm.hist_s, c_row, u_row, tid, 0);
+  SampleLoad<DTYPE, HAS_U, NT> sample;
+  sample.load(cfg, a.V, c_row, u_row, tid);
+  const SiftBinning bins = sift_sample<DTYPE, HAS_U, HAS_T, NT>(a, cfg, sm.row, sm.hist_s, sample, tid, 0);
   SiftTarget to;
   to.y_at = in_first_cta(list_y + (size_t)seg * cfg.seg_cap);
   to.id_at = in_first_cta(list_id + (size_t)seg * cfg.seg_cap);
-  to.hist_at = in_first_cta(sm.row.hist);
+  to.hist_at = in_first_cta(&sm.row.hist);
   to.scratch_at = smem_u32(csize > 1 ? local_id + (size_t)warp * cfg.seg_cap : list_id + (size_t)seg * cfg.seg_cap);
   const uint32_t cap = (uint32_t)cfg.seg_cap;
   const uint32_t bias = (uint32_t)((seg % (int)csize) * cfg.seg_len);  // ids are kept relative to the finishing warp's first one
@@ -1057,7 +1176,7 @@ rows_cluster_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ S
     return;
   }
   if (!finish_row<kClusterWarps>(a, cfg, sm.row, list_y, list_id, sm.seg_n, (int)csize, bins, row, r.pos, r.iter, r.draft, tid, 0))
-    sift_redo<DTYPE, NT>(a, row, tid, *reinterpret_cast<GenericSmem*>(sm.hist_s));
+    sift_redo<DTYPE, NT, 0>(a, row, tid, *reinterpret_cast<GenericSmem*>(&sm.hist_s));
 }
 
 }  // namespace sjd

@@ -13,7 +13,6 @@
 #include "device_utils.cuh"
 #include "row_kernels.cuh"
 #include "rows_pipeline.cuh"
-#include "rows_ranges.cuh"
 #include "rows_sift.cuh"
 #include "verify_kernel.cuh"
 #include "advance_kernel.cuh"
@@ -124,98 +123,6 @@ bool plan_pipeline(const sjd_params* P, int kcap, sjd::PipeCfg* cfg, size_t* sme
   return false;
 }
 
-// ---- the kernel with one id range per filter thread (rows_ranges.cuh) ----
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-// cuTensorMapEncodeTiled through the runtime (no link against the driver library); nullptr when unavailable.
-EncodeTiledFn encode_tiled_fn() {
-  static EncodeTiledFn fn = [] {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult qr;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &qr) != cudaSuccess ||
-        qr != cudaDriverEntryPointSuccess)
-      p = nullptr;
-    return reinterpret_cast<EncodeTiledFn>(p);
-  }();
-  return fn;
-}
-
-// Same sampling rule as plan_pipeline; the sample is stage 0, i.e. 1/S of the row.
-bool plan_ranges(const sjd_params* P, int kcap, sjd::RangeCfg* cfg, size_t* smem, bool need_encoder = true) {
-  const int V = P->V;
-  const int es = P->logits_dtype == SJD_F32 ? 4 : 2;
-  const int bw = 64 / es;  // elements per stage and range
-  if (kcap > sjd::kKcapMax || V % sjd::kRangeThreads != 0) return false;
-  const int R = V / sjd::kRangeThreads;
-  if (R % bw != 0) return false;
-  const int S = R / bw;
-  if (S < 2 || S > 16) return false;
-  // all rows must lie at one pitch: row r = b W + i starts at r * stride_w
-  if (P->B > 1 && P->stride_b != (int64_t)P->W * P->stride_w) return false;
-  if ((int64_t)P->B * P->W >= (1ll << 31)) return false;
-  const int mask_words = (R / 2 + 31) / 32;
-  if (mask_words > sjd::kMaskWordsMax) return false;
-  const int n_sample = sjd::kRangeThreads * bw;
-  const double a = (double)kcap / S;
-  int m = sample_rank(a);
-  if (m > n_sample / 2) return false;
-  // The element rank m can be taken as a rank among the maxima of the sample's groups of eight (see the
-  // sampler): directly while at most a tenth of the sample lies above the threshold.  Up to a fifth the group
-  // maxima still resolve the rank, but up to 1.6 times less sharply than the elements would: a margin of 6.5
-  // instead of 4.5 standard deviations keeps the row at least as safe.  Beyond that every element is binned.
-  bool by_groups = m <= n_sample / 8 && (double)m / n_sample <= 0.10;
-  if (!by_groups) {
-    const int m_wide = sample_rank(a, 6.5);
-    if ((double)m_wide / n_sample <= 0.20) {
-      m = m_wide;
-      by_groups = true;
-    }
-  }
-  const int sample_all = m > n_sample / 8 ? 1 : 0;  // the rank must exist among what an element-wise first pass bins
-  // candidates of a row: m S on average; pairs of neighbours with at least one candidate: a little fewer
-  const double cand = (double)m * S, cand_sd = (double)S * std::sqrt((double)m);
-  const double thin = 1.0 - 0.5 * cand / V;
-  if ((cand + 5.0 * cand_sd) * thin > (double)sjd::kRangePairCap) return false;
-  // pair entries per filter thread: a Poisson count; its list must hold it with a tail below 1e-6
-  const double per_thread = cand * thin / sjd::kRangeThreads;
-  if (per_thread + 5.0 * std::sqrt(per_thread) + 1.0 > (double)(sjd::kRangeListCap - 4)) return false;
-  if (need_encoder && encode_tiled_fn() == nullptr) return false;
-  cfg->sample_rank = m;
-  cfg->sample_all = sample_all;
-  {
-    const double p = (double)m / n_sample, groups = n_sample / 8.0;
-    cfg->group_rank = by_groups ? (int)std::ceil(groups * (1.0 - std::pow(1.0 - p, 8.0))) : 0;
-  }
-  cfg->stages = S;
-  cfg->range_len = R;
-  cfg->mask_words = mask_words;
-  cfg->row_begin = 0;
-  cfg->row_end = P->B * P->W;
-  *smem = sjd::range_smem_bytes(mask_words);
-  return *smem <= kSmemLimit;
-}
-
-// Tensor map over one logits array: dims {R ids, 256 ranges, rows}, box {64 bytes, 256, 1}, 64-byte swizzle.
-// L2 promotion stays at the box's own 64 bytes per range: wider promotion fetches the neighbouring stages
-// early, and measured slower (128 bytes: +1.6 us, 256 bytes: +5 us on the headline workload) than the kernel's
-// own prefetch one ring depth ahead.
-bool make_range_map(CUtensorMap* map, const void* base, const sjd_params* P, const sjd::RangeCfg& cfg) {
-  const int es = P->logits_dtype == SJD_F32 ? 4 : 2;
-  const cuuint64_t dims[3] = {(cuuint64_t)cfg.range_len, (cuuint64_t)sjd::kRangeThreads, (cuuint64_t)P->B * (cuuint64_t)P->W};
-  const cuuint64_t strides[2] = {(cuuint64_t)cfg.range_len * es, (cuuint64_t)P->stride_w * es};
-  const cuuint32_t box[3] = {(cuuint32_t)(64 / es), (cuuint32_t)sjd::kRangeThreads, 1};
-  const cuuint32_t estr[3] = {1, 1, 1};
-  const CUresult r = encode_tiled_fn()(map, P->logits_dtype == SJD_BF16  ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16
-                                       : P->logits_dtype == SJD_F16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16
-                                                                    : CU_TENSOR_MAP_DATA_TYPE_FLOAT32,
-                                       3, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                                       CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_64B,
-                                       CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS;
-}
-
 // Launch as a programmatic dependent of the stream's previous kernel: when that kernel allows it (ours do
 // near their end), this grid's blocks are placed and set up early and wait inside the kernel
 // (grid_dependency_wait) until the previous kernel has completed.  After a kernel that does not take part,
@@ -241,39 +148,6 @@ cudaError_t launch_after(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t s
     attr[lc.numAttrs++].val.clusterDim.z = 1;
   }
   return cudaLaunchKernelEx(&lc, kern, std::forward<Args>(args)...);
-}
-
-constexpr int kSamplerWarps = 3;
-constexpr int kRangeFinisherWarps = 16;
-
-// One kernel per logits type and per combination of (guidance given, temperature applied, thresholds by
-// group maxima): each holds only the code its launch runs, which matters because the roles' code does not fit
-// the instruction caches comfortably.
-template <int DTYPE, bool HAS_U, bool HAS_T, bool BY_GROUPS>
-cudaError_t launch_ranges_as(const sjd::RowArgs& ra, const sjd::RangeCfg& cfg, const CUtensorMap& mc, const CUtensorMap& mu,
-                             size_t smem, int grid, cudaStream_t st) {
-  auto kern = sjd::rows_ranges_kernel<DTYPE, kRangeFinisherWarps, kSamplerWarps, HAS_U, HAS_T, BY_GROUPS>;
-  static sjd::DeviceOnce configured;  // per instantiation
-  const cudaError_t e = allow_large_smem(kern, configured, (int)kSmemLimit);
-  if (e != cudaSuccess) return e;
-  return launch_after(kern, dim3((unsigned)grid), dim3((8 + kRangeFinisherWarps + kSamplerWarps + 1) * 32), smem, st, true, 1, ra,
-                      cfg, mc, mu);
-}
-
-template <int DTYPE>
-cudaError_t launch_ranges(const sjd::RowArgs& ra, const sjd::RangeCfg& cfg, const CUtensorMap& mc, const CUtensorMap& mu,
-                          size_t smem, int grid, cudaStream_t st) {
-  const int which = (ra.uncond != nullptr ? 4 : 0) | (ra.inv_T != 1.0f ? 2 : 0) | (cfg.group_rank > 0 ? 1 : 0);
-  switch (which) {
-    case 0: return launch_ranges_as<DTYPE, false, false, false>(ra, cfg, mc, mu, smem, grid, st);
-    case 1: return launch_ranges_as<DTYPE, false, false, true>(ra, cfg, mc, mu, smem, grid, st);
-    case 2: return launch_ranges_as<DTYPE, false, true, false>(ra, cfg, mc, mu, smem, grid, st);
-    case 3: return launch_ranges_as<DTYPE, false, true, true>(ra, cfg, mc, mu, smem, grid, st);
-    case 4: return launch_ranges_as<DTYPE, true, false, false>(ra, cfg, mc, mu, smem, grid, st);
-    case 5: return launch_ranges_as<DTYPE, true, false, true>(ra, cfg, mc, mu, smem, grid, st);
-    case 6: return launch_ranges_as<DTYPE, true, true, false>(ra, cfg, mc, mu, smem, grid, st);
-    default: return launch_ranges_as<DTYPE, true, true, true>(ra, cfg, mc, mu, smem, grid, st);
-  }
 }
 
 template <int DTYPE>
@@ -338,9 +212,6 @@ bool plan_sift(const sjd_params* P, int kcap, bool has_u, SiftPlan* plan) {
     return (int)std::ceil(c.by_vectors ? vecs * (1.0 - std::pow(1.0 - share, ev)) : share * vecs * ev);
   };
   c.rank = rank_of(p);
-  const double p_high = want - 3.0 * sd;
-  c.rank_high = p_high > 0 ? rank_of(p_high) : 1;
-  if (c.rank_high < 1) c.rank_high = 1;
   const int sms = sm_count();
   const int64_t rows = (int64_t)P->B * P->W;
   // few rows: as many CTAs per row as there are SMs for, as long as a warp has half a unit of its own
@@ -386,7 +257,7 @@ cudaError_t launch_sift_as(const sjd::RowArgs& ra, const SiftPlan& plan, cudaStr
     cfg.row_begin = (int)r0;
     cfg.row_end = (int)(r0 + per_launch < rows ? r0 + per_launch : rows);
     const int n = cfg.row_end - cfg.row_begin;
-    e = launch_after(kern, dim3((unsigned)(n < sm_count() ? n : sm_count())), dim3((unsigned)(cfg.teams * sjd::kTeamThreads)), plan.smem, st,
+    e = launch_after(kern, dim3((unsigned)(n < sm_count() ? n : sm_count())), dim3((unsigned)(cfg.teams * (sjd::kTeamThreads + 32))), plan.smem, st,
                      true, 1, ra, cfg);
     if (e == cudaSuccess && r0 > 0) ++g_launches;
   }
@@ -460,20 +331,6 @@ const char* sjd_last_cuda_error(void) { return g_cuda_error; }
 
 uint64_t sjd_launch_count(void) { return g_launches.load(); }
 
-#ifdef SJD_PHASE_TIMERS
-// Diagnostic builds only: copies the 48 phase counters to `out` (host) after a device synchronisation and
-// optionally clears them.
-int sjd_phase_cycles_read(unsigned long long* out, int reset) {
-  if (cudaDeviceSynchronize() != cudaSuccess) return SJD_ERR_CUDA;
-  if (cudaMemcpyFromSymbol(out, sjd::g_phase_cycles, sizeof(unsigned long long) * 48) != cudaSuccess) return SJD_ERR_CUDA;
-  if (reset) {
-    unsigned long long z[48] = {0};
-    if (cudaMemcpyToSymbol(sjd::g_phase_cycles, z, sizeof(z)) != cudaSuccess) return SJD_ERR_CUDA;
-  }
-  return SJD_OK;
-}
-#endif
-
 size_t sjd_workspace_bytes(const sjd_params* p) {
   if (!p || p->B < 0 || p->W < 1) return 0;
   const size_t rows = (size_t)p->B * (size_t)p->W;
@@ -533,28 +390,11 @@ int sjd_step(const void* logits_cond, const void* logits_uncond, const int32_t* 
   }
   {
     sjd::PipeCfg cfg;
-    sjd::RangeCfg rcfg;
     SiftPlan splan;
     size_t smem = 0;
     cudaError_t e;
-    CUtensorMap map_c, map_u;
     const bool fast = !(P->flags & (SJD_FLAG_FORCE_GENERIC | SJD_FLAG_FORCE_TILES));
-    if (fast && plan_ranges(P, kcap, &rcfg, &smem) && make_range_map(&map_c, logits_cond, P, rcfg) &&
-        make_range_map(&map_u, logits_uncond ? logits_uncond : logits_cond, P, rcfg)) {
-      // a CTA takes at most kRowsPerCta rows per launch: larger problems go in several launches
-      const int per_launch = sjd::kRowsPerCta * sm_count();
-      e = cudaSuccess;
-      for (int r0 = 0; r0 < rows && e == cudaSuccess; r0 += per_launch) {
-        rcfg.row_begin = r0;
-        rcfg.row_end = r0 + per_launch < rows ? r0 + per_launch : rows;
-        const int n = rcfg.row_end - r0;
-        const int grid = n < sm_count() ? n : sm_count();
-        e = P->logits_dtype == SJD_BF16  ? launch_ranges<1>(ra, rcfg, map_c, map_u, smem, grid, stream)
-            : P->logits_dtype == SJD_F16 ? launch_ranges<2>(ra, rcfg, map_c, map_u, smem, grid, stream)
-                                         : launch_ranges<0>(ra, rcfg, map_c, map_u, smem, grid, stream);
-        if (e == cudaSuccess && r0 > 0) ++g_launches;
-      }
-    } else if (fast && plan_sift(P, kcap, logits_uncond != nullptr, &splan)) {
+    if (fast && plan_sift(P, kcap, logits_uncond != nullptr, &splan)) {
       e = P->logits_dtype == SJD_BF16  ? launch_sift<1>(ra, splan, stream)
           : P->logits_dtype == SJD_F16 ? launch_sift<2>(ra, splan, stream)
                                        : launch_sift<0>(ra, splan, stream);
@@ -674,12 +514,10 @@ int sjd_row_kernel(const sjd_params* P) {
     return SJD_ERR_ALIGN;
   const int kcap = P->top_k < P->V ? P->top_k : P->V;
   sjd::PipeCfg cfg;
-  sjd::RangeCfg rcfg;
+  SiftPlan splan;
   size_t smem = 0;
   const bool fast = !(P->flags & (SJD_FLAG_FORCE_GENERIC | SJD_FLAG_FORCE_TILES));
-  SiftPlan splan;
-  if (fast && plan_ranges(P, kcap, &rcfg, &smem, false)) return SJD_ROWS_RANGES;
-  if (fast && plan_sift(P, kcap, true, &splan)) return SJD_ROWS_GENERIC;
+  if (fast && plan_sift(P, kcap, true, &splan)) return kcap <= sjd::kKcapMax ? SJD_ROWS_RANGES : SJD_ROWS_GENERIC;
   if (!(P->flags & SJD_FLAG_FORCE_GENERIC) && plan_pipeline(P, kcap, &cfg, &smem)) return SJD_ROWS_TILES;
   return SJD_ROWS_GENERIC;
 }

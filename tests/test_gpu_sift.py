@@ -26,6 +26,10 @@ def test_cutting_of_a_row(V, B, W, dtype):
     _check(f"cut{V}", B=B, W=W, V=V, dtype=dtype, top_k=1 + V // 40, seed=V + W, ragged_total=0 if B > 1 else 24)
 
 
+def test_more_rows_than_one_launch_takes():
+    _check("launches", B=20, W=500, V=2048, top_k=9, seed=11)
+
+
 @pytest.mark.parametrize("V,K,B,W", [(50264, 2000, 1, 8), (65536, 4096, 1, 5), (65536, 8192, 2, 76), (32776, 1, 2, 3),
                                      (131072, 3000, 1, 2), (20000, 5000, 1, 3),
                                      (65536, 9001, 1, 6), (65536, 2049, 3, 2)])
@@ -47,3 +51,32 @@ def test_rows_whose_lists_run_over_are_redone(B, W):
     prev = oracle_prime(inp)
     rep, got, ref = check_parity(inp.cond, inp.uncond, prev.tokens, prev.probs, step_kwargs(inp), inp.win_len)
     assert np.all(got.status & 16)
+
+
+def test_a_copy_that_never_lands_becomes_a_status_word_among_many_rows(tmp_path):
+    # as tests/test_gpu_timeout.py, for the kernel whose teams share a ring: CTAs with a second row lose one of its copies
+    import os
+    import subprocess
+    import sys
+    from paper_2512_07503_b200 import build
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    lib = build.build_variant(str(tmp_path / "libsjd_timeout_rows.so"), ["SJD_TEST_SPIN_CYCLES=2000000", "SJD_TEST_DROP_COPY=3"])
+    script = """
+import sys
+sys.path.insert(0, %r); sys.path.insert(0, %r)
+import numpy as np, torch, oracle
+from paper_2512_07503_b200 import workloads as wk
+from gpu_harness import gpu_step, step_kwargs
+wl = wk.CONFIGS["cfg2"].scaled(B=4, W=100, V=16384, top_k=200)
+inp = wk.make_step_inputs(wl)
+kw = step_kwargs(inp, flags=oracle.FLAG_DRAFT_ALL, iteration0=0)
+for _ in range(2):
+    got = gpu_step(inp.cond, inp.uncond, None, None, **kw)
+    lost = got.cnt == 0
+    assert np.any(lost) and np.any(~lost), lost.sum()
+    assert np.array_equal(np.any(lost, axis=1), (got.status & 8) != 0)
+assert torch.arange(10, device="cuda:0").sum().item() == 45
+print("ROWS_TIMEOUT_OK")
+""" % (root, os.path.join(root, "tests"))
+    out = subprocess.run([sys.executable, "-c", script], env=dict(os.environ, SJD_LIBRARY=lib), capture_output=True, text=True, timeout=600)
+    assert out.returncode == 0 and "ROWS_TIMEOUT_OK" in out.stdout, out.stdout[-2000:] + out.stderr[-4000:]
