@@ -40,30 +40,33 @@
 // kRowStatusTimeout, and the CTA waits (bounded) for its copies in flight before it exits.
 #pragma once
 
+#include <cuda_bf16.h>
+
 #include "rows_pipeline.cuh"
 
 namespace sjd {
 
 constexpr int kSiftPieces = 256;          // sample pieces per row
-constexpr int kSiftBins = 1024;           // bins of a row's histogram (the sample's, then the candidates')
+constexpr int kSiftGroups = 1024;         // sample groups per row (at most)
+constexpr int kSiftBins = 1024;           // bins of the candidates' histogram
 constexpr int kBinsLow = 768;             // candidates' bins 1 .. kBinsLow cover the lowest eighth of their values
 constexpr float kBinsCross = (8.0f * (kBinsLow + 1) - (kSiftBins - 2)) / 7.0f;  // where the upper bins' line starts
-constexpr int kSiftKeyShift = 22;         // key bits dropped by the sample's first pass: sign, exponent, one mantissa bit stay
 constexpr int kMemberCap = 512;           // members of the threshold bin ranked by brute force
 constexpr int kUnitBytes = 4096;          // bytes of one logits array per unit: 128 for each lane
 constexpr int kTeamWarps = 8;             // stream kernel: warps per team
 constexpr int kTeamThreads = kTeamWarps * 32;
 constexpr int kMaxTeams = 3;
 constexpr int kMaxSlots = 4;              // ring slots per warp
+constexpr int kAskAhead = 256 << 10;      // bytes of logits (whole rows) a CTA asks into the L2 before it may begin
 constexpr int kStreamRows = 64;           // live rows a CTA takes in one launch (the host splits larger problems)
 constexpr int kClusterWarps = 16;
 constexpr int kMaxCluster = 8;
 
 struct SiftCfg {
   int piece_stride;  // elements between the starts of two sample pieces (a multiple of 8)
-  int piece_vecs;    // 16-byte vectors per piece: 4 or 1
-  int by_vectors;    // 1: ranks among the vectors' maxima; 0: among all sampled elements
-  int rank;          // rank (from the top) of tau0
+  int piece_vecs;    // 16-byte vectors per piece: 4, 2 or 1
+  int groups;        // groups per vector, each represented by its largest element: 1, 2 or 4
+  int rank;          // rank of tau0 among the groups, from the top
   int seg_len;       // ids per segment, a multiple of 8
   int seg_cap;       // candidates a segment's list holds (a multiple of 8)
   int teams, slots;  // stream kernel: teams per CTA, ring slots per warp
@@ -95,7 +98,6 @@ struct alignas(16) SiftShared {
   uint64_t wtot[kClusterWarps];
   uint32_t wcnt[kClusterWarps];
   float wz[kClusterWarps];
-  uint32_t top_key;   // largest sample value
   uint32_t max_key;   // largest candidate
   uint32_t over;      // a list ran over, or a wait gave up
   int members;
@@ -231,14 +233,13 @@ static __device__ __noinline__ void rank_search(SiftShared* sm, SiftHist* h, uin
 }
 
 // ---------------------------------------------------------------------------------------------------
-// sample phase: tau0 and the candidates' bins, by the NT threads that work on the row.  hist is zero on entry and after.
+// sample phase
 // ---------------------------------------------------------------------------------------------------
-// First the maxima of the vectors (or, by_vectors == 0, all sampled elements) are binned by the top bits of their
-// order-preserving key, which gives a floor with enough of them above it; a second, linear histogram over
-// [floor, largest] resolves the wanted rank.  With exchangeable entries a vector of G elements has its maximum above t
-// with probability 1 - (1 - p(t))^G, which is how the host translates the wanted share of entries into a rank
-// among maxima: an eighth of the work for nearly the same sharpness while few entries lie above the threshold.
-// tau0 only steers how many candidates there are; the result is exact whatever it is.
+// A row's sample is cut into groups of G neighbouring elements, each represented by its largest.  With exchangeable entries
+// a group has its maximum above t with probability 1 - (1 - p(t))^G, which is how the host translates the wanted share p
+// of entries into a rank among maxima: a fraction of the work for nearly the same sharpness while few entries lie above the
+// threshold (where many do, it takes smaller groups of fewer vectors).  tau0 only steers how many candidates there are;
+// the result is exact whatever it is, so the maxima may be rounded to bf16.
 //
 // The candidates' bins are 1 .. kSiftBins - 1; bin 0 takes what is no candidate.  bin(y) is the smaller of two rising lines
 // over y - tau0, the first of which spends kBinsLow bins on the lowest eighth of [tau0, largest sample value], where
@@ -257,173 +258,136 @@ __device__ __forceinline__ SiftBinning sift_bins(float tau0, float top) {
   return SiftBinning{tau0, __fmul_rn(8.0f * kBinsLow, per), __fmul_rn((kSiftBins - 2) - kBinsCross, per)};
 }
 
-__device__ __forceinline__ uint4 ldg_now(const void* p) {  // issued where it stands: the values are wanted much later
+__device__ __forceinline__ uint4 ldg_now(const void* p) {  // issued where it stands
   uint4 v;
   asm volatile("ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
   return v;
 }
 
-__device__ __forceinline__ int sample_element(const SiftCfg& cfg, int vec, int ev, int V) {
-  const int piece = cfg.piece_vecs == 4 ? vec >> 2 : vec, k = cfg.piece_vecs == 4 ? vec & 3 : 0;
-  const int at = piece * cfg.piece_stride + k * ev;
-  return piece < kSiftPieces && k * ev < cfg.piece_stride && at < V ? at : -1;
-}
-
-// the sampled vectors of one thread
-template <int DTYPE, bool HAS_U, int NT>
-struct SampleLoad {
-  static constexpr int NV = 4 * kSiftPieces / NT;
-  uint4 c[NV], u[HAS_U ? NV : 1];
-  __device__ __forceinline__ void load(const SiftCfg& cfg, int V, const char* c_row, const char* u_row, int tid) {
-    constexpr int EV = SiftTraits<DTYPE>::kVec, ES = SiftTraits<DTYPE>::kElem;
-#pragma unroll
-    for (int j = 0; j < NV; ++j) {
-      const int e = max(sample_element(cfg, tid + j * NT, EV, V), 0);  // a vector that is not there: the row's first, not counted
-      c[j] = ldg_now(c_row + (size_t)e * ES);
-      if (HAS_U) u[HAS_U ? j : 0] = ldg_now(u_row + (size_t)e * ES);
-    }
-  }
+// what a row's threshold is found from
+struct alignas(16) SiftSample {
+  uint32_t m[kSiftGroups / 2];  // the groups' maxima as bf16 pairs, in no particular order
+  uint32_t top_key;             // largest sample value (0 between rows)
 };
 
-template <int DTYPE, bool HAS_U, bool HAS_T, int NT>
-__device__ __forceinline__ SiftBinning sift_sample(const RowArgs& a, const SiftCfg& cfg, SiftShared& sm, SiftHist& hist,
-                                                   const SampleLoad<DTYPE, HAS_U, NT>& in, int tid, int bar) {
-  constexpr int EV = SiftTraits<DTYPE>::kVec;
-  constexpr int NV = 4 * kSiftPieces / NT;  // vectors per thread
-  const int lane = tid & 31, warp = tid >> 5;
-  const float neg_inf = __int_as_float(0xff800000), lowest = -3.402823466e38f;
+// The groups' maxima of a row, by NT threads, four vectors per thread at a time (all there are when 256 threads share the
+// work).  `after_loads()` is called behind the first round's loads; the caller sees to the barrier behind it all.
+template <int DTYPE, bool HAS_U, bool HAS_T, int NT, typename AfterLoads>
+__device__ __forceinline__ void sift_sample(const RowArgs& a, const SiftCfg& cfg, SiftSample& out, const char* c_row, const char* u_row,
+                                            int tid, AfterLoads after_loads) {
+  constexpr int EV = SiftTraits<DTYPE>::kVec, ES = SiftTraits<DTYPE>::kElem;
+  constexpr int NV = NT >= 256 ? kSiftGroups / NT : 4;
+  const float neg_inf = __int_as_float(0xff800000);
   const uint64_t s2 = pack2(a.s, a.s), t2 = pack2(a.inv_T, a.inv_T);
-  float v[NV][EV];  // v[j][0]: the vector's maximum (by_vectors), or the vector's elements
+  const int vecs = kSiftPieces * cfg.piece_vecs;
+  const int shift = cfg.piece_vecs >> 1;  // log2 of 1, 2, 4
+  uint16_t* const m = reinterpret_cast<uint16_t*>(out.m);
+  auto put = [&](int x, float v) { m[x] = __bfloat16_as_ushort(__float2bfloat16_rn(v)); };
   float top = neg_inf;
-  const bool by_vectors = cfg.by_vectors != 0;
-#pragma unroll
-  for (int j = 0; j < NV; ++j) {
-    uint64_t y[EV / 2];
-    merge_vec<DTYPE, HAS_U, HAS_T>(in.c[j], in.u[HAS_U ? j : 0], s2, t2, y);
-    float m = neg_inf;
-#pragma unroll
-    for (int k = 0; k < EV / 2; ++k) {
-      unpack2(y[k], v[j][2 * k], v[j][2 * k + 1]);
-      m = max3(m, v[j][2 * k], v[j][2 * k + 1]);
-    }
-    const bool there = sample_element(cfg, tid + j * NT, EV, a.V) >= 0;
-    m = there ? canonical(m) : neg_inf;
-    top = fmaxf(top, m);
-    // an atomic with part of its lanes off runs several times slower than one with all lanes on: what is not there
-    // counts as -inf, below every threshold
-    if (by_vectors) {
-      v[j][0] = m;
-      hist.count(float_key(m) >> kSiftKeyShift);
-    } else {
-#pragma unroll
-      for (int k = 0; k < EV; ++k) {
-        v[j][k] = there ? canonical(v[j][k]) : neg_inf;
-        hist.count(float_key(v[j][k]) >> kSiftKeyShift);
-      }
-    }
-  }
-  const uint32_t warp_top = __reduce_max_sync(0xffffffffu, float_key(top));
-  if (lane == 0) atomicMax(&sm.top_key, warp_top);
-  row_sync<NT>(bar);
-  if (warp == 0) rank_search(&sm, &hist, (uint32_t)cfg.rank);
-  row_sync<NT>(bar);
-  float floor_y = key_float(sm.rank_bin << kSiftKeyShift);
-  if (!(floor_y >= lowest)) floor_y = lowest;  // the edge fell on -inf or into the NaN patterns
-  const float top_y = key_float(sm.top_key);
-  const bool refine = floor_y > lowest && top_y >= floor_y && top_y <= 3.402823466e38f;
-  const float range = __fsub_rn(top_y, floor_y);
-  const float scale = (refine && range > 0.0f) ? __fdiv_rn((float)kSiftBins - 1.5f, range) : 0.0f;
-  float tau0 = lowest;
-  if (refine) {
-    // bins 1 .. kSiftBins - 1; what lies below the floor counts in bin 0 (a negative argument converts to 0)
+#pragma unroll 1
+  for (int v0 = tid; v0 - tid < vecs; v0 += NT * NV) {
+    uint4 c[NV], u[HAS_U ? NV : 1];
+    uint32_t have = 0;
 #pragma unroll
     for (int j = 0; j < NV; ++j) {
+      const int v = v0 + j * NT, piece = v >> shift, k = v & (cfg.piece_vecs - 1);
+      const int e = piece * cfg.piece_stride + k * EV;
+      const bool in = v < vecs && k * EV < cfg.piece_stride && e < a.V;
+      have |= in ? 1u << j : 0u;
+      const size_t at = in ? (size_t)e * ES : 0;
+      c[j] = ldg_now(c_row + at);
+      if (HAS_U) u[HAS_U ? j : 0] = ldg_now(u_row + at);
+    }
+    if (v0 == tid) after_loads();
 #pragma unroll
-      for (int k = 0; k < EV; ++k) {
-        if (k > 0 && by_vectors) break;
-        const float x = v[j][k];
-        const uint32_t bin = x >= floor_y ? __float2uint_rz(__fmaf_rn(__fsub_rn(x, floor_y), scale, 1.0f)) : 0u;
-        hist.count(min(bin, (uint32_t)kSiftBins - 1u));
+    for (int j = 0; j < NV; ++j) {
+      uint64_t y2[EV / 2];
+      merge_vec<DTYPE, HAS_U, HAS_T>(c[j], u[HAS_U ? j : 0], s2, t2, y2);
+      float y[EV];
+#pragma unroll
+      for (int k = 0; k < EV / 2; ++k) unpack2(y2[k], y[2 * k], y[2 * k + 1]);
+      const int v = v0 + j * NT;
+      const bool in = (have >> j) & 1u;  // (a NaN is passed over by every maximum)
+      if (cfg.groups == 1) {
+        float all = neg_inf;
+#pragma unroll
+        for (int k = 0; k < EV / 2; ++k) all = max3(all, y[2 * k], y[2 * k + 1]);
+        all = in ? all : neg_inf;
+        top = fmaxf(top, all);
+        put(min(v, kSiftGroups - 1), all);
+      } else {
+        float q[4];  // maxima of the vector's quarters
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          q[k] = EV == 8 ? fmaxf(y[(2 * k) % EV], y[(2 * k + 1) % EV]) : y[k];
+          q[k] = in ? fmaxf(q[k], neg_inf) : neg_inf;
+          top = fmaxf(top, q[k]);
+        }
+        if (v < vecs) {
+          if (cfg.groups == 2) {
+            put(2 * v, fmaxf(q[0], q[1]));
+            put(2 * v + 1, fmaxf(q[2], q[3]));
+          } else {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) put(4 * v + k, q[k]);
+          }
+        }
       }
     }
-    row_sync<NT>(bar);
-    if (warp == 0) rank_search(&sm, &hist, (uint32_t)cfg.rank);
-    row_sync<NT>(bar);
-    const float tbin = (float)sm.rank_bin;
-    tau0 = floor_y;
-    // a little below the lower edge of the bin, so that rounding cannot exclude one of its members
-    if (tbin > 1.0f && scale > 0.0f) tau0 = __fmaf_rd(__fmul_rd(tbin - 1.0f, 0.9999f), __fdiv_rn(1.0f, scale), floor_y);
   }
-  return sift_bins(tau0, top_y);
+  // groups there are no vectors for
+  for (int x = vecs * cfg.groups + tid; x < kSiftGroups; x += NT) m[x] = 0xff80u;
+  const uint32_t warp_top = __reduce_max_sync(0xffffffffu, float_key(__fadd_rn(top, 0.0f)));
+  if ((tid & 31) == 0) atomicMax(&out.top_key, warp_top);
 }
 
-// The same by ONE warp, for a row that is not wanted yet: no barriers, and the vectors' maxima stay in registers, rounded
-// to bf16 pairs, through a binary search for the rank (sixteen packed comparisons and additions a step).  A few
-// thousand cycles that nobody waits for; the whole team would be held up by its barriers for as long.
-template <int DTYPE, bool HAS_U, bool HAS_T>
-__device__ __forceinline__ float2 sift_sample_ahead(const RowArgs& a, const SiftCfg& cfg, const char* c_row, const char* u_row, int lane) {
-  constexpr int EV = SiftTraits<DTYPE>::kVec, ES = SiftTraits<DTYPE>::kElem;
-  constexpr int NV = 4 * kSiftPieces / 32, BATCH = 4;
-  const uint64_t s2 = pack2(a.s, a.s), t2 = pack2(a.inv_T, a.inv_T);
-  uint32_t m2[NV / 2];  // maxima as bf16 pairs
-  float top = __int_as_float(0xff800000);
+// The search for the threshold goes over the bf16 values as 16-bit keys that are ordered like them: the largest key whose
+// value at least `rank` of the maxima reach.  How many do is counted by a warp that holds them all, a lane 16 pairs:
+// sixteen packed comparisons and additions.
+struct SiftMaxima {
+  static constexpr int NM = kSiftGroups / 64;
+  uint32_t m2[NM];
+  __device__ __forceinline__ void load(const SiftSample& in, int lane) {
 #pragma unroll
-  for (int j0 = 0; j0 < NV; j0 += BATCH) {
-    uint4 c[BATCH], u[BATCH];
-    int e[BATCH];
-#pragma unroll
-    for (int j = 0; j < BATCH; ++j) {
-      e[j] = sample_element(cfg, lane + 32 * (j0 + j), EV, a.V);
-      const size_t at = (size_t)max(e[j], 0) * ES;
-      c[j] = ldg_now(c_row + at);
-      u[j] = HAS_U ? ldg_now(u_row + at) : c[j];
-    }
-    float m[BATCH];
-#pragma unroll
-    for (int j = 0; j < BATCH; ++j) {
-      uint64_t y[EV / 2];
-      merge_vec<DTYPE, HAS_U, HAS_T>(c[j], u[j], s2, t2, y);
-      float x = __int_as_float(0xff800000);
-#pragma unroll
-      for (int k = 0; k < EV / 2; ++k) {
-        float y0, y1;
-        unpack2(y[k], y0, y1);
-        x = max3(x, y0, y1);
-      }
-      m[j] = e[j] >= 0 ? x : __int_as_float(0xff800000);
-      top = fmaxf(top, m[j]);
-    }
-#pragma unroll
-    for (int j = 0; j < BATCH; j += 2) {
-      asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(m2[(j0 + j) / 2]) : "f"(m[j + 1]), "f"(m[j]));
+    for (int x = 0; x < NM / 4; ++x) {
+      const uint4 v = reinterpret_cast<const uint4*>(in.m)[lane + 32 * x];
+      m2[4 * x] = v.x; m2[4 * x + 1] = v.y; m2[4 * x + 2] = v.z; m2[4 * x + 3] = v.w;
     }
   }
-  // largest 16-bit key whose value at least `rank` of the maxima reach (keys are ordered like the values)
-  uint32_t key = 0;
-#pragma unroll 1
-  for (uint32_t bit = 0x8000u; bit != 0u; bit >>= 1) {
-    const uint32_t k = key | bit;
-    const uint32_t v = (k & 0x8000u) ? k & 0x7fffu : ~k & 0xffffu;  // bf16 pattern of the key
+  __device__ __forceinline__ uint32_t reaching(uint32_t key) const {
+    const uint32_t v = (key & 0x8000u) ? key & 0x7fffu : ~key & 0xffffu;  // bf16 pattern of the key
     const uint32_t t = v | (v << 16);
-    uint32_t acc0 = 0, acc1 = 0;
+    uint32_t acc[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
-    for (int x = 0; x < NV / 2; x += 2) {
-      uint32_t g0, g1;
-      asm("set.ge.bf16x2.bf16x2 %0, %1, %2;" : "=r"(g0) : "r"(m2[x]), "r"(t));
-      asm("set.ge.bf16x2.bf16x2 %0, %1, %2;" : "=r"(g1) : "r"(m2[x + 1]), "r"(t));
-      asm("add.rn.bf16x2 %0, %0, %1;" : "+r"(acc0) : "r"(g0));
-      asm("add.rn.bf16x2 %0, %0, %1;" : "+r"(acc1) : "r"(g1));
+    for (int x = 0; x < NM; ++x) {
+      uint32_t g;
+      asm("set.ge.bf16x2.bf16x2 %0, %1, %2;" : "=r"(g) : "r"(m2[x]), "r"(t));
+      asm("add.rn.bf16x2 %0, %0, %1;" : "+r"(acc[x & 3]) : "r"(g));
     }
-    asm("add.rn.bf16x2 %0, %0, %1;" : "+r"(acc0) : "r"(acc1));
-    const uint32_t n = __reduce_add_sync(0xffffffffu, (uint32_t)(bf16_lo(acc0) + bf16_hi(acc0)));
-    if (n >= (uint32_t)cfg.rank) key = k;
+    asm("add.rn.bf16x2 %0, %0, %1;" : "+r"(acc[0]) : "r"(acc[1]));
+    asm("add.rn.bf16x2 %0, %0, %1;" : "+r"(acc[2]) : "r"(acc[3]));
+    asm("add.rn.bf16x2 %0, %0, %1;" : "+r"(acc[0]) : "r"(acc[2]));
+    return __reduce_add_sync(0xffffffffu, (uint32_t)(bf16_lo(acc[0]) + bf16_hi(acc[0])));
   }
-  top = key_float(__reduce_max_sync(0xffffffffu, float_key(canonical(top))));
-  // The maxima were rounded to nearest: the middle between this bf16 value and the one below is what they all reach.
+};
+// {tau0, largest sample value} for the key found
+__device__ __forceinline__ float2 sift_tau(uint32_t key, uint32_t top_key) {
+  const float top = key_float(top_key), lowest = -3.402823466e38f;  // lowest: every finite value is a candidate
+  // the maxima were rounded to nearest: the middle between this bf16 value and the one below is what they all reach
   const float at = key_float(key << 16), below = key_float((key - 1u) << 16);
   float tau0 = __fmaf_rd(__fsub_rn(at, below), -0.51f, at);
-  if (key == 0u || !(tau0 >= -3.402823466e38f) || !(top <= 3.402823466e38f)) tau0 = -3.402823466e38f;
+  if (key == 0u || !(tau0 >= lowest) || !(top <= 3.402823466e38f)) tau0 = lowest;
   return make_float2(tau0, top);
+}
+// by one warp, bit by bit
+__device__ __forceinline__ float2 sift_threshold(const SiftSample& in, uint32_t rank, int lane) {
+  SiftMaxima m;
+  m.load(in, lane);
+  uint32_t key = 0;
+#pragma unroll 1
+  for (uint32_t bit = 0x8000u; bit != 0u; bit >>= 1)
+    if (m.reaching(key | bit) >= rank) key |= bit;
+  return sift_tau(key, in.top_key);
 }
 
 // ---------------------------------------------------------------------------------------------------
@@ -597,7 +561,6 @@ __device__ __forceinline__ bool finish_row(const RowArgs& a, const SiftCfg& cfg,
   const uint32_t tbin = sm.rank_bin, need = kcap - sm.rank_above, nbin = sm.rank_count;
   if (tid == 0) {
     sm.max_key = 0u;
-    sm.top_key = 0u;
     sm.over = 0u;
   }
   // fewer than kcap candidates, a threshold bin too crowded for the ranking, or no finite maximum
@@ -615,7 +578,7 @@ __device__ __forceinline__ bool finish_row(const RowArgs& a, const SiftCfg& cfg,
     for (int g = 0; g < per_warp; ++g) {
       const uint32_t n = seg_n[first_seg + g];
       const float* const y_g = my_y + g * cfg.seg_cap;
-#pragma unroll 2
+#pragma unroll 4
       for (uint32_t i = (uint32_t)lane; i < n; i += 32u) {
         const float y = y_g[i], x = bins.at(y);
         if (x >= lo && x < hi) sm.hist.member[atomicAdd(&sm.members, 1)] = SiftMember{y, id0 + (int32_t)my_id[g * cfg.seg_cap + i]};
@@ -657,7 +620,8 @@ __device__ __forceinline__ bool finish_row(const RowArgs& a, const SiftCfg& cfg,
     thr_y = sm.thr_y;
     thr_id = sm.thr_id;
   }
-  // ---- survivors: exponentials and ids to the front of the warp's lists, their number and sum
+  // ---- survivors: exponentials and ids to the front of the warp's lists, their number and sum.  Four groups of 32 at a
+  // time: their loads and exponentials do not wait for one another, nor for the stores, which go to places already read.
   const int thr_rel = thr_id - id0;
   uint32_t cnt = 0;
   float z = 0.0f;
@@ -665,26 +629,36 @@ __device__ __forceinline__ bool finish_row(const RowArgs& a, const SiftCfg& cfg,
     const uint32_t n = seg_n[first_seg + g];
     const float* const y_g = my_y + g * cfg.seg_cap;
     const uint16_t* const id_g = my_id + g * cfg.seg_cap;
-#pragma unroll 2
-    for (uint32_t i0 = 0; i0 < n; i0 += 32u) {
-      const uint32_t i = i0 + (uint32_t)lane;
-      float y = __int_as_float(0xff800000);
-      int id = 0x7fffffff;
-      if (i < n) {
-        y = y_g[i];
-        id = (int)id_g[i];
+    constexpr int U = 4;
+#pragma unroll 1
+    for (uint32_t i0 = 0; i0 < n; i0 += 32u * U) {
+      float e[U];
+      int id[U];
+      uint32_t votes[U];
+#pragma unroll
+      for (int j = 0; j < U; ++j) {
+        const uint32_t i = i0 + 32u * j + (uint32_t)lane;
+        e[j] = i < n ? y_g[i] : __int_as_float(0xff800000);
+        id[j] = i < n ? (int)id_g[i] : 0x7fffffff;
       }
-      const bool alive = y > thr_y || (y == thr_y && id <= thr_rel);
-      const float e = exp_diff_finite(y, vmax);
-      const uint32_t votes = __ballot_sync(0xffffffffu, alive);
-      __syncwarp();  // every lane has read its entry: what follows overwrites entries up to this group's
-      if (alive) {
-        const uint32_t at = cnt + (uint32_t)__popc(votes & below);
-        my_y[at] = e;
-        my_id[at] = (uint16_t)id;
-        z += e;
+#pragma unroll
+      for (int j = 0; j < U; ++j) {
+        const bool alive = e[j] > thr_y || (e[j] == thr_y && id[j] <= thr_rel);
+        votes[j] = __ballot_sync(0xffffffffu, alive);  // (every lane has read its entries: they may be overwritten)
+        e[j] = exp_diff_finite(e[j], vmax);
       }
-      cnt += (uint32_t)__popc(votes);
+      __syncwarp();
+#pragma unroll
+      for (int j = 0; j < U; ++j) {
+        if ((votes[j] >> lane) & 1u) {
+          const uint32_t at = cnt + (uint32_t)__popc(votes[j] & below);
+          my_y[at] = e[j];
+          my_id[at] = (uint16_t)id[j];
+          z += e[j];
+        }
+        cnt += (uint32_t)__popc(votes[j]);
+      }
+      __syncwarp();
     }
   }
 #pragma unroll
@@ -707,7 +681,7 @@ __device__ __forceinline__ bool finish_row(const RowArgs& a, const SiftCfg& cfg,
   int32_t* const out_ids = a.out_ids + (size_t)row * kcap + before;
   float* const out_vals = a.out_vals + (size_t)row * kcap + before;
   uint64_t wsum = 0;
-#pragma unroll 2
+#pragma unroll 4
   for (uint32_t i = (uint32_t)lane; i < cnt; i += 32u) {
     const float p = __fmul_rn(my_y[i], inv_Z);
     const int id = id0 + (int)my_id[i];
@@ -777,7 +751,6 @@ __device__ __noinline__ void sift_redo(const RowArgs& a, int row, int tid, Gener
 __device__ __forceinline__ void init_shared(SiftShared& sm, int tid, int nt) {
   for (int k = tid; k < (int)sizeof(SiftHist) / 16; k += nt) reinterpret_cast<uint4*>(&sm.hist)[k] = make_uint4(0u, 0u, 0u, 0u);
   if (tid == 0) {
-    sm.top_key = 0u;
     sm.max_key = 0u;
     sm.over = 0u;
     sm.members = 0;
@@ -814,20 +787,28 @@ struct alignas(16) StreamShared {
   // parity wait tells a phase from its neighbours only, so each barrier is waited on by one warp, phase after phase.
   uint64_t full[kTeamWarps * kMaxTeams * kMaxSlots];
   uint32_t used[kTeamWarps * kMaxTeams * kMaxSlots];  // copies issued for that barrier so far
-  // thresholds of a team's rows after its first: {tau0, largest sample value}, two places used in turn
-  uint64_t tau_full[kMaxTeams * 2], tau_free[kMaxTeams * 2];
-  float2 tau[kMaxTeams * 2];
+  // for every team: a row's sample is complete, and {tau0, largest sample value} of rows to come, in two places used in turn
+  uint64_t sample_full[kMaxTeams], tau_full[2 * kMaxTeams], tau_free[2 * kMaxTeams];
+  float2 tau[2 * kMaxTeams];
   uint32_t seg_n[kMaxTeams * kTeamWarps];      // candidates per segment
   int32_t redo[kStreamRows];                   // rows the single pass could not finish (redone at the end)
   int n_live, n_redo, abort;
 };
-// shared memory: StreamShared | SiftShared x teams | list values | list ids | rings
+struct alignas(16) TeamShared {
+  SiftShared row;
+  SiftSample sample;  // the team's first row's is written by the team, the others' by its sampler
+};
+// shared memory: StreamShared | TeamShared x teams | list values | list ids | rings
 __host__ __device__ inline size_t sift_stream_rings(int teams, int seg_cap) {
-  const size_t b = sizeof(StreamShared) + teams * (sizeof(SiftShared) + (size_t)kTeamWarps * seg_cap * 6);
+  const size_t b = sizeof(StreamShared) + teams * (sizeof(TeamShared) + (size_t)kTeamWarps * seg_cap * 6);
   return (b + 127) & ~(size_t)127;
 }
 __host__ __device__ inline size_t sift_stream_smem(int teams, int seg_cap, int slots, bool has_u) {
   return sift_stream_rings(teams, seg_cap) + (size_t)kTeamWarps * slots * kUnitBytes * (has_u ? 2 : 1);
+}
+
+__device__ __forceinline__ void ask_l2(const void* p, uint32_t bytes) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
 }
 
 // bounded wait that also ends when another warp of the CTA has given up.  The wait stays suspended in hardware for up to
@@ -862,8 +843,9 @@ rows_stream_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ Si
   const bool sampler = (int)threadIdx.x >= teams * kTeamThreads;
   const int team = sampler ? ((int)threadIdx.x - teams * kTeamThreads) >> 5 : (int)threadIdx.x / kTeamThreads;
   const int tid = sampler ? (int)threadIdx.x & 31 : (int)threadIdx.x % kTeamThreads, lane = tid & 31, warp = tid >> 5, bar = 1 + team;
-  SiftShared* const team_sm = reinterpret_cast<SiftShared*>(smem_raw + sizeof(StreamShared));
-  SiftShared& sm = team_sm[team];
+  TeamShared* const team_sm = reinterpret_cast<TeamShared*>(smem_raw + sizeof(StreamShared));
+  SiftShared& sm = team_sm[team].row;
+  SiftSample& sample = team_sm[team].sample;
   float* const lists = reinterpret_cast<float*>(team_sm + teams);
   float* const list_y = lists + (size_t)team * kTeamWarps * cfg.seg_cap;
   uint16_t* const list_id = reinterpret_cast<uint16_t*>(lists + (size_t)teams * kTeamWarps * cfg.seg_cap) + (size_t)team * kTeamWarps * cfg.seg_cap;
@@ -873,16 +855,30 @@ rows_stream_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ Si
     mbar_init(&st.full[threadIdx.x], 1);
     st.used[threadIdx.x] = 0;
   }
-  if (threadIdx.x < kMaxTeams * 2) {
+  if (threadIdx.x < 2 * kMaxTeams) {
     mbar_init(&st.tau_full[threadIdx.x], 1);
     mbar_init(&st.tau_free[threadIdx.x], kTeamWarps);
+    if (threadIdx.x < kMaxTeams) mbar_init(&st.sample_full[threadIdx.x], kTeamWarps);
   }
+  if (tid == 0) sample.top_key = 0u;
   if (threadIdx.x == 0) {
     st.n_redo = 0;
     st.abort = 0;
   }
   fence_barrier_init();
-  grid_dependency_wait();  // shared memory only up to here; a launch that overlaps the previous kernel waits for its end
+  // What a launch that overlaps the previous kernel may do before that kernel's end is shared-memory set-up, and asking the
+  // CTA's first rows into the L2 (nothing is read; the L2 is where all writes meet): the memory would lie idle meanwhile.
+  if (threadIdx.x < 32) {
+    const int64_t bytes = (int64_t)a.V * ES, row = (int64_t)cfg.row_begin + blockIdx.x + (int64_t)lane * gridDim.x;
+    if (lane * bytes * (HAS_U ? 2 : 1) < kAskAhead && row < cfg.row_end) {
+      const int b = (int)(row / a.W), i = (int)(row - (int64_t)b * a.W);
+      const int64_t off = (int64_t)b * a.stride_b + (int64_t)i * a.stride_w;
+      ask_l2(row_ptr(a.cond, DTYPE, off), (uint32_t)bytes);
+      if (HAS_U) ask_l2(row_ptr(a.uncond, DTYPE, off), (uint32_t)bytes);
+    }
+    __syncwarp();
+  }
+  grid_dependency_wait();
   // ---- the CTA's rows: row_begin + blockIdx.x, + gridDim.x, ... (at most kStreamRows).  Rows beyond their sequence's window
   // length get their empty result; the others go into a table, so that no warp reads global memory for them later.
   if (threadIdx.x < 32) {
@@ -909,22 +905,26 @@ rows_stream_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ Si
   volatile int* const abort_flag = &st.abort;
   if (sampler) {
     // ======================================= samplers =======================================
-    // thresholds of the team's rows after its first, one or two rows ahead
-    int at = 0;
-    uint32_t round = 0;
-    for (int k = team + teams; k < n_live && cfg.by_vectors; k += teams) {
-      const int64_t off = st.tab[k].off;
-      const float2 tau = sift_sample_ahead<DTYPE, HAS_U, HAS_T>(a, cfg, static_cast<const char*>(row_ptr(a.cond, DTYPE, off)),
-                                                                HAS_U ? static_cast<const char*>(row_ptr(a.uncond, DTYPE, off)) : nullptr, lane);
-      const int x = 2 * team + at;
-      if (round > 0 && !sift_wait(&st.tau_free[x], (round - 1u) & 1u, abort_flag)) break;
+    // the thresholds of the team's rows, one or two rows ahead
+    for (int k = team, n = 0; k < n_live; k += teams, ++n) {
+      if (n == 0) {
+        if (!sift_wait(&st.sample_full[team], 0u, abort_flag)) break;
+      } else {
+        const int64_t off = st.tab[k].off;
+        sift_sample<DTYPE, HAS_U, HAS_T, 32>(a, cfg, sample, static_cast<const char*>(row_ptr(a.cond, DTYPE, off)),
+                                             HAS_U ? static_cast<const char*>(row_ptr(a.uncond, DTYPE, off)) : nullptr, lane, [] {});
+      }
+      __syncwarp();
+      const float2 tau = sift_threshold(sample, (uint32_t)cfg.rank, lane);
+      const int x = 2 * team + (n & 1);
+      if (n >= 2 && !sift_wait(&st.tau_free[x], (uint32_t)((n >> 1) - 1) & 1u, abort_flag)) break;
+      __syncwarp();
       if (lane == 0) {
+        sample.top_key = 0u;
         st.tau[x] = tau;
         mbar_arrive(&st.tau_full[x]);
       }
       __syncwarp();
-      round += (uint32_t)at;
-      at ^= 1;
     }
     __syncthreads();
     return;
@@ -952,8 +952,20 @@ rows_stream_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ Si
     bulk_g2s(dst, row_ptr(a.cond, DTYPE, off), bytes, &st.full[x]);
     if (HAS_U) bulk_g2s(dst + kUnitBytes, row_ptr(a.uncond, DTYPE, off), bytes, &st.full[x]);
   };
-  if (team == 0 && lane == 0 && units > 0) {
-    for (int k = 0; k < slots; ++k) issue(0, k, k);
+  if (team < n_live) {
+    // the team's first row: its sample's maxima, for the sampler
+    const int64_t off = st.tab[team].off;
+    sift_sample<DTYPE, HAS_U, HAS_T, kTeamThreads>(
+        a, cfg, sample, static_cast<const char*>(row_ptr(a.cond, DTYPE, off)),
+        HAS_U ? static_cast<const char*>(row_ptr(a.uncond, DTYPE, off)) : nullptr, tid, [&] {
+          // the first copies go out behind the first row's sample, not before it: everybody waits for that
+          if (team == 0 && lane == 0 && units > 0) {
+            for (int x = 0; x < slots; ++x) issue(0, x, x);
+          }
+          __syncwarp();
+        });
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&st.sample_full[team]);
   }
   const uint64_t s2 = pack2(a.s, a.s), t2 = pack2(a.inv_T, a.inv_T);
   SiftTarget to;
@@ -969,22 +981,13 @@ rows_stream_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ Si
     // from the CTA's last row on, the verification grid may be scheduled (it waits for this grid's end)
     if (k == n_live - 1) allow_dependent_launch();
     bool ok = *abort_flag == 0;
-    SiftBinning bins;
-    if (k == team || !cfg.by_vectors) {
-      SampleLoad<DTYPE, HAS_U, kTeamThreads> sample;
-      const int64_t off = st.tab[k].off;
-      sample.load(cfg, a.V, static_cast<const char*>(row_ptr(a.cond, DTYPE, off)),
-                  HAS_U ? static_cast<const char*>(row_ptr(a.uncond, DTYPE, off)) : nullptr, tid);
-      bins = sift_sample<DTYPE, HAS_U, HAS_T, kTeamThreads>(a, cfg, sm, sm.hist, sample, tid, bar);
-    } else {
-      const int x = 2 * team + tau_at;
-      if (ok) ok = sift_wait(&st.tau_full[x], tau_phase, abort_flag);
-      bins = sift_bins(st.tau[x].x, st.tau[x].y);
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&st.tau_free[x]);
-      tau_phase ^= (uint32_t)tau_at;
-      tau_at ^= 1;
-    }
+    const int x = 2 * team + tau_at;
+    if (ok) ok = sift_wait(&st.tau_full[x], tau_phase, abort_flag);
+    const SiftBinning bins = sift_bins(st.tau[x].x, st.tau[x].y);
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&st.tau_free[x]);
+    tau_phase ^= (uint32_t)tau_at;
+    tau_at ^= 1;
     uint32_t n = 0;
     float vmax = __int_as_float(0xff800000);
     int slot = (k * units) % slots;
@@ -1040,7 +1043,8 @@ rows_stream_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ Si
 // ---------------------------------------------------------------------------------------------------
 struct alignas(16) ClusterShared {
   SiftShared row;                                // the first CTA's: histogram of the candidates, finish phase
-  SiftHist hist_s;                               // the sample's histogram
+  SiftSample sample;
+  uint32_t key[kClusterWarps];                   // threshold search: what each warp's count says
   uint64_t full[kClusterWarps];                  // a warp's segment has landed
   uint32_t seg_n[kClusterWarps * kMaxCluster];   // candidates per segment (the first CTA's)
   uint32_t lost;                                 // a bounded wait of the cluster gave up (the first CTA's)
@@ -1095,13 +1099,25 @@ rows_cluster_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ S
   const int row = (int)(blockIdx.x / csize);
   const uint64_t s2 = pack2(a.s, a.s), t2 = pack2(a.inv_T, a.inv_T);
   init_shared(sm.row, tid, NT);
-  for (int k = tid; k < (int)sizeof(SiftHist) / 16; k += NT) reinterpret_cast<uint4*>(&sm.hist_s)[k] = make_uint4(0u, 0u, 0u, 0u);
   if (tid < kClusterWarps) mbar_init(&sm.full[tid], 1);
-  if (tid == 0) sm.lost = 0u;
+  if (tid == 0) {
+    sm.lost = 0u;
+    sm.sample.top_key = 0u;
+  }
   fence_barrier_init();
   __syncthreads();
-  cluster_arrive();        // from here on the first CTA's histogram and lists are ready for the others
-  grid_dependency_wait();  // shared memory only up to here
+  cluster_arrive();  // from here on the first CTA's histogram and lists are ready for the others
+  if (tid == 0) {    // this CTA's part of the row into the L2 (see rows_stream_kernel)
+    const int b = row / a.W, i = row - b * a.W, at = (int)crank * kClusterWarps * cfg.seg_len;
+    const int n = min(max(a.V - at, 0), kClusterWarps * cfg.seg_len);
+    const int64_t off = (int64_t)b * a.stride_b + (int64_t)i * a.stride_w + at;
+    if (n > 0) {
+      ask_l2(row_ptr(a.cond, DTYPE, off), (uint32_t)n * ES);
+      if (HAS_U) ask_l2(row_ptr(a.uncond, DTYPE, off), (uint32_t)n * ES);
+    }
+  }
+  __syncwarp();
+  grid_dependency_wait();
   allow_dependent_launch();
   const SiftRow r = sift_row(a, row);
   if (!r.live) {  // the whole cluster
@@ -1134,9 +1150,26 @@ rows_cluster_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ S
   }
   __syncwarp();
   // every CTA of the cluster finds the threshold for itself: the sample is small, an exchange would cost more
-  SampleLoad<DTYPE, HAS_U, NT> sample;
-  sample.load(cfg, a.V, c_row, u_row, tid);
-  const SiftBinning bins = sift_sample<DTYPE, HAS_U, HAS_T, NT>(a, cfg, sm.row, sm.hist_s, sample, tid, 0);
+  sift_sample<DTYPE, HAS_U, HAS_T, NT>(a, cfg, sm.sample, c_row, u_row, tid, [] {});
+  __syncthreads();
+  // the search four bits at a time: warp w counts for the digit w, the largest digit that is reached enough is taken
+  uint32_t key = 0;
+  {
+    static_assert(kClusterWarps == 16, "a warp per digit");
+    SiftMaxima m;
+    m.load(sm.sample, lane);
+#pragma unroll 1
+    for (int shift = 12; shift >= 0; shift -= 4) {
+      const uint32_t mine = key | ((uint32_t)warp << shift);
+      const bool reached = warp == 0 || m.reaching(mine) >= (uint32_t)cfg.rank;
+      if (lane == 0) sm.key[warp] = reached ? mine : 0u;
+      __syncthreads();
+      key = __reduce_max_sync(0xffffffffu, sm.key[lane & 15]);
+      __syncthreads();
+    }
+  }
+  const float2 tau = sift_tau(key, sm.sample.top_key);
+  const SiftBinning bins = sift_bins(tau.x, tau.y);
   SiftTarget to;
   to.y_at = in_first_cta(list_y + (size_t)seg * cfg.seg_cap);
   to.id_at = in_first_cta(list_id + (size_t)seg * cfg.seg_cap);
@@ -1176,7 +1209,7 @@ rows_cluster_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ S
     return;
   }
   if (!finish_row<kClusterWarps>(a, cfg, sm.row, list_y, list_id, sm.seg_n, (int)csize, bins, row, r.pos, r.iter, r.draft, tid, 0))
-    sift_redo<DTYPE, NT, 0>(a, row, tid, *reinterpret_cast<GenericSmem*>(&sm.hist_s));
+    sift_redo<DTYPE, NT, 0>(a, row, tid, *reinterpret_cast<GenericSmem*>(&sm.sample));
 }
 
 }  // namespace sjd

@@ -197,21 +197,27 @@ bool plan_sift(const sjd_params* P, int kcap, bool has_u, SiftPlan* plan) {
   sjd::SiftCfg& c = plan->cfg;
   std::memset(&c, 0, sizeof(c));
   c.piece_stride = (((V + sjd::kSiftPieces - 1) / sjd::kSiftPieces) + 7) & ~7;
-  c.piece_vecs = c.piece_stride * es >= 128 ? 4 : 1;
-  int vecs = 0;
-  for (int j = 0; j < sjd::kSiftPieces; ++j)
-    for (int k = 0; k < c.piece_vecs; ++k)
-      if (k * ev < c.piece_stride && j * c.piece_stride + k * ev < V) ++vecs;
+  // the sample: vectors per piece and groups per vector that let the threshold come closest, with 1,024 groups at most
   const double want = (double)kcap / V;
-  double sd_e, sd_v;
-  const double p_e = aimed_share(want, (double)vecs * ev, 1, &sd_e), p_v = aimed_share(want, vecs, ev, &sd_v);
-  c.by_vectors = p_v <= 1.1 * p_e ? 1 : 0;
-  const double p = c.by_vectors ? p_v : p_e, sd = c.by_vectors ? sd_v : sd_e;
+  double p = 2.0, sd = 0.0;
+  for (int pv = 4; pv >= 1; pv >>= 1) {
+    if (pv > 1 && c.piece_stride * es < 32 * pv) continue;  // pieces take half of the row at most
+    int vecs = 0;
+    for (int j = 0; j < sjd::kSiftPieces; ++j)
+      for (int k = 0; k < pv; ++k)
+        if (k * ev < c.piece_stride && j * c.piece_stride + k * ev < V) ++vecs;
+    for (int g = 1; g * pv <= 4; g <<= 1) {
+      double sd_g;
+      const double p_g = aimed_share(want, (double)vecs * g, ev / g, &sd_g);
+      if (p_g >= p) continue;
+      p = p_g;
+      sd = sd_g;
+      c.piece_vecs = pv;
+      c.groups = g;
+      c.rank = (int)std::ceil(vecs * g * (1.0 - std::pow(1.0 - p, ev / g)));
+    }
+  }
   if (p > 0.6) return false;
-  auto rank_of = [&](double share) {
-    return (int)std::ceil(c.by_vectors ? vecs * (1.0 - std::pow(1.0 - share, ev)) : share * vecs * ev);
-  };
-  c.rank = rank_of(p);
   const int sms = sm_count();
   const int64_t rows = (int64_t)P->B * P->W;
   // few rows: as many CTAs per row as there are SMs for, as long as a warp has half a unit of its own
