@@ -182,11 +182,11 @@ struct SiftPlan {
 };
 
 // Segments of equal length, each with a list that holds its share of the candidates with four standard deviations of
-// the threshold's estimate and 4.5 of the segment's own count to spare.
+// the threshold's estimate and four of the segment's own count to spare.
 void cut_segments(sjd::SiftCfg* c, int V, int segs, double p, double sd) {
   c->seg_len = (((V + segs - 1) / segs) + 7) & ~7;
   const double mean = c->seg_len * (p + 4.0 * sd);
-  int cap = (int)(mean + 4.5 * std::sqrt(mean) + 8.0);
+  int cap = (int)(mean + 4.0 * std::sqrt(mean) + 8.0);
   if (cap > c->seg_len) cap = c->seg_len;
   c->seg_cap = (cap + 7) & ~7;
 }
