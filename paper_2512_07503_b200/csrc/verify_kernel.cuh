@@ -70,7 +70,7 @@ struct VerifySmem {
 // One CTA per sequence.  Latency is all there is to it (it sits between two row kernels), so nothing is waited for
 // that could have been asked for earlier: what does not come from the row stage is loaded, and the accept tests' random
 // numbers are drawn, before the wait for that stage; both rows of the residual draw come in with one round of loads; the
-// lookups of a thread's four entries run side by side.  16 sequences of 64 rows, K=2,000: 8.4 us under ncu
+// lookups of a thread's four entries share one search.  16 sequences of 64 rows, K=2,000: 8.4 us under ncu
 // (12.1 before), and 3 us less of a step (one window of 32 rows: 25.5 -> 21.4 us).
 //
 // LONG: rows of more than 2,048 entries, taken in rounds (1,024 rows of K=8,192: 294 -> 235 us a step).
@@ -143,26 +143,32 @@ __global__ void __launch_bounds__(kVerifyThreads) verify_kernel(const VerifyArgs
     const int k0 = i * ITEMS * rounds;  // this thread's run of consecutive entries
     int id[ITEMS];
     float p[ITEMS], w[ITEMS];
-    auto load = [&](int k) {
+    // whole runs of four as one load each where the arrays' alignment allows it
+    const bool vec = (kcap & 3) == 0 && ((reinterpret_cast<uintptr_t>(a.p_ids) | reinterpret_cast<uintptr_t>(a.p_vals) |
+                                          reinterpret_cast<uintptr_t>(a.q_ids) | reinterpret_cast<uintptr_t>(a.q_vals)) & 15u) == 0;
+    auto load4 = [&](const int32_t* ids, const float* vals, int k, int (&to_id)[ITEMS], float (&to_val)[ITEMS]) {
+      if (vec) {
+        const int4 x = k < kcap ? *reinterpret_cast<const int4*>(ids + k) : make_int4(-1, -1, -1, -1);
+        const float4 y = k < kcap ? *reinterpret_cast<const float4*>(vals + k) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        to_id[0] = x.x; to_id[1] = x.y; to_id[2] = x.z; to_id[3] = x.w;
+        to_val[0] = y.x; to_val[1] = y.y; to_val[2] = y.z; to_val[3] = y.w;
+        return;
+      }
 #pragma unroll
       for (int j = 0; j < ITEMS; ++j) {
         const bool in = k + j < kcap;
-        id[j] = in ? pid[k + j] : -1;
-        p[j] = in ? pv[k + j] : 0.0f;
+        to_id[j] = in ? ids[k + j] : -1;
+        to_val[j] = in ? vals[k + j] : 0.0f;
       }
     };
+    auto load = [&](int k) { load4(pid, pv, k, id, p); };
     int n, stride = 1;
     if (!LONG) {
       // all loads at once: q's too, although only the first qc of its entries (if it has any) mean anything
       int qi[ITEMS];
       float qw[ITEMS];
       load(k0);
-#pragma unroll
-      for (int j = 0; j < ITEMS; ++j) {
-        const bool in = k0 + j < kcap;
-        qi[j] = in ? qid[k0 + j] : 0;
-        qw[j] = in ? qv[k0 + j] : 0.0f;
-      }
+      load4(qid, qv, k0, qi, qw);
       *reinterpret_cast<int4*>(&sm.q[k0]) = make_int4(qi[0], qi[1], qi[2], qi[3]);
       *reinterpret_cast<float4*>(&sm.q[NT * ITEMS + k0]) = make_float4(qw[0], qw[1], qw[2], qw[3]);
       n = min(max(qc, 0), kcap);
@@ -175,16 +181,22 @@ __global__ void __launch_bounds__(kVerifyThreads) verify_kernel(const VerifyArgs
     const int staged = n > 0 ? (n + stride - 1) / stride : 0;
     // weights of the four entries in id / p: what q leaves of p
     auto residual = [&](int k) {
-      int lo[ITEMS] = {0, 0, 0, 0};
+      // largest staged position whose id does not exceed the wanted one: by halving for the first of the four, by steps
+      // from there for the others: both rows ascend and hold about as many entries, so one or two steps do (four searches
+      // by halving in step: 5.7 K cycles of the kernel's 14 K, this 4.7 K; a hash table 7 K and 4 K to fill; neighbouring
+      // entries to neighbouring lanes 3.1 K, but more for locating the draw than that saves)
+      int lo[ITEMS];
+      int at = 0;
       if (n > 0) {
-        // largest staged position whose id does not exceed the wanted one: halving steps, the four lookups in step
-        for (int half = 1 << (31 - __clz(staged)); half > 0; half >>= 1) {
+        for (int half = 1 << (31 - __clz(staged)); half > 0; half >>= 1)
+          if (at + half < staged && sm.q[at + half] <= id[0]) at += half;
+      }
 #pragma unroll
-          for (int j = 0; j < ITEMS; ++j) {
-            const int at = lo[j] + half;
-            if (at < staged && sm.q[at] <= id[j]) lo[j] = at;
-          }
+      for (int j = 0; j < ITEMS; ++j) {
+        if (j > 0) {
+          while (at + 1 < staged && sm.q[at + 1] <= id[j]) ++at;
         }
+        lo[j] = at;
       }
 #pragma unroll
       for (int j = 0; j < ITEMS; ++j) {
