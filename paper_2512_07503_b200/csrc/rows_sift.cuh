@@ -271,10 +271,10 @@ struct alignas(16) SiftSample {
 };
 
 // The groups' maxima of a row, by NT threads, four vectors per thread at a time (all there are when 256 threads share the
-// work).  `after_loads()` is called behind the first round's loads; the caller sees to the barrier behind it all.
-template <int DTYPE, bool HAS_U, bool HAS_T, int NT, typename AfterLoads>
+// work).  The caller sees to the barrier behind it.
+template <int DTYPE, bool HAS_U, bool HAS_T, int NT>
 __device__ __forceinline__ void sift_sample(const RowArgs& a, const SiftCfg& cfg, SiftSample& out, const char* c_row, const char* u_row,
-                                            int tid, AfterLoads after_loads) {
+                                            int tid) {
   constexpr int EV = SiftTraits<DTYPE>::kVec, ES = SiftTraits<DTYPE>::kElem;
   constexpr int NV = NT >= 256 ? kSiftGroups / NT : 4;
   const float neg_inf = __int_as_float(0xff800000);
@@ -298,7 +298,6 @@ __device__ __forceinline__ void sift_sample(const RowArgs& a, const SiftCfg& cfg
       c[j] = ldg_now(c_row + at);
       if (HAS_U) u[HAS_U ? j : 0] = ldg_now(u_row + at);
     }
-    if (v0 == tid) after_loads();
 #pragma unroll
     for (int j = 0; j < NV; ++j) {
       uint64_t y2[EV / 2];
@@ -912,7 +911,7 @@ rows_stream_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ Si
       } else {
         const int64_t off = st.tab[k].off;
         sift_sample<DTYPE, HAS_U, HAS_T, 32>(a, cfg, sample, static_cast<const char*>(row_ptr(a.cond, DTYPE, off)),
-                                             HAS_U ? static_cast<const char*>(row_ptr(a.uncond, DTYPE, off)) : nullptr, lane, [] {});
+                                             HAS_U ? static_cast<const char*>(row_ptr(a.uncond, DTYPE, off)) : nullptr, lane);
       }
       __syncwarp();
       const float2 tau = sift_threshold(sample, (uint32_t)cfg.rank, lane);
@@ -952,21 +951,24 @@ rows_stream_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ Si
     bulk_g2s(dst, row_ptr(a.cond, DTYPE, off), bytes, &st.full[x]);
     if (HAS_U) bulk_g2s(dst + kUnitBytes, row_ptr(a.uncond, DTYPE, off), bytes, &st.full[x]);
   };
+  // The team's first row: its sample's maxima, for the sampler.  Everybody waits for the CTA's first threshold, so the other
+  // teams' samples and the first copies (which the second team sends off) come behind the first team's sample.
+  if (team > 0) sift_wait(&st.sample_full[0], 0u, abort_flag);  // (nothing depends on it)
+  if (team == 1 && lane == 0 && units > 0) {
+    for (int x = 0; x < slots; ++x) issue(0, x, x);
+  }
+  __syncwarp();
   if (team < n_live) {
-    // the team's first row: its sample's maxima, for the sampler
     const int64_t off = st.tab[team].off;
-    sift_sample<DTYPE, HAS_U, HAS_T, kTeamThreads>(
-        a, cfg, sample, static_cast<const char*>(row_ptr(a.cond, DTYPE, off)),
-        HAS_U ? static_cast<const char*>(row_ptr(a.uncond, DTYPE, off)) : nullptr, tid, [&] {
-          // the first copies go out behind the first row's sample, not before it: everybody waits for that
-          if (team == 0 && lane == 0 && units > 0) {
-            for (int x = 0; x < slots; ++x) issue(0, x, x);
-          }
-          __syncwarp();
-        });
+    sift_sample<DTYPE, HAS_U, HAS_T, kTeamThreads>(a, cfg, sample, static_cast<const char*>(row_ptr(a.cond, DTYPE, off)),
+                                                   HAS_U ? static_cast<const char*>(row_ptr(a.uncond, DTYPE, off)) : nullptr, tid);
     __syncwarp();
     if (lane == 0) mbar_arrive(&st.sample_full[team]);
   }
+  if (teams == 1 && lane == 0 && units > 0) {
+    for (int x = 0; x < slots; ++x) issue(0, x, x);
+  }
+  __syncwarp();
   const uint64_t s2 = pack2(a.s, a.s), t2 = pack2(a.inv_T, a.inv_T);
   SiftTarget to;
   to.y_at = smem_u32(list_y + warp * cfg.seg_cap);
@@ -1150,7 +1152,7 @@ rows_cluster_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ S
   }
   __syncwarp();
   // every CTA of the cluster finds the threshold for itself: the sample is small, an exchange would cost more
-  sift_sample<DTYPE, HAS_U, HAS_T, NT>(a, cfg, sm.sample, c_row, u_row, tid, [] {});
+  sift_sample<DTYPE, HAS_U, HAS_T, NT>(a, cfg, sm.sample, c_row, u_row, tid);
   __syncthreads();
   // the search four bits at a time: warp w counts for the digit w, the largest digit that is reached enough is taken
   uint32_t key = 0;
