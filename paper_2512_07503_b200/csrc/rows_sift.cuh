@@ -42,6 +42,8 @@
 
 #include <cuda_bf16.h>
 
+#include <type_traits>
+
 #include "rows_pipeline.cuh"
 
 namespace sjd {
@@ -67,9 +69,11 @@ struct SiftCfg {
   int piece_vecs;    // 16-byte vectors per piece: 4, 2 or 1
   int groups;        // groups per vector, each represented by its largest element: 1, 2 or 4
   int rank;          // rank of tau0 among the groups, from the top
+  int packed;        // 1: entries may be screened in packed 16-bit arithmetic (see SiftScreen)
   int seg_len;       // ids per segment, a multiple of 8
   int seg_cap;       // candidates a segment's list holds (a multiple of 8)
   int teams, slots;  // stream kernel: teams per CTA, ring slots per warp
+  int once;          // stream kernel: the logits of the call exceed the L2
   int row_begin, row_end;  // stream kernel: this launch covers rows [row_begin, row_end)
 };
 
@@ -202,10 +206,9 @@ __device__ __forceinline__ uint32_t scan_incl(uint32_t v, int lane) {
 // ---------------------------------------------------------------------------------------------------
 // rank search: the bin b with (entries above b) < target <= (entries in b and above), by one
 // warp, which also leaves the histogram zero.  A bin is 0 when there are fewer than `target` entries in bins 1 and
-// above.  A call of its own: all searches of a row run the same few instructions, which matters where every
-// instruction is fetched for the first time.
+// above.
 // ---------------------------------------------------------------------------------------------------
-static __device__ __noinline__ void rank_search(SiftShared* sm, SiftHist* h, uint32_t t) {
+__device__ __forceinline__ void rank_search(SiftShared* sm, SiftHist* h, uint32_t t) {
   const int lane = threadIdx.x & 31;
   const uint32_t sum = h->coarse[31 - lane];  // lane 0 takes the topmost
   const uint32_t upto = scan_incl(sum, lane);
@@ -258,16 +261,98 @@ __device__ __forceinline__ SiftBinning sift_bins(float tau0, float top) {
   return SiftBinning{tau0, __fmul_rn(8.0f * kBinsLow, per), __fmul_rn((kSiftBins - 2) - kBinsCross, per)};
 }
 
-__device__ __forceinline__ uint4 ldg_now(const void* p) {  // issued where it stands
+// A sample's load, issued where it stands.  It is to stay in the L2 until its row comes through the ring, half a dozen rows
+// later: without the hint an eighth of the logits came from memory twice.
+__device__ __forceinline__ uint4 ldg_now(const void* p) {
   uint4 v;
-  asm volatile("ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+  uint64_t pol;
+  asm("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol));
+  asm volatile("ld.global.nc.L2::cache_hint.v4.u32 {%0, %1, %2, %3}, [%4], %5;" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p), "l"(pol));
   return v;
+}
+
+// packed 16-bit arithmetic: DTYPE 1 bf16, 2 fp16
+template <int DTYPE>
+__device__ __forceinline__ uint32_t fma_pair(uint32_t a, uint32_t b, uint32_t c) {
+  uint32_t r;
+  if (DTYPE == 2) asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(c));
+  else asm("fma.rn.bf16x2 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(c));
+  return r;
+}
+template <int DTYPE>
+__device__ __forceinline__ uint32_t add_pair(uint32_t a, uint32_t b) {
+  uint32_t r;
+  if (DTYPE == 2) asm("add.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+  else asm("add.rn.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+  return r;
+}
+template <int DTYPE>
+__device__ __forceinline__ uint32_t largest2(uint32_t m, uint32_t w) {  // max(m, |w|) of both halves; a NaN is passed over
+  uint32_t r;
+  if (DTYPE == 2) asm("{\n\t.reg .b32 t;\n\tabs.f16x2 t, %2;\n\tmax.f16x2 %0, %1, t;\n\t}" : "=r"(r) : "r"(m), "r"(w));
+  else asm("{\n\t.reg .b32 t;\n\tabs.bf16x2 t, %2;\n\tmax.bf16x2 %0, %1, t;\n\t}" : "=r"(r) : "r"(m), "r"(w));
+  return r;
+}
+template <int DTYPE>
+__device__ __forceinline__ float largest_of(uint32_t m) {
+  if (DTYPE == 2) {
+    const float2 f = f16_pair(m);
+    return fmaxf(f.x, f.y);
+  }
+  return fmaxf(bf16_lo(m), bf16_hi(m));
+}
+// a float in the 16-bit type, rounded to nearest, twice in a word
+template <int DTYPE>
+__device__ __forceinline__ uint32_t pair_of(float x) {
+  uint32_t r;
+  if (DTYPE == 2) asm("cvt.rn.f16x2.f32 %0, %1, %1;" : "=r"(r) : "f"(x));
+  else asm("cvt.rn.bf16x2.f32 %0, %1, %1;" : "=r"(r) : "f"(x));
+  return r;
+}
+
+// 16-bit logits: entries are screened in packed 16-bit arithmetic, two to an instruction, and only what passes is merged
+// exactly.  With guidance g = s (c - u) + u reaches g0 (the value before the temperature) only if s c + ((1 - s) u - t) >= 0
+// for a t that lies below g0 by more than the bracket can be off: the product-sum's own rounding cannot change its sign, the
+// bracket is off by its rounding, 2^-8 (bf16) or 2^-11 (fp16) of |1 - s| |u| + |t| at most, and t by as much of |t|.  So s and
+// 1 - s have to be numbers of the type (the host sees to that), and |u| has to stay below a limit that t was chosen for: a
+// unit that holds a larger one is compared exactly.  About a tenth more entries pass than reach tau0; they end as
+// candidates below tau0, in bin 0.  Without guidance c is compared with the largest number of the type up to g0.
+// Two instructions per entry instead of four; worth it while few entries pass anyway (the host's rule): 1,000 rows of 65,536
+// fp16 entries, K=100: 59.7 -> 57.3 us.
+struct SiftScreen {
+  uint32_t s2, b2, t2;  // s, 1 - s and -t, pairs
+  float u_limit;        // negative: this row is compared exactly
+};
+template <int DTYPE, bool HAS_U, bool HAS_T>
+__device__ __forceinline__ SiftScreen sift_screen(const RowArgs& a, const SiftCfg& cfg, float tau0, float u_max) {
+  SiftScreen r{0u, 0u, 0u, -1.0f};
+  if (DTYPE == 0 || !cfg.packed) return r;
+  constexpr float kRound = DTYPE == 2 ? 0x1p-11f : 0x1p-8f;
+  float g0 = HAS_T ? __fdiv_rn(tau0, a.inv_T) : tau0;
+  g0 = __fmaf_rd(fabsf(g0), -0x1p-20f, g0);
+  if (HAS_U) {
+    const float b = 1.0f - a.s, limit = 1.25f * u_max, reach = fabsf(b) * limit + 2.0f * fabsf(g0);
+    if (!(reach < 3.0e4f)) return r;
+    r.s2 = pair_of<DTYPE>(a.s);
+    r.b2 = pair_of<DTYPE>(b);
+    r.t2 = pair_of<DTYPE>(__fmaf_rn(1.03f * kRound, reach, -g0));
+    r.u_limit = limit;
+  } else {
+    if (!(fabsf(g0) < 3.0e4f)) return r;
+    uint32_t t = pair_of<DTYPE>(g0);
+    const float back = DTYPE == 2 ? f16_pair(t).x : bf16_lo(t);
+    if (back > g0) t = (t & 0x7fffu) == 0u ? 0x80018001u : (t & 0x8000u) ? t + 0x00010001u : t - 0x00010001u;  // the number below
+    r.t2 = t ^ 0x80008000u;
+    r.u_limit = 0.0f;
+  }
+  return r;
 }
 
 // what a row's threshold is found from
 struct alignas(16) SiftSample {
   uint32_t m[kSiftGroups / 2];  // the groups' maxima as bf16 pairs, in no particular order
   uint32_t top_key;             // largest sample value (0 between rows)
+  uint32_t u_bits;              // largest |uncond| of the sample, 16-bit types (a float's bits; 0 between rows)
 };
 
 // The groups' maxima of a row, by NT threads, four vectors per thread at a time (all there are when 256 threads share the
@@ -284,6 +369,7 @@ __device__ __forceinline__ void sift_sample(const RowArgs& a, const SiftCfg& cfg
   uint16_t* const m = reinterpret_cast<uint16_t*>(out.m);
   auto put = [&](int x, float v) { m[x] = __bfloat16_as_ushort(__float2bfloat16_rn(v)); };
   float top = neg_inf;
+  uint32_t u_max = 0u;  // largest |uncond|, a pair
 #pragma unroll 1
   for (int v0 = tid; v0 - tid < vecs; v0 += NT * NV) {
     uint4 c[NV], u[HAS_U ? NV : 1];
@@ -302,6 +388,10 @@ __device__ __forceinline__ void sift_sample(const RowArgs& a, const SiftCfg& cfg
     for (int j = 0; j < NV; ++j) {
       uint64_t y2[EV / 2];
       merge_vec<DTYPE, HAS_U, HAS_T>(c[j], u[HAS_U ? j : 0], s2, t2, y2);
+      if (HAS_U && DTYPE != 0) {
+        const uint4 w = u[HAS_U ? j : 0];
+        u_max = largest2<DTYPE>(largest2<DTYPE>(largest2<DTYPE>(largest2<DTYPE>(u_max, w.x), w.y), w.z), w.w);
+      }
       float y[EV];
 #pragma unroll
       for (int k = 0; k < EV / 2; ++k) unpack2(y2[k], y[2 * k], y[2 * k + 1]);
@@ -338,6 +428,10 @@ __device__ __forceinline__ void sift_sample(const RowArgs& a, const SiftCfg& cfg
   for (int x = vecs * cfg.groups + tid; x < kSiftGroups; x += NT) m[x] = 0xff80u;
   const uint32_t warp_top = __reduce_max_sync(0xffffffffu, float_key(__fadd_rn(top, 0.0f)));
   if ((tid & 31) == 0) atomicMax(&out.top_key, warp_top);
+  if (HAS_U && DTYPE != 0) {
+    const uint32_t warp_u = __reduce_max_sync(0xffffffffu, __float_as_uint(largest_of<DTYPE>(u_max)));
+    if ((tid & 31) == 0) atomicMax(&out.u_bits, warp_u);
+  }
 }
 
 // The search for the threshold goes over the bf16 values as 16-bit keys that are ordered like them: the largest key whose
@@ -369,24 +463,28 @@ struct SiftMaxima {
     return __reduce_add_sync(0xffffffffu, (uint32_t)(bf16_lo(acc[0]) + bf16_hi(acc[0])));
   }
 };
-// {tau0, largest sample value} for the key found
-__device__ __forceinline__ float2 sift_tau(uint32_t key, uint32_t top_key) {
+// {tau0, largest sample value, largest |uncond| of the sample} for the key found
+struct SiftTau {
+  float tau0, top, u_max;
+};
+__device__ __forceinline__ SiftTau sift_tau(uint32_t key, const SiftSample& in) {
+  const uint32_t top_key = in.top_key;
   const float top = key_float(top_key), lowest = -3.402823466e38f;  // lowest: every finite value is a candidate
   // the maxima were rounded to nearest: the middle between this bf16 value and the one below is what they all reach
   const float at = key_float(key << 16), below = key_float((key - 1u) << 16);
   float tau0 = __fmaf_rd(__fsub_rn(at, below), -0.51f, at);
   if (key == 0u || !(tau0 >= lowest) || !(top <= 3.402823466e38f)) tau0 = lowest;
-  return make_float2(tau0, top);
+  return SiftTau{tau0, top, __uint_as_float(in.u_bits)};
 }
 // by one warp, bit by bit
-__device__ __forceinline__ float2 sift_threshold(const SiftSample& in, uint32_t rank, int lane) {
+__device__ __forceinline__ SiftTau sift_threshold(const SiftSample& in, uint32_t rank, int lane) {
   SiftMaxima m;
   m.load(in, lane);
   uint32_t key = 0;
 #pragma unroll 1
   for (uint32_t bit = 0x8000u; bit != 0u; bit >>= 1)
     if (m.reaching(key | bit) >= rank) key |= bit;
-  return sift_tau(key, in.top_key);
+  return sift_tau(key, in);
 }
 
 // ---------------------------------------------------------------------------------------------------
@@ -419,6 +517,41 @@ __device__ __forceinline__ uint32_t piece_hits(uint32_t c_at, uint32_t u_at, int
   if (DTYPE != 0) return __funnelshift_l(~miss, ~miss, 8 * rot);
   const uint32_t x = (~miss & 0xffffu) * 0x10001u;
   return (x >> (16 - 4 * rot)) & 0xffffu;
+}
+
+// The same by packed screening.  The signs of four entries are gathered as bytes of -1 by one permute; a dot product with
+// the powers of two makes them four bits.  u_max: largest |uncond| met.
+template <int DTYPE, bool HAS_U>
+__device__ __forceinline__ uint32_t piece_screened(uint32_t c_at, uint32_t u_at, int rot, const SiftScreen& sc, uint32_t& u_max) {
+  int32_t acc = 0;  // minus the missed entries' bits
+#pragma unroll
+  for (int j = 3; j >= 0; --j) {
+    const uint32_t off = (uint32_t)(((j + rot) & 3) << 4);
+    const uint4 cv = lds128(c_at + off);
+    const uint32_t c[4] = {cv.x, cv.y, cv.z, cv.w};
+    uint32_t w[4];
+    if (HAS_U) {
+      const uint4 uv = lds128(u_at + off);
+      const uint32_t u[4] = {uv.x, uv.y, uv.z, uv.w};
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        w[k] = fma_pair<DTYPE>(sc.s2, c[k], fma_pair<DTYPE>(sc.b2, u[k], sc.t2));
+        u_max = largest2<DTYPE>(u_max, u[k]);
+      }
+    } else {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) w[k] = add_pair<DTYPE>(c[k], sc.t2);
+    }
+    acc <<= 8;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      uint32_t signs;
+      asm("prmt.b32 %0, %1, %2, 0xfdb9;" : "=r"(signs) : "r"(w[2 * k]), "r"(w[2 * k + 1]));
+      asm("dp4a.s32.u32 %0, %1, %2, %0;" : "+r"(acc) : "r"(signs), "r"(k == 0 ? 0x08040201u : 0x80402010u));
+    }
+  }
+  const uint32_t hits = (uint32_t)acc - 1u;  // ~(-acc)
+  return __funnelshift_l(hits, hits, 8 * rot);
 }
 
 // ids of the set bits of x (bit 0: id `first`), from the highest down, to the halfwords below `put`
@@ -460,24 +593,34 @@ __device__ __forceinline__ void count_at(uint32_t at) {
 // what the list keeps plus `bias`.  n: candidates so far (cap + 1 or more: the list has run over).
 template <int DTYPE, bool HAS_U, bool HAS_T, bool REMOTE>
 __device__ __forceinline__ void sift_unit(const RowArgs& a, uint32_t c_unit, uint32_t u_unit, int valid, uint32_t rel, uint32_t bias,
-                                          uint64_t s2, uint64_t t2, const SiftBinning& bins, const SiftTarget& to, uint32_t cap,
-                                          int lane, uint32_t& n, float& vmax) {
+                                          uint64_t s2, uint64_t t2, const SiftBinning& bins, const SiftScreen& screen,
+                                          const SiftTarget& to, uint32_t cap, int lane, uint32_t& n, float& vmax) {
   constexpr int ES = SiftTraits<DTYPE>::kElem, EP = SiftTraits<DTYPE>::kPiece, EU = SiftTraits<DTYPE>::kUnit;
-  const uint64_t neg_tau2 = pack2(-bins.tau0, -bins.tau0);
-  uint32_t x0, x1 = 0;    // hits of the lane's first and second piece
-  uint32_t run = 2 * EP;  // consecutive elements of a lane
-  if (valid > EU / 2) {
-    const uint32_t at = 128u * (uint32_t)lane, swap = ((uint32_t)lane & 4u) << 4;
-    x0 = piece_hits<DTYPE, HAS_U, HAS_T>(c_unit + (at ^ swap), u_unit + (at ^ swap), lane & 3, s2, t2, neg_tau2);
-    x1 = piece_hits<DTYPE, HAS_U, HAS_T>(c_unit + (at ^ swap ^ 64u), u_unit + (at ^ swap ^ 64u), lane & 3, s2, t2, neg_tau2);
-    if (swap) {
-      const uint32_t x = x0;
-      x0 = x1;
-      x1 = x;
-    }
-  } else {
-    run = EP;
-    x0 = piece_hits<DTYPE, HAS_U, HAS_T>(c_unit + 64u * (uint32_t)lane, u_unit + 64u * (uint32_t)lane, (lane >> 1) & 3, s2, t2, neg_tau2);
+  uint32_t x0 = 0, x1 = 0;  // hits of the lane's first and second piece
+  const bool whole = valid > EU / 2;
+  const uint32_t run = whole ? 2 * EP : EP;  // consecutive elements of a lane
+  // where this lane's pieces lie and where it starts in them, so that the lanes served together touch different banks
+  const uint32_t swap = whole ? ((uint32_t)lane & 4u) << 4 : 0u;
+  const uint32_t at0 = whole ? (128u * (uint32_t)lane) ^ swap : 64u * (uint32_t)lane, at1 = at0 ^ 64u;
+  const int rot = whole ? lane & 3 : (lane >> 1) & 3;
+  // (a unit that is not full is compared exactly: what lies behind its end must not decide how it is compared, because the
+  // two ways pass different entries below tau0 and a sum over differently placed candidates rounds differently)
+  bool exact = DTYPE == 0 || screen.u_limit < 0.0f || (uint32_t)valid < 32u * run;
+  if (DTYPE != 0 && !exact) {
+    uint32_t u_max = 0u;
+    x0 = piece_screened<DTYPE, HAS_U>(c_unit + at0, u_unit + at0, rot, screen, u_max);
+    if (whole) x1 = piece_screened<DTYPE, HAS_U>(c_unit + at1, u_unit + at1, rot, screen, u_max);
+    if (HAS_U) exact = __any_sync(0xffffffffu, largest_of<DTYPE>(u_max) > screen.u_limit);
+  }
+  if (exact) {
+    const uint64_t neg_tau2 = pack2(-bins.tau0, -bins.tau0);
+    x0 = piece_hits<DTYPE, HAS_U, HAS_T>(c_unit + at0, u_unit + at0, rot, s2, t2, neg_tau2);
+    if (whole) x1 = piece_hits<DTYPE, HAS_U, HAS_T>(c_unit + at1, u_unit + at1, rot, s2, t2, neg_tau2);
+  }
+  if (swap) {
+    const uint32_t x = x0;
+    x0 = x1;
+    x1 = x;
   }
   if (DTYPE == 0) {
     x0 |= x1 << 16;
@@ -502,22 +645,34 @@ __device__ __forceinline__ void sift_unit(const RowArgs& a, uint32_t c_unit, uin
     put_ids(x0, first, put);
   }
   __syncwarp();
-  // candidates: merged, binned and kept
+  // candidates: merged, binned and kept, two groups of 32 at a time (their loads do not wait for one another)
   const uint32_t c_rel = c_unit - rel * (uint32_t)ES, u_rel = u_unit - rel * (uint32_t)ES;
-  for (uint32_t i = (uint32_t)lane; i < ((total + 31u) & ~31u); i += 32u) {
-    const bool in = i < total;
-    const uint32_t k = n + min(i, total - 1u);
-    const uint32_t id = lds16(to.scratch_at + 2u * k);
-    const float y = merge_entry<DTYPE, HAS_U, HAS_T>(c_rel + id * (uint32_t)ES, u_rel + id * (uint32_t)ES, a.s, a.inv_T);
-    const uint32_t bin = in ? min(__float2uint_rz(bins.at(y)), (uint32_t)kSiftBins - 1u) : 0u;
-    count_at<REMOTE>(to.hist_at + 4u * bin);
-    count_at<REMOTE>(to.hist_at + 4u * (kSiftBins + (bin >> 5)));
-    vmax = fmaxf(vmax, y);
-    if (in) {
-      put_f32<REMOTE>(to.y_at + 4u * k, y);
-      if (REMOTE) put_u16<true>(to.id_at + 2u * k, id + bias);
+  auto keep = [&](auto groups, uint32_t i0) {
+    constexpr int G = decltype(groups)::value;
+    uint32_t id[G];
+    float y[G];
+#pragma unroll
+    for (int j = 0; j < G; ++j) id[j] = lds16(to.scratch_at + 2u * (n + min(i0 + 32u * j + (uint32_t)lane, total - 1u)));
+#pragma unroll
+    for (int j = 0; j < G; ++j)
+      y[j] = merge_entry<DTYPE, HAS_U, HAS_T>(c_rel + id[j] * (uint32_t)ES, u_rel + id[j] * (uint32_t)ES, a.s, a.inv_T);
+#pragma unroll
+    for (int j = 0; j < G; ++j) {
+      const uint32_t i = i0 + 32u * j + (uint32_t)lane, k = n + i;
+      const bool in = i < total;
+      const uint32_t bin = in ? min(__float2uint_rz(bins.at(y[j])), (uint32_t)kSiftBins - 1u) : 0u;
+      count_at<REMOTE>(to.hist_at + 4u * bin);
+      count_at<REMOTE>(to.hist_at + 4u * (kSiftBins + (bin >> 5)));
+      vmax = fmaxf(vmax, y[j]);
+      if (in) {
+        put_f32<REMOTE>(to.y_at + 4u * k, y[j]);
+        if (REMOTE) put_u16<true>(to.id_at + 2u * k, id[j] + bias);
+      }
     }
-  }
+  };
+  uint32_t i0 = 0;
+  for (; i0 + 32u < total; i0 += 64u) keep(std::integral_constant<int, 2>(), i0);
+  if (i0 < total) keep(std::integral_constant<int, 1>(), i0);
   n += total;
 }
 
@@ -788,7 +943,7 @@ struct alignas(16) StreamShared {
   uint32_t used[kTeamWarps * kMaxTeams * kMaxSlots];  // copies issued for that barrier so far
   // for every team: a row's sample is complete, and {tau0, largest sample value} of rows to come, in two places used in turn
   uint64_t sample_full[kMaxTeams], tau_full[2 * kMaxTeams], tau_free[2 * kMaxTeams];
-  float2 tau[2 * kMaxTeams];
+  SiftTau tau[2 * kMaxTeams];
   uint32_t seg_n[kMaxTeams * kTeamWarps];      // candidates per segment
   int32_t redo[kStreamRows];                   // rows the single pass could not finish (redone at the end)
   int n_live, n_redo, abort;
@@ -806,6 +961,13 @@ __host__ __device__ inline size_t sift_stream_smem(int teams, int seg_cap, int s
   return sift_stream_rings(teams, seg_cap) + (size_t)kTeamWarps * slots * kUnitBytes * (has_u ? 2 : 1);
 }
 
+// bulk_g2s with an L2 hint
+__device__ __forceinline__ void bulk_g2s_hinted(void* dst, const void* src, uint32_t bytes, uint64_t* bar, uint64_t policy) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;" ::"r"(smem_u32(dst)),
+      "l"(src), "r"(bytes), "r"(smem_u32(bar)), "l"(policy)
+      : "memory");
+}
 __device__ __forceinline__ void ask_l2(const void* p, uint32_t bytes) {
   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
 }
@@ -859,7 +1021,7 @@ rows_stream_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ Si
     mbar_init(&st.tau_free[threadIdx.x], kTeamWarps);
     if (threadIdx.x < kMaxTeams) mbar_init(&st.sample_full[threadIdx.x], kTeamWarps);
   }
-  if (tid == 0) sample.top_key = 0u;
+  if (tid == 0) sample.top_key = sample.u_bits = 0u;
   if (threadIdx.x == 0) {
     st.n_redo = 0;
     st.abort = 0;
@@ -914,12 +1076,13 @@ rows_stream_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ Si
                                              HAS_U ? static_cast<const char*>(row_ptr(a.uncond, DTYPE, off)) : nullptr, lane);
       }
       __syncwarp();
-      const float2 tau = sift_threshold(sample, (uint32_t)cfg.rank, lane);
+      const SiftTau tau = sift_threshold(sample, (uint32_t)cfg.rank, lane);
       const int x = 2 * team + (n & 1);
       if (n >= 2 && !sift_wait(&st.tau_free[x], (uint32_t)((n >> 1) - 1) & 1u, abort_flag)) break;
       __syncwarp();
       if (lane == 0) {
         sample.top_key = 0u;
+        sample.u_bits = 0u;
         st.tau[x] = tau;
         mbar_arrive(&st.tau_full[x]);
       }
@@ -933,6 +1096,11 @@ rows_stream_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ Si
   const int units = (seg_n + EU - 1) / EU;
   // Copies go through the ring of the warp's segment in order: the units of the segment for row 0, row 1, ...; team t takes
   // rows t, t + teams, ...  Whoever has worked a unit through asks for the copy that goes into its slot next.
+  // Logits that exceed the L2 leave it first (they make room for samples and outputs: 1,024 rows of 65,536 74.4 -> 73.4 us);
+  // smaller ones are left where their writer put them (of 16,384: 45.7, with the hint 46.6).
+  uint64_t policy;
+  if (cfg.once) asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
+  else asm("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(policy));
   auto issue = [&](int k, int unit, int slot) {
     while (unit >= units) {
       ++k;
@@ -948,8 +1116,8 @@ rows_stream_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ Si
     const int x = (warp * kMaxTeams + k % teams) * kMaxSlots + slot;
     ++st.used[x];
     mbar_arrive_expect_tx(&st.full[x], bytes * (HAS_U ? 2u : 1u));
-    bulk_g2s(dst, row_ptr(a.cond, DTYPE, off), bytes, &st.full[x]);
-    if (HAS_U) bulk_g2s(dst + kUnitBytes, row_ptr(a.uncond, DTYPE, off), bytes, &st.full[x]);
+    bulk_g2s_hinted(dst, row_ptr(a.cond, DTYPE, off), bytes, &st.full[x], policy);
+    if (HAS_U) bulk_g2s_hinted(dst + kUnitBytes, row_ptr(a.uncond, DTYPE, off), bytes, &st.full[x], policy);
   };
   // The team's first row: its sample's maxima, for the sampler.  Everybody waits for the CTA's first threshold, so the other
   // teams' samples and the first copies (which the second team sends off) come behind the first team's sample.
@@ -985,7 +1153,8 @@ rows_stream_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ Si
     bool ok = *abort_flag == 0;
     const int x = 2 * team + tau_at;
     if (ok) ok = sift_wait(&st.tau_full[x], tau_phase, abort_flag);
-    const SiftBinning bins = sift_bins(st.tau[x].x, st.tau[x].y);
+    const SiftBinning bins = sift_bins(st.tau[x].tau0, st.tau[x].top);
+    const SiftScreen screen = sift_screen<DTYPE, HAS_U, HAS_T>(a, cfg, st.tau[x].tau0, st.tau[x].u_max);
     __syncwarp();
     if (lane == 0) mbar_arrive(&st.tau_free[x]);
     tau_phase ^= (uint32_t)tau_at;
@@ -999,7 +1168,7 @@ rows_stream_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ Si
       phase ^= 1u << slot;
       const uint32_t c_unit = ring_at + (uint32_t)slot * kSlot;
       sift_unit<DTYPE, HAS_U, HAS_T, false>(a, c_unit, c_unit + kUnitBytes, seg_n - unit * EU, (uint32_t)(unit * EU), 0u, s2, t2, bins,
-                                            to, cap, lane, n, vmax);
+                                            screen, to, cap, lane, n, vmax);
       __syncwarp();
       if (lane == 0) issue(k, unit + slots, slot);
       if (++slot == slots) slot = 0;
@@ -1104,7 +1273,7 @@ rows_cluster_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ S
   if (tid < kClusterWarps) mbar_init(&sm.full[tid], 1);
   if (tid == 0) {
     sm.lost = 0u;
-    sm.sample.top_key = 0u;
+    sm.sample.top_key = sm.sample.u_bits = 0u;
   }
   fence_barrier_init();
   __syncthreads();
@@ -1170,8 +1339,9 @@ rows_cluster_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ S
       __syncthreads();
     }
   }
-  const float2 tau = sift_tau(key, sm.sample.top_key);
-  const SiftBinning bins = sift_bins(tau.x, tau.y);
+  const SiftTau tau = sift_tau(key, sm.sample);
+  const SiftBinning bins = sift_bins(tau.tau0, tau.top);
+  const SiftScreen screen = sift_screen<DTYPE, HAS_U, HAS_T>(a, cfg, tau.tau0, tau.u_max);
   SiftTarget to;
   to.y_at = in_first_cta(list_y + (size_t)seg * cfg.seg_cap);
   to.id_at = in_first_cta(list_id + (size_t)seg * cfg.seg_cap);
@@ -1187,7 +1357,7 @@ rows_cluster_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ S
     const uint32_t c_at = smem_u32(stage), u_at = smem_u32(u_stage);
     for (int k = 0; k < units; ++k)
       sift_unit<DTYPE, HAS_U, HAS_T, true>(a, c_at + (uint32_t)k * kUnitBytes, u_at + (uint32_t)k * kUnitBytes, seg_n - k * EU,
-                                           (uint32_t)(k * EU), bias, s2, t2, bins, to, cap, lane, n, vmax);
+                                           (uint32_t)(k * EU), bias, s2, t2, bins, screen, to, cap, lane, n, vmax);
   }
   __syncwarp();
   const uint32_t wmax = __reduce_max_sync(0xffffffffu, float_key(vmax));

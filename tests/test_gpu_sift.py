@@ -80,3 +80,24 @@ print("ROWS_TIMEOUT_OK")
 """ % (root, os.path.join(root, "tests"))
     out = subprocess.run([sys.executable, "-c", script], env=dict(os.environ, SJD_LIBRARY=lib), capture_output=True, text=True, timeout=600)
     assert out.returncode == 0 and "ROWS_TIMEOUT_OK" in out.stdout, out.stdout[-2000:] + out.stderr[-4000:]
+
+
+@pytest.mark.parametrize("scale,temperature", [(3.0, 1.0), (7.5, 0.8), (1.0, 1.0), (3.1, 1.3), (0.0, 1.0)])
+@pytest.mark.parametrize("dtype", [wk.BF16, wk.F16])
+@pytest.mark.parametrize("B,W", [(1, 4), (2, 90)])
+def test_screening_keeps_what_cancels(B, W, dtype, scale, temperature):
+    # the merged logit is a small difference of large ones, and some unconditional logits exceed everything the sample
+    # shows: what the packed 16-bit screening must not lose
+    from gpu_harness import check_parity, oracle_prime, step_kwargs
+    wl = wk.CONFIGS["cfg2"].scaled(B=B, W=W, V=8192, dtype=dtype, top_k=150, cfg_scale=scale, temperature=temperature, seed=W)
+    inp = wk.make_step_inputs(wl)
+    rng = np.random.default_rng(W + dtype)
+    shape = inp.cond.shape
+    y = rng.standard_normal(shape).astype(np.float32) * 3
+    u = rng.standard_normal(shape).astype(np.float32) * 40
+    u[rng.random(shape) < 0.003] *= 30
+    c = u + (y - u) / scale if scale else u + y
+    for arr, x in ((inp.cond, c), (inp.uncond, u), (inp.prev_cond, c + 0.5), (inp.prev_uncond, u)):
+        arr[:] = wk._store(x.astype(np.float32), dtype)
+    prev = oracle_prime(inp)
+    check_parity(inp.cond, inp.uncond, prev.tokens, prev.probs, step_kwargs(inp), inp.win_len)
