@@ -164,11 +164,19 @@ cudaError_t launch_pipeline(const sjd::RowArgs& ra, const sjd::PipeCfg& cfg, siz
 // kcap candidates when the estimate is off by 4.5 standard deviations (probability below 4e-6): p - 4.5 sd(p) =
 // kcap / V.  From the n sampled elements themselves sd(p) = sqrt(p (1 - p) / n); from the maxima of N vectors of G
 // elements, of which the share q = 1 - (1 - p)^G lies above the threshold, sd(p) = sqrt(q (1 - q) / N) / (dq/dp).
+// (Part of every call: a handful of multiplications, no pow.)
+double power(double x, int G) {  // G: 1, 2, 4 or 8
+  if (G > 1) x *= x;
+  if (G > 2) x *= x;
+  if (G > 4) x *= x;
+  return x;
+}
 double aimed_share(double want, double N, int G, double* sd) {
-  double p = want;
-  for (int it = 0; it < 40; ++it) {
-    const double q = 1.0 - std::pow(1.0 - p, G);
-    *sd = std::sqrt(q * (1.0 - q) / N) / (G * std::pow(1.0 - p, G - 1));
+  double p = want, last = 0.0;
+  for (int it = 0; it < 40 && std::fabs(p - last) > 1e-5 * p; ++it) {
+    const double rest = power(1.0 - p, G), q = 1.0 - rest;
+    *sd = std::sqrt(q * rest / N) * (1.0 - p) / (G * rest);
+    last = p;
     p = want + 4.5 * *sd;
     if (!(p < 0.9)) return 1.0;
   }
@@ -204,9 +212,10 @@ bool plan_sift(const sjd_params* P, int kcap, bool has_u, SiftPlan* plan) {
   for (int pv = 4; pv >= 1; pv >>= 1) {
     if (pv > 1 && c.piece_stride * es < 32 * pv) continue;  // pieces take half of the row at most
     int vecs = 0;
-    for (int j = 0; j < sjd::kSiftPieces; ++j)
-      for (int k = 0; k < pv; ++k)
-        if (k * ev < c.piece_stride && j * c.piece_stride + k * ev < V) ++vecs;
+    for (int k = 0; k < pv && k * ev < c.piece_stride; ++k) {  // pieces that have a k-th vector
+      const int with = (V - k * ev + c.piece_stride - 1) / c.piece_stride;
+      vecs += with < sjd::kSiftPieces ? with : sjd::kSiftPieces;
+    }
     for (int g = 1; g * pv <= 4; g <<= 1) {
       double sd_g;
       const double p_g = aimed_share(want, (double)vecs * g, ev / g, &sd_g);
@@ -215,7 +224,7 @@ bool plan_sift(const sjd_params* P, int kcap, bool has_u, SiftPlan* plan) {
       sd = sd_g;
       c.piece_vecs = pv;
       c.groups = g;
-      c.rank = (int)std::ceil(vecs * g * (1.0 - std::pow(1.0 - p, ev / g)));
+      c.rank = (int)std::ceil(vecs * g * (1.0 - power(1.0 - p, ev / g)));
     }
   }
   if (p > 0.6) return false;
