@@ -43,6 +43,30 @@ class SjdError(RuntimeError):
     pass
 
 
+_f32, _i32 = torch.float32, torch.int32
+
+
+class _on:
+    """``torch.cuda.device(...)`` for the common case that the device is current already: entering and leaving that
+    context costs as much as a kernel launch."""
+    __slots__ = ("index", "prev")
+
+    def __init__(self, device: torch.device):
+        self.index = device.index
+
+    def __enter__(self):
+        cur = torch.cuda.current_device()
+        self.prev = -1
+        if self.index is not None and self.index != cur:
+            self.prev = cur
+            torch.cuda.set_device(self.index)
+
+    def __exit__(self, *exc):
+        if self.prev >= 0:
+            torch.cuda.set_device(self.prev)
+        return False
+
+
 _lib = None
 
 
@@ -118,17 +142,18 @@ class DeviceProbs:
         return p
 
     def c_struct(self) -> sjd_probs:
-        for t, dt in ((self.tok_prob, torch.float32), (self.ids, torch.int32), (self.vals, torch.float32),
-                      (self.cnt, torch.int32)):
-            if not (t.is_cuda and t.is_contiguous() and t.dtype == dt):
-                raise SjdError("sjd_probs arrays must be contiguous CUDA tensors of the documented dtypes")
-        return sjd_probs(self.tok_prob.data_ptr(), self.ids.data_ptr(), self.vals.data_ptr(), self.cnt.data_ptr())
+        a, b, c, d = self.tok_prob, self.ids, self.vals, self.cnt
+        if not (a.is_cuda and b.is_cuda and c.is_cuda and d.is_cuda and a.dtype is _f32 and b.dtype is _i32 and
+                c.dtype is _f32 and d.dtype is _i32 and a.is_contiguous() and b.is_contiguous() and c.is_contiguous() and
+                d.is_contiguous()):
+            raise SjdError("sjd_probs arrays must be contiguous CUDA tensors of the documented dtypes")
+        return sjd_probs(a.data_ptr(), b.data_ptr(), c.data_ptr(), d.data_ptr())
 
 
-def _opt_ptr(t: Optional[torch.Tensor], dtype=torch.int32) -> Optional[int]:
+def _opt_ptr(t: Optional[torch.Tensor], dtype=_i32) -> Optional[int]:
     if t is None:
         return None
-    if not (t.is_cuda and t.is_contiguous() and t.dtype == dtype):
+    if not (t.is_cuda and t.dtype is dtype and t.is_contiguous()):
         raise SjdError("optional arrays must be contiguous CUDA tensors of the documented dtype")
     return t.data_ptr()
 
@@ -212,21 +237,20 @@ def sjd_step(logits_cond: torch.Tensor, logits_uncond: Optional[torch.Tensor], d
              out_tokens: torch.Tensor, out_probs: DeviceProbs) -> None:
     """Enqueue one verify-and-redraft step on ``params.stream``.  Same arguments as the C entry point."""
     _check_logits(logits_cond, logits_uncond)
-    q = draft_probs.c_struct() if draft_probs is not None else None
-    o = out_probs.c_struct()
-    with torch.cuda.device(logits_cond.device):
-        code = lib().sjd_step(logits_cond.data_ptr(), None if logits_uncond is None else logits_uncond.data_ptr(),
-                              _opt_ptr(drafts), C.byref(q) if q is not None else None, C.byref(params),
-                              int(philox_seed) & 0xFFFFFFFFFFFFFFFF, _opt_ptr(out_accept_len), _opt_ptr(out_tokens),
-                              C.byref(o))
-    _check(code)
+    q = C.byref(draft_probs.c_struct()) if draft_probs is not None else None
+    with _on(logits_cond.device):
+        code = (_lib or lib()).sjd_step(logits_cond.data_ptr(), None if logits_uncond is None else logits_uncond.data_ptr(),
+                                        _opt_ptr(drafts), q, C.byref(params), int(philox_seed) & 0xFFFFFFFFFFFFFFFF,
+                                        _opt_ptr(out_accept_len), _opt_ptr(out_tokens), C.byref(out_probs.c_struct()))
+    if code != 0:
+        _check(code)
 
 
 def sjd_window_init(params: sjd_params, n_total: int, philox_seed: int, win_len: torch.Tensor, pos_base: torch.Tensor,
                     iteration: torch.Tensor, drafts: torch.Tensor, draft_probs: DeviceProbs) -> None:
     """Fill the first window with randomly initialised drafts (uniform reference distribution)."""
     q = draft_probs.c_struct()
-    with torch.cuda.device(drafts.device):
+    with _on(drafts.device):
         code = lib().sjd_window_init(C.byref(params), int(n_total), int(philox_seed) & 0xFFFFFFFFFFFFFFFF,
                                      _opt_ptr(win_len), _opt_ptr(pos_base), _opt_ptr(iteration), _opt_ptr(drafts),
                                      C.byref(q))
@@ -240,7 +264,7 @@ def sjd_window_advance(params: sjd_params, n_total: int, philox_seed: int, accep
     """Commit the accepted prefix and the residual token, shift the window and refill it (same arguments as
     the C entry point)."""
     sp, nq = step_probs.c_struct(), next_probs.c_struct()
-    with torch.cuda.device(step_tokens.device):
+    with _on(step_tokens.device):
         code = lib().sjd_window_advance(C.byref(params), int(n_total), int(philox_seed) & 0xFFFFFFFFFFFFFFFF,
                                         _opt_ptr(accept_len), _opt_ptr(step_tokens), C.byref(sp), _opt_ptr(win_len),
                                         _opt_ptr(pos_base), _opt_ptr(iteration), _opt_ptr(next_drafts), C.byref(nq),
@@ -261,7 +285,7 @@ def sjd_step_static(logits_cond: torch.Tensor, logits_uncond: Optional[torch.Ten
     _check_logits(logits_cond, logits_uncond)
     q = draft_probs.c_struct() if draft_probs is not None else None
     o = out_probs.c_struct()
-    with torch.cuda.device(logits_cond.device):
+    with _on(logits_cond.device):
         code = lib().sjd_step_static(logits_cond.data_ptr(),
                                      None if logits_uncond is None else logits_uncond.data_ptr(), _opt_ptr(drafts),
                                      C.byref(q) if q is not None else None, C.byref(params),

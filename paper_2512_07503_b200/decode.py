@@ -25,19 +25,35 @@ class DecodeLoop:
         self.seed, self.device = seed, torch.device(device)
         dev = self.device
         i32 = dict(dtype=torch.int32, device=dev)
-        self.win_len = torch.full((batch,), min(window, n_total), **i32)
-        self.pos_base = torch.zeros(batch, **i32)
-        self.iteration = torch.zeros(batch, **i32)
+        # One zeroed allocation for everything the loop keeps (a launch instead of two dozen), cut into 256-byte aligned pieces.
+        # What done() looks at lies together: one copy to the host (page-locked: no staging).
+        kcap, rows = self.kcap, batch * window
+        sizes = [3 * batch] + [batch] * 3 + [rows] * 3 + [rows, rows * kcap, rows * kcap, rows] * 3
+        starts = [0]
+        for n in sizes:
+            starts.append(starts[-1] + (n + 63) // 64 * 64)
+        self._arena = torch.zeros(starts[-1], **i32)
+        piece = iter([self._arena[a:a + n] for a, n in zip(starts, sizes)])
+        self._state = next(piece).view(3, batch)
+        self._host_state = torch.empty(3, batch, dtype=torch.int32, pin_memory=True)
+        self.win_len, self.status, self.n_committed = self._state.unbind(0)
+        self.win_len.fill_(min(window, n_total))
+        self.pos_base, self.iteration, self.acc = (next(piece) for _ in range(3))
+        self.drafts = [next(piece).view(batch, window) for _ in range(2)]
+        self.toks = next(piece).view(batch, window)
+
+        def probs():
+            tok_prob, ids, vals, cnt = (next(piece) for _ in range(4))
+            f32 = torch.float32
+            return B.DeviceProbs(tok_prob.view(f32).view(batch, window), ids.view(batch, window, kcap),
+                                 vals.view(f32).view(batch, window, kcap), cnt.view(batch, window))
+
+        self.q = [probs(), probs()]
+        self.out = probs()
         self.committed = torch.full((batch, n_total), -1, **i32)
-        self.n_committed = torch.zeros(batch, **i32)
-        self.drafts = [torch.zeros(batch, window, **i32) for _ in range(2)]
-        self.q = [B.DeviceProbs.empty(batch, window, self.kcap, dev) for _ in range(2)]
-        self.out = B.DeviceProbs.empty(batch, window, self.kcap, dev)
-        self.acc = torch.zeros(batch, **i32)
-        self.toks = torch.zeros(batch, window, **i32)
-        self.status = torch.zeros(batch, **i32)
         self.cur = 0
-        proto = torch.empty(batch, window, vocab, dtype=logits_dtype, device=dev)
+        # (only the type and the shape count here: step() sets the strides of the logits it is given)
+        proto = torch.empty(vocab, dtype=logits_dtype, device=dev).as_strided((batch, window, vocab), (0, 0, 1))
         self.params = B.make_params(proto, top_k=top_k, cfg_scale=cfg_scale, inv_temperature=inv_temperature,
                                     reuse_tau=reuse_tau,
                                     flags=(B.SJD_FLAG_REUSE if reuse else 0) | (0 if refine else B.SJD_FLAG_NO_REFINE),
@@ -99,21 +115,25 @@ class DecodeLoop:
         """True when every sequence is complete.  This is the loop's one synchronisation point per iteration: the
         status words of the last step come back with it, and a step whose on-chip wait gave up (its outputs are
         invalid, and the window was advanced on them) raises here instead of passing unnoticed."""
-        state = torch.stack([(self.win_len != 0).any().to(torch.int32),
-                             (self.status & B.SJD_STATUS_INTERNAL_TIMEOUT).any().to(torch.int32)]).cpu()
-        if int(state[1]) != 0:
+        self._host_state.copy_(self._state, non_blocking=True)
+        torch.cuda.current_stream(self.device).synchronize()
+        win_len, status, _ = self._host_state.tolist()
+        if any(s & B.SJD_STATUS_INTERNAL_TIMEOUT for s in status):
             raise B.SjdError("a step reported SJD_STATUS_INTERNAL_TIMEOUT: its outputs are invalid")
-        return int(state[0]) == 0
+        return not any(win_len)
 
     def run(self, logit_source: Callable[["DecodeLoop"], Tuple[torch.Tensor, Optional[torch.Tensor]]],
             max_steps: Optional[int] = None):
         """Iterate until every sequence is complete.  Returns (committed tokens, steps, committed counts per step)."""
-        history = []
-        while not self.done():
-            if max_steps is not None and self.steps >= max_steps:
+        # done() brings the counts of the step before it to the host along with the window lengths.
+        first, history = self.steps, []
+        while True:
+            done = self.done()
+            if self.steps > first + len(history):
+                history.append(self._host_state[2].tolist())
+            if done or (max_steps is not None and self.steps >= max_steps):
                 break
             cond, uncond = logit_source(self)
             self.step(cond, uncond)
-            history.append(self.n_committed.clone())
-        counts = torch.stack(history).cpu() if history else torch.zeros(0, self.B, dtype=torch.int32)
+        counts = torch.tensor(history, dtype=torch.int32).reshape(len(history), self.B)
         return self.committed.cpu(), self.steps, counts
