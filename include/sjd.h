@@ -274,10 +274,11 @@ int sjd_step_static(const void* logits_cond, const void* logits_uncond, const in
  *
  * sjd_host_ctx_create() allocates, on the current device, device copies of every argument of sjd_step()
  * for the shape in `shape` (B, W, V, logits_dtype, top_k are read; strides are taken as contiguous
- * [B,W,V]) plus the workspace and a stream, and returns an opaque handle.  sjd_step_host() copies the
+ * [B,W,V]) plus the workspace and three streams, and returns an opaque handle.  sjd_step_host() copies the
  * HOST arrays in (pinned memory makes the copies asynchronous and fast, pageable memory works), runs
- * sjd_step() on the context's stream, copies every output back and returns after the stream has
- * drained, so the host arrays are ready on return.  In `params`, B/W/V/dtype/top_k must equal the
+ * sjd_step() on the context's streams (a large batch in several parts, whose copies and kernels overlap), copies
+ * every output back and returns after the streams have drained, so the host arrays are ready on return.  Of pinned
+ * draft_probs only the rows that the residual draws need cross the link.  In `params`, B/W/V/dtype/top_k must equal the
  * context's; win_len, pos_base, iteration, out_flags and status are HOST pointers here (or NULL);
  * workspace, stream and the event fields are ignored.  draft_probs / out_probs hold HOST pointers.
  * Returns SJD_OK or a negative SJD_ERR_*.  sjd_host_ctx_destroy() frees everything (NULL is allowed).

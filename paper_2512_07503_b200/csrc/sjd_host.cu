@@ -1,5 +1,16 @@
 // Host-buffer variant of the step (declared in include/sjd.h): device mirrors of every argument are
 // allocated once per context; each call copies in, runs sjd_step() and copies out.
+//
+// The link to the host is what bounds it: 50 GB/s, and some 4 us for every copy whatever its size.  So
+//   - the batch goes through in parts of whole sequences: while a part's logits are on their way in, the part before it is
+//     in the kernels and the one before that on its way out (three streams; the parts use the mirrors' own ranges, and
+//     sequence numbers by seq_base, so the results are those of one call);
+//   - the small arrays of a call are gathered in page-locked memory, from which a kernel fetches them while the
+//     first logits come in, and into which the kernels write the small results: no copies of their own;
+//   - of the previous iteration's distributions one row per sequence is needed, and only the verification knows which: it
+//     reads that row out of the caller's arrays if they are page-locked.  Pageable ones are copied whole.
+// Pinned bf16 logits, W=32, V=16,384, K=1,000, both logit arrays: B=4 (8.4 MB of logits, 168 us of the link) 296 -> 233 us, B=32
+// 1,640 -> 1,370 us (1,340 of the link).  One part only: 238 us at B=4.
 #include "../../include/sjd.h"
 
 #include <cuda_runtime.h>
@@ -7,39 +18,174 @@
 #include <cstdlib>
 #include <cstring>
 
+namespace {
+
+// A part has at least this many bytes of logits: each costs two to four copies more, and hides its kernels and
+// its copies out behind the others.  The case above in parts of 2, 3, 4 and 8 MB: 252, 250, 233, 238 us; B=32: at most four
+// parts 1,402 us, eight 1,383.
+constexpr size_t kPartBytes = 4 << 20;
+constexpr int kMaxParts = 8;
+
+}  // namespace
+
 struct sjd_host_ctx {
   int32_t B, W, V, dtype, top_k, kcap;
-  size_t rows, logits_bytes;
-  void* d_cond;
-  void* d_uncond;
-  int32_t* d_drafts;
-  sjd_probs d_q, d_out;
-  int32_t *d_acc, *d_tokens, *d_flags, *d_status, *d_win, *d_pos, *d_iter;
+  size_t rows, row_bytes;
+  char* arena;  // the device mirrors, one allocation
+  char *d_cond, *d_uncond;
+  sjd_probs d_q, d_out;  // (only the lists: ids and vals)
+  int32_t* d_small;      // window lengths, positions, iterations; drafts and their probabilities and list lengths
+  int32_t *h_small, *h_results, *m_small, *m_results;  // page-locked: the same, and the small results; as the device sees them
   void* d_ws;
   size_t ws_bytes;
-  cudaStream_t stream;
+  cudaStream_t in, run, out;
+  cudaEvent_t arrived[kMaxParts], stepped[kMaxParts];
 };
 
 namespace {
 
+__global__ void fetch_words(const int32_t* __restrict__ from, int32_t* __restrict__ to, int n) {
+  const int i = (int)(blockIdx.x * blockDim.x + threadIdx.x);
+  if (i < n) to[i] = from[i];
+}
+
+// The device's address of a page-locked host array, null if any end of it is not.
 template <typename T>
-bool dev_alloc(T** p, size_t bytes) {
-  return cudaMalloc(reinterpret_cast<void**>(p), bytes ? bytes : 16) == cudaSuccess;
+T* mapped(T* p, size_t bytes) {
+  cudaPointerAttributes first, last;
+  const char* end = reinterpret_cast<const char*>(p) + bytes - 1;
+  if (cudaPointerGetAttributes(&first, p) != cudaSuccess || cudaPointerGetAttributes(&last, end) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return nullptr;
+  }
+  if (first.type != cudaMemoryTypeHost || last.type != cudaMemoryTypeHost || !first.devicePointer ||
+      static_cast<char*>(last.devicePointer) - static_cast<char*>(first.devicePointer) != (ptrdiff_t)(bytes - 1))
+    return nullptr;
+  return static_cast<T*>(first.devicePointer);
 }
 
-bool alloc_probs(sjd_probs* p, size_t rows, size_t kcap) {
-  return dev_alloc(&p->tok_prob, rows * 4) && dev_alloc(&p->ids, rows * kcap * 4) &&
-         dev_alloc(&p->vals, rows * kcap * 4) && dev_alloc(&p->cnt, rows * 4);
+void drain(sjd_host_ctx* c) {
+  if (c->in) cudaStreamSynchronize(c->in);
+  if (c->run) cudaStreamSynchronize(c->run);
+  if (c->out) cudaStreamSynchronize(c->out);
 }
 
-void free_probs(sjd_probs* p) {
-  cudaFree(p->tok_prob); cudaFree(p->ids); cudaFree(p->vals); cudaFree(p->cnt);
+bool create(sjd_host_ctx* c) {
+  const size_t rows = c->rows, B = (size_t)c->B, lists = rows * (size_t)c->kcap * 4, logits = rows * c->row_bytes;
+  const size_t n_in = (3 * B + 3 * rows) * 4, n_out = (2 * B + 4 * rows) * 4;
+  const size_t sizes[] = {logits, logits, lists, lists, lists, lists, n_in, c->ws_bytes};
+  size_t at[9] = {0};
+  for (int i = 0; i < 8; ++i) at[i + 1] = at[i] + ((sizes[i] + 255) & ~(size_t)255);
+  if (cudaMalloc(reinterpret_cast<void**>(&c->arena), at[8]) != cudaSuccess) return false;
+  auto words = [&](int i) { return reinterpret_cast<int32_t*>(c->arena + at[i]); };
+  c->d_cond = c->arena;
+  c->d_uncond = c->arena + at[1];
+  c->d_q.ids = words(2);
+  c->d_q.vals = reinterpret_cast<float*>(words(3));
+  c->d_out.ids = words(4);
+  c->d_out.vals = reinterpret_cast<float*>(words(5));
+  c->d_small = words(6);
+  c->d_ws = words(7);
+  if (cudaHostAlloc(reinterpret_cast<void**>(&c->h_small), n_in + n_out, cudaHostAllocMapped) != cudaSuccess ||
+      cudaHostGetDevicePointer(reinterpret_cast<void**>(&c->m_small), c->h_small, 0) != cudaSuccess)
+    return false;
+  c->h_results = c->h_small + n_in / 4;
+  c->m_results = c->m_small + n_in / 4;
+  for (cudaStream_t* st : {&c->in, &c->run, &c->out})
+    if (cudaStreamCreateWithFlags(st, cudaStreamNonBlocking) != cudaSuccess) return false;
+  for (int i = 0; i < kMaxParts; ++i)
+    if (cudaEventCreateWithFlags(&c->arrived[i], cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&c->stepped[i], cudaEventDisableTiming) != cudaSuccess)
+      return false;
+  return true;
 }
 
 #define SJD_TRY(expr)                   \
   do {                                  \
     if ((expr) != cudaSuccess) return SJD_ERR_CUDA; \
   } while (0)
+
+// Everything that a call enqueues; the caller drains the streams whatever it returns.
+int enqueue(sjd_host_ctx* c, const char* cond, const char* uncond, const int32_t* drafts, const sjd_probs* q,
+            const sjd_params* P, uint64_t seed, sjd_probs* out) {
+  const cudaMemcpyKind H2D = cudaMemcpyHostToDevice, D2H = cudaMemcpyDeviceToHost;
+  const size_t rows = c->rows, B = (size_t)c->B, W = (size_t)c->W, kc = (size_t)c->kcap, n_logits = W * c->row_bytes;
+  const size_t total = B * n_logits * (uncond ? 2 : 1);
+  size_t parts = total / kPartBytes;
+  if (parts > kMaxParts) parts = kMaxParts;
+  if (parts > B) parts = B;
+  if (parts < 1) parts = 1;
+  int32_t* const d_win = c->d_small;
+  int32_t* const d_drafts = c->d_small + 3 * B;
+  int32_t* const m_tokens = c->m_results + 2 * B;
+  sjd_probs d_q = c->d_q;
+  bool q_copied = false;
+  for (size_t k = 0; k < parts; ++k) {
+    const size_t b0 = k * B / parts, nb = (k + 1) * B / parts - b0, r0 = b0 * W, n_lists = nb * W * kc * 4;
+    SJD_TRY(cudaMemcpyAsync(c->d_cond + b0 * n_logits, cond + b0 * n_logits, nb * n_logits, H2D, c->in));
+    if (uncond) SJD_TRY(cudaMemcpyAsync(c->d_uncond + b0 * n_logits, uncond + b0 * n_logits, nb * n_logits, H2D, c->in));
+    if (k == 0) {  // the small arrays, while the first logits are on their way
+      const int n = (int)(3 * B + (q ? 3 * rows : 0));
+      if (P->win_len) std::memcpy(c->h_small, P->win_len, B * 4);
+      if (P->pos_base) std::memcpy(c->h_small + B, P->pos_base, B * 4);
+      if (P->iteration) std::memcpy(c->h_small + 2 * B, P->iteration, B * 4);
+      if (q) {
+        std::memcpy(c->h_small + 3 * B, drafts, rows * 4);
+        std::memcpy(c->h_small + 3 * B + rows, q->tok_prob, rows * 4);
+        std::memcpy(c->h_small + 3 * B + 2 * rows, q->cnt, rows * 4);
+        int32_t* const m_ids = mapped(q->ids, rows * kc * 4);
+        float* const m_vals = mapped(q->vals, rows * kc * 4);
+        q_copied = !m_ids || !m_vals;
+        if (!q_copied) d_q.ids = m_ids, d_q.vals = m_vals;
+      }
+      fetch_words<<<(n + 255) / 256, 256, 0, c->run>>>(c->m_small, c->d_small, n);
+      SJD_TRY(cudaGetLastError());
+    }
+    if (q_copied) {
+      SJD_TRY(cudaMemcpyAsync(d_q.ids + r0 * kc, q->ids + r0 * kc, n_lists, H2D, c->in));
+      SJD_TRY(cudaMemcpyAsync(d_q.vals + r0 * kc, q->vals + r0 * kc, n_lists, H2D, c->in));
+    }
+    sjd_probs part_q, part_out;
+    part_q.tok_prob = reinterpret_cast<float*>(d_drafts + rows + r0);
+    part_q.ids = d_q.ids + r0 * kc;
+    part_q.vals = d_q.vals + r0 * kc;
+    part_q.cnt = d_drafts + 2 * rows + r0;
+    part_out.tok_prob = reinterpret_cast<float*>(m_tokens + rows + r0);
+    part_out.ids = c->d_out.ids + r0 * kc;
+    part_out.vals = c->d_out.vals + r0 * kc;
+    part_out.cnt = m_tokens + 2 * rows + r0;
+    SJD_TRY(cudaEventRecord(c->arrived[k], c->in));
+    SJD_TRY(cudaStreamWaitEvent(c->run, c->arrived[k], 0));
+
+    sjd_params D = *P;
+    D.B = (int32_t)nb;
+    D.seq_base = P->seq_base + (int32_t)b0;
+    D.stride_b = (int64_t)c->W * c->V;
+    D.stride_w = c->V;
+    D.win_len = P->win_len ? d_win + b0 : nullptr;
+    D.pos_base = P->pos_base ? d_win + B + b0 : nullptr;
+    D.iteration = P->iteration ? d_win + 2 * B + b0 : nullptr;
+    D.status = P->status ? c->m_results + B + b0 : nullptr;
+    D.out_flags = P->out_flags ? m_tokens + 3 * rows + r0 : nullptr;
+    D.workspace = c->d_ws;
+    D.workspace_bytes = c->ws_bytes;
+    D.stream = c->run;
+    D.ev_rows_begin = nullptr;
+    D.ev_rows_end = nullptr;
+    const int rc = sjd_step(c->d_cond + b0 * n_logits, uncond ? c->d_uncond + b0 * n_logits : nullptr, d_drafts + r0,
+                            q ? &part_q : nullptr, &D, seed, c->m_results + b0, m_tokens + r0, &part_out);
+    if (rc != SJD_OK) return rc;
+    SJD_TRY(cudaEventRecord(c->stepped[k], c->run));
+  }
+  // (Copies to pageable memory hold the caller up, so none is issued before the last part is on its way.)
+  for (size_t k = 0; k < parts; ++k) {
+    const size_t b0 = k * B / parts, nb = (k + 1) * B / parts - b0, r0 = b0 * W, n_lists = nb * W * kc * 4;
+    SJD_TRY(cudaStreamWaitEvent(c->out, c->stepped[k], 0));
+    SJD_TRY(cudaMemcpyAsync(out->ids + r0 * kc, c->d_out.ids + r0 * kc, n_lists, D2H, c->out));
+    SJD_TRY(cudaMemcpyAsync(out->vals + r0 * kc, c->d_out.vals + r0 * kc, n_lists, D2H, c->out));
+  }
+  return SJD_OK;
+}
 
 }  // namespace
 
@@ -55,20 +201,12 @@ int sjd_host_ctx_create(const sjd_params* s, sjd_host_ctx** out_ctx) {
   c->B = s->B; c->W = s->W; c->V = s->V; c->dtype = s->logits_dtype; c->top_k = s->top_k;
   c->kcap = s->top_k < s->V ? s->top_k : s->V;
   c->rows = (size_t)s->B * s->W;
-  c->logits_bytes = c->rows * (size_t)s->V * (s->logits_dtype == SJD_F32 ? 4 : 2);
+  c->row_bytes = (size_t)s->V * (s->logits_dtype == SJD_F32 ? 4 : 2);
   sjd_params shape;
   std::memset(&shape, 0, sizeof(shape));
   shape.B = s->B; shape.W = s->W;
   c->ws_bytes = sjd_workspace_bytes(&shape);
-  const bool ok = dev_alloc(&c->d_cond, c->logits_bytes) && dev_alloc(&c->d_uncond, c->logits_bytes) &&
-                  dev_alloc(&c->d_drafts, c->rows * 4) && alloc_probs(&c->d_q, c->rows, c->kcap) &&
-                  alloc_probs(&c->d_out, c->rows, c->kcap) && dev_alloc(&c->d_acc, (size_t)s->B * 4) &&
-                  dev_alloc(&c->d_tokens, c->rows * 4) && dev_alloc(&c->d_flags, c->rows * 4) &&
-                  dev_alloc(&c->d_status, (size_t)s->B * 4) && dev_alloc(&c->d_win, (size_t)s->B * 4) &&
-                  dev_alloc(&c->d_pos, (size_t)s->B * 4) && dev_alloc(&c->d_iter, (size_t)s->B * 4) &&
-                  dev_alloc(&c->d_ws, c->ws_bytes) &&
-                  cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking) == cudaSuccess;
-  if (!ok) {
+  if (!create(c)) {
     sjd_host_ctx_destroy(c);
     return SJD_ERR_CUDA;
   }
@@ -78,14 +216,15 @@ int sjd_host_ctx_create(const sjd_params* s, sjd_host_ctx** out_ctx) {
 
 void sjd_host_ctx_destroy(sjd_host_ctx* c) {
   if (!c) return;
-  if (c->stream) {
-    cudaStreamSynchronize(c->stream);
-    cudaStreamDestroy(c->stream);
+  drain(c);
+  for (cudaStream_t st : {c->in, c->run, c->out})
+    if (st) cudaStreamDestroy(st);
+  for (int i = 0; i < kMaxParts; ++i) {
+    if (c->arrived[i]) cudaEventDestroy(c->arrived[i]);
+    if (c->stepped[i]) cudaEventDestroy(c->stepped[i]);
   }
-  cudaFree(c->d_cond); cudaFree(c->d_uncond); cudaFree(c->d_drafts);
-  free_probs(&c->d_q); free_probs(&c->d_out);
-  cudaFree(c->d_acc); cudaFree(c->d_tokens); cudaFree(c->d_flags); cudaFree(c->d_status);
-  cudaFree(c->d_win); cudaFree(c->d_pos); cudaFree(c->d_iter); cudaFree(c->d_ws);
+  cudaFreeHost(c->h_small);
+  cudaFree(c->arena);
   std::free(c);
 }
 
@@ -99,50 +238,21 @@ int sjd_step_host(sjd_host_ctx* c, const void* logits_cond, const void* logits_u
     return SJD_ERR_SHAPE;
   const bool draft_all = (P->flags & SJD_FLAG_DRAFT_ALL) != 0;
   if (!draft_all && (!drafts || !q || !q->tok_prob || !q->ids || !q->vals || !q->cnt)) return SJD_ERR_NULL;
-  cudaStream_t st = c->stream;
-  const size_t rows = c->rows, kc = (size_t)c->kcap, B = (size_t)c->B;
-  const cudaMemcpyKind H2D = cudaMemcpyHostToDevice, D2H = cudaMemcpyDeviceToHost;
-  SJD_TRY(cudaMemcpyAsync(c->d_cond, logits_cond, c->logits_bytes, H2D, st));
-  if (logits_uncond) SJD_TRY(cudaMemcpyAsync(c->d_uncond, logits_uncond, c->logits_bytes, H2D, st));
-  if (!draft_all) {
-    SJD_TRY(cudaMemcpyAsync(c->d_drafts, drafts, rows * 4, H2D, st));
-    SJD_TRY(cudaMemcpyAsync(c->d_q.tok_prob, q->tok_prob, rows * 4, H2D, st));
-    SJD_TRY(cudaMemcpyAsync(c->d_q.ids, q->ids, rows * kc * 4, H2D, st));
-    SJD_TRY(cudaMemcpyAsync(c->d_q.vals, q->vals, rows * kc * 4, H2D, st));
-    SJD_TRY(cudaMemcpyAsync(c->d_q.cnt, q->cnt, rows * 4, H2D, st));
-  }
-  if (P->win_len) SJD_TRY(cudaMemcpyAsync(c->d_win, P->win_len, B * 4, H2D, st));
-  if (P->pos_base) SJD_TRY(cudaMemcpyAsync(c->d_pos, P->pos_base, B * 4, H2D, st));
-  if (P->iteration) SJD_TRY(cudaMemcpyAsync(c->d_iter, P->iteration, B * 4, H2D, st));
-
-  sjd_params D = *P;
-  D.stride_b = (int64_t)c->W * c->V;
-  D.stride_w = c->V;
-  D.win_len = P->win_len ? c->d_win : nullptr;
-  D.pos_base = P->pos_base ? c->d_pos : nullptr;
-  D.iteration = P->iteration ? c->d_iter : nullptr;
-  D.out_flags = P->out_flags ? c->d_flags : nullptr;
-  D.status = P->status ? c->d_status : nullptr;
-  D.workspace = c->d_ws;
-  D.workspace_bytes = c->ws_bytes;
-  D.stream = st;
-  D.ev_rows_begin = nullptr;
-  D.ev_rows_end = nullptr;
-  const int rc = sjd_step(c->d_cond, logits_uncond ? c->d_uncond : nullptr, c->d_drafts, draft_all ? nullptr : &c->d_q,
-                          &D, seed, c->d_acc, c->d_tokens, &c->d_out);
+  const int rc = enqueue(c, static_cast<const char*>(logits_cond), static_cast<const char*>(logits_uncond), drafts,
+                         draft_all ? nullptr : q, P, seed, out);
   if (rc != SJD_OK) {
-    cudaStreamSynchronize(st);
+    drain(c);  // nothing of the caller's is touched after the return
     return rc;
   }
-  SJD_TRY(cudaMemcpyAsync(out_accept_len, c->d_acc, B * 4, D2H, st));
-  SJD_TRY(cudaMemcpyAsync(out_tokens, c->d_tokens, rows * 4, D2H, st));
-  SJD_TRY(cudaMemcpyAsync(out->tok_prob, c->d_out.tok_prob, rows * 4, D2H, st));
-  SJD_TRY(cudaMemcpyAsync(out->ids, c->d_out.ids, rows * kc * 4, D2H, st));
-  SJD_TRY(cudaMemcpyAsync(out->vals, c->d_out.vals, rows * kc * 4, D2H, st));
-  SJD_TRY(cudaMemcpyAsync(out->cnt, c->d_out.cnt, rows * 4, D2H, st));
-  if (P->out_flags) SJD_TRY(cudaMemcpyAsync(P->out_flags, c->d_flags, rows * 4, D2H, st));
-  if (P->status) SJD_TRY(cudaMemcpyAsync(P->status, c->d_status, B * 4, D2H, st));
-  SJD_TRY(cudaStreamSynchronize(st));
+  SJD_TRY(cudaStreamSynchronize(c->out));  // behind every part's step, and so behind every copy in
+  const size_t rows = c->rows, B = (size_t)c->B;
+  const int32_t* o = c->h_results;
+  std::memcpy(out_accept_len, o, B * 4);
+  if (P->status) std::memcpy(P->status, o + B, B * 4);
+  std::memcpy(out_tokens, o + 2 * B, rows * 4);
+  std::memcpy(out->tok_prob, o + 2 * B + rows, rows * 4);
+  std::memcpy(out->cnt, o + 2 * B + 2 * rows, rows * 4);
+  if (P->out_flags) std::memcpy(P->out_flags, o + 2 * B + 3 * rows, rows * 4);
   return SJD_OK;
 }
 
