@@ -54,6 +54,37 @@ __device__ __forceinline__ int random_token(int pos, int seq, int iter, int V, u
   return (int)(((uint64_t)r.x0 * (uint64_t)(uint32_t)V) >> 32);
 }
 
+// Copy n entries of a row's two lists.  Latency is all there is to it: the loads of up to two rounds are in flight before the
+// first store (which the compiler, not knowing that the lists do not overlap, would have waited for each time).  Word by word
+// where a list is not 16-byte aligned (an odd K).  One window of 32 rows, K=2,000: an iteration's kernels 35.9 -> 31.2 us; 16 of
+// 16 rows, K=1,000: 30.9 -> 28.3 us.
+template <int NT, typename T>
+__device__ __forceinline__ void copy_lists(const T* sid, const T* sv, T* nid, T* nv, int n) {
+  for (int k = threadIdx.x; k < n; k += 2 * NT) {
+    const bool more = k + NT < n;
+    const T i0 = sid[k], v0 = sv[k];
+    T i1 = i0, v1 = v0;
+    if (more) i1 = sid[k + NT], v1 = sv[k + NT];
+    nid[k] = i0;
+    nv[k] = v0;
+    if (more) nid[k + NT] = i1, nv[k + NT] = v1;
+  }
+}
+
+template <int NT>
+__device__ __forceinline__ void copy_row(const int32_t* sid, const float* sv, int32_t* nid, float* nv, int n) {
+  n = max(n, 0);
+  int done = 0;
+  if (((reinterpret_cast<uintptr_t>(sid) | reinterpret_cast<uintptr_t>(sv) | reinterpret_cast<uintptr_t>(nid) |
+        reinterpret_cast<uintptr_t>(nv)) & 15u) == 0) {
+    done = n & ~3;
+    copy_lists<NT>(reinterpret_cast<const uint4*>(sid), reinterpret_cast<const uint4*>(sv), reinterpret_cast<uint4*>(nid),
+                   reinterpret_cast<uint4*>(nv), n >> 2);
+  }
+  copy_lists<NT>(reinterpret_cast<const uint32_t*>(sid) + done, reinterpret_cast<const uint32_t*>(sv) + done,
+                 reinterpret_cast<uint32_t*>(nid) + done, reinterpret_cast<uint32_t*>(nv) + done, n - done);
+}
+
 // One block per (sequence, next-window row).
 template <int NT>
 __global__ void __launch_bounds__(NT) advance_rows_kernel(const AdvanceArgs a) {
@@ -89,10 +120,7 @@ __global__ void __launch_bounds__(NT) advance_rows_kernel(const AdvanceArgs a) {
     const int32_t* sid = a.step_ids + srow * a.kcap;
     const float* sv = a.step_vals + srow * a.kcap;
     const int n = a.step_cnt[srow];
-    for (int k = threadIdx.x; k < n; k += NT) {
-      nid[k] = sid[k];
-      nv[k] = sv[k];
-    }
+    copy_row<NT>(sid, sv, nid, nv, n);
     if (threadIdx.x == 0) {
       a.next_drafts[row] = a.step_tokens[srow];
       a.next_tok_prob[row] = a.step_tok_prob[srow];
@@ -149,10 +177,7 @@ __global__ void __launch_bounds__(NT) advance_rows_kernel(const AdvanceArgs a) {
   const int32_t* sid = a.step_ids + srow * a.kcap;
   const float* sv = a.step_vals + srow * a.kcap;
   const int n = min(max(a.step_cnt[srow], 0), a.kcap);
-  for (int k = threadIdx.x; k < n; k += NT) {
-    nid[k] = sid[k];
-    nv[k] = sv[k];
-  }
+  copy_row<NT>(sid, sv, nid, nv, n);
   const Philox4 rnd = philox4x32_10((uint32_t)p, (uint32_t)(a.seq_base + b), (uint32_t)iter, kPurposePriorInit,
                                     a.seed_lo, a.seed_hi);
   int k = group_icdf<NT, 0>([&](int j) { return fixed_weight(sv[j]); }, n, random64(rnd), threadIdx.x, scratch);
