@@ -29,7 +29,7 @@
 //                        memory at once.  The candidates go straight into the first CTA's lists (distributed shared
 //                        memory), which finishes the row.
 //
-// What bounds it: at V=65,536 and K=2,000 a row is about 35 K warp instructions at 60 % of the issue slots; a row of the
+// What bounds it: at V=65,536 and K=2,000 a row is about 40 K warp instructions at 56 % of the issue slots; a row of the
 // memory stream alone would be 12.3 K cycles.  us a step against the kernels that took these shapes before: 1,024 rows of
 // 65,536 bf16, K=2,000: 82.4 (85.4 with a kernel of one id range per filter thread); of 16,384: 53.0 (65.0); 1,024 ragged
 // rows of 16,384 fp32, K=1,000: 51.8 (58.5); 1,024 rows of 32,768 bf16 without guidance: 50.2 (63.4); 231 rows of
