@@ -1120,8 +1120,9 @@ rows_stream_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ Si
     if (HAS_U) bulk_g2s_hinted(dst + kUnitBytes, row_ptr(a.uncond, DTYPE, off), bytes, &st.full[x], policy);
   };
   // The team's first row: its sample's maxima, for the sampler.  Everybody waits for the CTA's first threshold, so the other
-  // teams' samples and the first copies (which the second team sends off) come behind the first team's sample.
-  if (team > 0) sift_wait(&st.sample_full[0], 0u, abort_flag);  // (nothing depends on it)
+  // teams' samples and the first copies (which the second team sends off) come behind the first team's sample.  (Nothing but
+  // time depends on it; a CTA whose rows all lie beyond their windows takes no sample.)
+  if (team > 0 && n_live > 0) sift_wait(&st.sample_full[0], 0u, abort_flag);
   if (team == 1 && lane == 0 && units > 0) {
     for (int x = 0; x < slots; ++x) issue(0, x, x);
   }
