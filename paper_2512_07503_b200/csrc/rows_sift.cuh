@@ -258,7 +258,9 @@ struct SiftBinning {
 __device__ __forceinline__ SiftBinning sift_bins(float tau0, float top) {
   const float range = __fsub_rn(top, tau0);
   const float per = range > 0.0f ? __fdiv_rn(1.0f, range) : 0.0f;
-  return SiftBinning{tau0, __fmul_rn(8.0f * kBinsLow, per), __fmul_rn((kSiftBins - 2) - kBinsCross, per)};
+  // (finite slopes however narrow the range: tau0 itself has to fall into bin 1)
+  const float most = 3.0e38f;
+  return SiftBinning{tau0, fminf(__fmul_rn(8.0f * kBinsLow, per), most), fminf(__fmul_rn((kSiftBins - 2) - kBinsCross, per), most)};
 }
 
 // A sample's load, issued where it stands.  It is to stay in the L2 until its row comes through the ring, half a dozen rows
@@ -728,14 +730,19 @@ __device__ __forceinline__ bool finish_row(const RowArgs& a, const SiftCfg& cfg,
   const int id0 = warp * per_warp * cfg.seg_len;
   // ---- the threshold bin's members
   {
-    const float lo = (float)tbin, hi = tbin == (uint32_t)kSiftBins - 1u ? __int_as_float(0x7f800000) : (float)(tbin + 1u);
+    // (the last bin also holds what lies above its end)
+    const bool last = tbin == (uint32_t)kSiftBins - 1u;
+    const float lo = (float)tbin, hi = (float)(tbin + 1u);
     for (int g = 0; g < per_warp; ++g) {
       const uint32_t n = seg_n[first_seg + g];
       const float* const y_g = my_y + g * cfg.seg_cap;
 #pragma unroll 4
       for (uint32_t i = (uint32_t)lane; i < n; i += 32u) {
         const float y = y_g[i], x = bins.at(y);
-        if (x >= lo && x < hi) sm.hist.member[atomicAdd(&sm.members, 1)] = SiftMember{y, id0 + (int32_t)my_id[g * cfg.seg_cap + i]};
+        if (x >= lo && (x < hi || last)) {
+          const int at = atomicAdd(&sm.members, 1);  // (as many as the histogram counted: the check keeps the store in bounds)
+          if (at < kMemberCap) sm.hist.member[at] = SiftMember{y, id0 + (int32_t)my_id[g * cfg.seg_cap + i]};
+        }
       }
     }
   }
@@ -826,7 +833,10 @@ __device__ __forceinline__ bool finish_row(const RowArgs& a, const SiftCfg& cfg,
   if (tid == 0) sm.members = 0;
   const uint32_t cw = lane < NW ? sm.wcnt[lane] : 0u;
   const uint32_t before = __reduce_add_sync(0xffffffffu, lane < warp ? cw : 0u);
-  if (__reduce_add_sync(0xffffffffu, cw) != kcap) return false;  // cannot happen; the result stays exact anyway
+  if (__reduce_add_sync(0xffffffffu, cw) != kcap) {  // cannot happen; the result stays exact anyway
+    row_sync<NT>(bar);  // (the histogram's words are zero before anybody counts in them again)
+    return false;
+  }
   float Z = sm.wz[lane & (NW - 1)];
 #pragma unroll
   for (int d = NW / 2; d > 0; d >>= 1) Z += __shfl_xor_sync(0xffffffffu, Z, d);

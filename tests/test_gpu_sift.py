@@ -101,3 +101,27 @@ def test_screening_keeps_what_cancels(B, W, dtype, scale, temperature):
         arr[:] = wk._store(x.astype(np.float32), dtype)
     prev = oracle_prime(inp)
     check_parity(inp.cond, inp.uncond, prev.tokens, prev.probs, step_kwargs(inp), inp.win_len)
+
+
+@pytest.mark.parametrize("unit", [1e-36, 3e-38, 1e-40])
+@pytest.mark.parametrize("B,W", [(1, 3), (2, 90)])
+def test_rows_whose_candidates_differ_by_next_to_nothing(B, W, unit):
+    # a few hundred entries between 0 and `unit` (normal and subnormal numbers), everything else at -1: the candidates' bins
+    # are as narrow as floats allow, and the threshold lies among them
+    from gpu_harness import check_parity, step_kwargs
+    wl = wk.CONFIGS["cfg1"].scaled(B=B, W=W, V=4096, top_k=64, seed=W)
+    inp = wk.make_step_inputs(wl)
+    rng = np.random.default_rng(W)
+    for arr in (inp.cond, inp.prev_cond):
+        arr[:] = -1.0
+        pick = rng.random(arr.shape) < 0.15
+        arr[pick] = (rng.random(int(pick.sum())) * unit).astype(np.float32)
+    prev = _prime_without_guidance(inp)
+    check_parity(inp.cond, None, prev.tokens, prev.probs, step_kwargs(inp), inp.win_len)
+
+
+def _prime_without_guidance(inp):
+    import oracle
+    from gpu_harness import step_kwargs
+    kw = step_kwargs(inp, flags=oracle.FLAG_DRAFT_ALL, iteration0=inp.iteration - 1)
+    return oracle.sjd_step(inp.prev_cond, None, None, None, V=inp.wl.V, n_threads=8, diag=True, **kw)
