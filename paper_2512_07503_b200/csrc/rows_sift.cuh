@@ -315,10 +315,12 @@ __device__ __forceinline__ uint32_t pair_of(float x) {
 // 16-bit logits: entries are screened in packed 16-bit arithmetic, two to an instruction, and only what passes is merged
 // exactly.  With guidance g = s (c - u) + u reaches g0 (the value before the temperature) only if s c + ((1 - s) u - t) >= 0
 // for a t that lies below g0 by more than the bracket can be off: the product-sum's own rounding cannot change its sign, the
-// bracket is off by its rounding, 2^-8 (bf16) or 2^-11 (fp16) of |1 - s| |u| + |t| at most, and t by as much of |t|.  So s and
-// 1 - s have to be numbers of the type (the host sees to that), and |u| has to stay below a limit that t was chosen for: a
-// unit that holds a larger one is compared exactly.  About a tenth more entries pass than reach tau0; they end as
-// candidates below tau0, in bin 0.  Without guidance c is compared with the largest number of the type up to g0.
+// bracket is off by its rounding, 2^-8 (bf16) or 2^-11 (fp16) of |1 - s| |u| + |t| at most, and t by as much of |t|.  The exact
+// path rounds as well: c - u and the sum, in 32 bits, put g off by 2^-24 of |g| and of |u| each, which matters where s is 1 and
+// |u| outweighs the threshold.  So s and 1 - s have to be numbers of the type (the host sees to that), and |u| has to stay
+// below a limit that t was chosen for: a unit that holds a larger one is compared exactly, and so is a row for which the 32-bit
+// roundings outweigh the 16-bit ones, or whose products with 1/T may be subnormal.  About a tenth more entries pass than reach
+// tau0; they end as candidates below tau0, in bin 0.  Without guidance c is compared with the largest number of the type up to g0.
 // Two instructions per entry instead of four; worth it while few entries pass anyway (the host's rule): 1,000 rows of 65,536
 // fp16 entries, K=100: 59.7 -> 57.3 us.
 struct SiftScreen {
@@ -329,15 +331,17 @@ template <int DTYPE, bool HAS_U, bool HAS_T>
 __device__ __forceinline__ SiftScreen sift_screen(const RowArgs& a, const SiftCfg& cfg, float tau0, float u_max) {
   SiftScreen r{0u, 0u, 0u, -1.0f};
   if (DTYPE == 0 || !cfg.packed) return r;
+  if (HAS_T && !(fabsf(tau0) >= 1.0e-30f)) return r;
   constexpr float kRound = DTYPE == 2 ? 0x1p-11f : 0x1p-8f;
   float g0 = HAS_T ? __fdiv_rn(tau0, a.inv_T) : tau0;
   g0 = __fmaf_rd(fabsf(g0), -0x1p-20f, g0);
   if (HAS_U) {
     const float b = 1.0f - a.s, limit = 1.25f * u_max, reach = fabsf(b) * limit + 2.0f * fabsf(g0);
-    if (!(reach < 3.0e4f)) return r;
+    const float narrow = 0x1p-22f * limit;  // the 32-bit roundings, with room
+    if (!(reach < 3.0e4f) || !(narrow <= kRound * reach)) return r;
     r.s2 = pair_of<DTYPE>(a.s);
     r.b2 = pair_of<DTYPE>(b);
-    r.t2 = pair_of<DTYPE>(__fmaf_rn(1.03f * kRound, reach, -g0));
+    r.t2 = pair_of<DTYPE>(__fmaf_rn(1.03f * kRound, reach, narrow - g0));
     r.u_limit = limit;
   } else {
     if (!(fabsf(g0) < 3.0e4f)) return r;

@@ -125,3 +125,20 @@ def _prime_without_guidance(inp):
     from gpu_harness import step_kwargs
     kw = step_kwargs(inp, flags=oracle.FLAG_DRAFT_ALL, iteration0=inp.iteration - 1)
     return oracle.sjd_step(inp.prev_cond, None, None, None, V=inp.wl.V, n_threads=8, diag=True, **kw)
+
+
+@pytest.mark.parametrize("dtype,u_size,c_size", [(wk.BF16, 1e7, 3.0), (wk.BF16, 1e5, 0.03), (wk.F16, 6e4, 0.01), (wk.BF16, 3e3, 3.0)])
+@pytest.mark.parametrize("B,W", [(1, 4), (2, 90)])
+def test_screening_keeps_what_32_bit_rounding_lifts(B, W, dtype, u_size, c_size):
+    # guidance scale 1: the merged logit is c - u + u, off from c by 2^-24 of a |u| that dwarfs the threshold
+    from gpu_harness import check_parity, oracle_prime, step_kwargs
+    wl = wk.CONFIGS["cfg2"].scaled(B=B, W=W, V=16384, dtype=dtype, top_k=150, cfg_scale=1.0, seed=W)
+    inp = wk.make_step_inputs(wl)
+    rng = np.random.default_rng(W + dtype)
+    shape = inp.cond.shape
+    c = rng.standard_normal(shape).astype(np.float32) * c_size
+    u = np.clip(rng.standard_normal(shape).astype(np.float32), -1, 1) * u_size
+    for arr, x in ((inp.cond, c), (inp.uncond, u), (inp.prev_cond, c + c_size / 8), (inp.prev_uncond, u)):
+        arr[:] = wk._store(x.astype(np.float32), dtype)
+    prev = oracle_prime(inp)
+    check_parity(inp.cond, inp.uncond, prev.tokens, prev.probs, step_kwargs(inp), inp.win_len)
