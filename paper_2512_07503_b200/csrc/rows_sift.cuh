@@ -282,10 +282,10 @@ __device__ __forceinline__ uint32_t fma_pair(uint32_t a, uint32_t b, uint32_t c)
   return r;
 }
 template <int DTYPE>
-__device__ __forceinline__ uint32_t add_pair(uint32_t a, uint32_t b) {
+__device__ __forceinline__ uint32_t sub_pair(uint32_t a, uint32_t b) {
   uint32_t r;
-  if (DTYPE == 2) asm("add.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
-  else asm("add.rn.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+  if (DTYPE == 2) asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+  else asm("sub.rn.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
   return r;
 }
 template <int DTYPE>
@@ -312,19 +312,25 @@ __device__ __forceinline__ uint32_t pair_of(float x) {
   return r;
 }
 
+// the largest number of the type below the one that a word holds twice (zero: the negative number next to it)
+__device__ __forceinline__ uint32_t pair_below(uint32_t t) {
+  return (t & 0x7fffu) == 0u ? 0x80018001u : (t & 0x8000u) ? t + 0x00010001u : t - 0x00010001u;
+}
+
 // 16-bit logits: entries are screened in packed 16-bit arithmetic, two to an instruction, and only what passes is merged
-// exactly.  With guidance g = s (c - u) + u reaches g0 (the value before the temperature) only if s c + ((1 - s) u - t) >= 0
+// exactly.  With guidance g = s (c - u) + u reaches g0 (the value before the temperature) only if (t - (1 - s) u) - s c < 0
 // for a t that lies below g0 by more than the bracket can be off: the product-sum's own rounding cannot change its sign, the
 // bracket is off by its rounding, 2^-8 (bf16) or 2^-11 (fp16) of |1 - s| |u| + |t| at most, and t by as much of |t|.  The exact
 // path rounds as well: c - u and the sum, in 32 bits, put g off by 2^-24 of |g| and of |u| each, which matters where s is 1 and
 // |u| outweighs the threshold.  So s and 1 - s have to be numbers of the type (the host sees to that), and |u| has to stay
 // below a limit that t was chosen for: a unit that holds a larger one is compared exactly, and so is a row for which the 32-bit
 // roundings outweigh the 16-bit ones, or whose products with 1/T may be subnormal.  About a tenth more entries pass than reach
-// tau0; they end as candidates below tau0, in bin 0.  Without guidance c is compared with the largest number of the type up to g0.
+// tau0; they end as candidates below tau0, in bin 0.  Without guidance c is compared with the largest number of the type below
+// g0.  A NaN (the merge of two tokens masked with -inf) has no sign and does not pass.
 // Two instructions per entry instead of four; worth it while few entries pass anyway (the host's rule): 1,000 rows of 65,536
 // fp16 entries, K=100: 59.7 -> 57.3 us.
 struct SiftScreen {
-  uint32_t s2, b2, t2;  // s, 1 - s and -t, pairs
+  uint32_t s2, b2, t2;  // -s, s - 1 and t, pairs
   float u_limit;        // negative: this row is compared exactly
 };
 template <int DTYPE, bool HAS_U, bool HAS_T>
@@ -339,16 +345,15 @@ __device__ __forceinline__ SiftScreen sift_screen(const RowArgs& a, const SiftCf
     const float b = 1.0f - a.s, limit = 1.25f * u_max, reach = fabsf(b) * limit + 2.0f * fabsf(g0);
     const float narrow = 0x1p-22f * limit;  // the 32-bit roundings, with room
     if (!(reach < 3.0e4f) || !(narrow <= kRound * reach)) return r;
-    r.s2 = pair_of<DTYPE>(a.s);
-    r.b2 = pair_of<DTYPE>(b);
-    r.t2 = pair_of<DTYPE>(__fmaf_rn(1.03f * kRound, reach, narrow - g0));
+    r.s2 = pair_of<DTYPE>(-a.s);
+    r.b2 = pair_of<DTYPE>(-b);
+    r.t2 = pair_below(pair_of<DTYPE>(__fmaf_rn(-1.03f * kRound, reach, g0 - narrow)));
     r.u_limit = limit;
   } else {
     if (!(fabsf(g0) < 3.0e4f)) return r;
-    uint32_t t = pair_of<DTYPE>(g0);
+    const uint32_t t = pair_of<DTYPE>(g0);
     const float back = DTYPE == 2 ? f16_pair(t).x : bf16_lo(t);
-    if (back > g0) t = (t & 0x7fffu) == 0u ? 0x80018001u : (t & 0x8000u) ? t + 0x00010001u : t - 0x00010001u;  // the number below
-    r.t2 = t ^ 0x80008000u;
+    r.t2 = back >= g0 ? pair_below(t) : t;
     r.u_limit = 0.0f;
   }
   return r;
@@ -496,14 +501,14 @@ __device__ __forceinline__ SiftTau sift_threshold(const SiftSample& in, uint32_t
 // ---------------------------------------------------------------------------------------------------
 // sift phase
 // ---------------------------------------------------------------------------------------------------
-// Hit bits of 64 bytes per array of a lane: bit k is set when element k reaches tau0 (or is a NaN, sorted out when the
-// candidate is merged).  The sign of y - tau0 is exact (a difference rounds to zero only when it is zero) and is
-// moved in with one funnel shift per element.  Lanes start at different 16-byte pieces (`rot`), so that the eight lanes
+// Hit bits of 64 bytes per array of a lane: bit k is set when element k reaches tau0, that is when it lies above `below`, the
+// number next to tau0.  The sign of below - y is exact (a difference rounds to zero only when it is zero), is not set for a
+// NaN (tokens masked with -inf in both arrays merge to one) and is moved in with one funnel shift per element.  Lanes start at different 16-byte pieces (`rot`), so that the eight lanes
 // served together touch different banks; the word is rotated back afterwards.
 template <int DTYPE, bool HAS_U, bool HAS_T>
-__device__ __forceinline__ uint32_t piece_hits(uint32_t c_at, uint32_t u_at, int rot, uint64_t s2, uint64_t t2, uint64_t neg_tau2) {
+__device__ __forceinline__ uint32_t piece_hits(uint32_t c_at, uint32_t u_at, int rot, uint64_t s2, uint64_t t2, uint64_t below2) {
   constexpr int EV = SiftTraits<DTYPE>::kVec;
-  uint32_t miss = 0;
+  uint32_t hits = 0;
 #pragma unroll
   for (int j = 3; j >= 0; --j) {
     const uint32_t off = (uint32_t)(((j + rot) & 3) << 4);
@@ -514,14 +519,13 @@ __device__ __forceinline__ uint32_t piece_hits(uint32_t c_at, uint32_t u_at, int
     merge_vec<DTYPE, HAS_U, HAS_T>(c, u, s2, t2, y);
 #pragma unroll
     for (int k = EV / 2 - 1; k >= 0; --k) {
-      uint64_t t;
-      asm("add.rn.f32x2 %0, %1, %2;" : "=l"(t) : "l"(y[k]), "l"(neg_tau2));
-      miss = __funnelshift_l((uint32_t)(t >> 32), miss, 1);
-      miss = __funnelshift_l((uint32_t)t, miss, 1);
+      const uint64_t t = sub2(below2, y[k]);
+      hits = __funnelshift_l((uint32_t)(t >> 32), hits, 1);
+      hits = __funnelshift_l((uint32_t)t, hits, 1);
     }
   }
-  if (DTYPE != 0) return __funnelshift_l(~miss, ~miss, 8 * rot);
-  const uint32_t x = (~miss & 0xffffu) * 0x10001u;
+  if (DTYPE != 0) return __funnelshift_l(hits, hits, 8 * rot);
+  const uint32_t x = (hits & 0xffffu) * 0x10001u;
   return (x >> (16 - 4 * rot)) & 0xffffu;
 }
 
@@ -529,7 +533,7 @@ __device__ __forceinline__ uint32_t piece_hits(uint32_t c_at, uint32_t u_at, int
 // the powers of two makes them four bits.  u_max: largest |uncond| met.
 template <int DTYPE, bool HAS_U>
 __device__ __forceinline__ uint32_t piece_screened(uint32_t c_at, uint32_t u_at, int rot, const SiftScreen& sc, uint32_t& u_max) {
-  int32_t acc = 0;  // minus the missed entries' bits
+  int32_t acc = 0;  // minus the hit bits
 #pragma unroll
   for (int j = 3; j >= 0; --j) {
     const uint32_t off = (uint32_t)(((j + rot) & 3) << 4);
@@ -546,7 +550,7 @@ __device__ __forceinline__ uint32_t piece_screened(uint32_t c_at, uint32_t u_at,
       }
     } else {
 #pragma unroll
-      for (int k = 0; k < 4; ++k) w[k] = add_pair<DTYPE>(c[k], sc.t2);
+      for (int k = 0; k < 4; ++k) w[k] = sub_pair<DTYPE>(sc.t2, c[k]);
     }
     acc <<= 8;
 #pragma unroll
@@ -556,7 +560,7 @@ __device__ __forceinline__ uint32_t piece_screened(uint32_t c_at, uint32_t u_at,
       asm("dp4a.s32.u32 %0, %1, %2, %0;" : "+r"(acc) : "r"(signs), "r"(k == 0 ? 0x08040201u : 0x80402010u));
     }
   }
-  const uint32_t hits = (uint32_t)acc - 1u;  // ~(-acc)
+  const uint32_t hits = 0u - (uint32_t)acc;
   return __funnelshift_l(hits, hits, 8 * rot);
 }
 
@@ -619,9 +623,10 @@ __device__ __forceinline__ void sift_unit(const RowArgs& a, uint32_t c_unit, uin
     if (HAS_U) exact = __any_sync(0xffffffffu, largest_of<DTYPE>(u_max) > screen.u_limit);
   }
   if (exact) {
-    const uint64_t neg_tau2 = pack2(-bins.tau0, -bins.tau0);
-    x0 = piece_hits<DTYPE, HAS_U, HAS_T>(c_unit + at0, u_unit + at0, rot, s2, t2, neg_tau2);
-    if (whole) x1 = piece_hits<DTYPE, HAS_U, HAS_T>(c_unit + at1, u_unit + at1, rot, s2, t2, neg_tau2);
+    const float below = bins.tau0 == 0.0f ? __int_as_float(0x80000001) : key_float(float_key(bins.tau0) - 1u);
+    const uint64_t below2 = pack2(below, below);
+    x0 = piece_hits<DTYPE, HAS_U, HAS_T>(c_unit + at0, u_unit + at0, rot, s2, t2, below2);
+    if (whole) x1 = piece_hits<DTYPE, HAS_U, HAS_T>(c_unit + at1, u_unit + at1, rot, s2, t2, below2);
   }
   if (swap) {
     const uint32_t x = x0;

@@ -142,3 +142,20 @@ def test_screening_keeps_what_32_bit_rounding_lifts(B, W, dtype, u_size, c_size)
         arr[:] = wk._store(x.astype(np.float32), dtype)
     prev = oracle_prime(inp)
     check_parity(inp.cond, inp.uncond, prev.tokens, prev.probs, step_kwargs(inp), inp.win_len)
+
+
+@pytest.mark.parametrize("mask", ["a tenth in one piece", "every other token"])
+@pytest.mark.parametrize("V,K,dtype,B,W,temperature", [(65536, 2000, wk.BF16, 2, 76, 1.0), (50264, 500, wk.BF16, 1, 6, 0.8),
+                                                       (50264, 500, wk.F16, 3, 53, 1.0), (16384, 300, wk.F32, 2, 80, 1.0)])
+def test_masked_tokens_are_no_candidates(V, K, dtype, B, W, temperature, mask):
+    # tokens forbidden with -inf in both arrays: their merge is a NaN, and no row is redone for them
+    from gpu_harness import check_parity, oracle_prime, step_kwargs
+    wl = wk.CONFIGS["cfg2"].scaled(B=B, W=W, V=V, dtype=dtype, top_k=K, temperature=temperature, seed=W)
+    inp = wk.make_step_inputs(wl)
+    ids = np.arange(V)
+    out = (ids // (V // 10) == 3) if mask.startswith("a tenth") else (np.random.default_rng(V).random(V) < 0.5)
+    for arr in (inp.cond, inp.uncond, inp.prev_cond, inp.prev_uncond):
+        arr[:, :, out] = wk._store(np.full(1, -np.inf, np.float32), dtype)[0]
+    prev = oracle_prime(inp)
+    rep, got, ref = check_parity(inp.cond, inp.uncond, prev.tokens, prev.probs, step_kwargs(inp), inp.win_len)
+    assert not np.any(got.status & 16)
