@@ -201,7 +201,7 @@ void cut_segments(sjd::SiftCfg* c, int V, int segs, double p, double sd, double 
 }
 
 bool plan_sift(const sjd_params* P, int kcap, bool has_u, SiftPlan* plan) {
-  const int V = P->V, es = P->logits_dtype == SJD_F32 ? 4 : 2, ev = 16 / es, unit = sjd::kUnitBytes / es;
+  const int V = P->V, es = P->logits_dtype == SJD_F32 ? 4 : 2, ev = 16 / es;
   if (V < 2048 || V > 65536 * sjd::kTeamWarps) return false;
   sjd::SiftCfg& c = plan->cfg;
   std::memset(&c, 0, sizeof(c));
@@ -245,15 +245,17 @@ bool plan_sift(const sjd_params* P, int kcap, bool has_u, SiftPlan* plan) {
   const int sms = sm_count();
   const int64_t rows = (int64_t)P->B * P->W;
   const double more = !c.packed ? 1.0 : P->logits_dtype == SJD_F16 || !has_u ? 1.05 : 1.15;
-  // few rows: as many CTAs per row as there are SMs for, as long as a warp has half a unit of its own
-  for (int n_cta = sjd::kMaxCluster; n_cta >= 1; n_cta >>= 1) {
-    if (rows * n_cta > sms) continue;
-    if (n_cta > 1 && (int64_t)V < (int64_t)unit * sjd::kClusterWarps * n_cta / 4) continue;
+  // few rows: the fewest CTAs that hold a row, while all rows' clusters find their SMs at once (clusters of four and eight do
+  // not fill the GPU: their SMs lie in one GPC).  Sharing a row costs more than it saves: every CTA takes the whole sample,
+  // and the candidates, the barriers and the launch of a cluster are slow.  16 rows, us a step with clusters of 1, 2, 4, 8 CTAs and
+  // by the stream kernel: of 16,384 bf16, K=500: 12.8, 14.1, 16.5, 32.3, 13.7; of 65,536 bf16 (do not fit one): -, 15.5, 16.7, 32.8,
+  // 18.1; of 65,536 fp32: -, -, 16.7, 31.9, 21.3 (32 rows: 18.8 with four; 36 rows: 25.0, two rounds of clusters, and 21.8).
+  for (int n_cta = 1; n_cta <= sjd::kMaxCluster; n_cta <<= 1) {
+    if (rows * n_cta > (n_cta <= 2 ? sms : n_cta == 4 ? sms * 7 / 8 : sms / 2)) break;
     cut_segments(&c, V, sjd::kClusterWarps * n_cta, p, sd, more);
     plan->cluster = n_cta;
     plan->smem = sjd::sift_cluster_smem(c, n_cta, es, has_u);
     if (plan->smem <= kSmemLimit && (int64_t)n_cta * c.seg_len <= 65536) return true;
-    break;
   }
   cut_segments(&c, V, sjd::kTeamWarps, p, sd, more);
   c.once = rows * V * es * (has_u ? 2 : 1) > (96ll << 20) ? 1 : 0;

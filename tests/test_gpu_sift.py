@@ -159,3 +159,12 @@ def test_masked_tokens_are_no_candidates(V, K, dtype, B, W, temperature, mask):
     prev = oracle_prime(inp)
     rep, got, ref = check_parity(inp.cond, inp.uncond, prev.tokens, prev.probs, step_kwargs(inp), inp.win_len)
     assert not np.any(got.status & 16)
+
+
+# rows that one CTA does not hold: clusters of two, four and eight with ragged last segments, and more rows than there is
+# room for their clusters (which the kernel for many rows takes)
+@pytest.mark.parametrize("V,K,dtype,B,W", [(40008, 300, wk.F32, 1, 3), (65528, 700, wk.F16, 2, 5), (65544, 300, wk.F32, 1, 4), (65536, 500, wk.F32, 4, 9),
+                                           (131080, 2000, wk.BF16, 1, 3), (262152, 1500, wk.F16, 1, 2), (262144, 500, wk.BF16, 2, 5),
+                                           (300008, 100, wk.F32, 1, 1)])
+def test_rows_shared_by_a_cluster(V, K, dtype, B, W):
+    _check(f"cluster{V}", B=B, W=W, V=V, dtype=dtype, top_k=K, seed=V % 1000)
