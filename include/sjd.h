@@ -61,7 +61,7 @@ extern "C" {
                                 newly initialised; sjd_step() ignores it                                   */
 
 #define SJD_FLAG_FORCE_GENERIC 4 /* diagnostics: use the any-shape multi-pass row kernel even where a
-                                   single-pass kernel applies (results are identical)                    */
+                                   single-pass kernel applies (same ids; probabilities agree to rounding) */
 #define SJD_FLAG_FORCE_TILES 8   /* diagnostics: skip the single-pass kernels that cut a row into one id
                                    range per warp; the tile-dealing one is used where it applies          */
 

@@ -167,6 +167,14 @@ __device__ __forceinline__ uint64_t shfl_up_u64(uint64_t v, int d) {
   return (uint64_t)lo | ((uint64_t)hi << 32);
 }
 
+// Sum over the warp's lanes (modulo 2^64), in pieces that the warp-wide 32-bit sum holds.
+__device__ __forceinline__ uint64_t warp_sum_u64(uint64_t v) {
+  const uint32_t a = __reduce_add_sync(0xffffffffu, (uint32_t)v & 0x3ffffffu);
+  const uint32_t b = __reduce_add_sync(0xffffffffu, (uint32_t)(v >> 26) & 0x3ffffffu);
+  const uint32_t c = __reduce_add_sync(0xffffffffu, (uint32_t)(v >> 52));
+  return (uint64_t)a + ((uint64_t)b << 26) + ((uint64_t)c << 52);
+}
+
 // Exclusive prefix sum of one value per thread in rank order; *total receives the group sum.
 template <int NT, int BAR, typename T>
 __device__ __forceinline__ T group_exclusive_scan(T v, int tid, uint64_t* scratch, T* total) {

@@ -168,3 +168,21 @@ def test_masked_tokens_are_no_candidates(V, K, dtype, B, W, temperature, mask):
                                            (300008, 100, wk.F32, 1, 1)])
 def test_rows_shared_by_a_cluster(V, K, dtype, B, W):
     _check(f"cluster{V}", B=B, W=W, V=V, dtype=dtype, top_k=K, seed=V % 1000)
+
+
+@pytest.mark.parametrize("V,K,dtype,B,W,temperature", [(8192, 300, wk.BF16, 3, 60, 1.0), (65536, 2000, wk.BF16, 3, 60, 1.0),
+                                                       (65536, 500, wk.F32, 6, 30, 0.9), (50264, 100, wk.F16, 4, 50, 1.0)])
+def test_a_sequence_alone_gives_the_same_bits(V, K, dtype, B, W, temperature):
+    # one sequence's rows by clusters, the same rows in a batch by the kernel for many rows
+    from gpu_harness import gpu_step, oracle_prime, step_kwargs
+    import oracle
+    wl = wk.CONFIGS["cfg2"].scaled(B=B, W=W, V=V, dtype=dtype, top_k=K, temperature=temperature, seed=V % 77)
+    inp = wk.make_step_inputs(wl)
+    prev = oracle_prime(inp)
+    batch = gpu_step(inp.cond, inp.uncond, prev.tokens, prev.probs, **step_kwargs(inp))
+    one = lambda a: None if a is None else np.ascontiguousarray(a[:1])
+    q = oracle.Probs(one(prev.probs.tok_prob), one(prev.probs.ids), one(prev.probs.vals), one(prev.probs.cnt))
+    kw = step_kwargs(inp, win_len=one(inp.win_len), pos_base=one(inp.pos_base))
+    alone = gpu_step(one(inp.cond), one(inp.uncond), one(prev.tokens), q, **kw)
+    for name in ("accept_len", "tokens", "tok_prob", "ids", "vals", "cnt", "flags", "status"):
+        assert getattr(alone, name).tobytes() == getattr(batch, name)[:1].tobytes(), name
