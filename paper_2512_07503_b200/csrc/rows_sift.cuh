@@ -14,7 +14,15 @@
 //             lower id), softmax, output, inverse-CDF draw.  Every warp works on its own candidates, which are in
 //             ascending id order already; what the warps exchange is a histogram and a few sums.
 //
-// A row whose candidates cannot contain its top-K for sure (fewer than K), do not fit the lists, or have no finite
+// A row whose largest entries crowd into one block of ids (image tokens in a vocabulary with text) overruns one segment's list
+// while the others are empty.  What finds no room is still counted, and the histogram of all candidates gives a threshold that
+// hardly more than K entries reach: with that the row is sifted once more, every unit taking a run of one list for the
+// whole row.  us a step with the top-K in an eighth of the ids, all of it redone by
+// row_generic() before: 1,024 rows of 65,536 bf16, K=2,000: 598 -> 259; 1,000 of 65,536 fp16, K=100: 560 -> 124; 231 of 50,264, K=500:
+// 136 -> 71; 1,024 of 65,536, K=8,192: 907 -> 436 (ordinary rows of these shapes: 75.7 -> 76.8, 55.3 -> 55.9, 27.9 -> 27.9, 169 -> 170).  One list for
+// all rows from the start costs ordinary rows a tenth (a barrier per row, an atomic per unit, loops over short runs).
+//
+// A row whose candidates cannot contain its top-K for sure (fewer than K), do not fit the list even so, or have no finite
 // maximum is redone by row_generic() from global memory: results are exact for any input.
 //
 // Two kernels share the phases:
@@ -71,7 +79,10 @@ struct SiftCfg {
   int rank;          // rank of tau0 among the groups, from the top
   int packed;        // 1: entries may be screened in packed 16-bit arithmetic (see SiftScreen)
   int seg_len;       // ids per segment, a multiple of 8
+  int units;         // units per segment
   int seg_cap;       // candidates a segment's list holds (a multiple of 8)
+  int pool;          // entries of all lists of a row (a multiple of 8, below 65,536)
+  int scratch;       // cluster kernel: ids that a warp can list apart from these
   int teams, slots;  // stream kernel: teams per CTA, ring slots per warp
   int once;          // stream kernel: the logits of the call exceed the L2
   int row_begin, row_end;  // stream kernel: this launch covers rows [row_begin, row_end)
@@ -104,6 +115,7 @@ struct alignas(16) SiftShared {
   uint64_t wz[kClusterWarps];
   uint32_t max_key;   // largest candidate
   uint32_t over;      // a list ran over, or a wait gave up
+  uint32_t taken;     // a row that crowds: entries of its list that are given out
   int members;
   uint32_t rank_bin, rank_above, rank_count;  // results of a rank search
   float thr_y;
@@ -581,7 +593,12 @@ struct SiftTarget {
   uint32_t y_at, id_at;    // shared-memory addresses of the segment's lists (of the cluster's first CTA when REMOTE)
   uint32_t hist_at;        // of the candidates' histogram (a SiftHist)
   uint32_t scratch_at;     // local id list (the same as id_at unless REMOTE)
+  uint32_t cap;            // candidates the lists hold
+  // a row that crowds: the lists are the row's
+  uint32_t taken_at;       // of the number of entries given out
+  uint32_t scratch;        // ids the local list holds (0: it is the row's)
 };
+constexpr uint32_t kNoRoom = 0xffffffffu;
 
 template <bool REMOTE>
 __device__ __forceinline__ void put_f32(uint32_t at, float v) {
@@ -599,12 +616,25 @@ __device__ __forceinline__ void count_at(uint32_t at) {
   else asm volatile("red.relaxed.cta.shared::cta.add.u32 [%0], 1;" ::"r"(at) : "memory");
 }
 
+// `n` entries of the row's list, n being lane 31's
+template <bool REMOTE>
+__device__ __forceinline__ uint32_t take_entries(uint32_t at, uint32_t n, int lane) {
+  uint32_t first = 0;
+  if (lane == 31) {
+    if (REMOTE) asm volatile("atom.relaxed.cluster.shared::cluster.add.u32 %0, [%1], %2;" : "=r"(first) : "r"(at), "r"(n) : "memory");
+    else asm volatile("atom.relaxed.cta.shared::cta.add.u32 %0, [%1], %2;" : "=r"(first) : "r"(at), "r"(n) : "memory");
+  }
+  return __shfl_sync(0xffffffffu, first, 31);
+}
+
 // One unit: `valid` elements of it belong to the segment; element 0 has id `rel` in the segment's numbering, which is
-// what the list keeps plus `bias`.  n: candidates so far (cap + 1 or more: the list has run over).
-template <int DTYPE, bool HAS_U, bool HAS_T, bool REMOTE>
+// what the list keeps plus `bias`.  n: candidates so far (cap + 1: the list has run over).
+// CROWDS: the unit takes a run of the row's list, which n becomes: its first entry, and from bit 16 its length (kNoRoom: there was
+// none).  Candidates that find no room are counted all the same, so that the row's histogram is complete.
+template <int DTYPE, bool HAS_U, bool HAS_T, bool REMOTE, bool CROWDS>
 __device__ __forceinline__ void sift_unit(const RowArgs& a, uint32_t c_unit, uint32_t u_unit, int valid, uint32_t rel, uint32_t bias,
                                           uint64_t s2, uint64_t t2, const SiftBinning& bins, const SiftScreen& screen,
-                                          const SiftTarget& to, uint32_t cap, int lane, uint32_t& n, float& vmax) {
+                                          const SiftTarget& to, int lane, uint32_t& n, float& vmax) {
   constexpr int ES = SiftTraits<DTYPE>::kElem, EP = SiftTraits<DTYPE>::kPiece, EU = SiftTraits<DTYPE>::kUnit;
   uint32_t x0 = 0, x1 = 0;  // hits of the lane's first and second piece
   const bool whole = valid > EU / 2;
@@ -643,32 +673,55 @@ __device__ __forceinline__ void sift_unit(const RowArgs& a, uint32_t c_unit, uin
   }
   const uint32_t inc = scan_incl((uint32_t)(__popc(x0) + __popc(x1)), lane);
   const uint32_t total = __shfl_sync(0xffffffffu, inc, 31);
-  if (n + total > cap) {
-    n = cap + 1u;
+  const uint32_t first = rel + (uint32_t)lane * run;  // id of the lane's first bit
+  const uint32_t c_rel = c_unit - rel * (uint32_t)ES, u_rel = u_unit - rel * (uint32_t)ES;
+  const bool own_ids = CROWDS && REMOTE && to.scratch != 0u;  // ids are listed apart from the row's list
+  uint32_t at = n;  // first entry of the unit's candidates
+  if (CROWDS) at = take_entries<REMOTE>(to.taken_at, inc, lane);
+  if (__builtin_expect(at + total > to.cap || (own_ids && total > to.scratch), 0)) {
+    n = CROWDS ? kNoRoom : to.cap + 1u;
+    while ((x0 | x1) != 0u) {  // one of each piece at a time
+      float y[2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const uint32_t x = h == 0 ? x0 : x1, id = x != 0u ? first + 32u * h + (uint32_t)__ffs((int)x) - 1u : first;
+        y[h] = merge_entry<DTYPE, HAS_U, HAS_T>(c_rel + id * (uint32_t)ES, u_rel + id * (uint32_t)ES, a.s, a.inv_T);
+        if (x == 0u) y[h] = __int_as_float(0xff800000);
+      }
+      x0 &= x0 - 1u;
+      x1 &= x1 - 1u;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const uint32_t bin = min(__float2uint_rz(bins.at(y[h])), (uint32_t)kSiftBins - 1u);
+        count_at<REMOTE>(to.hist_at + 4u * bin);
+        count_at<REMOTE>(to.hist_at + 4u * (kSiftBins + (bin >> 5)));
+        vmax = fmaxf(vmax, y[h]);
+      }
+    }
+    __syncwarp();
     return;
   }
   // ids, from the lane's highest one down
+  const uint32_t ids_at = own_ids ? to.scratch_at : to.scratch_at + 2u * at;
   {
-    const uint32_t first = rel + (uint32_t)lane * run;
-    uint32_t put = to.scratch_at + 2u * (n + inc);
+    uint32_t put = ids_at + 2u * inc;
     if (DTYPE != 0) put = put_ids(x1, first + 32u, put);
     put_ids(x0, first, put);
   }
   __syncwarp();
   // candidates: merged, binned and kept, two groups of 32 at a time (their loads do not wait for one another)
-  const uint32_t c_rel = c_unit - rel * (uint32_t)ES, u_rel = u_unit - rel * (uint32_t)ES;
   auto keep = [&](auto groups, uint32_t i0) {
     constexpr int G = decltype(groups)::value;
     uint32_t id[G];
     float y[G];
 #pragma unroll
-    for (int j = 0; j < G; ++j) id[j] = lds16(to.scratch_at + 2u * (n + min(i0 + 32u * j + (uint32_t)lane, total - 1u)));
+    for (int j = 0; j < G; ++j) id[j] = lds16(ids_at + 2u * min(i0 + 32u * j + (uint32_t)lane, total - 1u));
 #pragma unroll
     for (int j = 0; j < G; ++j)
       y[j] = merge_entry<DTYPE, HAS_U, HAS_T>(c_rel + id[j] * (uint32_t)ES, u_rel + id[j] * (uint32_t)ES, a.s, a.inv_T);
 #pragma unroll
     for (int j = 0; j < G; ++j) {
-      const uint32_t i = i0 + 32u * j + (uint32_t)lane, k = n + i;
+      const uint32_t i = i0 + 32u * j + (uint32_t)lane, k = at + i;
       const bool in = i < total;
       const uint32_t bin = in ? min(__float2uint_rz(bins.at(y[j])), (uint32_t)kSiftBins - 1u) : 0u;
       count_at<REMOTE>(to.hist_at + 4u * bin);
@@ -683,7 +736,7 @@ __device__ __forceinline__ void sift_unit(const RowArgs& a, uint32_t c_unit, uin
   uint32_t i0 = 0;
   for (; i0 + 32u < total; i0 += 64u) keep(std::integral_constant<int, 2>(), i0);
   if (i0 < total) keep(std::integral_constant<int, 1>(), i0);
-  n += total;
+  n = CROWDS ? at | (total << 16) : at + total;
 }
 
 // exp(y - m) with the rounding of the difference compensated (exp_diff without its case for y = -inf)
@@ -705,13 +758,40 @@ __device__ __forceinline__ uint64_t fixed_exp(float e) { return __float2ull_rz(_
 // ---------------------------------------------------------------------------------------------------
 // finish phase, by the NW warps that work on the row
 // ---------------------------------------------------------------------------------------------------
-// Warp w holds the candidates of `per_warp` consecutive segments in lists of seg_cap entries each, ids relative to
-// the warp's first id.  Starts with a barrier.  Returns false when the row has to be redone; the histogram is zero
-// again and the counters are reset either way.
+// where the runs of a row that crowds lie in it: run r holds candidates of the ids from (r / units) * seg_len + (r % units) * unit on
+struct SiftRuns {
+  uint32_t* run;  // first entry in the row's list, and from bit 16 their number
+  int n, units, seg_len, unit;
+  __device__ __forceinline__ int id0(int r) const { return r / units * seg_len + r % units * unit; }
+};
+// The first run of warp `part`'s share when NW warps share the candidates about evenly: the number of runs that begin before
+// that part of all candidates.
 template <int NW>
-__device__ __forceinline__ bool finish_row(const RowArgs& a, const SiftCfg& cfg, SiftShared& sm, float* list_y, uint16_t* list_id,
-                                           const uint32_t* seg_n, int per_warp, const SiftBinning& bins, int row, int pos, int iter,
-                                           int draft, int tid, int bar) {
+__device__ __forceinline__ int first_run(const SiftRuns& runs, int part, int lane) {
+  uint32_t total = 0;
+  for (int r = lane; r < runs.n; r += 32) total += runs.run[r] >> 16;
+  total = __reduce_add_sync(0xffffffffu, total);
+  const uint32_t bound = (uint32_t)((uint64_t)total * (uint32_t)part / NW);
+  uint32_t before = 0;
+  int n = 0;
+  for (int r0 = 0; r0 < runs.n; r0 += 32) {
+    const uint32_t len = r0 + lane < runs.n ? runs.run[r0 + lane] >> 16 : 0u;
+    const uint32_t upto = scan_incl(len, lane);
+    n += __popc(__ballot_sync(0xffffffffu, r0 + lane < runs.n && before + upto - len < bound));
+    before += __shfl_sync(0xffffffffu, upto, 31);
+  }
+  return part >= NW ? runs.n : n;
+}
+
+// Warp w holds the candidates of `per_warp` consecutive segments in lists of seg_cap entries each, seg_n of them in use, ids
+// relative to the warp's first one.  CROWDS: the row has one list, `runs` of it in ascending order, of which each warp takes a share;
+// their ids are relative to the run's first one.
+// Starts with a barrier.  The histogram is zero again and the counters are reset whatever comes of it.
+enum { kRowDone = 0, kRowOver = 1, kRowElse = 2 };  // finished; a list had run over; not to be finished here for another reason
+template <int NW, bool CROWDS>
+__device__ __forceinline__ int finish_row(const RowArgs& a, const SiftCfg& cfg, SiftShared& sm, float* list_y, uint16_t* list_id,
+                                          const uint32_t* seg_n, int per_warp, const SiftRuns& runs, const SiftBinning& bins, int row, int pos,
+                                          int iter, int draft, int status, int tid, int bar) {
   constexpr int NT = NW * 32;
   const int lane = tid & 31, warp = tid >> 5;
   const uint32_t kcap = (uint32_t)a.kcap;
@@ -733,30 +813,37 @@ __device__ __forceinline__ bool finish_row(const RowArgs& a, const SiftCfg& cfg,
   if (tid == 0) {
     sm.max_key = 0u;
     sm.over = 0u;
+    if (CROWDS) sm.taken = 0u;
+    sm.thr_y = vmax;  // (for raise_threshold)
   }
   // fewer than kcap candidates, a threshold bin too crowded for the ranking, or no finite maximum
   if (over || tbin == 0u || nbin > (uint32_t)kMemberCap || !(vmax <= 3.402823466e38f)) {
     row_sync<NT>(bar);
-    return false;
+    return over ? kRowOver : kRowElse;
   }
-  const size_t first_seg = (size_t)warp * per_warp;
+  // the warp's segments, or its share of the runs: from g0 on, up to g1
+  const int g0 = CROWDS ? first_run<NW>(runs, warp, lane) : 0, g1 = CROWDS ? first_run<NW>(runs, warp + 1, lane) : per_warp;
+  if (CROWDS) row_sync<NT>(bar);  // (their lengths are changed below)
+  const size_t first_seg = CROWDS ? 0 : (size_t)warp * per_warp;
   float* const my_y = list_y + first_seg * cfg.seg_cap;
   uint16_t* const my_id = list_id + first_seg * cfg.seg_cap;
-  const int id0 = warp * per_warp * cfg.seg_len;
+  const int warp_id0 = warp * per_warp * cfg.seg_len;
   // ---- the threshold bin's members
   {
     // (the last bin also holds what lies above its end)
     const bool last = tbin == (uint32_t)kSiftBins - 1u;
     const float lo = (float)tbin, hi = (float)(tbin + 1u);
-    for (int g = 0; g < per_warp; ++g) {
-      const uint32_t n = seg_n[first_seg + g];
-      const float* const y_g = my_y + g * cfg.seg_cap;
+    for (int g = g0; g < g1; ++g) {
+      const uint32_t run = CROWDS ? runs.run[g] : 0u, n = CROWDS ? run >> 16 : seg_n[first_seg + g];
+      const uint32_t at_g = CROWDS ? run & 0xffffu : (uint32_t)(g * cfg.seg_cap);
+      const int id0 = CROWDS ? runs.id0(g) : warp_id0;
+      const float* const y_g = my_y + at_g;
 #pragma unroll 4
       for (uint32_t i = (uint32_t)lane; i < n; i += 32u) {
         const float y = y_g[i], x = bins.at(y);
         if (x >= lo && (x < hi || last)) {
           const int at = atomicAdd(&sm.members, 1);  // (as many as the histogram counted: the check keeps the store in bounds)
-          if (at < kMemberCap) sm.hist.member[at] = SiftMember{y, id0 + (int32_t)my_id[g * cfg.seg_cap + i]};
+          if (at < kMemberCap) sm.hist.member[at] = SiftMember{y, id0 + (int32_t)my_id[at_g + i]};
         }
       }
     }
@@ -796,15 +883,18 @@ __device__ __forceinline__ bool finish_row(const RowArgs& a, const SiftCfg& cfg,
     thr_y = sm.thr_y;
     thr_id = sm.thr_id;
   }
-  // ---- survivors: exponentials and ids to the front of the warp's lists, their number and sum.  Four groups of 32 at a
-  // time: their loads and exponentials do not wait for one another, nor for the stores, which go to places already read.
-  const int thr_rel = thr_id - id0;
+  // ---- survivors: exponentials and ids to the front of the warp's lists (of each run), their number and sum.  Four groups of 32
+  // at a time: their loads and exponentials do not wait for one another, nor for the stores, which go to places already read.
+  int thr_rel = thr_id - warp_id0;
   uint32_t cnt = 0;
   uint64_t z = 0;
-  for (int g = 0; g < per_warp; ++g) {
-    const uint32_t n = seg_n[first_seg + g];
-    const float* const y_g = my_y + g * cfg.seg_cap;
-    const uint16_t* const id_g = my_id + g * cfg.seg_cap;
+  for (int g = g0; g < g1; ++g) {
+    const uint32_t run = CROWDS ? runs.run[g] : 0u, n = CROWDS ? run >> 16 : seg_n[first_seg + g];
+    const uint32_t at_g = CROWDS ? run & 0xffffu : (uint32_t)(g * cfg.seg_cap);
+    const float* const y_g = my_y + at_g;
+    const uint16_t* const id_g = my_id + at_g;
+    const uint32_t cnt0 = cnt;
+    if (CROWDS) thr_rel = thr_id - runs.id0(g);
     constexpr int U = 4;
 #pragma unroll 1
     for (uint32_t i0 = 0; i0 < n; i0 += 32u * U) {
@@ -827,7 +917,7 @@ __device__ __forceinline__ bool finish_row(const RowArgs& a, const SiftCfg& cfg,
 #pragma unroll
       for (int j = 0; j < U; ++j) {
         if ((votes[j] >> lane) & 1u) {
-          const uint32_t at = cnt + (uint32_t)__popc(votes[j] & below);
+          const uint32_t at = (CROWDS ? at_g + cnt - cnt0 : cnt) + (uint32_t)__popc(votes[j] & below);
           my_y[at] = e[j];
           my_id[at] = (uint16_t)id[j];
           z += fixed_exp(e[j]);
@@ -836,6 +926,7 @@ __device__ __forceinline__ bool finish_row(const RowArgs& a, const SiftCfg& cfg,
       }
       __syncwarp();
     }
+    if (CROWDS && lane == 0) runs.run[g] = at_g | ((cnt - cnt0) << 16);
   }
   z = warp_sum_u64(z);
   if (lane == 0) {
@@ -849,22 +940,30 @@ __device__ __forceinline__ bool finish_row(const RowArgs& a, const SiftCfg& cfg,
   const uint32_t before = __reduce_add_sync(0xffffffffu, lane < warp ? cw : 0u);
   if (__reduce_add_sync(0xffffffffu, cw) != kcap) {  // cannot happen; the result stays exact anyway
     row_sync<NT>(bar);  // (the histogram's words are zero before anybody counts in them again)
-    return false;
+    return kRowElse;
   }
   const uint64_t Z = warp_sum_u64(lane < NW ? sm.wz[lane] : 0ull);
   const float inv_Z = __fdiv_rn(0x1p45f, __ull2float_rn(Z));  // p = e / Z within 2 ulp
   // ---- output and fixed-point weights
-  int32_t* const out_ids = a.out_ids + (size_t)row * kcap + before;
-  float* const out_vals = a.out_vals + (size_t)row * kcap + before;
+  const int p0 = CROWDS ? g0 : 0, p1 = CROWDS ? g1 : 1;  // where the warp's survivors lie: in the front of its runs, or of its lists
+  int32_t* out_ids = a.out_ids + (size_t)row * kcap + before;
+  float* out_vals = a.out_vals + (size_t)row * kcap + before;
   uint64_t wsum = 0;
+  for (int g = p0; g < p1; ++g) {
+    const uint32_t n = CROWDS ? runs.run[g] >> 16 : cnt, at_g = CROWDS ? runs.run[g] & 0xffffu : 0u;
+    const int id0 = CROWDS ? runs.id0(g) : warp_id0;
+    const float* const y_g = my_y + at_g;
+    const uint16_t* const id_g = my_id + at_g;
 #pragma unroll 4
-  for (uint32_t i = (uint32_t)lane; i < cnt; i += 32u) {
-    const float p = __fmul_rn(my_y[i], inv_Z);
-    const int id = id0 + (int)my_id[i];
-    out_ids[i] = id;
-    out_vals[i] = p;
-    wsum += fixed_weight(p);
-    if (id == draft) sm.ptok = p;
+    for (uint32_t i = (uint32_t)lane; i < n; i += 32u) {
+      const float p = __fmul_rn(y_g[i], inv_Z);
+      const int id = id0 + (int)id_g[i];
+      out_ids[i] = id;
+      out_vals[i] = p;
+      wsum += fixed_weight(p);
+      if (id == draft) sm.ptok = p;
+    }
+    if (CROWDS) out_ids += n, out_vals += n;
   }
   wsum = warp_sum_u64(wsum);
   if (lane == 0) sm.wtot[warp] = wsum;
@@ -884,33 +983,68 @@ __device__ __forceinline__ bool finish_row(const RowArgs& a, const SiftCfg& cfg,
   const uint64_t hi = shfl_u64(xi, warp);
   if (total == 0ull) {  // all weights rounded to zero: the first survivor
     if (lane == 0 && before == 0u && cnt > 0u) {
-      a.out_cnt[row] = (int)kcap;
-      a.scratch[row] = RowScratch{sm.ptok, id0 + (int32_t)my_id[0], __fmul_rn(my_y[0], inv_Z), 0};
-    }
-  } else if (t >= lo && t < hi) {
-    const uint32_t run = (cnt + 31u) / 32u;
-    const uint32_t beg = min((uint32_t)lane * run, cnt), end = min(beg + run, cnt);
-    uint64_t own = 0;
-    for (uint32_t i = beg; i < end; ++i) own += fixed_weight(__fmul_rn(my_y[i], inv_Z));
-    uint64_t inc = own;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-      const uint64_t o = shfl_up_u64(inc, d);
-      if (lane >= d) inc += o;
-    }
-    lo += inc - own;
-    if (t >= lo && t < lo + own) {
-      uint32_t i = beg;
-      float p;
-      for (;; ++i) {  // ends before `end`: the run's weights sum to more than t - lo
-        p = __fmul_rn(my_y[i], inv_Z);
-        lo += fixed_weight(p);
-        if (t < lo || i + 1u >= end) break;
+      uint32_t at = 0u;
+      int id0 = warp_id0;
+      if (CROWDS) {
+        int g = g0;
+        while ((runs.run[g] >> 16) == 0u) ++g;
+        at = runs.run[g] & 0xffffu;
+        id0 = runs.id0(g);
       }
       a.out_cnt[row] = (int)kcap;
-      a.scratch[row] = RowScratch{sm.ptok, id0 + (int32_t)my_id[i], p, 0};
+      a.scratch[row] = RowScratch{sm.ptok, id0 + (int32_t)my_id[at], __fmul_rn(my_y[at], inv_Z), status};
+    }
+  } else if (t >= lo && t < hi) {
+    for (int g = p0; g < p1; ++g) {
+      const uint32_t n = CROWDS ? runs.run[g] >> 16 : cnt, at_g = CROWDS ? runs.run[g] & 0xffffu : 0u;
+      const int id0 = CROWDS ? runs.id0(g) : warp_id0;
+      const float* const y_g = my_y + at_g;
+      const uint32_t run = (n + 31u) / 32u;
+      const uint32_t beg = min((uint32_t)lane * run, n), end = min(beg + run, n);
+      uint64_t own = 0;
+      for (uint32_t i = beg; i < end; ++i) own += fixed_weight(__fmul_rn(y_g[i], inv_Z));
+      uint64_t inc = own;
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const uint64_t o = shfl_up_u64(inc, d);
+        if (lane >= d) inc += o;
+      }
+      uint64_t sum = lo + inc - own;
+      if (CROWDS) {
+        lo += shfl_u64(inc, 31);
+        if (t >= lo) continue;  // the whole warp: the draw lies behind this run
+      }
+      if (t >= sum && t < sum + own) {
+        uint32_t i = beg;
+        float p;
+        for (;; ++i) {  // ends before `end`: the lane's weights sum to more than t - sum
+          p = __fmul_rn(y_g[i], inv_Z);
+          sum += fixed_weight(p);
+          if (t < sum || i + 1u >= end) break;
+        }
+        a.out_cnt[row] = (int)kcap;
+        a.scratch[row] = RowScratch{sm.ptok, id0 + (int32_t)my_id[at_g + i], p, status};
+      }
+      break;
     }
   }
+  if (CROWDS) row_sync<NT>(bar);  // (the next row's runs may lie anywhere in the list)
+  return kRowDone;
+}
+
+// By the thread that resets the counters, after a row has run over its lists: from the row's complete histogram a
+// threshold that only the entries of the K-th largest one's bin and above reach.  False when even they do not fit, or when
+// that would be the threshold there was.
+__device__ __forceinline__ bool raise_threshold(const SiftShared& sm, const SiftBinning& bins, int room, SiftTau& tau) {
+  const uint32_t bin = sm.rank_bin;
+  const float vmax = sm.thr_y;
+  if (bin < 2u || (int)(sm.rank_above + sm.rank_count) + 64 > room || !(vmax <= 3.402823466e38f)) return false;
+  // the least difference to tau0 that falls into the bin, a little less (some entries of the bin below come along)
+  const float d = fmaxf(__fdiv_rn((float)bin - 1.0f, bins.s1), __fdiv_rn((float)bin - kBinsCross, bins.s2));
+  const float raised = __fadd_rd(bins.tau0, __fmul_rd(d, 1.0f - 0x1p-14f));
+  if (!(raised > bins.tau0)) return false;
+  tau.tau0 = raised;
+  tau.top = vmax;
   return true;
 }
 
@@ -925,6 +1059,7 @@ __device__ __forceinline__ void init_shared(SiftShared& sm, int tid, int nt) {
   if (tid == 0) {
     sm.max_key = 0u;
     sm.over = 0u;
+    sm.taken = 0u;
     sm.members = 0;
   }
 }
@@ -963,20 +1098,23 @@ struct alignas(16) StreamShared {
   uint64_t sample_full[kMaxTeams], tau_full[2 * kMaxTeams], tau_free[2 * kMaxTeams];
   SiftTau tau[2 * kMaxTeams];
   uint32_t seg_n[kMaxTeams * kTeamWarps];      // candidates per segment
-  int32_t redo[kStreamRows];                   // rows the single pass could not finish (redone at the end)
-  int n_live, n_redo, abort;
+  // Rows that were not finished: those to be redone from the front; from the back places in `tab` of those to be sifted again as
+  // rows that crowd (their thresholds wait in their records).
+  int32_t redo[kStreamRows];
+  int n_live, n_redo, n_again, abort;
 };
 struct alignas(16) TeamShared {
   SiftShared row;
   SiftSample sample;  // the team's first row's is written by the team, the others' by its sampler
 };
-// shared memory: StreamShared | TeamShared x teams | list values | list ids | rings
-__host__ __device__ inline size_t sift_stream_rings(int teams, int seg_cap) {
-  const size_t b = sizeof(StreamShared) + teams * (sizeof(TeamShared) + (size_t)kTeamWarps * seg_cap * 6);
+// shared memory: StreamShared | TeamShared x teams | list values | list ids | rings.  A team's lists of its segments lie one behind the
+// other; a row that crowds has them as one, the last entries of whose values hold its runs.
+__host__ __device__ inline size_t sift_stream_rings(const SiftCfg& cfg) {
+  const size_t b = sizeof(StreamShared) + cfg.teams * (sizeof(TeamShared) + (size_t)cfg.pool * 6);
   return (b + 127) & ~(size_t)127;
 }
-__host__ __device__ inline size_t sift_stream_smem(int teams, int seg_cap, int slots, bool has_u) {
-  return sift_stream_rings(teams, seg_cap) + (size_t)kTeamWarps * slots * kUnitBytes * (has_u ? 2 : 1);
+__host__ __device__ inline size_t sift_stream_smem(const SiftCfg& cfg, bool has_u) {
+  return sift_stream_rings(cfg) + (size_t)kTeamWarps * cfg.slots * kUnitBytes * (has_u ? 2 : 1);
 }
 
 // bulk_g2s with an L2 hint
@@ -1010,6 +1148,159 @@ __device__ __forceinline__ bool sift_wait(uint64_t* bar, uint32_t parity, volati
   return false;
 }
 
+// Copies go through the ring of a warp in order: its units of row 0, row 1, ...; team t takes rows t, t + teams, ...  Whoever has worked a
+// unit through asks for the copy that goes into its slot next.  The units of a warp begin `step` ids apart, from seg0 on.
+template <int DTYPE, bool HAS_U>
+__device__ __forceinline__ void issue_unit(const RowArgs& a, StreamShared& st, unsigned char* ring, uint64_t policy, int warp, int teams,
+                                           int units, int seg0, int seg_n, int step, int n_live, int k, int unit, int slot) {
+  constexpr int ES = SiftTraits<DTYPE>::kElem, EU = SiftTraits<DTYPE>::kUnit;
+  while (unit >= units) {
+    ++k;
+    unit -= units;
+  }
+  if (k >= n_live) return;
+  const uint32_t bytes = (uint32_t)min(seg_n - unit * step, EU) * ES;
+  const int64_t off = st.tab[k].off + seg0 + (int64_t)unit * step;
+  unsigned char* const dst = ring + (size_t)slot * kUnitBytes * (HAS_U ? 2 : 1);
+#ifdef SJD_TEST_DROP_COPY
+  if (warp == SJD_TEST_DROP_COPY && k == 1 && unit == 0) return;  // test builds only, see rows_cluster_kernel
+#endif
+  const int x = (warp * kMaxTeams + k % teams) * kMaxSlots + slot;
+  ++st.used[x];
+  mbar_arrive_expect_tx(&st.full[x], bytes * (HAS_U ? 2u : 1u));
+  bulk_g2s_hinted(dst, row_ptr(a.cond, DTYPE, off), bytes, &st.full[x], policy);
+  if (HAS_U) bulk_g2s_hinted(dst + kUnitBytes, row_ptr(a.uncond, DTYPE, off), bytes, &st.full[x], policy);
+}
+// Logits that exceed the L2 leave it first (they make room for samples and outputs: 1,024 rows of 65,536 74.4 -> 73.4 us);
+// smaller ones are left where their writer put them (of 16,384: 45.7, with the hint 46.6).
+__device__ __forceinline__ uint64_t ring_policy(const SiftCfg& cfg) {
+  uint64_t policy;
+  if (cfg.once) asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
+  else asm("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(policy));
+  return policy;
+}
+// A row that is to be sifted again, by one thread: its place in `tab`, and its threshold, which waits in its record.
+__device__ __forceinline__ void sift_again(const RowArgs& a, StreamShared& st, int k, const SiftTau& tau) {
+  a.scratch[st.tab[k].row] = RowScratch{tau.tau0, (int32_t)__float_as_uint(tau.u_max), tau.top, 0};
+  st.redo[kStreamRows - 1 - atomicAdd(&st.n_again, 1)] = k;
+}
+
+// A row that crowds, by the team that calls: the part of rows_stream_kernel's loop from the sift on, with one list for the whole
+// row and every eighth unit for a warp, so that a block of ids is shared by all.  Returns the ring barriers' parities (`phase` of
+// the kernel).
+template <int DTYPE, bool HAS_U, bool HAS_T>
+__device__ __noinline__ uint32_t stream_crowded_row(const RowArgs& a, const SiftCfg& cfg, unsigned char* smem, int k, uint32_t phase, SiftTau tau) {
+  constexpr int EU = SiftTraits<DTYPE>::kUnit, kStep = kTeamWarps * EU;
+  constexpr uint32_t kSlot = kUnitBytes * (HAS_U ? 2u : 1u);
+  StreamShared& st = *reinterpret_cast<StreamShared*>(smem);
+  const int teams = cfg.teams, slots = cfg.slots;
+  const int team = (int)threadIdx.x / kTeamThreads, tid = (int)threadIdx.x % kTeamThreads, lane = tid & 31, warp = tid >> 5, bar = 1 + team;
+  TeamShared* const team_sm = reinterpret_cast<TeamShared*>(smem + sizeof(StreamShared));
+  SiftShared& sm = team_sm[team].row;
+  float* const lists = reinterpret_cast<float*>(team_sm + teams);
+  float* const list_y = lists + team * cfg.pool;
+  uint16_t* const list_id = reinterpret_cast<uint16_t*>(lists + teams * cfg.pool) + team * cfg.pool;
+  const int row_units = (a.V + EU - 1) / EU, room = cfg.pool - row_units;
+  const SiftRuns runs{reinterpret_cast<uint32_t*>(list_y + room), row_units, row_units, 0, EU};
+  unsigned char* const ring = smem + sift_stream_rings(cfg) + (size_t)warp * slots * kSlot;
+  const int seg0 = warp * EU, seg_n = max(a.V - seg0, 0), units = (seg_n + kStep - 1) / kStep;
+  volatile int* const abort_flag = &st.abort;
+  uint64_t* const full = st.full + (warp * kMaxTeams + team) * kMaxSlots;
+  const uint64_t s2 = pack2(a.s, a.s), t2 = pack2(a.inv_T, a.inv_T), policy = ring_policy(cfg);
+  const SiftBinning bins = sift_bins(tau.tau0, tau.top);
+  const SiftScreen screen = sift_screen<DTYPE, HAS_U, HAS_T>(a, cfg, tau.tau0, tau.u_max);
+  SiftTarget to;
+  to.y_at = smem_u32(list_y);
+  to.id_at = to.scratch_at = smem_u32(list_id);
+  to.hist_at = smem_u32(&sm.hist);
+  to.cap = (uint32_t)room;
+  to.taken_at = smem_u32(&sm.taken);
+  to.scratch = 0u;
+  bool ok = true, over = false;
+  float vmax = __int_as_float(0xff800000);
+  int slot = (k * units) % slots;
+  for (int unit = 0; unit < units; ++unit) {
+    ok = sift_wait(&full[slot], (phase >> slot) & 1u, abort_flag);
+    if (!ok) break;
+    phase ^= 1u << slot;
+    const uint32_t c_unit = smem_u32(ring) + (uint32_t)slot * kSlot;
+    uint32_t run = 0u;
+    sift_unit<DTYPE, HAS_U, HAS_T, false, true>(a, c_unit, c_unit + kUnitBytes, seg_n - unit * kStep, 0u, 0u, s2, t2, bins, screen, to, lane,
+                                                run, vmax);
+    over = over || run == kNoRoom;
+    __syncwarp();
+    if (lane == 0) {
+      runs.run[unit * kTeamWarps + warp] = run;
+      issue_unit<DTYPE, HAS_U>(a, st, ring, policy, warp, teams, units, seg0, seg_n, kStep, st.n_live, k, unit + slots, slot);
+    }
+    if (++slot == slots) slot = 0;
+  }
+  const uint32_t wmax = __reduce_max_sync(0xffffffffu, float_key(vmax));
+  if (lane == 0) {
+    atomicMax(&sm.max_key, wmax);
+    if (over || !ok) sm.over = 1u;
+    if (!ok) *abort_flag = 1;
+  }
+  const SiftRow& r = st.tab[k];
+  const int result = finish_row<kTeamWarps, true>(a, cfg, sm, list_y, list_id, nullptr, 0, runs, bins, r.row, r.pos, r.iter, r.draft, kRowStatusRedone,
+                                                  tid, bar);
+  if (result != kRowDone && tid == 0) {
+    if (*abort_flag != 0) {
+      a.out_cnt[r.row] = 0;
+      a.scratch[r.row] = RowScratch{0.0f, -1, 0.0f, kRowStatusTimeout};
+    } else {
+      st.redo[atomicAdd(&st.n_redo, 1)] = r.row;
+    }
+  }
+  return phase;
+}
+
+// After the CTA's last row, by all teams: the rows that are to be sifted again, through the ring as before.
+template <int DTYPE, bool HAS_U, bool HAS_T>
+__device__ __noinline__ uint32_t stream_again(const RowArgs& a, const SiftCfg& cfg, unsigned char* smem, uint32_t phase) {
+  constexpr int EU = SiftTraits<DTYPE>::kUnit, kStep = kTeamWarps * EU;
+  StreamShared& st = *reinterpret_cast<StreamShared*>(smem);
+  const int teams = cfg.teams, team = (int)threadIdx.x / kTeamThreads, lane = (int)threadIdx.x & 31;
+  const int warp = ((int)threadIdx.x % kTeamThreads) >> 5, n = st.n_again;
+  const bool lost = st.abort != 0;
+  auto sync = [&] { asm volatile("bar.sync %0, %1;" ::"n"(1 + kMaxTeams), "r"(teams * kTeamThreads) : "memory"); };
+  sync();  // (everybody has read what is changed now)
+  if (threadIdx.x < 32) {
+    SiftRow r[kStreamRows / 32];
+#pragma unroll
+    for (int j = 0; j < kStreamRows / 32; ++j)
+      if (lane + 32 * j < n) r[j] = st.tab[st.redo[kStreamRows - 1 - lane - 32 * j]];
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < kStreamRows / 32; ++j) {
+      if (lane + 32 * j >= n) continue;
+      st.tab[lane + 32 * j] = r[j];
+      if (lost) {
+        a.out_cnt[r[j].row] = 0;
+        a.scratch[r[j].row] = RowScratch{0.0f, -1, 0.0f, kRowStatusTimeout};
+      }
+    }
+    if (lane == 0) st.n_live = n;
+  }
+  sync();
+  if (lost) return phase;
+  const int seg0 = warp * EU, seg_n = max(a.V - seg0, 0), units = (seg_n + kStep - 1) / kStep;
+  unsigned char* const ring = smem + sift_stream_rings(cfg) + (size_t)warp * cfg.slots * kUnitBytes * (HAS_U ? 2 : 1);
+  if (team == 0 && lane == 0 && units > 0) {
+    const uint64_t policy = ring_policy(cfg);
+    for (int x = 0; x < cfg.slots; ++x)
+      issue_unit<DTYPE, HAS_U>(a, st, ring, policy, warp, teams, units, seg0, seg_n, kStep, n, 0, x, x);
+  }
+  __syncwarp();
+  for (int k = team; k < n; k += teams) {
+    const RowScratch what = a.scratch[st.tab[k].row];
+    phase = stream_crowded_row<DTYPE, HAS_U, HAS_T>(a, cfg, smem, k, phase,
+                                                    SiftTau{what.p_tok, what.samp_prob, __uint_as_float((uint32_t)what.samp_tok)});
+  }
+  sync();
+  return phase;
+}
+
 template <int DTYPE, bool HAS_U, bool HAS_T>
 __global__ void __launch_bounds__((kTeamThreads + 32) * kMaxTeams, 1)
 rows_stream_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ SiftCfg cfg) {
@@ -1026,9 +1317,9 @@ rows_stream_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ Si
   SiftShared& sm = team_sm[team].row;
   SiftSample& sample = team_sm[team].sample;
   float* const lists = reinterpret_cast<float*>(team_sm + teams);
-  float* const list_y = lists + (size_t)team * kTeamWarps * cfg.seg_cap;
-  uint16_t* const list_id = reinterpret_cast<uint16_t*>(lists + (size_t)teams * kTeamWarps * cfg.seg_cap) + (size_t)team * kTeamWarps * cfg.seg_cap;
-  unsigned char* const ring = smem_raw + sift_stream_rings(teams, cfg.seg_cap) + (size_t)warp * slots * kSlot;
+  float* const list_y = lists + team * cfg.pool;
+  uint16_t* const list_id = reinterpret_cast<uint16_t*>(lists + teams * cfg.pool) + team * cfg.pool;
+  unsigned char* const ring = smem_raw + sift_stream_rings(cfg) + (size_t)warp * slots * kSlot;
   if (!sampler) init_shared(sm, tid, kTeamThreads);
   if (threadIdx.x < kTeamWarps * kMaxTeams * kMaxSlots) {
     mbar_init(&st.full[threadIdx.x], 1);
@@ -1041,7 +1332,7 @@ rows_stream_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ Si
   }
   if (tid == 0) sample.top_key = sample.u_bits = 0u;
   if (threadIdx.x == 0) {
-    st.n_redo = 0;
+    st.n_redo = st.n_again = 0;
     st.abort = 0;
   }
   fence_barrier_init();
@@ -1112,30 +1403,9 @@ rows_stream_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ Si
   const int seg0 = warp * cfg.seg_len;
   const int seg_n = min(max(a.V - seg0, 0), cfg.seg_len);  // ids of this warp's segment
   const int units = (seg_n + EU - 1) / EU;
-  // Copies go through the ring of the warp's segment in order: the units of the segment for row 0, row 1, ...; team t takes
-  // rows t, t + teams, ...  Whoever has worked a unit through asks for the copy that goes into its slot next.
-  // Logits that exceed the L2 leave it first (they make room for samples and outputs: 1,024 rows of 65,536 74.4 -> 73.4 us);
-  // smaller ones are left where their writer put them (of 16,384: 45.7, with the hint 46.6).
-  uint64_t policy;
-  if (cfg.once) asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
-  else asm("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(policy));
+  const uint64_t policy = ring_policy(cfg);
   auto issue = [&](int k, int unit, int slot) {
-    while (unit >= units) {
-      ++k;
-      unit -= units;
-    }
-    if (k >= n_live) return;
-    const uint32_t bytes = (uint32_t)min(seg_n - unit * EU, EU) * ES;
-    const int64_t off = st.tab[k].off + seg0 + (int64_t)unit * EU;
-    unsigned char* const dst = ring + (size_t)slot * kSlot;
-#ifdef SJD_TEST_DROP_COPY
-    if (warp == SJD_TEST_DROP_COPY && k == 1 && unit == 0) return;  // test builds only, see rows_cluster_kernel
-#endif
-    const int x = (warp * kMaxTeams + k % teams) * kMaxSlots + slot;
-    ++st.used[x];
-    mbar_arrive_expect_tx(&st.full[x], bytes * (HAS_U ? 2u : 1u));
-    bulk_g2s_hinted(dst, row_ptr(a.cond, DTYPE, off), bytes, &st.full[x], policy);
-    if (HAS_U) bulk_g2s_hinted(dst + kUnitBytes, row_ptr(a.uncond, DTYPE, off), bytes, &st.full[x], policy);
+    issue_unit<DTYPE, HAS_U>(a, st, ring, policy, warp, teams, units, seg0, seg_n, EU, n_live, k, unit, slot);
   };
   // The team's first row: its sample's maxima, for the sampler.  Everybody waits for the CTA's first threshold, so the other
   // teams' samples and the first copies (which the second team sends off) come behind the first team's sample.  (Nothing but
@@ -1161,7 +1431,8 @@ rows_stream_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ Si
   to.y_at = smem_u32(list_y + warp * cfg.seg_cap);
   to.id_at = to.scratch_at = smem_u32(list_id + warp * cfg.seg_cap);
   to.hist_at = smem_u32(&sm.hist);
-  const uint32_t ring_at = smem_u32(ring), cap = (uint32_t)cfg.seg_cap;
+  to.cap = (uint32_t)cfg.seg_cap;
+  const uint32_t ring_at = smem_u32(ring);
   uint64_t* const full = st.full + (warp * kMaxTeams + team) * kMaxSlots;
   uint32_t phase = 0;      // bit s: parity of the next phase of full[s]
   int tau_at = 0;          // thresholds come through two places in turn
@@ -1186,8 +1457,8 @@ rows_stream_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ Si
       if (!ok) break;
       phase ^= 1u << slot;
       const uint32_t c_unit = ring_at + (uint32_t)slot * kSlot;
-      sift_unit<DTYPE, HAS_U, HAS_T, false>(a, c_unit, c_unit + kUnitBytes, seg_n - unit * EU, (uint32_t)(unit * EU), 0u, s2, t2, bins,
-                                            screen, to, cap, lane, n, vmax);
+      sift_unit<DTYPE, HAS_U, HAS_T, false, false>(a, c_unit, c_unit + kUnitBytes, seg_n - unit * EU, (uint32_t)(unit * EU), 0u, s2, t2,
+                                                   bins, screen, to, lane, n, vmax);
       __syncwarp();
       if (lane == 0) issue(k, unit + slots, slot);
       if (++slot == slots) slot = 0;
@@ -1196,21 +1467,25 @@ rows_stream_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ Si
     if (lane == 0) {
       st.seg_n[team * kTeamWarps + warp] = n;
       atomicMax(&sm.max_key, wmax);
-      if (n > cap || !ok) sm.over = 1u;
+      if (n > to.cap || !ok) sm.over = 1u;
       if (!ok) *abort_flag = 1;
     }
     const SiftRow& r = st.tab[k];
-    if (!finish_row<kTeamWarps>(a, cfg, sm, list_y, list_id, st.seg_n + team * kTeamWarps, 1, bins, r.row, r.pos, r.iter, r.draft, tid, bar) &&
-        tid == 0) {
+    const int result = finish_row<kTeamWarps, false>(a, cfg, sm, list_y, list_id, st.seg_n + team * kTeamWarps, 1, SiftRuns{}, bins, r.row, r.pos,
+                                                     r.iter, r.draft, 0, tid, bar);
+    if (result != kRowDone && tid == 0) {
       if (*abort_flag != 0) {
         a.out_cnt[r.row] = 0;
         a.scratch[r.row] = RowScratch{0.0f, -1, 0.0f, kRowStatusTimeout};
       } else {
-        st.redo[atomicAdd(&st.n_redo, 1)] = r.row;
+        SiftTau raised{0.0f, 0.0f, __int_as_float(0x7f800000)};  // (|uncond| not known any more: compared exactly)
+        if (result == kRowOver && raise_threshold(sm, bins, cfg.pool - (a.V + EU - 1) / EU, raised)) sift_again(a, st, k, raised);
+        else st.redo[atomicAdd(&st.n_redo, 1)] = r.row;
       }
     }
   }
   __syncthreads();
+  if (st.n_again != 0) phase = stream_again<DTYPE, HAS_U, HAS_T>(a, cfg, smem_raw, phase);
   if (st.abort != 0 && lane == 0) {
     // a wait gave up: the copies in flight have to land (the wait is bounded) before the CTA may go
     for (int s = 0; s < slots; ++s) {
@@ -1238,12 +1513,14 @@ struct alignas(16) ClusterShared {
   uint64_t full[kClusterWarps];                  // a warp's segment has landed
   uint32_t seg_n[kClusterWarps * kMaxCluster];   // candidates per segment (the first CTA's)
   uint32_t lost;                                 // a bounded wait of the cluster gave up (the first CTA's)
+  uint32_t again;                                // a list of the cluster ran over (in every CTA)
+  uint32_t go;                                   // a row that crowds is sifted once more, with `next` (the first CTA's)
+  SiftTau next;
 };
-// shared memory: ClusterShared | list values | list ids | local ids | cond | uncond.  Only the cluster's first CTA uses the
-// lists (one per segment of the row).
+// shared memory: ClusterShared | list values | list ids | the warps' own ids | cond | uncond.  Only the cluster's first CTA uses the
+// lists (one per segment of the row, or one for the whole row, see rows_stream_kernel).
 __host__ __device__ inline size_t sift_cluster_lists(const SiftCfg& cfg, int n_cta) {
-  const size_t segs = (size_t)kClusterWarps * n_cta;
-  const size_t b = sizeof(ClusterShared) + segs * cfg.seg_cap * 6 + (n_cta > 1 ? (size_t)kClusterWarps * cfg.seg_cap * 2 : 0);
+  const size_t b = sizeof(ClusterShared) + (size_t)cfg.pool * 6 + (n_cta > 1 ? (size_t)kClusterWarps * cfg.scratch * 2 : 0);
   return (b + 127) & ~(size_t)127;
 }
 __host__ __device__ inline size_t sift_cluster_stage(const SiftCfg& cfg, int elem_bytes) {  // one array of one segment
@@ -1272,6 +1549,74 @@ __device__ __forceinline__ uint32_t in_first_cta(const void* p) {
   return at;
 }
 
+// what a warp of the cluster has to say about its segment, to the first CTA (by one lane)
+__device__ __forceinline__ void tell_first_cta(ClusterShared& sm, uint32_t max_key, bool over, bool lost) {
+  asm volatile("red.relaxed.cluster.shared::cluster.max.u32 [%0], %1;" ::"r"(in_first_cta(&sm.row.max_key)), "r"(max_key) : "memory");
+  if (over) asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(in_first_cta(&sm.row.over)), "r"(1u) : "memory");
+  if (lost) asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(in_first_cta(&sm.lost)), "r"(1u) : "memory");
+}
+
+// A row that crowds, by the whole cluster: sifted once more out of shared memory, with the first CTA's `next` threshold and one
+// list for the row.  ok: the warp's segment has landed.  Returns the first CTA's result (kRowElse to the others).
+template <int DTYPE, bool HAS_U, bool HAS_T>
+__device__ __noinline__ int cluster_crowded_row(const RowArgs& a, const SiftCfg& cfg, unsigned char* smem, int row, bool ok) {
+  constexpr int ES = SiftTraits<DTYPE>::kElem, EU = SiftTraits<DTYPE>::kUnit;
+  ClusterShared& sm = *reinterpret_cast<ClusterShared*>(smem);
+  const uint32_t crank = cluster_rank(), csize = cluster_size();
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  float* const list_y = reinterpret_cast<float*>(smem + sizeof(ClusterShared));
+  uint16_t* const list_id = reinterpret_cast<uint16_t*>(list_y + cfg.pool);
+  const int room = cfg.pool - kClusterWarps * (int)csize * cfg.units;
+  const SiftRuns runs{reinterpret_cast<uint32_t*>(list_y + room), kClusterWarps * (int)csize * cfg.units, cfg.units, cfg.seg_len, EU};
+  const size_t stage_bytes = sift_cluster_stage(cfg, ES);
+  const uint32_t c_at = smem_u32(smem + sift_cluster_lists(cfg, (int)csize) + (size_t)warp * stage_bytes * (HAS_U ? 2 : 1));
+  const int seg = (int)crank * kClusterWarps + warp;
+  const int seg_n = min(max(a.V - seg * cfg.seg_len, 0), cfg.seg_len), units = (seg_n + EU - 1) / EU;
+  const uint64_t s2 = pack2(a.s, a.s), t2 = pack2(a.inv_T, a.inv_T);
+  // whether, and with which threshold, from the first CTA, which stays until everybody knows
+  uint32_t go, word[3];
+  asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(go) : "r"(in_first_cta(&sm.go)) : "memory");
+#pragma unroll
+  for (int k = 0; k < 3; ++k)
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(word[k]) : "r"(in_first_cta(&sm.next) + 4u * k) : "memory");
+  __syncwarp();
+  cluster_arrive();
+  cluster_wait();
+  if (go == 0u) return kRowElse;
+  const SiftTau tau{__uint_as_float(word[0]), __uint_as_float(word[1]), __uint_as_float(word[2])};
+  const SiftBinning bins = sift_bins(tau.tau0, tau.top);
+  const SiftScreen screen = sift_screen<DTYPE, HAS_U, HAS_T>(a, cfg, tau.tau0, tau.u_max);
+  SiftTarget to;
+  to.y_at = in_first_cta(list_y);
+  to.id_at = in_first_cta(list_id);
+  to.hist_at = in_first_cta(&sm.row.hist);
+  to.cap = (uint32_t)room;
+  to.taken_at = in_first_cta(&sm.row.taken);
+  to.scratch = csize > 1 ? (uint32_t)cfg.scratch : 0u;
+  to.scratch_at = smem_u32(csize > 1 ? list_id + cfg.pool + warp * cfg.scratch : list_id);
+  const uint32_t runs_at = in_first_cta(runs.run + seg * cfg.units);
+  float vmax = __int_as_float(0xff800000);
+  bool over = false;
+  for (int k = 0; k < cfg.units; ++k) {
+    uint32_t run = 0u;  // (segments at the row's end have fewer units)
+    if (ok && k < units)
+      sift_unit<DTYPE, HAS_U, HAS_T, true, true>(a, c_at + (uint32_t)k * kUnitBytes, c_at + (uint32_t)(stage_bytes + (size_t)k * kUnitBytes),
+                                                 seg_n - k * EU, 0u, 0u, s2, t2, bins, screen, to, lane, run, vmax);
+    over = over || run == kNoRoom;
+    if (lane == 0) asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(runs_at + 4u * k), "r"(run) : "memory");
+    __syncwarp();  // (the warp's own ids are listed again)
+  }
+  const uint32_t wmax = __reduce_max_sync(0xffffffffu, float_key(vmax));
+  if (lane == 0) tell_first_cta(sm, wmax, over, !ok);
+  __syncwarp();
+  cluster_arrive();
+  cluster_wait();
+  if (crank != 0 || sm.lost != 0u) return kRowElse;
+  const SiftRow r = sift_row(a, row);
+  return finish_row<kClusterWarps, true>(a, cfg, sm.row, list_y, list_id, nullptr, 0, runs, bins, row, r.pos, r.iter, r.draft, kRowStatusRedone,
+                                         tid, 0);
+}
+
 template <int DTYPE, bool HAS_U, bool HAS_T>
 __global__ void __launch_bounds__(kClusterWarps * 32, 1)
 rows_cluster_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ SiftCfg cfg) {
@@ -1282,8 +1627,8 @@ rows_cluster_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ S
   const uint32_t crank = cluster_rank(), csize = cluster_size();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   float* const list_y = reinterpret_cast<float*>(smem_raw + sizeof(ClusterShared));
-  uint16_t* const list_id = reinterpret_cast<uint16_t*>(list_y + kClusterWarps * csize * cfg.seg_cap);
-  uint16_t* const local_id = list_id + kClusterWarps * csize * cfg.seg_cap;
+  uint16_t* const list_id = reinterpret_cast<uint16_t*>(list_y + cfg.pool);
+  uint16_t* const local_id = list_id + cfg.pool;
   const size_t stage_bytes = sift_cluster_stage(cfg, ES);
   unsigned char* const stage = smem_raw + sift_cluster_lists(cfg, (int)csize) + (size_t)warp * stage_bytes * (HAS_U ? 2 : 1);
   const int row = (int)(blockIdx.x / csize);
@@ -1291,7 +1636,7 @@ rows_cluster_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ S
   init_shared(sm.row, tid, NT);
   if (tid < kClusterWarps) mbar_init(&sm.full[tid], 1);
   if (tid == 0) {
-    sm.lost = 0u;
+    sm.lost = sm.again = 0u;
     sm.sample.top_key = sm.sample.u_bits = 0u;
   }
   fence_barrier_init();
@@ -1365,8 +1710,8 @@ rows_cluster_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ S
   to.y_at = in_first_cta(list_y + (size_t)seg * cfg.seg_cap);
   to.id_at = in_first_cta(list_id + (size_t)seg * cfg.seg_cap);
   to.hist_at = in_first_cta(&sm.row.hist);
-  to.scratch_at = smem_u32(csize > 1 ? local_id + (size_t)warp * cfg.seg_cap : list_id + (size_t)seg * cfg.seg_cap);
-  const uint32_t cap = (uint32_t)cfg.seg_cap;
+  to.scratch_at = smem_u32(csize > 1 ? local_id + (size_t)warp * cfg.scratch : list_id + (size_t)seg * cfg.seg_cap);
+  to.cap = (uint32_t)cfg.seg_cap;
   const uint32_t bias = (uint32_t)((seg % (int)csize) * cfg.seg_len);  // ids are kept relative to the finishing warp's first one
   uint32_t n = 0;
   float vmax = __int_as_float(0xff800000);
@@ -1375,23 +1720,43 @@ rows_cluster_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ S
   if (ok) {
     const uint32_t c_at = smem_u32(stage), u_at = smem_u32(u_stage);
     for (int k = 0; k < units; ++k)
-      sift_unit<DTYPE, HAS_U, HAS_T, true>(a, c_at + (uint32_t)k * kUnitBytes, u_at + (uint32_t)k * kUnitBytes, seg_n - k * EU,
-                                           (uint32_t)(k * EU), bias, s2, t2, bins, screen, to, cap, lane, n, vmax);
+      sift_unit<DTYPE, HAS_U, HAS_T, true, false>(a, c_at + (uint32_t)k * kUnitBytes, u_at + (uint32_t)k * kUnitBytes, seg_n - k * EU,
+                                                  (uint32_t)(k * EU), bias, s2, t2, bins, screen, to, lane, n, vmax);
   }
   __syncwarp();
   const uint32_t wmax = __reduce_max_sync(0xffffffffu, float_key(vmax));
   if (lane == 0) {
-    const uint32_t n_at = in_first_cta(&sm.seg_n[seg]), max_at = in_first_cta(&sm.row.max_key);
-    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(n_at), "r"(n) : "memory");
-    asm volatile("red.relaxed.cluster.shared::cluster.max.u32 [%0], %1;" ::"r"(max_at), "r"(wmax) : "memory");
-    if (n > cap) asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(in_first_cta(&sm.row.over)), "r"(1u) : "memory");
-    if (!ok) asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(in_first_cta(&sm.lost)), "r"(1u) : "memory");
+    const bool over = n > to.cap;
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(in_first_cta(&sm.seg_n[seg])), "r"(n) : "memory");
+    tell_first_cta(sm, wmax, over, !ok);
+    for (uint32_t c = 0; over && c < csize; ++c) {  // every CTA has to know
+      uint32_t at;
+      asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"(smem_u32(&sm.again)), "r"(c));
+      asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(at), "r"(1u) : "memory");
+    }
   }
   if (!ok && copied) mbar_wait(&sm.full[warp], 0u);  // bounded: no copy of this CTA outlives it
   __syncwarp();
   cluster_arrive();
   cluster_wait();
-  if (crank != 0) return;
+  const bool again = sm.again != 0u;  // (the same in every CTA)
+  if (crank != 0 && !again) return;
+  int result = kRowElse;
+  if (crank == 0 && sm.lost == 0u)
+    result = finish_row<kClusterWarps, false>(a, cfg, sm.row, list_y, list_id, sm.seg_n, (int)csize, SiftRuns{}, bins, row, r.pos, r.iter, r.draft,
+                                              0, tid, 0);
+  if (again) {
+    if (crank == 0 && tid == 0) {
+      SiftTau next = tau;
+      sm.go = result == kRowOver && raise_threshold(sm.row, bins, cfg.pool - kClusterWarps * (int)csize * cfg.units, next) ? 1u : 0u;
+      sm.next = next;
+    }
+    __syncwarp();
+    cluster_arrive();  // (the first CTA has reset what the others count in)
+    cluster_wait();
+    result = cluster_crowded_row<DTYPE, HAS_U, HAS_T>(a, cfg, smem_raw, row, ok);
+    if (crank != 0) return;
+  }
   if (sm.lost != 0u) {
     if (tid == 0) {
       a.out_cnt[row] = 0;
@@ -1399,8 +1764,7 @@ rows_cluster_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ S
     }
     return;
   }
-  if (!finish_row<kClusterWarps>(a, cfg, sm.row, list_y, list_id, sm.seg_n, (int)csize, bins, row, r.pos, r.iter, r.draft, tid, 0))
-    sift_redo<DTYPE, NT, 0>(a, row, tid, *reinterpret_cast<GenericSmem*>(&sm.sample));
+  if (result != kRowDone) sift_redo<DTYPE, NT, 0>(a, row, tid, *reinterpret_cast<GenericSmem*>(&sm.sample));
 }
 
 }  // namespace sjd

@@ -190,18 +190,23 @@ struct SiftPlan {
 };
 
 // Segments of equal length, each with a list that holds its share of the candidates with four standard deviations of
-// the threshold's estimate and four of the segment's own count to spare.
-// Packed screening lets some more pass.
-void cut_segments(sjd::SiftCfg* c, int V, int segs, double p, double sd, double more) {
+// the threshold's estimate and four of the segment's own count to spare.  Packed screening lets some more pass.  Together the
+// lists also hold what a row that crowds needs: the entries a second threshold leaves, and a word per unit.  False where they would
+// be too long for 16-bit positions.
+bool cut_segments(sjd::SiftCfg* c, int V, int kcap, int segs, int unit, double p, double sd, double more) {
   c->seg_len = (((V + segs - 1) / segs) + 7) & ~7;
+  c->units = (c->seg_len + unit - 1) / unit;
   const double mean = c->seg_len * (p + 4.0 * sd) * more;
   int cap = (int)(mean + 4.0 * std::sqrt(mean) + 8.0);
   if (cap > c->seg_len) cap = c->seg_len;
   c->seg_cap = (cap + 7) & ~7;
+  const int crowded = (kcap + 128 + segs * c->units + 7) & ~7;
+  c->pool = c->seg_cap * segs > crowded ? c->seg_cap * segs : crowded;
+  return c->pool <= 65528;
 }
 
 bool plan_sift(const sjd_params* P, int kcap, bool has_u, SiftPlan* plan) {
-  const int V = P->V, es = P->logits_dtype == SJD_F32 ? 4 : 2, ev = 16 / es;
+  const int V = P->V, es = P->logits_dtype == SJD_F32 ? 4 : 2, ev = 16 / es, unit = sjd::kUnitBytes / es;
   if (V < 2048 || V > 65536 * sjd::kTeamWarps) return false;
   sjd::SiftCfg& c = plan->cfg;
   std::memset(&c, 0, sizeof(c));
@@ -252,19 +257,30 @@ bool plan_sift(const sjd_params* P, int kcap, bool has_u, SiftPlan* plan) {
   // 18.1; of 65,536 fp32: -, -, 16.7, 31.9, 21.3 (32 rows: 18.8 with four; 36 rows: 25.0, two rounds of clusters, and 21.8).
   for (int n_cta = 1; n_cta <= sjd::kMaxCluster; n_cta <<= 1) {
     if (rows * n_cta > (n_cta <= 2 ? sms : n_cta == 4 ? sms * 7 / 8 : sms / 2)) break;
-    cut_segments(&c, V, sjd::kClusterWarps * n_cta, p, sd, more);
+    if (!cut_segments(&c, V, kcap, sjd::kClusterWarps * n_cta, unit, p, sd, more) || (int64_t)n_cta * c.seg_len > 65536) continue;
+    c.scratch = c.seg_cap;
     plan->cluster = n_cta;
     plan->smem = sjd::sift_cluster_smem(c, n_cta, es, has_u);
-    if (plan->smem <= kSmemLimit && (int64_t)n_cta * c.seg_len <= 65536) return true;
+    if (plan->smem > kSmemLimit) continue;
+    // A row that crowds lists the ids of a unit apart from the row's list: room for all of a unit's, as long as the verification's
+    // blocks still find room beside this kernel's.
+    const size_t beside = 36u << 10;
+    const int most = c.seg_len < unit ? c.seg_len : unit;
+    if (n_cta > 1 && most > c.scratch && plan->smem + beside < kSmemLimit) {
+      const int room = c.scratch + (int)((kSmemLimit - beside - plan->smem) / (2 * sjd::kClusterWarps));
+      c.scratch = (room < most ? room : most) & ~7;
+      plan->smem = sjd::sift_cluster_smem(c, n_cta, es, has_u);
+    }
+    return true;
   }
-  cut_segments(&c, V, sjd::kTeamWarps, p, sd, more);
+  if (!cut_segments(&c, V, kcap, sjd::kTeamWarps, unit, p, sd, more)) return false;
   c.once = rows * V * es * (has_u ? 2 : 1) > (96ll << 20) ? 1 : 0;
   plan->cluster = 0;
   static const int choices[][2] = {{3, 4}, {3, 3}, {3, 2}, {2, 2}, {2, 1}, {1, 2}, {1, 1}};
   for (const auto& ch : choices) {
     c.teams = ch[0];
     c.slots = ch[1];
-    plan->smem = sjd::sift_stream_smem(c.teams, c.seg_cap, c.slots, has_u);
+    plan->smem = sjd::sift_stream_smem(c, has_u);
     if (plan->smem <= kSmemLimit) return true;
   }
   return false;

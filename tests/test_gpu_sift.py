@@ -186,3 +186,23 @@ def test_a_sequence_alone_gives_the_same_bits(V, K, dtype, B, W, temperature):
     alone = gpu_step(one(inp.cond), one(inp.uncond), one(prev.tokens), q, **kw)
     for name in ("accept_len", "tokens", "tok_prob", "ids", "vals", "cnt", "flags", "status"):
         assert getattr(alone, name).tobytes() == getattr(batch, name)[:1].tobytes(), name
+
+
+# One CTA per row, clusters of two and four, many rows; more candidates than the lists hold and fewer; blocks at the row's ends;
+# several rows to a CTA, some of them ordinary.
+@pytest.mark.parametrize("V,K,dtype,B,W", [(16384, 500, wk.BF16, 1, 3), (65536, 2000, wk.BF16, 1, 4), (65536, 300, wk.F32, 1, 3),
+                                           (65536, 100, wk.F16, 2, 77), (65536, 2000, wk.BF16, 2, 80), (5000, 300, wk.BF16, 3, 110),
+                                           (16384, 1000, wk.F32, 2, 90), (50264, 5000, wk.F16, 2, 75), (2056, 64, wk.F32, 4, 100)])
+@pytest.mark.parametrize("where", ["start", "middle", "end"])
+def test_top_k_in_one_block_of_ids(V, K, dtype, B, W, where):
+    from gpu_harness import check_parity, oracle_prime, step_kwargs
+    wl = wk.CONFIGS["cfg2"].scaled(B=B, W=W, V=V, dtype=dtype, top_k=K, seed=V + W, peaks=0)
+    inp = wk.make_step_inputs(wl)
+    n = max(V // 8, K + K // 2)
+    begin = {"start": 0, "middle": (V - n) // 3, "end": V - n}[where]
+    for arr in (inp.cond, inp.uncond, inp.prev_cond, inp.prev_uncond):
+        f = wk._as_f32(arr, dtype).copy()
+        f[:, : W - W // 3, begin:begin + n] += 12.0  # (the last third of the rows is ordinary)
+        arr[:] = wk._store(f, dtype)
+    prev = oracle_prime(inp)
+    check_parity(inp.cond, inp.uncond, prev.tokens, prev.probs, step_kwargs(inp), inp.win_len)
