@@ -490,12 +490,17 @@ struct SiftMaxima {
 struct SiftTau {
   float tau0, top, u_max;
 };
-__device__ __forceinline__ SiftTau sift_tau(uint32_t key, const SiftSample& in) {
+// Below this value (a bf16 key: -8,192) a token counts as masked.  Where so much of a row is masked that the wanted rank lies among
+// the masked groups, the rest of the row is taken whole, so to speak: the threshold goes as far below the least unmasked
+// maximum as the largest lies above it, and the row comes again with the threshold that its histogram gives.
+constexpr uint32_t kMaskedKey = 0x39ffu;
+__device__ __forceinline__ SiftTau sift_tau(uint32_t key, bool whole, const SiftSample& in) {
   const uint32_t top_key = in.top_key;
   const float top = key_float(top_key), lowest = -3.402823466e38f;  // lowest: every finite value is a candidate
   // the maxima were rounded to nearest: the middle between this bf16 value and the one below is what they all reach
   const float at = key_float(key << 16), below = key_float((key - 1u) << 16);
   float tau0 = __fmaf_rd(__fsub_rn(at, below), -0.51f, at);
+  if (whole) tau0 = __fsub_rn(tau0, __fsub_rn(top, tau0));
   if (key == 0u || !(tau0 >= lowest) || !(top <= 3.402823466e38f)) tau0 = lowest;
   return SiftTau{tau0, top, __uint_as_float(in.u_bits)};
 }
@@ -503,11 +508,16 @@ __device__ __forceinline__ SiftTau sift_tau(uint32_t key, const SiftSample& in) 
 __device__ __forceinline__ SiftTau sift_threshold(const SiftSample& in, uint32_t rank, int lane) {
   SiftMaxima m;
   m.load(in, lane);
-  uint32_t key = 0;
+  uint32_t key;
+  for (bool whole = false;; whole = true) {
+    key = 0;
 #pragma unroll 1
-  for (uint32_t bit = 0x8000u; bit != 0u; bit >>= 1)
-    if (m.reaching(key | bit) >= rank) key |= bit;
-  return sift_tau(key, in);
+    for (uint32_t bit = 0x8000u; bit != 0u; bit >>= 1)
+      if (m.reaching(key | bit) >= rank) key |= bit;
+    if (key >= kMaskedKey || whole) return sift_tau(key, whole, in);
+    rank = m.reaching(kMaskedKey);
+    if (rank == 0u) return sift_tau(key, false, in);
+  }
 }
 
 // ---------------------------------------------------------------------------------------------------
@@ -1688,22 +1698,30 @@ rows_cluster_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ S
   sift_sample<DTYPE, HAS_U, HAS_T, NT>(a, cfg, sm.sample, c_row, u_row, tid);
   __syncthreads();
   // the search four bits at a time: warp w counts for the digit w, the largest digit that is reached enough is taken
-  uint32_t key = 0;
+  uint32_t key;
+  bool whole = false;
   {
     static_assert(kClusterWarps == 16, "a warp per digit");
     SiftMaxima m;
     m.load(sm.sample, lane);
+    for (uint32_t rank = (uint32_t)cfg.rank;;) {
+      key = 0;
 #pragma unroll 1
-    for (int shift = 12; shift >= 0; shift -= 4) {
-      const uint32_t mine = key | ((uint32_t)warp << shift);
-      const bool reached = warp == 0 || m.reaching(mine) >= (uint32_t)cfg.rank;
-      if (lane == 0) sm.key[warp] = reached ? mine : 0u;
-      __syncthreads();
-      key = __reduce_max_sync(0xffffffffu, sm.key[lane & 15]);
-      __syncthreads();
+      for (int shift = 12; shift >= 0; shift -= 4) {
+        const uint32_t mine = key | ((uint32_t)warp << shift);
+        const bool reached = warp == 0 || m.reaching(mine) >= rank;
+        if (lane == 0) sm.key[warp] = reached ? mine : 0u;
+        __syncthreads();
+        key = __reduce_max_sync(0xffffffffu, sm.key[lane & 15]);
+        __syncthreads();
+      }
+      if (key >= kMaskedKey || whole) break;
+      rank = m.reaching(kMaskedKey);  // (the same in every warp)
+      if (rank == 0u) break;
+      whole = true;
     }
   }
-  const SiftTau tau = sift_tau(key, sm.sample);
+  const SiftTau tau = sift_tau(key, whole, sm.sample);
   const SiftBinning bins = sift_bins(tau.tau0, tau.top);
   const SiftScreen screen = sift_screen<DTYPE, HAS_U, HAS_T>(a, cfg, tau.tau0, tau.u_max);
   SiftTarget to;

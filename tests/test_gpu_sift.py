@@ -206,3 +206,20 @@ def test_top_k_in_one_block_of_ids(V, K, dtype, B, W, where):
         arr[:] = wk._store(f, dtype)
     prev = oracle_prime(inp)
     check_parity(inp.cond, inp.uncond, prev.tokens, prev.probs, step_kwargs(inp), inp.win_len)
+
+
+@pytest.mark.parametrize("lowest", [-np.inf, -65504.0])
+@pytest.mark.parametrize("V,K,dtype,B,W,left", [(16384, 500, wk.BF16, 1, 3, 2048), (65536, 2000, wk.BF16, 1, 4, 8192), (65536, 2000, wk.BF16, 2, 80, 8192),
+                                                (65536, 100, wk.F16, 2, 77, 8192), (50264, 500, wk.BF16, 2, 75, 6000), (16384, 1000, wk.F32, 2, 90, 1500),
+                                                (8192, 300, wk.F32, 2, 90, 290)])
+def test_all_but_a_block_masked(V, K, dtype, B, W, left, lowest):
+    # image tokens only: fewer of the sample's groups are unmasked than the threshold's rank; the last shape has fewer tokens than K left
+    from gpu_harness import check_parity, oracle_prime, step_kwargs
+    wl = wk.CONFIGS["cfg2"].scaled(B=B, W=W, V=V, dtype=dtype, top_k=K, seed=V + W, peaks=0)
+    inp = wk.make_step_inputs(wl)
+    out = np.ones(V, bool)
+    out[V // 5:V // 5 + left] = False
+    for arr in (inp.cond, inp.uncond, inp.prev_cond, inp.prev_uncond):
+        arr[:, :, out] = wk._store(np.full(1, lowest, np.float32), dtype)[0]
+    prev = oracle_prime(inp)
+    check_parity(inp.cond, inp.uncond, prev.tokens, prev.probs, step_kwargs(inp), inp.win_len)
