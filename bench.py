@@ -309,10 +309,10 @@ def run_ours(args):
     if rank == 0 and world == 1 and not args.no_cpu_baseline:
         cpu, parity = run_cpu_baseline(wl, sets[0])
 
-    # status words of the last step of every input set: sequences with a row the single-pass kernel handed to
-    # the any-shape path (exact, but many times slower), and the selected row kernel
+    # status words of the last step of every input set: sequences with a row that did not fit the row kernel's lists and
+    # was done again (exact, but slower), and the selected row kernel
     redone = sum(int(((d.status & 16) != 0).sum().item()) for d in sets)
-    row_kernel = ["generic", "tiles", "ranges"][sjd.sjd_row_kernel(sets[0].params)]
+    row_kernel = ["any_shape", "tiles", "stream", "cluster"][sjd.sjd_row_path(sets[0].params, sets[0].uncond is not None)]
     if rank == 0:
         line = {"metric": METRIC, "value": round(value, 1), "unit": UNIT, "n_gpus": world, "steps": K, "warmup": Wm,
                 "ms_per_step": round(ms_per_step, 5), "higher_is_better": True, "scaling": "weak",
@@ -333,7 +333,7 @@ def run_ours(args):
 # the capture is summarised under profiles/.  None = not captured yet.
 NCU_TRAFFIC_BYTES = {"cfg4": 273_000_000}
 NCU_TRAFFIC_SOURCE = ("stored figure, not measured by this run: dram__bytes_read.sum + dram__bytes_write.sum of one launch, "
-                      "from the ncu capture summarised in profiles/rows_stream_cfg4.md")
+                      "from an ncu capture of the row kernel on this workload")
 
 
 def run_e2e(sjd, wl, dset, device, n, world, tokens_per_step, barrier):

@@ -156,15 +156,26 @@ uint64_t sjd_launch_count(void);
 size_t sjd_workspace_bytes(const sjd_params* params);
 
 /*
- * Which row kernel sjd_step() selects for this shape and these flags (Section 3.1's sampling head has three
- * implementations that give identical results): SJD_ROWS_RANGES, SJD_ROWS_TILES or SJD_ROWS_GENERIC, or a
- * negative SJD_ERR_* for a shape, dtype or strides sjd_step() would refuse (pointers and the workspace are not
+ * Which row kernel sjd_step() takes for this shape and these flags, with logits_uncond (guidance != 0) or without (Section 3.1's
+ * sampling head has several implementations: the same ids, tokens and counts, probabilities that agree to rounding;
+ * SJD_PATH_STREAM and SJD_PATH_CLUSTER, which share their rows by the number of rows in the call, give the same bits), or
+ * a negative SJD_ERR_* for a shape, dtype or strides sjd_step() would refuse (pointers and the workspace are not
  * looked at).  Decided from the shape alone.  Launches nothing.
  */
-#define SJD_ROWS_GENERIC 0 /* any shape: several passes over a row in global memory (kcap > 2,048: one pass where V and
-                              K allow it)                                                                    */
-#define SJD_ROWS_TILES 1   /* V a multiple of 2,048: one pass, tiles dealt to the filter warps               */
-#define SJD_ROWS_RANGES 2  /* V >= 2,048, kcap <= 2,048 and a modest share of V: one pass, one id range per warp */
+#define SJD_PATH_ANY_SHAPE 0 /* several passes over a row in global memory: V < 2,048, V > 524,288 or K more than about half of V,
+                                and SJD_FLAG_FORCE_GENERIC                                                        */
+#define SJD_PATH_TILES 1     /* SJD_FLAG_FORCE_TILES only: one pass, tiles dealt to the filter warps                */
+#define SJD_PATH_STREAM 2    /* one pass, rows sifted by a sampled threshold, many rows to a block                  */
+#define SJD_PATH_CLUSTER 3   /* the same for few rows: a cluster of blocks for each                                 */
+int sjd_row_path(const sjd_params* params, int guidance);
+
+/*
+ * The same in an older, coarser division, with guidance: SJD_ROWS_GENERIC for every kcap > 2,048, whichever kernel takes it,
+ * else SJD_ROWS_RANGES for both SJD_PATH_STREAM and SJD_PATH_CLUSTER.
+ */
+#define SJD_ROWS_GENERIC 0
+#define SJD_ROWS_TILES 1
+#define SJD_ROWS_RANGES 2
 int sjd_row_kernel(const sjd_params* params);
 
 /*

@@ -85,6 +85,8 @@ def lib() -> C.CDLL:
         L.sjd_workspace_bytes.restype = C.c_size_t
         L.sjd_row_kernel.argtypes = [C.POINTER(sjd_params)]
         L.sjd_row_kernel.restype = C.c_int
+        L.sjd_row_path.argtypes = [C.POINTER(sjd_params), C.c_int]
+        L.sjd_row_path.restype = C.c_int
         L.sjd_step.argtypes = [C.c_void_p, C.c_void_p, C.c_void_p, C.POINTER(sjd_probs), C.POINTER(sjd_params),
                                C.c_uint64, C.c_void_p, C.c_void_p, C.POINTER(sjd_probs)]
         L.sjd_step.restype = C.c_int
@@ -159,10 +161,19 @@ def _opt_ptr(t: Optional[torch.Tensor], dtype=_i32) -> Optional[int]:
 
 
 SJD_ROWS_GENERIC, SJD_ROWS_TILES, SJD_ROWS_RANGES = 0, 1, 2
+SJD_PATH_ANY_SHAPE, SJD_PATH_TILES, SJD_PATH_STREAM, SJD_PATH_CLUSTER = 0, 1, 2, 3
+
+
+def sjd_row_path(params: "sjd_params", guidance: bool = True) -> int:
+    """Which row kernel sjd_step() takes for these parameters, with or without unconditional logits (SJD_PATH_*)."""
+    code = lib().sjd_row_path(C.byref(params), int(guidance))
+    if code < 0:
+        _check(code)
+    return code
 
 
 def sjd_row_kernel(params: "sjd_params") -> int:
-    """Which row kernel sjd_step() takes for these parameters (SJD_ROWS_*)."""
+    """The same in the older, coarser division (SJD_ROWS_*): SJD_ROWS_GENERIC for every top_k above 2,048."""
     code = lib().sjd_row_kernel(C.byref(params))
     if code < 0:
         _check(code)

@@ -286,6 +286,23 @@ bool plan_sift(const sjd_params* P, int kcap, bool has_u, SiftPlan* plan) {
   return false;
 }
 
+// Which row kernel a step takes, and how.  The tile-dealing one is only there for SJD_FLAG_FORCE_TILES: what plan_sift() refuses,
+// plan_pipeline() refuses as well.
+struct RowPlan {
+  int path;  // SJD_PATH_*
+  SiftPlan sift;
+  sjd::PipeCfg tiles;
+  size_t tiles_smem;
+};
+void plan_rows(const sjd_params* P, int kcap, bool has_u, RowPlan* plan) {
+  plan->path = SJD_PATH_ANY_SHAPE;
+  if (P->flags & SJD_FLAG_FORCE_GENERIC) return;
+  if (!(P->flags & SJD_FLAG_FORCE_TILES) && plan_sift(P, kcap, has_u, &plan->sift))
+    plan->path = plan->sift.cluster > 0 ? SJD_PATH_CLUSTER : SJD_PATH_STREAM;
+  else if (plan_pipeline(P, kcap, &plan->tiles, &plan->tiles_smem))
+    plan->path = SJD_PATH_TILES;
+}
+
 template <int DTYPE, bool HAS_U, bool HAS_T>
 cudaError_t launch_sift_as(const sjd::RowArgs& ra, const SiftPlan& plan, cudaStream_t st) {
   const int rows = ra.B * ra.W;
@@ -439,20 +456,18 @@ int sjd_step(const void* logits_cond, const void* logits_uncond, const int32_t* 
     if (e != cudaSuccess) return cuda_fail(e, "event record");
   }
   {
-    sjd::PipeCfg cfg;
-    SiftPlan splan;
-    size_t smem = 0;
+    RowPlan plan;
     cudaError_t e;
-    const bool fast = !(P->flags & (SJD_FLAG_FORCE_GENERIC | SJD_FLAG_FORCE_TILES));
-    if (fast && plan_sift(P, kcap, logits_uncond != nullptr, &splan)) {
-      e = P->logits_dtype == SJD_BF16  ? launch_sift<1>(ra, splan, stream)
-          : P->logits_dtype == SJD_F16 ? launch_sift<2>(ra, splan, stream)
-                                       : launch_sift<0>(ra, splan, stream);
-    } else if (!(P->flags & SJD_FLAG_FORCE_GENERIC) && plan_pipeline(P, kcap, &cfg, &smem)) {
+    plan_rows(P, kcap, logits_uncond != nullptr, &plan);
+    if (plan.path == SJD_PATH_STREAM || plan.path == SJD_PATH_CLUSTER) {
+      e = P->logits_dtype == SJD_BF16  ? launch_sift<1>(ra, plan.sift, stream)
+          : P->logits_dtype == SJD_F16 ? launch_sift<2>(ra, plan.sift, stream)
+                                       : launch_sift<0>(ra, plan.sift, stream);
+    } else if (plan.path == SJD_PATH_TILES) {
       const int grid = rows < sm_count() ? rows : sm_count();
-      e = P->logits_dtype == SJD_BF16  ? launch_pipeline<1>(ra, cfg, smem, grid, stream)
-          : P->logits_dtype == SJD_F16 ? launch_pipeline<2>(ra, cfg, smem, grid, stream)
-                                       : launch_pipeline<0>(ra, cfg, smem, grid, stream);
+      e = P->logits_dtype == SJD_BF16  ? launch_pipeline<1>(ra, plan.tiles, plan.tiles_smem, grid, stream)
+          : P->logits_dtype == SJD_F16 ? launch_pipeline<2>(ra, plan.tiles, plan.tiles_smem, grid, stream)
+                                       : launch_pipeline<0>(ra, plan.tiles, plan.tiles_smem, grid, stream);
     } else {
       const int grid = rows < 4 * sm_count() ? rows : 4 * sm_count();
       e = P->logits_dtype == SJD_BF16
@@ -554,7 +569,7 @@ int fill_advance(sjd::AdvanceArgs* a, const sjd_params* P, int32_t n_total, uint
 
 extern "C" {
 
-int sjd_row_kernel(const sjd_params* P) {
+int sjd_row_path(const sjd_params* P, int guidance) {
   if (!P) return SJD_ERR_NULL;
   if (P->struct_size != (int32_t)sizeof(sjd_params)) return SJD_ERR_STRUCT;
   if (P->B < 0 || P->W < 1 || P->W > SJD_W_MAX || P->V < 8 || (P->V % 8) != 0 || P->top_k < 1) return SJD_ERR_SHAPE;
@@ -562,14 +577,15 @@ int sjd_row_kernel(const sjd_params* P) {
   const int64_t esize = P->logits_dtype == SJD_F32 ? 4 : 2;
   if ((P->stride_b * esize) % 16 != 0 || (P->stride_w * esize) % 16 != 0 || P->stride_w < P->V || P->stride_b < 0)
     return SJD_ERR_ALIGN;
-  const int kcap = P->top_k < P->V ? P->top_k : P->V;
-  sjd::PipeCfg cfg;
-  SiftPlan splan;
-  size_t smem = 0;
-  const bool fast = !(P->flags & (SJD_FLAG_FORCE_GENERIC | SJD_FLAG_FORCE_TILES));
-  if (fast && plan_sift(P, kcap, true, &splan)) return kcap <= sjd::kKcapMax ? SJD_ROWS_RANGES : SJD_ROWS_GENERIC;
-  if (!(P->flags & SJD_FLAG_FORCE_GENERIC) && plan_pipeline(P, kcap, &cfg, &smem)) return SJD_ROWS_TILES;
-  return SJD_ROWS_GENERIC;
+  RowPlan plan;
+  plan_rows(P, P->top_k < P->V ? P->top_k : P->V, guidance != 0, &plan);
+  return plan.path;
+}
+
+int sjd_row_kernel(const sjd_params* P) {
+  const int path = sjd_row_path(P, 1);
+  if (path != SJD_PATH_STREAM && path != SJD_PATH_CLUSTER) return path;  // (the two names' values agree)
+  return (P->top_k < P->V ? P->top_k : P->V) <= sjd::kKcapMax ? SJD_ROWS_RANGES : SJD_ROWS_GENERIC;
 }
 
 int sjd_window_init(const sjd_params* P, int32_t n_total, uint64_t philox_seed, int32_t* win_len, int32_t* pos_base,
