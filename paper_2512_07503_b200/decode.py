@@ -52,7 +52,7 @@ class DecodeLoop:
         self.out = probs()
         self.committed = torch.full((batch, n_total), -1, **i32)
         self.cur = 0
-        # (only the type and the shape count here: step() sets the strides of the logits it is given)
+        # (no memory for a whole window of logits: step() sets the strides of those it is given, until then they are contiguous)
         proto = torch.empty(vocab, dtype=logits_dtype, device=dev).as_strided((batch, window, vocab), (0, 0, 1))
         self.params = B.make_params(proto, top_k=top_k, cfg_scale=cfg_scale, inv_temperature=inv_temperature,
                                     reuse_tau=reuse_tau,
@@ -60,6 +60,7 @@ class DecodeLoop:
                                     win_len=self.win_len,
                                     pos_base=self.pos_base, iteration=self.iteration, status=self.status,
                                     seq_base=seq_base, init_mode=init_mode, grid_width=grid_width)
+        self.params.stride_b, self.params.stride_w = window * vocab, vocab
         del proto
         self.use_graphs = use_graphs
         self.graphs = [None, None]   # one per buffer parity
