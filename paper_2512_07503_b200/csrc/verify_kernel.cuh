@@ -61,6 +61,7 @@ struct VerifySmem {
   // ids of the previous iteration's row (of a very long one every stride-th), and behind the first 2,048 the
   // probabilities when the whole row fits in 2,048 entries
   alignas(16) int32_t q[kVerifyStage];
+  int32_t q_cnt[kVerifyThreads];  // of every window row
   int first_reject;
   int status;
   int res_tok;
@@ -92,6 +93,7 @@ __global__ void __launch_bounds__(kVerifyThreads) verify_kernel(const VerifyArgs
   if (!draft_all && i < L) {
     q_tok = a.q_tok[base + i];
     draft = a.drafts[base + i];
+    sm.q_cnt[i] = a.q_cnt[base + i];
     u = uniform24(philox4x32_10((uint32_t)(pos0 + i), seq, (uint32_t)iter, kPurposeAccept, a.seed_lo, a.seed_hi).x0);
   }
   if (i == 0) {
@@ -136,7 +138,7 @@ __global__ void __launch_bounds__(kVerifyThreads) verify_kernel(const VerifyArgs
     const float* pv = a.p_vals + r * kcap;
     const int32_t* qid = a.q_ids + r * kcap;
     const float* qv = a.q_vals + r * kcap;
-    const int qc = a.q_cnt[r];
+    const int qc = sm.q_cnt[acc];
     const float q_uniform = __fdiv_rn(1.0f, (float)a.V);
     const uint64_t R = random64(philox4x32_10((uint32_t)(pos0 + acc), seq, (uint32_t)iter, kPurposeResidual, a.seed_lo, a.seed_hi));
     const int rounds = LONG ? (kcap + NT * ITEMS - 1) / (NT * ITEMS) : 1;
@@ -146,34 +148,33 @@ __global__ void __launch_bounds__(kVerifyThreads) verify_kernel(const VerifyArgs
     // whole runs of four as one load each where the arrays' alignment allows it
     const bool vec = (kcap & 3) == 0 && ((reinterpret_cast<uintptr_t>(a.p_ids) | reinterpret_cast<uintptr_t>(a.p_vals) |
                                           reinterpret_cast<uintptr_t>(a.q_ids) | reinterpret_cast<uintptr_t>(a.q_vals)) & 15u) == 0;
-    auto load4 = [&](const int32_t* ids, const float* vals, int k, int (&to_id)[ITEMS], float (&to_val)[ITEMS]) {
+    auto load4 = [&](const int32_t* ids, const float* vals, int k, int len, int (&to_id)[ITEMS], float (&to_val)[ITEMS]) {
       if (vec) {
-        const int4 x = k < kcap ? *reinterpret_cast<const int4*>(ids + k) : make_int4(-1, -1, -1, -1);
-        const float4 y = k < kcap ? *reinterpret_cast<const float4*>(vals + k) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        const int4 x = k < len ? *reinterpret_cast<const int4*>(ids + k) : make_int4(-1, -1, -1, -1);
+        const float4 y = k < len ? *reinterpret_cast<const float4*>(vals + k) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         to_id[0] = x.x; to_id[1] = x.y; to_id[2] = x.z; to_id[3] = x.w;
         to_val[0] = y.x; to_val[1] = y.y; to_val[2] = y.z; to_val[3] = y.w;
         return;
       }
 #pragma unroll
       for (int j = 0; j < ITEMS; ++j) {
-        const bool in = k + j < kcap;
+        const bool in = k + j < len;
         to_id[j] = in ? ids[k + j] : -1;
         to_val[j] = in ? vals[k + j] : 0.0f;
       }
     };
-    auto load = [&](int k) { load4(pid, pv, k, id, p); };
-    int n, stride = 1;
+    auto load = [&](int k) { load4(pid, pv, k, kcap, id, p); };
+    const int n = min(max(qc, 0), kcap);  // a uniform row has no list
+    int stride = 1;
     if (!LONG) {
-      // all loads at once: q's too, although only the first qc of its entries (if it has any) mean anything
+      // all loads at once
       int qi[ITEMS];
       float qw[ITEMS];
       load(k0);
-      load4(qid, qv, k0, qi, qw);
+      load4(qid, qv, k0, n, qi, qw);
       *reinterpret_cast<int4*>(&sm.q[k0]) = make_int4(qi[0], qi[1], qi[2], qi[3]);
       *reinterpret_cast<float4*>(&sm.q[NT * ITEMS + k0]) = make_float4(qw[0], qw[1], qw[2], qw[3]);
-      n = min(max(qc, 0), kcap);
     } else {
-      n = min(max(qc, 0), kcap);
       stride = (n + kVerifyStage - 1) / kVerifyStage;
       for (int k = i; k * stride < n; k += NT) sm.q[k] = qid[k * stride];
     }
