@@ -185,17 +185,21 @@ __global__ void __launch_bounds__(kVerifyThreads) verify_kernel(const VerifyArgs
       // largest staged position whose id does not exceed the wanted one: by halving for the first of the four, by steps
       // from there for the others: both rows ascend and hold about as many entries, so one or two steps do (four searches
       // by halving in step: 5.7 K cycles of the kernel's 14 K, this 4.7 K; a hash table 7 K and 4 K to fill; neighbouring
-      // entries to neighbouring lanes 3.1 K, but more for locating the draw than that saves)
+      // entries to neighbouring lanes 3.1 K, but more for locating the draw than that saves).  Where the other row's ids crowd
+      // between two of these eight steps do not get there, and the rest goes by halving again.
       int lo[ITEMS];
       int at = 0;
-      if (n > 0) {
-        for (int half = 1 << (31 - __clz(staged)); half > 0; half >>= 1)
-          if (at + half < staged && sm.q[at + half] <= id[0]) at += half;
-      }
+      auto halve = [&](int wanted) {
+        for (int half = n > 0 ? 1 << (31 - __clz(staged)) : 0; half > 0; half >>= 1)
+          if (at + half < staged && sm.q[at + half] <= wanted) at += half;
+      };
+      halve(id[0]);
 #pragma unroll
       for (int j = 0; j < ITEMS; ++j) {
         if (j > 0) {
-          while (at + 1 < staged && sm.q[at + 1] <= id[j]) ++at;
+          int steps = 8;
+          while (at + 1 < staged && sm.q[at + 1] <= id[j] && steps > 0) ++at, --steps;
+          if (steps == 0) halve(id[j]);
         }
         lo[j] = at;
       }

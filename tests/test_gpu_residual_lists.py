@@ -1,4 +1,4 @@
-"""The residual draw's look at the previous iteration's row: rows without a list."""
+"""The residual draw's look at the previous iteration's row: lists that lie anywhere against this row's, and rows without a list."""
 import numpy as np
 import pytest
 import torch
@@ -12,6 +12,32 @@ pytestmark = pytest.mark.gpu
 def _inputs(V, K, W, seed):
     wl = wk.CONFIGS["cfg2"].scaled(B=2, W=W, V=V, top_k=K, seed=seed, peaks=0)
     return wl, wk.make_step_inputs(wl)
+
+
+# all of the previous row's ids between two neighbours of this row's, below all of them, above all of them, every other one the same
+@pytest.mark.parametrize("K", [5, 2000, 2048, 5000])
+@pytest.mark.parametrize("where", ["between", "below", "above", "interleaved"])
+def test_previous_ids_anywhere(K, where):
+    from gpu_harness import check_parity, step_kwargs
+    V, W = 65536, 4
+    wl, inp = _inputs(V, K, W, K)
+    # this row's largest entries: the ids [a, a + half) and [b, b + rest); the previous row's elsewhere
+    half = K // 2
+    a, b = {"between": (100, 40000), "below": (20000, 40000), "above": (100, 8000), "interleaved": (100, 40000)}[where]
+    own = np.r_[a:a + half, b:b + K - half]
+    q0 = {"between": 9000, "below": 100, "above": 50000, "interleaved": 0}[where]
+    q_ids = np.arange(q0, q0 + K) if where != "interleaved" else np.unique(np.r_[own[::2], 50000 + np.arange(K)])[:K]
+    for arr in (inp.cond, inp.uncond):
+        f = wk._as_f32(arr, wl.dtype).copy()
+        f[:, :, own] += 30.0
+        arr[:] = wk._store(f, wl.dtype)
+    rng = np.random.default_rng(K)
+    vals = rng.random((2, W, K)).astype(np.float32)
+    vals /= vals.sum(-1, keepdims=True)
+    ids = np.ascontiguousarray(np.broadcast_to(q_ids.astype(np.int32), (2, W, K)))
+    drafts = np.ascontiguousarray(ids[:, :, K // 2])
+    q = oracle.Probs(np.ascontiguousarray(vals[:, :, K // 2]), ids, vals, np.full((2, W), K, np.int32))
+    check_parity(inp.cond, inp.uncond, drafts, q, step_kwargs(inp), inp.win_len)
 
 
 @pytest.mark.parametrize("K", [64, 2048, 3000])
