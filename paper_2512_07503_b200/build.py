@@ -27,7 +27,7 @@ def sources():
 
 
 def _deps():
-    return sources() + glob.glob(os.path.join(_CSRC, "*.cuh")) + glob.glob(os.path.join(_INC, "*.h"))
+    return sources() + glob.glob(os.path.join(_CSRC, "*.cuh")) + glob.glob(os.path.join(_CSRC, "*.h")) + glob.glob(os.path.join(_INC, "*.h"))
 
 
 def is_stale() -> bool:

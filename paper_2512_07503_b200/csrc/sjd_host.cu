@@ -13,10 +13,13 @@
 // 1,640 -> 1,370 us (1,340 of the link).  One part only: 238 us at B=4.
 #include "../../include/sjd.h"
 
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <cstdlib>
 #include <cstring>
+
+#include "host_piece.h"
 
 namespace {
 
@@ -49,19 +52,28 @@ __global__ void fetch_words(const int32_t* __restrict__ from, int32_t* __restric
   if (i < n) to[i] = from[i];
 }
 
-// The device's address of a page-locked host array, null if any end of it is not.
+// The device's address of a host array that one page-locked and mapped piece of memory holds, else null.
 template <typename T>
 T* mapped(T* p, size_t bytes) {
-  cudaPointerAttributes first, last;
-  const char* end = reinterpret_cast<const char*>(p) + bytes - 1;
-  if (cudaPointerGetAttributes(&first, p) != cudaSuccess || cudaPointerGetAttributes(&last, end) != cudaSuccess) {
-    (void)cudaGetLastError();
-    return nullptr;
-  }
-  if (first.type != cudaMemoryTypeHost || last.type != cudaMemoryTypeHost || !first.devicePointer ||
-      static_cast<char*>(last.devicePointer) - static_cast<char*>(first.devicePointer) != (ptrdiff_t)(bytes - 1))
-    return nullptr;
-  return static_cast<T*>(first.devicePointer);
+  using Query = CUresult (*)(void*, CUpointer_attribute, CUdeviceptr);
+  static const Query query = [] {  // (through the runtime: no link against the driver library)
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult found;
+    if (cudaGetDriverEntryPoint("cuPointerGetAttribute", &f, cudaEnableDefault, &found) != cudaSuccess || found != cudaDriverEntryPointSuccess) f = nullptr;
+    return reinterpret_cast<Query>(f);
+  }();
+  return static_cast<T*>(sjd::device_address_of(p, bytes, [](const void* at, sjd::HostPiece* piece) {
+    cudaPointerAttributes attr;
+    if (cudaPointerGetAttributes(&attr, at) != cudaSuccess) {
+      (void)cudaGetLastError();
+      return false;
+    }
+    if (attr.type != cudaMemoryTypeHost || !attr.devicePointer || !query) return false;
+    piece->device = static_cast<char*>(attr.devicePointer);
+    const CUdeviceptr d = reinterpret_cast<CUdeviceptr>(attr.devicePointer);
+    return query(&piece->start, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, d) == CUDA_SUCCESS &&
+           query(&piece->size, CU_POINTER_ATTRIBUTE_RANGE_SIZE, d) == CUDA_SUCCESS;
+  }));
 }
 
 void drain(sjd_host_ctx* c) {
