@@ -4,7 +4,8 @@
 // The link to the host is what bounds it: 50 GB/s, and some 4 us for every copy whatever its size.  So
 //   - the batch goes through in parts of whole sequences: while a part's logits are on their way in, the part before it is
 //     in the kernels and the one before that on its way out (three streams; the parts use the mirrors' own ranges, and
-//     sequence numbers by seq_base, so the results are those of one call);
+//     sequence numbers by seq_base; a row's result does not depend on how many rows a call has, except that a row which one of
+//     the row kernels has to redo agrees with the other's to rounding only);
 //   - the small arrays of a call are gathered in page-locked memory, from which a kernel fetches them while the
 //     first logits come in, and into which the kernels write the small results: no copies of their own;
 //   - of the previous iteration's distributions one row per sequence is needed, and only the verification knows which: it
@@ -23,9 +24,9 @@
 
 namespace {
 
-// A part has at least this many bytes of logits: each costs two to four copies more, and hides its kernels and
-// its copies out behind the others.  The case above in parts of 2, 3, 4 and 8 MB: 252, 250, 233, 238 us; B=32: at most four
-// parts 1,402 us, eight 1,383.
+// Every part has at least this many bytes of logits (where there is more than one): each costs two to four copies more, and hides its
+// kernels and its copies out behind the others.  The case above in parts of 2, 3, 4 and 8 MB: 252, 250, 233, 238 us; B=32: at
+// most four parts 1,402 us, eight 1,383.
 constexpr size_t kPartBytes = 4 << 20;
 constexpr int kMaxParts = 8;
 
@@ -122,11 +123,8 @@ int enqueue(sjd_host_ctx* c, const char* cond, const char* uncond, const int32_t
             const sjd_params* P, uint64_t seed, sjd_probs* out) {
   const cudaMemcpyKind H2D = cudaMemcpyHostToDevice, D2H = cudaMemcpyDeviceToHost;
   const size_t rows = c->rows, B = (size_t)c->B, W = (size_t)c->W, kc = (size_t)c->kcap, n_logits = W * c->row_bytes;
-  const size_t total = B * n_logits * (uncond ? 2 : 1);
-  size_t parts = total / kPartBytes;
-  if (parts > kMaxParts) parts = kMaxParts;
-  if (parts > B) parts = B;
-  if (parts < 1) parts = 1;
+  size_t parts = B < kMaxParts ? B : kMaxParts;
+  while (parts > 1 && B / parts * n_logits * (uncond ? 2 : 1) < kPartBytes) --parts;  // (the smallest part)
   int32_t* const d_win = c->d_small;
   int32_t* const d_drafts = c->d_small + 3 * B;
   int32_t* const m_tokens = c->m_results + 2 * B;
