@@ -81,8 +81,8 @@ extern "C" {
 #define SJD_STATUS_EMPTY_RESIDUAL 2   /* fixed-point residual total was 0: drawn from p instead          */
 #define SJD_STATUS_DEGENERATE_ROW 4   /* a row had no finite logit: its probabilities are all 0          */
 #define SJD_STATUS_INTERNAL_TIMEOUT 8 /* a bounded on-chip wait gave up: the sequence's outputs are invalid */
-#define SJD_STATUS_ROW_REDONE 16      /* informational: a row did not fit the single-pass kernel's on-chip lists
-                                         and was redone by the any-shape path; its result is exact, the step slower */
+#define SJD_STATUS_ROW_REDONE 16      /* informational: a row did not fit the single-pass kernel's on-chip lists and was sifted
+                                         once more or redone by the any-shape path; its result is exact, the step slower */
 
 /* return codes */
 #define SJD_OK 0
