@@ -338,6 +338,23 @@ cudaError_t launch_sift(const sjd::RowArgs& ra, const SiftPlan& plan, cudaStream
   return t ? launch_sift_as<DTYPE, false, true>(ra, plan, st) : launch_sift_as<DTYPE, false, false>(ra, plan, st);
 }
 
+template <bool LONG, int LOOK>
+cudaError_t launch_verify_as(const sjd::VerifyArgs& va, cudaStream_t st, bool dependent) {
+  auto kern = sjd::verify_kernel<LONG, LOOK>;
+  static sjd::DeviceOnce configured;
+  const cudaError_t e = allow_large_smem(kern, configured, (int)kSmemLimit);
+  if (e != cudaSuccess) return e;
+  return launch_after(kern, dim3((unsigned)va.B), dim3(sjd::kVerifyThreads), sjd::verify_smem(va.V, va.kcap, LONG, LOOK), st, dependent, 1, va);
+}
+cudaError_t launch_verify(const sjd::VerifyArgs& va, cudaStream_t st, bool dependent) {
+  const bool is_long = va.kcap > sjd::kVerifyShort;
+  const int look = sjd::verify_map(va.V, va.kcap, is_long, kSmemLimit);
+  if (!is_long) return look == sjd::kMapVals ? launch_verify_as<false, sjd::kMapVals>(va, st, dependent) : launch_verify_as<false, sjd::kNoMap>(va, st, dependent);
+  return look == sjd::kMapVals ? launch_verify_as<true, sjd::kMapVals>(va, st, dependent)
+         : look == sjd::kMap   ? launch_verify_as<true, sjd::kMap>(va, st, dependent)
+                               : launch_verify_as<true, sjd::kNoMap>(va, st, dependent);
+}
+
 // Scratch of sjd_step_static(): lives in the library's device image, so every GPU that loads the library
 // holds these bytes until the process exits.  Sized for SJD_STATIC_MAX_ROWS rows of RowScratch.
 constexpr size_t kStaticScratchBytes = (((size_t)SJD_STATIC_MAX_ROWS * sizeof(sjd::RowScratch) + 256) + 255) & ~(size_t)255;
@@ -512,10 +529,7 @@ int sjd_step(const void* logits_cond, const void* logits_uncond, const int32_t* 
     // directly behind the row kernel the verification grid is launched as its programmatic dependent: its
     // blocks are placed as the row kernel's last blocks retire and wait inside the kernel for its completion.
     // An event recorded in between makes it an ordinary launch.
-    const bool longer = kcap > sjd::kVerifyThreads * sjd::kVerifyItems;
-    const cudaError_t e = launch_after(longer ? sjd::verify_kernel<true> : sjd::verify_kernel<false>, dim3((unsigned)P->B),
-                                       dim3(sjd::kVerifyThreads), 0, stream,
-                                       P->ev_rows_end == nullptr, 1, va);
+    const cudaError_t e = launch_verify(va, stream, P->ev_rows_end == nullptr);
     if (e != cudaSuccess) return cuda_fail(e, "verify kernel launch");
     ++g_launches;
   }

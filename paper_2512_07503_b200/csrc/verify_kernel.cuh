@@ -16,6 +16,9 @@ constexpr int kQUniform = -1;
 constexpr int kOutInvalid = 0, kOutAccepted = 1, kOutResidual = 2, kOutReused = 3, kOutResampled = 4;
 constexpr int kStatusQtok = 1, kStatusEmptyResidual = 2, kStatusDegenerate = 4, kStatusTimeout = 8, kStatusRedone = 16;
 
+// a cache line into the L2
+__device__ __forceinline__ void ask_line(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
 struct VerifyArgs {
   int B, W, V, kcap;
   int flags;
@@ -53,33 +56,57 @@ __device__ __forceinline__ float likelihood_ratio(float p, float q) {
 }
 
 constexpr int kVerifyThreads = 512;     // >= SJD_W_MAX: a thread per window row
-constexpr int kVerifyItems = 4;         // entries of the rejected row per thread and round: 2,048 a round
-constexpr int kVerifyStage = 8192;      // words of the previous iteration's row staged in shared memory
+constexpr int kVerifyShort = 4 * kVerifyThreads;  // entries of a row that is not LONG
+constexpr int kVerifyStage = 8192;      // without the map: words of the previous iteration's row staged in shared memory
+constexpr int kVerifyAsked = 4;         // rows of the previous iteration's distributions asked into the L2 early
 
 struct VerifySmem {
-  uint64_t scan[2 * 32 + 8];
-  // ids of the previous iteration's row (of a very long one every stride-th), and behind the first 2,048 the
-  // probabilities when the whole row fits in 2,048 entries
-  alignas(16) int32_t q[kVerifyStage];
-  int32_t q_cnt[kVerifyThreads];  // of every window row
+  uint64_t warp_sum[2][kVerifyThreads / 32];
+  uint64_t random;                // of the rejected row
   int first_reject;
   int status;
-  int res_tok;
-  float res_prob;
+  int q_cnt[kVerifyThreads];      // of every window row
 };
+static_assert(sizeof(VerifySmem) % 16 == 0, "the map behind it is cleared sixteen bytes at a time");
+// Behind it, where an id lies in the previous iteration's row.  kMapVals: a bit for every id of the vocabulary, for each word of bits the
+// position of its first entry (16 bits), and the row's probabilities: a lookup is a bit, a population count and an addition.  kMap:
+// without the probabilities, where they would be too much.  kNoMap (vocabularies of a million ids): the ids themselves, of a very
+// long row every stride-th, to be searched by halving, and the probabilities of a row that is not LONG.
+enum { kNoMap = 0, kMap = 1, kMapVals = 2 };
+__host__ __device__ inline int verify_map_words(int V) { return V / 128 * 4 + 4; }
+__host__ __device__ inline size_t verify_smem(int V, int kcap, bool is_long, int map) {
+  if (map == kNoMap) return sizeof(VerifySmem) + (is_long ? (size_t)kVerifyStage * 4 : (size_t)kVerifyShort * 8);
+  return sizeof(VerifySmem) + (size_t)verify_map_words(V) * 6 + (map == kMapVals ? (size_t)(kcap + 3) / 4 * 16 : 0);
+}
+// the best that fits
+inline int verify_map(int V, int kcap, bool is_long, size_t limit) {
+  if (kcap > 65536) return kNoMap;
+  return verify_smem(V, kcap, is_long, kMapVals) <= limit ? kMapVals : is_long && verify_smem(V, kcap, is_long, kMap) <= limit ? kMap : kNoMap;
+}
 
 // One CTA per sequence.  Latency is all there is to it (it sits between two row kernels), so nothing is waited for
-// that could have been asked for earlier: what does not come from the row stage is loaded, and the accept tests' random
-// numbers are drawn, before the wait for that stage; both rows of the residual draw come in with one round of loads; the
-// lookups of a thread's four entries share one search.  16 sequences of 64 rows, K=2,000: 8.4 us under ncu
-// (12.1 before), and 3 us less of a step (one window of 32 rows: 25.5 -> 21.4 us).
+// that could have been asked for earlier: what does not come from the row stage is loaded, the random numbers are drawn and the
+// map is cleared before the wait for that stage; both rows of the residual draw come in with one round of loads, without
+// branches (a load in one is waited for where the branch ends); what does not depend on the draw is written meanwhile.  A warp
+// owns consecutive entries of the rejected row, a lane every 32nd of them; only the warp that the draw falls to locates it.
 //
-// LONG: rows of more than 2,048 entries, taken in rounds (1,024 rows of K=8,192: 294 -> 235 us a step).
-template <bool LONG>
+// LONG: rows of more than 2,048 entries, a warp's taken sixteen groups of 32 at a time.
+//
+// The map, the loads without branches and the early requests against a search by halving in the row itself, from the row stage's end to a
+// CTA's own, thousands of cycles: 16 rows of K=64 7.4 -> 4.9, 1,024 rows of K=2,000 11.3 -> 7.3, of K=8,192 85 -> 14.7 (a step: 77.9 -> 74.6
+// us, 171 -> 142 us); 128 rows of V=131,072, K=8,192 73.2 -> 55.8 us a step; 32 rows of K=V=65,536 (without probabilities in the map) 597 -> 378 us.
+template <bool LONG, int LOOK>
 __global__ void __launch_bounds__(kVerifyThreads) verify_kernel(const VerifyArgs a) {
-  constexpr int NT = kVerifyThreads, ITEMS = kVerifyItems;
-  __shared__ VerifySmem sm;
-  const int b = blockIdx.x, i = threadIdx.x, W = a.W;
+  constexpr int NT = kVerifyThreads, NW = NT / 32, E = LONG ? 16 : 4;
+  constexpr bool MAP = LOOK != kNoMap, VALS = LOOK == kMapVals || (LOOK == kNoMap && !LONG);  // VALS: the probabilities are staged
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  VerifySmem& sm = *reinterpret_cast<VerifySmem*>(smem_raw);
+  const int words = MAP ? verify_map_words(a.V) : 0;
+  uint32_t* const map_bits = reinterpret_cast<uint32_t*>(smem_raw + sizeof(VerifySmem));
+  uint16_t* const map_first = reinterpret_cast<uint16_t*>(map_bits + words);
+  int32_t* const look_id = reinterpret_cast<int32_t*>(map_bits);
+  float* const look_val = MAP ? reinterpret_cast<float*>(map_first + words) : reinterpret_cast<float*>(look_id + kVerifyShort);
+  const int b = blockIdx.x, i = threadIdx.x, lane = i & 31, warp = i >> 5, W = a.W, kcap = a.kcap;
   const bool draft_all = (a.flags & kFlagDraftAll) != 0;
   const bool reuse_on = (a.flags & kFlagReuse) != 0;
   const size_t base = (size_t)b * W;
@@ -90,17 +117,34 @@ __global__ void __launch_bounds__(kVerifyThreads) verify_kernel(const VerifyArgs
   const uint32_t seq = (uint32_t)(a.seq_base + b);
   float q_tok = 0.0f, u = 0.0f;
   int draft = -1;
+  uint64_t random = 0;
   if (!draft_all && i < L) {
     q_tok = a.q_tok[base + i];
     draft = a.drafts[base + i];
     sm.q_cnt[i] = a.q_cnt[base + i];
     u = uniform24(philox4x32_10((uint32_t)(pos0 + i), seq, (uint32_t)iter, kPurposeAccept, a.seed_lo, a.seed_hi).x0);
+    random = random64(philox4x32_10((uint32_t)(pos0 + i), seq, (uint32_t)iter, kPurposeResidual, a.seed_lo, a.seed_hi));
+  }
+  if constexpr (MAP) {
+    if (!draft_all)
+      for (int k = i; k < words / 4; k += NT) reinterpret_cast<uint4*>(map_bits)[k] = make_uint4(0u, 0u, 0u, 0u);
+  }
+  // (the draw most often falls to one of the first rows; an address that this SM has not met lately is found out as well)
+  if (!draft_all && warp < min(kVerifyAsked, L)) {
+    const size_t at = (base + warp) * (size_t)kcap;
+    const int n = min(a.q_cnt[base + warp], kcap);
+    for (int k = 32 * lane; k < n; k += 1024) {
+      ask_line(a.q_ids + at + k);
+      ask_line(a.q_vals + at + k);
+    }
+    if (lane == 0) {
+      ask_line(a.p_ids + at);
+      ask_line(a.p_vals + at);
+    }
   }
   if (i == 0) {
     sm.first_reject = L;
     sm.status = 0;
-    sm.res_tok = -1;
-    sm.res_prob = 0.0f;
   }
   __syncthreads();
   // Launched with programmatic stream serialisation right behind the row kernel: the grid may be scheduled while that
@@ -114,183 +158,232 @@ __global__ void __launch_bounds__(kVerifyThreads) verify_kernel(const VerifyArgs
   // they are all tested at once
   RowScratch rs{0.0f, -1, 0.0f, 0};
   float ratio = 0.0f;
-  if (i < L) {
-    rs = a.scratch[base + i];
-    int st = (rs.status & kRowStatusDegenerate) ? kStatusDegenerate : 0;
-    if (rs.status & kRowStatusTimeout) st |= kStatusTimeout;
-    if (rs.status & kRowStatusRedone) st |= kStatusRedone;
-    if (!draft_all) {
-      ratio = likelihood_ratio(rs.p_tok, q_tok);
-      if (!(u < fminf(ratio, 1.0f))) atomicMin(&sm.first_reject, i);
-      if (!(q_tok > 0.0f)) st |= kStatusQtok;
+  {
+    int st = 0;
+    bool rejected = false;
+    if (i < L) {
+      rs = a.scratch[base + i];
+      if (rs.status & kRowStatusDegenerate) st |= kStatusDegenerate;
+      if (rs.status & kRowStatusTimeout) st |= kStatusTimeout;
+      if (rs.status & kRowStatusRedone) st |= kStatusRedone;
+      if (!draft_all) {
+        ratio = likelihood_ratio(rs.p_tok, q_tok);
+        rejected = !(u < fminf(ratio, 1.0f));
+        if (!(q_tok > 0.0f)) st |= kStatusQtok;
+      }
     }
+    const uint32_t votes = __ballot_sync(0xffffffffu, rejected);
+    if (lane == 0 && votes != 0u) atomicMin(&sm.first_reject, i + __ffs((int)votes) - 1);
     if (st) atomicOr(&sm.status, st);
   }
   __syncthreads();
   const int acc = draft_all ? 0 : sm.first_reject;
+  const bool draw = !draft_all && acc < L;
 
-  // Step 4, first rejected row: draw from max(0, p - q) / sum max(0, p - q).  Every thread owns a run of consecutive entries
-  // of p_a (ascending token id), so one scan of the per-thread sums locates the draw.
-  if (!draft_all && acc < L) {
-    const size_t r = base + acc;
-    const int kcap = a.kcap;
-    const int32_t* pid = a.p_ids + r * kcap;
-    const float* pv = a.p_vals + r * kcap;
-    const int32_t* qid = a.q_ids + r * kcap;
-    const float* qv = a.q_vals + r * kcap;
-    const int qc = sm.q_cnt[acc];
-    const float q_uniform = __fdiv_rn(1.0f, (float)a.V);
-    const uint64_t R = random64(philox4x32_10((uint32_t)(pos0 + acc), seq, (uint32_t)iter, kPurposeResidual, a.seed_lo, a.seed_hi));
-    const int rounds = LONG ? (kcap + NT * ITEMS - 1) / (NT * ITEMS) : 1;
-    const int k0 = i * ITEMS * rounds;  // this thread's run of consecutive entries
-    int id[ITEMS];
-    float p[ITEMS], w[ITEMS];
-    // whole runs of four as one load each where the arrays' alignment allows it
-    const bool vec = (kcap & 3) == 0 && ((reinterpret_cast<uintptr_t>(a.p_ids) | reinterpret_cast<uintptr_t>(a.p_vals) |
-                                          reinterpret_cast<uintptr_t>(a.q_ids) | reinterpret_cast<uintptr_t>(a.q_vals)) & 15u) == 0;
-    auto load4 = [&](const int32_t* ids, const float* vals, int k, int len, int (&to_id)[ITEMS], float (&to_val)[ITEMS]) {
-      if (vec) {
-        const int4 x = k < len ? *reinterpret_cast<const int4*>(ids + k) : make_int4(-1, -1, -1, -1);
-        const float4 y = k < len ? *reinterpret_cast<const float4*>(vals + k) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        to_id[0] = x.x; to_id[1] = x.y; to_id[2] = x.z; to_id[3] = x.w;
-        to_val[0] = y.x; to_val[1] = y.y; to_val[2] = y.z; to_val[3] = y.w;
-        return;
+  // Step 4, the rows that do not wait for a draw, and the outputs
+  auto put_rows = [&] {
+    if (i < W && !(draw && i == acc)) {
+      int tok = -1, flag = kOutInvalid;
+      float pr = 0.0f;
+      if (i < L) {
+        if (draft_all) {
+          tok = rs.samp_tok; pr = rs.samp_prob; flag = kOutResampled;
+        } else if (i < acc) {
+          tok = draft; pr = rs.p_tok; flag = kOutAccepted;
+        } else if (reuse_on && rs.p_tok > 0.0f && ratio > a.tau) {  // the ratio is the confidence of Eq. (C)
+          tok = draft; pr = rs.p_tok; flag = kOutReused;
+        } else {
+          tok = rs.samp_tok; pr = rs.samp_prob; flag = kOutResampled;
+        }
       }
-#pragma unroll
-      for (int j = 0; j < ITEMS; ++j) {
-        const bool in = k + j < len;
-        to_id[j] = in ? ids[k + j] : -1;
-        to_val[j] = in ? vals[k + j] : 0.0f;
-      }
-    };
-    auto load = [&](int k) { load4(pid, pv, k, kcap, id, p); };
-    const int n = min(max(qc, 0), kcap);  // a uniform row has no list
-    int stride = 1;
-    if (!LONG) {
-      // all loads at once
-      int qi[ITEMS];
-      float qw[ITEMS];
-      load(k0);
-      load4(qid, qv, k0, n, qi, qw);
-      *reinterpret_cast<int4*>(&sm.q[k0]) = make_int4(qi[0], qi[1], qi[2], qi[3]);
-      *reinterpret_cast<float4*>(&sm.q[NT * ITEMS + k0]) = make_float4(qw[0], qw[1], qw[2], qw[3]);
-    } else {
-      stride = (n + kVerifyStage - 1) / kVerifyStage;
-      for (int k = i; k * stride < n; k += NT) sm.q[k] = qid[k * stride];
+      a.out_tokens[base + i] = tok;
+      a.out_tok_prob[base + i] = pr;
+      if (a.out_flags) a.out_flags[base + i] = flag;
     }
-    __syncthreads();
-    const int staged = n > 0 ? (n + stride - 1) / stride : 0;
-    // weights of the four entries in id / p: what q leaves of p
-    auto residual = [&](int k) {
-      // largest staged position whose id does not exceed the wanted one: by halving for the first of the four, by steps
-      // from there for the others: both rows ascend and hold about as many entries, so one or two steps do (four searches
-      // by halving in step: 5.7 K cycles of the kernel's 14 K, this 4.7 K; a hash table 7 K and 4 K to fill; neighbouring
-      // entries to neighbouring lanes 3.1 K, but more for locating the draw than that saves).  Where the other row's ids crowd
-      // between two of these eight steps do not get there, and the rest goes by halving again.
-      int lo[ITEMS];
-      int at = 0;
-      auto halve = [&](int wanted) {
-        for (int half = n > 0 ? 1 << (31 - __clz(staged)) : 0; half > 0; half >>= 1)
-          if (at + half < staged && sm.q[at + half] <= wanted) at += half;
-      };
-      halve(id[0]);
+    if (i == 0) a.out_accept_len[b] = acc;
+  };
+  if (!draw) {
+    put_rows();
+    if (i == 0 && a.status) a.status[b] = sm.status;
+    return;
+  }
+  if (i == acc) sm.random = random;
+
+  // Step 4, first rejected row: draw from max(0, p - q) / sum max(0, p - q).  Warp w owns 32 * per consecutive entries of p_a
+  // (ascending token id).
+  const size_t row = (base + acc) * (size_t)kcap;
+  const int32_t* const pid = a.p_ids + row;
+  const float* const pv = a.p_vals + row;
+  const int32_t* const qid = a.q_ids + row;
+  const float* const qv = a.q_vals + row;
+  const int per = (kcap + NT - 1) / NT;  // groups of 32 per warp: up to E unless LONG
+  const int own0 = warp * per * 32 + lane;
+  int id[E];
+  float p[E];
+  auto load = [&](int j0) {
 #pragma unroll
-      for (int j = 0; j < ITEMS; ++j) {
-        if (j > 0) {
-          int steps = 8;
-          while (at + 1 < staged && sm.q[at + 1] <= id[j] && steps > 0) ++at, --steps;
-          if (steps == 0) halve(id[j]);
-        }
-        lo[j] = at;
+    for (int j = 0; j < E; ++j) {
+      const int k = own0 + 32 * (j0 + j);
+      id[j] = -1;
+      p[j] = 0.0f;
+      if (j0 + j < per && k < kcap) {
+        id[j] = pid[k];
+        p[j] = pv[k];
       }
-#pragma unroll
-      for (int j = 0; j < ITEMS; ++j) {
-        float q = qc == kQUniform ? q_uniform : 0.0f;
-        if (n > 0) {
-          if (!LONG) {
-            if (sm.q[lo[j]] == id[j]) q = reinterpret_cast<const float*>(sm.q)[NT * ITEMS + lo[j]];
-          } else {
-            int at = lo[j] * stride;
-            const int end = min(at + stride, n);
-            while (at + 1 < end && qid[at + 1] <= id[j]) ++at;
-            if (qid[at] == id[j]) q = qv[at];
-          }
-        }
-        w[j] = k + j < kcap ? __fsub_rn(p[j], q) : 0.0f;
-      }
-    };
-    int flip = 0;
-    uint64_t T = 0, before = 0, local = 0;
-    bool from_p = false;
-    for (;;) {
-      // residual weights first; p itself only when they sum to zero after rounding
-      local = 0;
-      for (int r = 0; r < rounds; ++r) {
-        if (LONG) load(k0 + ITEMS * r);
-        if (!from_p) residual(k0 + ITEMS * r);
-#pragma unroll
-        for (int j = 0; j < ITEMS; ++j) {
-          if (from_p) w[j] = p[j];
-          local += fixed_weight(w[j]);
-        }
-      }
-      before = group_scan1<NT, 0, uint64_t>(local, i, sm.scan, flip, &T);
-      if (T != 0 || from_p) break;
-      if (i == 0) sm.status |= kStatusEmptyResidual;
-      from_p = true;
     }
-    const uint64_t t = __umul64hi(R, T);
-    if (T == 0 ? i == 0 : (t >= before && t < before + local)) {
-      int j = 0;
-      if (T == 0) {
-        load(0);  // nothing but zeros: the first entry
-      } else {
-        for (int r = 0; r < rounds; ++r) {
-          if (LONG) {
-            load(k0 + ITEMS * r);
-            if (!from_p) residual(k0 + ITEMS * r);
-          }
-          uint64_t sum = 0;
-          j = 0;
+  };
+  load(0);
+  // the previous iteration's row
+  const int qc = sm.q_cnt[acc];
+  const int n = min(max(qc, 0), kcap);  // a uniform row has no list
+  int stride = 1;
+  int x[E], last[E];  // ids, and (first lane) the id before them
+  float y[E];
+  auto load_reference = [&](int k0) {
 #pragma unroll
-          for (int x = 0; x < ITEMS; ++x) {
-            sum += fixed_weight(LONG && from_p ? p[x] : w[x]);
-            if (t >= before + sum) j = x + 1;
-          }
-          if (j < ITEMS) break;  // comes true: t < before + local
-          before += sum;
+    for (int j = 0; j < E; ++j) {
+      const int k = k0 + j * NT;
+      x[j] = last[j] = -1;  // (of another word than any there is)
+      y[j] = 0.0f;
+      if (k < n) x[j] = qid[k];
+      if (MAP && lane == 0 && k > 0 && k < n) last[j] = qid[k - 1];
+      if (VALS && k < n) y[j] = qv[k];
+    }
+  };
+  if constexpr (MAP || !LONG) load_reference(i);
+  put_rows();
+  if constexpr (MAP) {
+    for (int k0 = i;;) {
+#pragma unroll
+      for (int j = 0; j < E; ++j) {
+        const int k = k0 + j * NT, own = x[j];
+        int before = __shfl_up_sync(0xffffffffu, own, 1);
+        if (lane == 0) before = last[j];
+        if (VALS && k < n) look_val[k] = y[j];
+        if ((uint32_t)own < (uint32_t)a.V) {  // (-1 beyond the list's end)
+          atomicOr(&map_bits[own >> 5], 1u << (own & 31));
+          if ((before >> 5) != (own >> 5)) map_first[own >> 5] = (uint16_t)k;
         }
       }
-      sm.res_tok = j == 0 ? id[0] : j == 1 ? id[1] : j == 2 ? id[2] : id[3];
-      sm.res_prob = j == 0 ? p[0] : j == 1 ? p[1] : j == 2 ? p[2] : p[3];
+      k0 += E * NT;
+      if (!LONG || k0 - i >= n) break;
+      load_reference(k0);
     }
+  } else if constexpr (!LONG) {
+#pragma unroll
+    for (int j = 0; j < E; ++j) {
+      look_id[i + j * NT] = x[j];
+      look_val[i + j * NT] = y[j];
+    }
+  } else {
+    stride = (n + kVerifyStage - 1) / kVerifyStage;
+    for (int k = i; k * stride < n; k += NT) look_id[k] = qid[k * stride];
   }
   __syncthreads();
-
-  // Step 4, remaining rows, and the outputs
-  if (i < W) {
-    int tok = -1, flag = kOutInvalid;
-    float pr = 0.0f;
-    if (i < L) {
-      if (draft_all) {
-        tok = rs.samp_tok; pr = rs.samp_prob; flag = kOutResampled;
-      } else if (i < acc) {
-        tok = draft; pr = rs.p_tok; flag = kOutAccepted;
-      } else if (i == acc) {
-        tok = sm.res_tok; pr = sm.res_prob; flag = kOutResidual;
-      } else if (reuse_on && rs.p_tok > 0.0f && ratio > a.tau) {  // the ratio is the confidence of Eq. (C)
-        tok = draft; pr = rs.p_tok; flag = kOutReused;
+  const float unlisted = qc == kQUniform ? __fdiv_rn(1.0f, (float)a.V) : 0.0f;
+  const int staged = n > 0 ? (n + stride - 1) / stride : 0;
+  // the previous iteration's probability of a token
+  auto reference = [&](int token) {
+    float q = unlisted;
+    if constexpr (MAP) {
+      const uint32_t at_word = min((uint32_t)token, (uint32_t)a.V - 1u) >> 5, bit = 1u << (token & 31);
+      const uint32_t word = map_bits[at_word];
+      const int at = max(min((int)map_first[at_word] + __popc(word & (bit - 1u)), n - 1), 0);
+      if constexpr (VALS) {
+        const float v = look_val[at];  // (whether or not: a load is cheaper than a branch)
+        q = (word & bit) != 0u ? v : q;
       } else {
-        tok = rs.samp_tok; pr = rs.samp_prob; flag = kOutResampled;
+        if ((word & bit) != 0u) q = qv[at];
+      }
+    } else if (n > 0) {
+      // largest staged position whose id does not exceed the wanted one
+      int at = 0;
+      for (int half = 1 << (31 - __clz(staged)); half > 0; half >>= 1)
+        if (at + half < staged && look_id[at + half] <= token) at += half;
+      if constexpr (!LONG) {
+        if (look_id[at] == token) q = look_val[at];
+      } else {
+        at *= stride;
+        const int end = min(at + stride, n);
+        while (at + 1 < end && qid[at + 1] <= token) ++at;
+        if (qid[at] == token) q = qv[at];
       }
     }
-    a.out_tokens[base + i] = tok;
-    a.out_tok_prob[base + i] = pr;
-    if (a.out_flags) a.out_flags[base + i] = flag;
-  }
-  if (i == 0) {
-    a.out_accept_len[b] = acc;
-    if (a.status) a.status[b] = sm.status;
+    return q;
+  };
+  // what q leaves of the loaded entries, or p itself (nothing where there is no entry: its p is zero)
+  float w[E];
+  bool from_p = false;
+  auto weigh = [&] {
+#pragma unroll
+    for (int j = 0; j < E; ++j) w[j] = from_p ? p[j] : __fsub_rn(p[j], reference(id[j]));
+  };
+  for (;;) {
+    uint64_t local = 0;
+    for (int j0 = 0; j0 < per; j0 += E) {
+      if (LONG && per > E && (j0 > 0 || from_p)) load(j0);
+      weigh();
+#pragma unroll
+      for (int j = 0; j < E; ++j) local += fixed_weight(w[j]);
+    }
+    local = warp_sum_u64(local);
+    if (lane == 0) sm.warp_sum[from_p][warp] = local;
+    __syncthreads();
+    const uint64_t sum = lane < NW ? sm.warp_sum[from_p][lane] : 0ull;
+    const uint64_t T = warp_sum_u64(sum);
+    uint64_t before = warp_sum_u64(lane < warp ? sum : 0ull);
+    if (T == 0 && !from_p) {  // the residual weights sum to zero after rounding: p itself
+      from_p = true;
+      continue;
+    }
+    if (i == 0 && a.status) a.status[b] = sm.status | (from_p ? kStatusEmptyResidual : 0);
+    auto emit = [&](int token, float prob) {
+      a.out_tokens[base + acc] = token;
+      a.out_tok_prob[base + acc] = prob;
+      if (a.out_flags) a.out_flags[base + acc] = kOutResidual;
+    };
+    if (T == 0) {  // nothing but zeros: the first entry
+      if (i == 0) emit(pid[0], pv[0]);
+      return;
+    }
+    const uint64_t t = __umul64hi(sm.random, T);
+    if (!(t >= before && t < before + local)) return;  // the whole warp
+    for (int j0 = 0; j0 < per; j0 += E) {
+      if (LONG && per > E) {
+        load(j0);
+        weigh();
+      }
+      // the group of 32 that the draw falls to, then the entry
+      uint64_t group[E];
+#pragma unroll
+      for (int j = 0; j < E; ++j) group[j] = warp_sum_u64(fixed_weight(w[j]));
+      int at_id = 0;
+      float at_p = 0.0f;
+      uint64_t own = 0;
+      bool found = false;
+#pragma unroll
+      for (int j = 0; j < E; ++j) {
+        if (found) continue;
+        found = t < before + group[j];
+        if (found) {
+          own = fixed_weight(w[j]);
+          at_id = id[j];
+          at_p = p[j];
+        } else {
+          before += group[j];
+        }
+      }
+      if (!found) continue;
+      uint64_t upto = own;
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const uint64_t o = shfl_up_u64(upto, d);
+        if (lane >= d) upto += o;
+      }
+      upto += before;
+      if (t < upto && t >= upto - own) emit(at_id, at_p);
+      return;
+    }
   }
 }
 
