@@ -7,6 +7,7 @@ loaded, importing a symbol from it raises.
 from __future__ import annotations
 
 import ctypes as C
+import importlib.util
 from dataclasses import dataclass
 from typing import Optional
 
@@ -68,11 +69,21 @@ class _on:
 
 
 _lib = None
+_native = None
+
+
+def _load_native(L: C.CDLL):
+    """The extension module, pointed at the loaded library's functions."""
+    spec = importlib.util.spec_from_file_location(__package__ + "._native", _build.build_native())
+    mod = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(mod)
+    mod.set_entries(C.cast(L.sjd_step, C.c_void_p).value, C.cast(L.sjd_window_advance, C.c_void_p).value)
+    return mod
 
 
 def lib() -> C.CDLL:
     """The loaded CUDA library; built in-tree with nvcc when missing or stale.  Raises when that fails."""
-    global _lib
+    global _lib, _native
     if _lib is None:
         path = _build.build()
         L = C.CDLL(path)
@@ -99,6 +110,7 @@ def lib() -> C.CDLL:
                                          C.POINTER(sjd_probs), C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p,
                                          C.POINTER(sjd_probs), C.c_void_p, C.c_void_p]
         L.sjd_window_advance.restype = C.c_int
+        _native = _load_native(L)
         _lib = L
     return _lib
 
@@ -247,6 +259,13 @@ def sjd_step(logits_cond: torch.Tensor, logits_uncond: Optional[torch.Tensor], d
              draft_probs: Optional[DeviceProbs], params: sjd_params, philox_seed: int, out_accept_len: torch.Tensor,
              out_tokens: torch.Tensor, out_probs: DeviceProbs) -> None:
     """Enqueue one verify-and-redraft step on ``params.stream``.  Same arguments as the C entry point."""
+    if type(params) is sjd_params:
+        code = (_native or (lib(), _native)[1]).step(C.addressof(params), logits_cond, logits_uncond, drafts, draft_probs, philox_seed,
+                                                     out_accept_len, out_tokens, out_probs)
+        if code <= 0:
+            if code < 0:
+                _check(code)
+            return
     _check_logits(logits_cond, logits_uncond)
     q = C.byref(draft_probs.c_struct()) if draft_probs is not None else None
     with _on(logits_cond.device):
@@ -274,6 +293,13 @@ def sjd_window_advance(params: sjd_params, n_total: int, philox_seed: int, accep
                        committed: torch.Tensor, n_committed: Optional[torch.Tensor] = None) -> None:
     """Commit the accepted prefix and the residual token, shift the window and refill it (same arguments as
     the C entry point)."""
+    if type(params) is sjd_params:
+        code = (_native or (lib(), _native)[1]).advance(C.addressof(params), n_total, philox_seed, accept_len, step_tokens, step_probs, win_len,
+                                                        pos_base, iteration, next_drafts, next_probs, committed, n_committed)
+        if code <= 0:
+            if code < 0:
+                _check(code)
+            return
     sp, nq = step_probs.c_struct(), next_probs.c_struct()
     with _on(step_tokens.device):
         code = lib().sjd_window_advance(C.byref(params), int(n_total), int(philox_seed) & 0xFFFFFFFFFFFFFFFF,
