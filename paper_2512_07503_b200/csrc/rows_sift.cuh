@@ -875,18 +875,29 @@ __device__ __forceinline__ int finish_row(const RowArgs& a, const SiftCfg& cfg, 
     thr_y = __shfl_sync(0xffffffffu, me.y, who);
     thr_id = __shfl_sync(0xffffffffu, me.id, who);
   } else {
-    // a warp per member, a lane per rival
-    for (uint32_t x = (uint32_t)warp; x < nbin; x += NW) {
-      const SiftMember me = sm.hist.member[x];
-      uint32_t ahead = 0;
+    // A warp per member, a lane per rival; three members at a time, whose chains do not wait for one another.  (bf16 logits leave some
+    // forty members with hardly a different value: 1,024 rows of 65,536, K=2,000: 74.4 -> 73.6 us; K=8,192: 142.0 -> 140.0.)
+    constexpr int M = 3;
+    for (uint32_t x = (uint32_t)warp; x < nbin; x += M * NW) {
+      SiftMember me[M];
+      uint32_t ahead[M];
+#pragma unroll
+      for (int k = 0; k < M; ++k) {
+        me[k] = sm.hist.member[min(x + (uint32_t)(k * NW), nbin - 1u)];
+        ahead[k] = 0;
+      }
       for (uint32_t z = (uint32_t)lane; z < nbin; z += 32u) {
         const SiftMember o = sm.hist.member[z];
-        ahead += (o.y > me.y || (o.y == me.y && o.id < me.id)) ? 1u : 0u;
+#pragma unroll
+        for (int k = 0; k < M; ++k) ahead[k] += (o.y > me[k].y || (o.y == me[k].y && o.id < me[k].id)) ? 1u : 0u;
       }
-      ahead = __reduce_add_sync(0xffffffffu, ahead);
-      if (lane == 0 && ahead == need - 1u) {
-        sm.thr_y = me.y;
-        sm.thr_id = me.id;
+#pragma unroll
+      for (int k = 0; k < M; ++k) {
+        ahead[k] = __reduce_add_sync(0xffffffffu, ahead[k]);
+        if (lane == 0 && ahead[k] == need - 1u) {  // (the last member may come twice: the same values)
+          sm.thr_y = me[k].y;
+          sm.thr_id = me[k].id;
+        }
       }
     }
     row_sync<NT>(bar);
