@@ -34,8 +34,8 @@
 //                        phase (its first row's) is 9-14 K cycles of barriers and short searches that would hold up
 //                        eight warps (with every row sampled by its team: 94 us where this takes 82).
 //   rows_cluster_kernel  few rows: one cluster of up to eight CTAs of sixteen warps per row, the whole row in shared
-//                        memory at once.  The candidates go straight into the first CTA's lists (distributed shared
-//                        memory), which finishes the row.
+//                        memory at once.  Every CTA sifts into lists of its own and sends them to the first one (distributed
+//                        shared memory), which finishes the row.
 //
 // What bounds it: at V=65,536 and K=2,000 a row is about 40 K warp instructions at 56 % of the issue slots; a row of the
 // memory stream alone would be 12.3 K cycles, and takes 14 K.  us a step against the kernels that took these shapes before:
@@ -82,7 +82,7 @@ struct SiftCfg {
   int units;         // units per segment
   int seg_cap;       // candidates a segment's list holds (a multiple of 8)
   int pool;          // entries of all lists of a row (a multiple of 8, below 65,536)
-  int scratch;       // cluster kernel: ids that a warp can list apart from these
+  int scratch;       // cluster kernel, rows that crowd: ids that a warp can list apart from these
   int teams, slots;  // stream kernel: teams per CTA, ring slots per warp
   int once;          // stream kernel: the logits of the call exceed the L2
   int row_begin, row_end;  // stream kernel: this launch covers rows [row_begin, row_end)
@@ -620,9 +620,12 @@ __device__ __forceinline__ void put_u16(uint32_t at, uint32_t v) {
   if (REMOTE) asm volatile("st.shared::cluster.u16 [%0], %1;" ::"r"(at), "h"((uint16_t)v) : "memory");
   else asm volatile("st.shared.u16 [%0], %1;" ::"r"(at), "h"((uint16_t)v) : "memory");
 }
-template <bool REMOTE>
+// whose lists and histogram a sift fills: the CTA's own; the cluster's first CTA's; its own, to the histogram of which other CTAs add
+enum { kToOwn = 0, kToFirst = 1, kToShared = 2 };
+template <int TO>
 __device__ __forceinline__ void count_at(uint32_t at) {
-  if (REMOTE) asm volatile("red.relaxed.cluster.shared::cluster.add.u32 [%0], 1;" ::"r"(at) : "memory");
+  if (TO == kToFirst) asm volatile("red.relaxed.cluster.shared::cluster.add.u32 [%0], 1;" ::"r"(at) : "memory");
+  else if (TO == kToShared) asm volatile("red.relaxed.cluster.shared::cta.add.u32 [%0], 1;" ::"r"(at) : "memory");
   else asm volatile("red.relaxed.cta.shared::cta.add.u32 [%0], 1;" ::"r"(at) : "memory");
 }
 
@@ -641,11 +644,12 @@ __device__ __forceinline__ uint32_t take_entries(uint32_t at, uint32_t n, int la
 // what the list keeps plus `bias`.  n: candidates so far (cap + 1: the list has run over).
 // CROWDS: the unit takes a run of the row's list, which n becomes: its first entry, and from bit 16 its length (kNoRoom: there was
 // none).  Candidates that find no room are counted all the same, so that the row's histogram is complete.
-template <int DTYPE, bool HAS_U, bool HAS_T, bool REMOTE, bool CROWDS>
+template <int DTYPE, bool HAS_U, bool HAS_T, int TO, bool CROWDS>
 __device__ __forceinline__ void sift_unit(const RowArgs& a, uint32_t c_unit, uint32_t u_unit, int valid, uint32_t rel, uint32_t bias,
                                           uint64_t s2, uint64_t t2, const SiftBinning& bins, const SiftScreen& screen,
                                           const SiftTarget& to, int lane, uint32_t& n, float& vmax) {
   constexpr int ES = SiftTraits<DTYPE>::kElem, EP = SiftTraits<DTYPE>::kPiece, EU = SiftTraits<DTYPE>::kUnit;
+  constexpr bool REMOTE = TO == kToFirst;
   uint32_t x0 = 0, x1 = 0;  // hits of the lane's first and second piece
   const bool whole = valid > EU / 2;
   const uint32_t run = whole ? 2 * EP : EP;  // consecutive elements of a lane
@@ -703,8 +707,8 @@ __device__ __forceinline__ void sift_unit(const RowArgs& a, uint32_t c_unit, uin
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const uint32_t bin = min(__float2uint_rz(bins.at(y[h])), (uint32_t)kSiftBins - 1u);
-        count_at<REMOTE>(to.hist_at + 4u * bin);
-        count_at<REMOTE>(to.hist_at + 4u * (kSiftBins + (bin >> 5)));
+        count_at<TO>(to.hist_at + 4u * bin);
+        count_at<TO>(to.hist_at + 4u * (kSiftBins + (bin >> 5)));
         vmax = fmaxf(vmax, y[h]);
       }
     }
@@ -734,8 +738,8 @@ __device__ __forceinline__ void sift_unit(const RowArgs& a, uint32_t c_unit, uin
       const uint32_t i = i0 + 32u * j + (uint32_t)lane, k = at + i;
       const bool in = i < total;
       const uint32_t bin = in ? min(__float2uint_rz(bins.at(y[j])), (uint32_t)kSiftBins - 1u) : 0u;
-      count_at<REMOTE>(to.hist_at + 4u * bin);
-      count_at<REMOTE>(to.hist_at + 4u * (kSiftBins + (bin >> 5)));
+      count_at<TO>(to.hist_at + 4u * bin);
+      count_at<TO>(to.hist_at + 4u * (kSiftBins + (bin >> 5)));
       vmax = fmaxf(vmax, y[j]);
       if (in) {
         put_f32<REMOTE>(to.y_at + 4u * k, y[j]);
@@ -1246,7 +1250,7 @@ __device__ __noinline__ uint32_t stream_crowded_row(const RowArgs& a, const Sift
     phase ^= 1u << slot;
     const uint32_t c_unit = smem_u32(ring) + (uint32_t)slot * kSlot;
     uint32_t run = 0u;
-    sift_unit<DTYPE, HAS_U, HAS_T, false, true>(a, c_unit, c_unit + kUnitBytes, seg_n - unit * kStep, 0u, 0u, s2, t2, bins, screen, to, lane,
+    sift_unit<DTYPE, HAS_U, HAS_T, kToOwn, true>(a, c_unit, c_unit + kUnitBytes, seg_n - unit * kStep, 0u, 0u, s2, t2, bins, screen, to, lane,
                                                 run, vmax);
     over = over || run == kNoRoom;
     __syncwarp();
@@ -1478,7 +1482,7 @@ rows_stream_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ Si
       if (!ok) break;
       phase ^= 1u << slot;
       const uint32_t c_unit = ring_at + (uint32_t)slot * kSlot;
-      sift_unit<DTYPE, HAS_U, HAS_T, false, false>(a, c_unit, c_unit + kUnitBytes, seg_n - unit * EU, (uint32_t)(unit * EU), 0u, s2, t2,
+      sift_unit<DTYPE, HAS_U, HAS_T, kToOwn, false>(a, c_unit, c_unit + kUnitBytes, seg_n - unit * EU, (uint32_t)(unit * EU), 0u, s2, t2,
                                                    bins, screen, to, lane, n, vmax);
       __syncwarp();
       if (lane == 0) issue(k, unit + slots, slot);
@@ -1538,8 +1542,9 @@ struct alignas(16) ClusterShared {
   uint32_t go;                                   // a row that crowds is sifted once more, with `next` (the first CTA's)
   SiftTau next;
 };
-// shared memory: ClusterShared | list values | list ids | the warps' own ids | cond | uncond.  Only the cluster's first CTA uses the
-// lists (one per segment of the row, or one for the whole row, see rows_stream_kernel).
+// shared memory: ClusterShared | list values | list ids | the warps' own ids | cond | uncond.  The lists (one per segment of the row) are
+// complete in the cluster's first CTA, the others fill their segments'; of a row that crowds, one for the whole row in the first CTA
+// (see rows_stream_kernel).
 __host__ __device__ inline size_t sift_cluster_lists(const SiftCfg& cfg, int n_cta) {
   const size_t b = sizeof(ClusterShared) + (size_t)cfg.pool * 6 + (n_cta > 1 ? (size_t)kClusterWarps * cfg.scratch * 2 : 0);
   return (b + 127) & ~(size_t)127;
@@ -1568,6 +1573,10 @@ __device__ __forceinline__ uint32_t in_first_cta(const void* p) {
   uint32_t at;
   asm("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(at) : "r"(smem_u32(p)));
   return at;
+}
+
+__device__ __forceinline__ void put_16_bytes(uint32_t at, const uint4& v) {
+  asm volatile("st.shared::cluster.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(at), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
 
 // what a warp of the cluster has to say about its segment, to the first CTA (by one lane)
@@ -1621,7 +1630,7 @@ __device__ __noinline__ int cluster_crowded_row(const RowArgs& a, const SiftCfg&
   for (int k = 0; k < cfg.units; ++k) {
     uint32_t run = 0u;  // (segments at the row's end have fewer units)
     if (ok && k < units)
-      sift_unit<DTYPE, HAS_U, HAS_T, true, true>(a, c_at + (uint32_t)k * kUnitBytes, c_at + (uint32_t)(stage_bytes + (size_t)k * kUnitBytes),
+      sift_unit<DTYPE, HAS_U, HAS_T, kToFirst, true>(a, c_at + (uint32_t)k * kUnitBytes, c_at + (uint32_t)(stage_bytes + (size_t)k * kUnitBytes),
                                                  seg_n - k * EU, 0u, 0u, s2, t2, bins, screen, to, lane, run, vmax);
     over = over || run == kNoRoom;
     if (lane == 0) asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(runs_at + 4u * k), "r"(run) : "memory");
@@ -1649,7 +1658,6 @@ rows_cluster_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ S
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   float* const list_y = reinterpret_cast<float*>(smem_raw + sizeof(ClusterShared));
   uint16_t* const list_id = reinterpret_cast<uint16_t*>(list_y + cfg.pool);
-  uint16_t* const local_id = list_id + cfg.pool;
   const size_t stage_bytes = sift_cluster_stage(cfg, ES);
   unsigned char* const stage = smem_raw + sift_cluster_lists(cfg, (int)csize) + (size_t)warp * stage_bytes * (HAS_U ? 2 : 1);
   const int row = (int)(blockIdx.x / csize);
@@ -1736,24 +1744,38 @@ rows_cluster_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ S
   const SiftBinning bins = sift_bins(tau.tau0, tau.top);
   const SiftScreen screen = sift_screen<DTYPE, HAS_U, HAS_T>(a, cfg, tau.tau0, tau.u_max);
   SiftTarget to;
-  to.y_at = in_first_cta(list_y + (size_t)seg * cfg.seg_cap);
-  to.id_at = in_first_cta(list_id + (size_t)seg * cfg.seg_cap);
-  to.hist_at = in_first_cta(&sm.row.hist);
-  to.scratch_at = smem_u32(csize > 1 ? local_id + (size_t)warp * cfg.scratch : list_id + (size_t)seg * cfg.seg_cap);
+  // Every CTA sifts into its own lists and histogram (a segment's place in the lists is the same in all CTAs), and the others send
+  // theirs to the first one as a whole.  (Entry by entry, stores and counts into the first CTA's memory held the others up by 3.6 K cycles:
+  // 32 rows of 65,536 bf16, K=2,000: 18.8 -> 17.3 us a step; 16 rows of 4,096, a CTA each: 11.9 -> 11.7.)
+  to.y_at = smem_u32(list_y + (size_t)seg * cfg.seg_cap);
+  to.id_at = to.scratch_at = smem_u32(list_id + (size_t)seg * cfg.seg_cap);
+  to.hist_at = smem_u32(&sm.row.hist);
   to.cap = (uint32_t)cfg.seg_cap;
   const uint32_t bias = (uint32_t)((seg % (int)csize) * cfg.seg_len);  // ids are kept relative to the finishing warp's first one
   uint32_t n = 0;
   float vmax = __int_as_float(0xff800000);
-  cluster_wait();  // every CTA of the cluster has begun
   const bool ok = seg_n == 0 || mbar_wait(&sm.full[warp], 0u);
   if (ok) {
     const uint32_t c_at = smem_u32(stage), u_at = smem_u32(u_stage);
     for (int k = 0; k < units; ++k)
-      sift_unit<DTYPE, HAS_U, HAS_T, true, false>(a, c_at + (uint32_t)k * kUnitBytes, u_at + (uint32_t)k * kUnitBytes, seg_n - k * EU,
-                                                  (uint32_t)(k * EU), bias, s2, t2, bins, screen, to, lane, n, vmax);
+      sift_unit<DTYPE, HAS_U, HAS_T, kToShared, false>(a, c_at + (uint32_t)k * kUnitBytes, u_at + (uint32_t)k * kUnitBytes, seg_n - k * EU,
+                                                       (uint32_t)(k * EU) + bias, 0u, s2, t2, bins, screen, to, lane, n, vmax);
   }
   __syncwarp();
   const uint32_t wmax = __reduce_max_sync(0xffffffffu, float_key(vmax));
+  cluster_wait();  // every CTA of the cluster has begun
+  if (crank != 0) {
+    if (n <= to.cap) {  // (lists end on sixteen bytes)
+      const uint32_t y_to = in_first_cta(list_y + (size_t)seg * cfg.seg_cap), id_to = in_first_cta(list_id + (size_t)seg * cfg.seg_cap);
+      for (uint32_t k = 16u * (uint32_t)lane; k < 4u * n; k += 512u) put_16_bytes(y_to + k, lds128(to.y_at + k));
+      for (uint32_t k = 16u * (uint32_t)lane; k < 2u * n; k += 512u) put_16_bytes(id_to + k, lds128(to.id_at + k));
+    }
+    __syncthreads();  // (this CTA's histogram is complete)
+    const uint32_t* const words = reinterpret_cast<const uint32_t*>(&sm.row.hist);  // the fine bins and behind them the coarse ones
+    const uint32_t to_words = in_first_cta(words);
+    for (int k = tid; k < kSiftBins + kSiftBins / 32; k += NT)
+      if (words[k] != 0u) asm volatile("red.relaxed.cluster.shared::cluster.add.u32 [%0], %1;" ::"r"(to_words + 4u * k), "r"(words[k]) : "memory");
+  }
   if (lane == 0) {
     const bool over = n > to.cap;
     asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(in_first_cta(&sm.seg_n[seg])), "r"(n) : "memory");
