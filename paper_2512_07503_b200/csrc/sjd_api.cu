@@ -255,6 +255,8 @@ bool plan_sift(const sjd_params* P, int kcap, bool has_u, SiftPlan* plan) {
   // and the candidates, the barriers and the launch of a cluster are slow.  16 rows, us a step with clusters of 1, 2, 4, 8 CTAs and
   // by the stream kernel: of 16,384 bf16, K=500: 12.8, 14.1, 16.5, 32.3, 13.7; of 65,536 bf16 (do not fit one): -, 15.5, 16.7, 32.8,
   // 18.1; of 65,536 fp32: -, -, 16.7, 31.9, 21.3 (32 rows: 18.8 with four; 36 rows: 25.0, two rounds of clusters, and 21.8).
+  // (Those with the candidates sent one by one.  Sent as whole lists: 16 rows of 4,096 fp32 by one CTA each 11.4, by four 14.4; 32 rows of
+  // 65,536 bf16 by two 17.2, by four 17.9.)
   for (int n_cta = 1; n_cta <= sjd::kMaxCluster; n_cta <<= 1) {
     if (rows * n_cta > (n_cta <= 2 ? sms : n_cta == 4 ? sms * 7 / 8 : sms / 2)) break;
     if (!cut_segments(&c, V, kcap, sjd::kClusterWarps * n_cta, unit, p, sd, more) || (int64_t)n_cta * c.seg_len > 65536) continue;
