@@ -38,11 +38,11 @@
 //                        shared memory), which finishes the row.
 //
 // What bounds it: at V=65,536 and K=2,000 a row is about 40 K warp instructions at 56 % of the issue slots; a row of the
-// memory stream alone would be 12.3 K cycles, and takes 14 K.  us a step against the kernels that took these shapes before:
-// 1,024 rows of 65,536 bf16, K=2,000: 76.9 (88.4 with a kernel of one id range per filter thread); of 16,384: 47.5 (68.2);
-// 1,024 ragged rows of 16,384 fp32, K=1,000: 44.8 (59.4); 1,024 rows of 32,768 bf16 without guidance: 47.3 (64.7); 231 rows of
-// 50,264, K=500: 27.9 (100.8, four radix passes and a compaction over the row in the L2); 1,024 rows of 65,536, K=8,192:
-// 170 (524); 16 rows of 4,096 fp32, K=64: 12.9 (16.7, tiles dealt to filter warps).
+// memory stream alone would be 12.3 K cycles, and takes 14 K.  us a step (in brackets the kernels that took these shapes before):
+// 1,024 rows of 65,536 bf16, K=2,000: 73.5 (88.4 with a kernel of one id range per filter thread); of 16,384: 44.9 (68.2);
+// 1,024 ragged rows of 16,384 fp32, K=1,000: 41.7 (59.4); 1,024 rows of 32,768 bf16 without guidance: 44.5 (64.7); 231 rows of
+// 50,264, K=500: 27.4 (100.8, four radix passes and a compaction over the row in the L2); 1,024 rows of 65,536, K=8,192:
+// 139.0 (524); 16 rows of 4,096 fp32, K=64: 11.2 (16.7, tiles dealt to filter warps).
 //
 // Every wait on an mbarrier is bounded; a wait that gives up marks the row (and the CTA's unfinished rows) with
 // kRowStatusTimeout, and the CTA waits (bounded) for its copies in flight before it exits.
