@@ -1547,7 +1547,7 @@ rows_stream_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ Si
 struct alignas(16) ClusterShared {
   SiftShared row;                                // the first CTA's: histogram of the candidates, finish phase
   SiftSample sample;
-  uint32_t key[kClusterWarps];                   // threshold search: what each warp's count says
+  uint32_t key[2][kClusterWarps];                // threshold search: what each warp's count says, in two places used in turn
   uint64_t full[kClusterWarps];                  // a warp's segment has landed
   uint32_t seg_n[kClusterWarps * kMaxCluster];   // candidates per segment (the first CTA's)
   uint32_t lost;                                 // a bounded wait of the cluster gave up (the first CTA's)
@@ -1744,10 +1744,11 @@ rows_cluster_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ S
       for (int shift = near ? 4 : 12; shift >= 0; shift -= 4) {
         const uint32_t mine = key + ((uint32_t)warp << shift);
         const bool reached = warp == 0 || m.reaching(mine) >= rank;  // (a key beyond the largest maximum's is reached by none)
-        if (lane == 0) sm.key[warp] = reached ? mine : 0u;
+        // (Nobody is more than one barrier ahead; with a second barrier for every digit few rows took 0.1 to 0.2 us longer: 17.2 -> 17.1, 11.8 -> 11.6.)
+        uint32_t* const said = sm.key[(shift >> 2) & 1];
+        if (lane == 0) said[warp] = reached ? mine : 0u;
         __syncthreads();
-        key = __reduce_max_sync(0xffffffffu, sm.key[lane & 15]);
-        __syncthreads();
+        key = __reduce_max_sync(0xffffffffu, said[lane & 15]);
       }
       if (key >= kMaskedKey || whole) break;
       rank = m.reaching(kMaskedKey);  // (the same in every warp)
