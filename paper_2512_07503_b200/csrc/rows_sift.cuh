@@ -88,17 +88,20 @@ struct SiftCfg {
   int row_begin, row_end;  // stream kernel: this launch covers rows [row_begin, row_end)
 };
 
-struct SiftMember {  // member of the threshold bin: value and id
-  float y;
-  int32_t id;
-};
+// Member of the threshold bin: value and id as one number, the larger the earlier it ranks (value descending, id ascending; the two
+// zeros are equal values).
+__device__ __forceinline__ uint64_t sift_member(float y, int id) {
+  return (uint64_t)float_key(__fadd_rn(y, 0.0f)) << 32 | (uint32_t)~id;
+}
+__device__ __forceinline__ float member_value(uint64_t member) { return key_float((uint32_t)(member >> 32)); }
+__device__ __forceinline__ int member_id(uint64_t member) { return (int)~(uint32_t)member; }
 
 // Fine bins and one coarse bin per 32 of them: whoever counts in a fine bin counts in its coarse bin as well, which costs
 // next to nothing and makes the search for a rank two scans of 32 words, done while everybody waits.
 struct alignas(16) SiftHist {
   union {
     uint32_t fine[kSiftBins];        // zero whenever it is not in use
-    SiftMember member[kMemberCap];   // the threshold bin's members, after the histogram's last search
+    uint64_t member[kMemberCap];     // the threshold bin's members, after the histogram's last search
   };
   uint32_t coarse[kSiftBins / 32];
   __device__ __forceinline__ void count(uint32_t bin) {
@@ -872,7 +875,7 @@ __device__ __forceinline__ int finish_row(const RowArgs& a, const SiftCfg& cfg, 
         const float y = y_g[i], x = bins.at(y);
         if (x >= lo && (x < hi || last)) {
           const int at = atomicAdd(&sm.members, 1);  // (as many as the histogram counted: the check keeps the store in bounds)
-          if (at < kMemberCap) sm.hist.member[at] = SiftMember{y, id0 + (int32_t)my_id[at_g + i]};
+          if (at < kMemberCap) sm.hist.member[at] = sift_member(y, id0 + (int32_t)my_id[at_g + i]);
         }
       }
     }
@@ -883,39 +886,41 @@ __device__ __forceinline__ int finish_row(const RowArgs& a, const SiftCfg& cfg, 
   int thr_id;
   if (nbin <= 32u) {
     // every warp ranks them for itself, a lane per member
-    const SiftMember me = sm.hist.member[min(lane, (int)nbin - 1)];
+    const uint64_t me = sm.hist.member[min(lane, (int)nbin - 1)];
     uint32_t ahead = 0;
 #pragma unroll 4
-    for (int x = 0; x < (int)nbin; ++x) {
-      const SiftMember o = sm.hist.member[x];
-      ahead += (o.y > me.y || (o.y == me.y && o.id < me.id)) ? 1u : 0u;
-    }
+    for (int x = 0; x < (int)nbin; ++x) ahead += sm.hist.member[x] > me ? 1u : 0u;
     const int who = __ffs((int)__ballot_sync(0xffffffffu, lane < (int)nbin && ahead == need - 1u)) - 1;
-    thr_y = __shfl_sync(0xffffffffu, me.y, who);
-    thr_id = __shfl_sync(0xffffffffu, me.id, who);
+    const uint64_t found = shfl_u64(me, who);
+    thr_y = member_value(found);
+    thr_id = member_id(found);
   } else {
     // A warp per member, a lane per rival; three members at a time, whose chains do not wait for one another.  (bf16 logits leave some
-    // forty members with hardly a different value: 1,024 rows of 65,536, K=2,000: 74.4 -> 73.6 us; K=8,192: 142.0 -> 140.0.)
+    // forty members with hardly a different value: 1,024 rows of 65,536, K=2,000: 74.4 -> 73.6 us; K=8,192: 142.0 -> 140.0.)  A comparison is
+    // one of numbers: with values and ids compared apart it branched, and a row with 327 members, a few entries far above the rest, took 50 K
+    // cycles to finish (32 K one member at a time).  64 rows of 524,288 bf16, K=100: 79.1 -> 61.0 us a step (one at a time: 70.2), without guidance
+    // 73.3 -> 51.7 (61.8); 64 of 262,144 fp32: 65.7 -> 54.2 (62.1).
     constexpr int M = 3;
     for (uint32_t x = (uint32_t)warp; x < nbin; x += M * NW) {
-      SiftMember me[M];
+      uint64_t me[M];
       uint32_t ahead[M];
 #pragma unroll
       for (int k = 0; k < M; ++k) {
         me[k] = sm.hist.member[min(x + (uint32_t)(k * NW), nbin - 1u)];
         ahead[k] = 0;
       }
+#pragma unroll 2
       for (uint32_t z = (uint32_t)lane; z < nbin; z += 32u) {
-        const SiftMember o = sm.hist.member[z];
+        const uint64_t o = sm.hist.member[z];
 #pragma unroll
-        for (int k = 0; k < M; ++k) ahead[k] += (o.y > me[k].y || (o.y == me[k].y && o.id < me[k].id)) ? 1u : 0u;
+        for (int k = 0; k < M; ++k) ahead[k] += o > me[k] ? 1u : 0u;
       }
 #pragma unroll
       for (int k = 0; k < M; ++k) {
         ahead[k] = __reduce_add_sync(0xffffffffu, ahead[k]);
         if (lane == 0 && ahead[k] == need - 1u) {  // (the last member may come twice: the same values)
-          sm.thr_y = me[k].y;
-          sm.thr_id = me[k].id;
+          sm.thr_y = member_value(me[k]);
+          sm.thr_id = member_id(me[k]);
         }
       }
     }
@@ -974,7 +979,7 @@ __device__ __forceinline__ int finish_row(const RowArgs& a, const SiftCfg& cfg, 
     sm.wz[warp] = z;
   }
   row_sync<NT>(bar);
-  for (uint32_t x = (uint32_t)tid; x < nbin; x += NT) sm.hist.member[x] = SiftMember{0.0f, 0};  // the histogram's words again
+  for (uint32_t x = (uint32_t)tid; x < nbin; x += NT) sm.hist.member[x] = 0ull;  // the histogram's words again
   if (tid == 0) sm.members = 0;
   const uint32_t cw = lane < NW ? sm.wcnt[lane] : 0u;
   const uint32_t before = __reduce_add_sync(0xffffffffu, lane < warp ? cw : 0u);
