@@ -1453,8 +1453,11 @@ rows_stream_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ Si
     issue_unit<DTYPE, HAS_U>(a, st, ring, policy, warp, teams, units, seg0, seg_n, EU, n_live, k, unit, slot);
   };
   // The first copies are sent off before anything else (behind the first team's sample: 1,024 rows of 16,384 bf16 46.2 us a step, now 45.3;
-  // ragged fp32 ones 42.0 and 41.5; of 65,536 73.2 and 73.7).
+  // ragged fp32 ones 42.0 and 41.5; of 65,536 73.2 and 73.7; 444 of 32,768, K=2,500, 41.8 and 40.8), but behind its sample where the CTA has
+  // a single row of several units a warp: no other row hides a sample that waits for copies (148 rows of 65,536, K=10: 19.4 before the
+  // sample, now 18.6; of fp32 25.0 and 23.7; of 262,144, K=700, 39.7 and 38.8; a unit a warp, 200 rows of 4,096: 12.7 before it, 12.9 behind it).
   if (team == (teams > 1 ? 1 : 0) && lane == 0 && units > 0) {
+    if (n_live == 1 && team > 0 && units > 1) mbar_wait(&st.sample_full[0], 0u);
     for (int x = 0; x < slots; ++x) issue(0, x, x);
   }
   __syncwarp();
