@@ -340,21 +340,29 @@ cudaError_t launch_sift(const sjd::RowArgs& ra, const SiftPlan& plan, cudaStream
   return t ? launch_sift_as<DTYPE, false, true>(ra, plan, st) : launch_sift_as<DTYPE, false, false>(ra, plan, st);
 }
 
-template <bool LONG, int LOOK>
+template <bool LONG, int LOOK, bool MANY>
 cudaError_t launch_verify_as(const sjd::VerifyArgs& va, cudaStream_t st, bool dependent) {
-  auto kern = sjd::verify_kernel<LONG, LOOK>;
+  auto kern = sjd::verify_kernel<LONG, LOOK, MANY>;
   static sjd::DeviceOnce configured;
   const cudaError_t e = allow_large_smem(kern, configured, (int)kSmemLimit);
   if (e != cudaSuccess) return e;
   return launch_after(kern, dim3((unsigned)va.B), dim3(sjd::kVerifyThreads), sjd::verify_smem(va.V, va.kcap, LONG, LOOK), st, dependent, 1, va);
 }
+template <bool LONG, int LOOK>
+cudaError_t launch_verify_of(const sjd::VerifyArgs& va, cudaStream_t st, bool dependent) {
+  // Two CTAs to an SM where they would go in rounds otherwise, us a step (V, K, sequences x rows; one to an SM, two): 4,096, 64, 170 x 1: 14.0, 14.0;
+  // 300 x 1: 16.8, 15.3; 1,024 x 1: 39.2, 33.1; 1,024, 64, 2,048 x 1: 98.0, 85.6; 65,536, 2,000, 200 x 4: 64.6, 63.2; 4,096, 2,100, 1,024 x 1: 68.0, 52.6;
+  // 65,536, 8,192, 200 x 4: 129.4, 124.1.  A few more than one to an SM end about as early the one way as the other: 4,096, 64, 149 x 1: 13.7, 13.8;
+  // 524,288, 2,000, 150 x 1: 133.1, 135.0.
+  return va.B > sm_count() + sm_count() / 8 ? launch_verify_as<LONG, LOOK, true>(va, st, dependent) : launch_verify_as<LONG, LOOK, false>(va, st, dependent);
+}
 cudaError_t launch_verify(const sjd::VerifyArgs& va, cudaStream_t st, bool dependent) {
   const bool is_long = va.kcap > sjd::kVerifyShort;
   const int look = sjd::verify_map(va.V, va.kcap, is_long, kSmemLimit);
-  if (!is_long) return look == sjd::kMapVals ? launch_verify_as<false, sjd::kMapVals>(va, st, dependent) : launch_verify_as<false, sjd::kNoMap>(va, st, dependent);
-  return look == sjd::kMapVals ? launch_verify_as<true, sjd::kMapVals>(va, st, dependent)
-         : look == sjd::kMap   ? launch_verify_as<true, sjd::kMap>(va, st, dependent)
-                               : launch_verify_as<true, sjd::kNoMap>(va, st, dependent);
+  if (!is_long) return look == sjd::kMapVals ? launch_verify_of<false, sjd::kMapVals>(va, st, dependent) : launch_verify_of<false, sjd::kNoMap>(va, st, dependent);
+  return look == sjd::kMapVals ? launch_verify_of<true, sjd::kMapVals>(va, st, dependent)
+         : look == sjd::kMap   ? launch_verify_of<true, sjd::kMap>(va, st, dependent)
+                               : launch_verify_of<true, sjd::kNoMap>(va, st, dependent);
 }
 
 // Scratch of sjd_step_static(): lives in the library's device image, so every GPU that loads the library

@@ -91,13 +91,16 @@ inline int verify_map(int V, int kcap, bool is_long, size_t limit) {
 // owns consecutive entries of the rejected row, a lane every 32nd of them; only the warp that the draw falls to locates it.
 //
 // LONG: rows of more than 2,048 entries, a warp's taken sixteen groups of 32 at a time.
+// MANY: more sequences than SMs (launch_verify()): two CTAs to an SM.  One CTA of 72 registers a thread (128 where it is LONG) fills an SM, and then
+// the sequences go in rounds; where there is one round, registers shorten the only CTA's way (1,024 rows in 32 sequences 73.2 us a step with 64
+// registers, 70.8 with 72; in 512 of two rows 78.7, 81.4).  LONG rows then come four groups at a time: sixteen do not fit, eight are no faster.
 //
 // The map, the loads without branches and the early requests against a search by halving in the row itself, from the row stage's end to a
 // CTA's own, thousands of cycles: 16 rows of K=64 7.4 -> 4.9, 1,024 rows of K=2,000 11.3 -> 7.3, of K=8,192 85 -> 14.7 (a step: 77.9 -> 74.6
 // us, 171 -> 142 us); 128 rows of V=131,072, K=8,192 73.2 -> 55.8 us a step; 32 rows of K=V=65,536 (without probabilities in the map) 597 -> 378 us.
-template <bool LONG, int LOOK>
-__global__ void __launch_bounds__(kVerifyThreads) verify_kernel(const VerifyArgs a) {
-  constexpr int NT = kVerifyThreads, NW = NT / 32, E = LONG ? 16 : 4;
+template <bool LONG, int LOOK, bool MANY>
+__global__ void __launch_bounds__(kVerifyThreads, MANY ? 2 : 1) verify_kernel(const VerifyArgs a) {
+  constexpr int NT = kVerifyThreads, NW = NT / 32, E = LONG && !MANY ? 16 : 4;
   constexpr bool MAP = LOOK != kNoMap, VALS = LOOK == kMapVals || (LOOK == kNoMap && !LONG);  // VALS: the probabilities are staged
   extern __shared__ __align__(128) unsigned char smem_raw[];
   VerifySmem& sm = *reinterpret_cast<VerifySmem*>(smem_raw);
