@@ -1,17 +1,17 @@
-"""Compile the CUDA library (libsjd.so) in-tree for sm_100a with nvcc, and the binding's extension module (_native.so) with the host compiler."""
+"""Compile the CUDA library (libsjd.so) in-tree for sm_100a with nvcc, and the binding's extension module (_native.*.so) with the host compiler."""
 from __future__ import annotations
 
 import glob
 import os
 import shutil
 import subprocess
+import sysconfig
 
 _PKG = os.path.dirname(os.path.abspath(__file__))
 _CSRC = os.path.join(_PKG, "csrc")
 _INC = os.path.join(os.path.dirname(_PKG), "include")
 LIB_PATH = os.path.join(_PKG, "libsjd.so")
 NATIVE_SOURCE = os.path.join(_CSRC, "binding_native.cpp")
-NATIVE_PATH = os.path.join(_PKG, "_native.so")
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17", "-shared",
               "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr", "--extended-lambda"]
@@ -39,24 +39,32 @@ def is_stale() -> bool:
     return any(os.path.getmtime(p) > t for p in _deps())
 
 
+def native_path() -> str:
+    """Where the extension module lies that fits this interpreter and this PyTorch.  It is compiled against the layouts of both, so their versions
+    are part of its name: after a change of either it is another file, and one that fits the new ones is built."""
+    import torch
+    fits = [sysconfig.get_config_var("SOABI"), "torch" + torch.__version__, (torch.version.git_version or "")[:8],
+            "cxx11" if torch.compiled_with_cxx11_abi() else "cxx98"]
+    return os.path.join(_PKG, "_native." + ".".join(str(x) for x in fits) + ".so")
+
+
 def build_native(force: bool = False) -> str:
     """The extension module that binding.py calls the library's per-step functions through."""
+    path = native_path()
     deps = [NATIVE_SOURCE] + glob.glob(os.path.join(_INC, "*.h"))
-    if not force and os.path.exists(NATIVE_PATH) and all(os.path.getmtime(p) <= os.path.getmtime(NATIVE_PATH) for p in deps):
-        return NATIVE_PATH
-    import sysconfig
-
+    if not force and os.path.exists(path) and all(os.path.getmtime(p) <= os.path.getmtime(path) for p in deps):
+        return path
     import torch
     at = os.path.join(os.path.dirname(torch.__file__), "include")
     libs = ["-L" + os.path.join(os.path.dirname(torch.__file__), "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10_cuda", "-lc10"]
     cuda = os.path.join(os.path.dirname(os.path.dirname(_nvcc())), "include")
     includes = [at, os.path.join(at, "torch", "csrc", "api", "include"), cuda, sysconfig.get_paths()["include"]]
-    tmp = NATIVE_PATH + f".tmp{os.getpid()}"
+    tmp = path + f".tmp{os.getpid()}"
     # (torch is imported before the module: the libraries named here are loaded already)
     cmd = [shutil.which("g++") or "g++", "-O2", "-std=c++20", "-shared", "-fPIC", *[f"-I{d}" for d in includes], NATIVE_SOURCE, "-o", tmp, *libs]
     subprocess.check_call(cmd)
-    os.replace(tmp, NATIVE_PATH)
-    return NATIVE_PATH
+    os.replace(tmp, path)
+    return path
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
