@@ -8,6 +8,8 @@ from __future__ import annotations
 
 import ctypes as C
 import importlib.util
+import subprocess
+import warnings
 from dataclasses import dataclass
 from typing import Optional
 
@@ -69,7 +71,7 @@ class _on:
 
 
 _lib = None
-_native = None
+_native = None  # the extension module; False where there is none
 
 
 def _load_native(L: C.CDLL):
@@ -110,9 +112,21 @@ def lib() -> C.CDLL:
                                          C.POINTER(sjd_probs), C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p,
                                          C.POINTER(sjd_probs), C.c_void_p, C.c_void_p]
         L.sjd_window_advance.restype = C.c_int
-        _native = _load_native(L)
+        try:
+            _native = _load_native(L)
+        except (OSError, RuntimeError, ImportError, subprocess.SubprocessError) as e:
+            # a library built elsewhere needs no compiler here, nor the headers of Python, PyTorch and CUDA
+            warnings.warn(f"no extension module for the binding ({e}): calls take some microseconds longer", RuntimeWarning, stacklevel=2)
+            _native = False
         _lib = L
     return _lib
+
+
+def _native_module():
+    """The extension module, or False."""
+    if _native is None:
+        lib()
+    return _native
 
 
 def sjd_version() -> int:
@@ -259,9 +273,9 @@ def sjd_step(logits_cond: torch.Tensor, logits_uncond: Optional[torch.Tensor], d
              draft_probs: Optional[DeviceProbs], params: sjd_params, philox_seed: int, out_accept_len: torch.Tensor,
              out_tokens: torch.Tensor, out_probs: DeviceProbs) -> None:
     """Enqueue one verify-and-redraft step on ``params.stream``.  Same arguments as the C entry point."""
-    if type(params) is sjd_params:
-        code = (_native or (lib(), _native)[1]).step(C.addressof(params), logits_cond, logits_uncond, drafts, draft_probs, philox_seed,
-                                                     out_accept_len, out_tokens, out_probs)
+    native = _native or _native_module()
+    if native and type(params) is sjd_params:
+        code = native.step(C.addressof(params), logits_cond, logits_uncond, drafts, draft_probs, philox_seed, out_accept_len, out_tokens, out_probs)
         if code <= 0:
             if code < 0:
                 _check(code)
@@ -293,9 +307,10 @@ def sjd_window_advance(params: sjd_params, n_total: int, philox_seed: int, accep
                        committed: torch.Tensor, n_committed: Optional[torch.Tensor] = None) -> None:
     """Commit the accepted prefix and the residual token, shift the window and refill it (same arguments as
     the C entry point)."""
-    if type(params) is sjd_params:
-        code = (_native or (lib(), _native)[1]).advance(C.addressof(params), n_total, philox_seed, accept_len, step_tokens, step_probs, win_len,
-                                                        pos_base, iteration, next_drafts, next_probs, committed, n_committed)
+    native = _native or _native_module()
+    if native and type(params) is sjd_params:
+        code = native.advance(C.addressof(params), n_total, philox_seed, accept_len, step_tokens, step_probs, win_len, pos_base, iteration,
+                              next_drafts, next_probs, committed, n_committed)
         if code <= 0:
             if code < 0:
                 _check(code)
