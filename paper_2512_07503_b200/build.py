@@ -48,23 +48,32 @@ def native_path() -> str:
     return os.path.join(_PKG, "_native." + ".".join(str(x) for x in fits) + ".so")
 
 
+def _native_command(out: str, first_includes=()) -> list:
+    import torch
+    at = os.path.join(os.path.dirname(torch.__file__), "include")
+    libs = ["-L" + os.path.join(os.path.dirname(torch.__file__), "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10_cuda", "-lc10"]
+    cuda = os.path.join(os.path.dirname(os.path.dirname(_nvcc())), "include")
+    includes = [*first_includes, at, os.path.join(at, "torch", "csrc", "api", "include"), cuda, sysconfig.get_paths()["include"]]
+    # (torch is imported before the module: the libraries named here are loaded already)
+    return [shutil.which("g++") or "g++", "-O2", "-std=c++20", "-shared", "-fPIC", *[f"-I{d}" for d in includes], NATIVE_SOURCE, "-o", out, *libs]
+
+
 def build_native(force: bool = False) -> str:
     """The extension module that binding.py calls the library's per-step functions through."""
     path = native_path()
     deps = [NATIVE_SOURCE] + glob.glob(os.path.join(_INC, "*.h"))
     if not force and os.path.exists(path) and all(os.path.getmtime(p) <= os.path.getmtime(path) for p in deps):
         return path
-    import torch
-    at = os.path.join(os.path.dirname(torch.__file__), "include")
-    libs = ["-L" + os.path.join(os.path.dirname(torch.__file__), "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10_cuda", "-lc10"]
-    cuda = os.path.join(os.path.dirname(os.path.dirname(_nvcc())), "include")
-    includes = [at, os.path.join(at, "torch", "csrc", "api", "include"), cuda, sysconfig.get_paths()["include"]]
     tmp = path + f".tmp{os.getpid()}"
-    # (torch is imported before the module: the libraries named here are loaded already)
-    cmd = [shutil.which("g++") or "g++", "-O2", "-std=c++20", "-shared", "-fPIC", *[f"-I{d}" for d in includes], NATIVE_SOURCE, "-o", tmp, *libs]
-    subprocess.check_call(cmd)
+    subprocess.check_call(_native_command(tmp))
     os.replace(tmp, path)
     return path
+
+
+def build_native_variant(out_path: str, first_includes) -> str:
+    """The extension module with other headers found first (test builds: a stand-in for the CUDA device functions), written to `out_path`."""
+    subprocess.check_call(_native_command(out_path, first_includes))
+    return out_path
 
 
 def build(force: bool = False, verbose: bool = False) -> str:

@@ -1,7 +1,7 @@
 // The per-step calls of the binding as a CPython extension: the same checks as binding.py makes, on the tensors themselves instead of through
 // attribute lookups, which bounded small steps and the decode loop's critical path: 16 rows of 4,096 13.1 -> 11.9 us a step, 32 iterations of
 // one window 2,058 -> 1,655 us, 16 of sixteen windows 1,130 -> 934 us.
-// Whatever is not the ordinary case (another type, a device that is not current, a check that fails) is handed back untouched
+// Whatever is not the ordinary case (another type, a check that fails) is handed back untouched
 // and takes the way through binding.py, which also words the errors.
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
@@ -68,9 +68,29 @@ uint64_t word_of(PyObject* o) {
   }
   return v;
 }
-void check_current(const at::Tensor& t) {
-  if (!t.is_cuda() || t.get_device() != c10::cuda::current_device()) throw HandBack{};
-}
+// A CUDA tensor's device is current as long as this lives: a process that drives several GPUs need not switch itself.
+class OnDeviceOf {
+ public:
+  explicit OnDeviceOf(const at::Tensor& t) {
+    if (!t.is_cuda()) throw HandBack{};
+    const c10::DeviceIndex current = c10::cuda::current_device();
+    if (t.get_device() == current) return;
+    c10::cuda::set_device(t.get_device());
+    before_ = current;
+  }
+  ~OnDeviceOf() {
+    if (before_ < 0) return;
+    try {
+      c10::cuda::set_device(before_);
+    } catch (...) {  // (it was current before: the next CUDA call says what has happened to it)
+    }
+  }
+  OnDeviceOf(const OnDeviceOf&) = delete;
+  OnDeviceOf& operator=(const OnDeviceOf&) = delete;
+
+ private:
+  c10::DeviceIndex before_ = -1;
+};
 
 // step(params address, cond, uncond, drafts, draft_probs, seed, accept_len, tokens, out_probs)
 PyObject* py_step(PyObject*, PyObject* const* a, Py_ssize_t n) {
@@ -82,7 +102,7 @@ PyObject* py_step(PyObject*, PyObject* const* a, Py_ssize_t n) {
   try {
     const sjd_params* const params = reinterpret_cast<const sjd_params*>(word_of(a[0]));
     const at::Tensor& cond = tensor_of(a[1]);
-    check_current(cond);
+    const OnDeviceOf on(cond);
     const void* uncond = nullptr;
     if (a[2] != Py_None) {
       const at::Tensor& u = tensor_of(a[2]);
@@ -124,7 +144,7 @@ PyObject* py_advance(PyObject*, PyObject* const* a, Py_ssize_t n) {
     if (overflow != 0 || total != (int32_t)total) throw HandBack{};
     const uint64_t seed = word_of(a[2]);
     auto words = [&](int i) { return static_cast<int32_t*>(optional_array_of(a[i], at::kInt)); };
-    check_current(tensor_of(a[4]));
+    const OnDeviceOf on(tensor_of(a[4]));
     sjd_probs step = probs_of(a[5]), next = probs_of(a[10]);
     int32_t *const acc = words(3), *const tok = words(4), *const win = words(6), *const pos = words(7), *const iter = words(8), *const drafts = words(9),
                    *const committed = words(11), *const count = words(12);
