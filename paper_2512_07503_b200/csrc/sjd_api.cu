@@ -264,12 +264,15 @@ bool plan_sift(const sjd_params* P, int kcap, bool has_u, SiftPlan* plan) {
     plan->cluster = n_cta;
     plan->smem = sjd::sift_cluster_smem(c, n_cta, es, has_u);
     if (plan->smem > kSmemLimit) continue;
-    // A row that crowds lists the ids of a unit apart from the row's list: room for all of a unit's, as long as the verification's
-    // blocks still find room beside this kernel's.
-    const size_t beside = 36u << 10;
+    // A row that crowds lists the ids of a unit apart from the row's list: room for all of a unit's, as far as the division of an SM's
+    // memory that the row needs anyway goes (196 KB shared, or all of it: with less left to the L1 ordinary rows take up to 1 % longer).  The
+    // verification's blocks need nothing kept free: beside these, 512 threads of 72 registers and more, they find no registers.  (With 36 KB
+    // kept free for them rows of K=8,192 got no more room at all: 32 of 65,536 bf16 that crowd 163 us a step, now 87; 8 of fp32 144 and 106.)
     const int most = c.seg_len < unit ? c.seg_len : unit;
-    if (n_cta > 1 && most > c.scratch && plan->smem + beside < kSmemLimit) {
-      const int room = c.scratch + (int)((kSmemLimit - beside - plan->smem) / (2 * sjd::kClusterWarps));
+    const size_t division = 195u << 10;  // (a block's own kilobyte comes on top)
+    const size_t limit = plan->smem <= division ? division : kSmemLimit;
+    if (n_cta > 1 && most > c.scratch) {
+      const int room = c.scratch + (int)((limit - plan->smem) / (2 * sjd::kClusterWarps));
       c.scratch = (room < most ? room : most) & ~7;
       plan->smem = sjd::sift_cluster_smem(c, n_cta, es, has_u);
     }
