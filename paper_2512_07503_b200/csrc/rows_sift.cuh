@@ -618,9 +618,9 @@ __device__ __forceinline__ uint32_t put_ids(uint32_t x, uint32_t first, uint32_t
 
 // where a warp's candidates go
 struct SiftTarget {
-  uint32_t y_at, id_at;    // shared-memory addresses of the segment's lists (of the cluster's first CTA when REMOTE)
+  uint32_t y_at, id_at;    // shared-memory addresses of the segment's lists (a cluster's row that crowds: of the row's, in the first CTA)
   uint32_t hist_at;        // of the candidates' histogram (a SiftHist)
-  uint32_t scratch_at;     // local id list (the same as id_at unless REMOTE)
+  uint32_t scratch_at;     // where ids are listed first: the same as id_at unless that is in another CTA
   uint32_t cap;            // candidates the lists hold
   // a row that crowds: the lists are the row's
   uint32_t taken_at;       // of the number of entries given out
@@ -658,13 +658,13 @@ __device__ __forceinline__ uint32_t take_entries(uint32_t at, uint32_t n, int la
   return __shfl_sync(0xffffffffu, first, 31);
 }
 
-// One unit: `valid` elements of it belong to the segment; element 0 has id `rel` in the segment's numbering, which is
-// what the list keeps plus `bias`.  n: candidates so far (cap + 1: the list has run over).
+// One unit: `valid` elements of it belong to the segment; element 0 has id `rel` in the list's numbering.  n: candidates so far (cap + 1:
+// the list has run over).
 // CROWDS: the unit takes a run of the row's list, which n becomes: its first entry, and from bit 16 its length (kNoRoom: there was
 // none).  Candidates that find no room are counted all the same, so that the row's histogram is complete.
 template <int DTYPE, bool HAS_U, bool HAS_T, int TO, bool CROWDS>
-__device__ __forceinline__ void sift_unit(const RowArgs& a, uint32_t c_unit, uint32_t u_unit, int valid, uint32_t rel, uint32_t bias,
-                                          uint64_t s2, uint64_t t2, const SiftBinning& bins, const SiftScreen& screen,
+__device__ __forceinline__ void sift_unit(const RowArgs& a, uint32_t c_unit, uint32_t u_unit, int valid, uint32_t rel, uint64_t s2,
+                                          uint64_t t2, const SiftBinning& bins, const SiftScreen& screen,
                                           const SiftTarget& to, int lane, uint32_t& n, float& vmax) {
   constexpr int ES = SiftTraits<DTYPE>::kElem, EP = SiftTraits<DTYPE>::kPiece, EU = SiftTraits<DTYPE>::kUnit;
   constexpr bool REMOTE = TO == kToFirst;
@@ -761,7 +761,7 @@ __device__ __forceinline__ void sift_unit(const RowArgs& a, uint32_t c_unit, uin
       vmax = fmaxf(vmax, y[j]);
       if (in) {
         put_f32<REMOTE>(to.y_at + 4u * k, y[j]);
-        if (REMOTE) put_u16<true>(to.id_at + 2u * k, id[j] + bias);
+        if (REMOTE) put_u16<true>(to.id_at + 2u * k, id[j]);
       }
     }
   };
@@ -1270,8 +1270,8 @@ __device__ __noinline__ uint32_t stream_crowded_row(const RowArgs& a, const Sift
     phase ^= 1u << slot;
     const uint32_t c_unit = smem_u32(ring) + (uint32_t)slot * kSlot;
     uint32_t run = 0u;
-    sift_unit<DTYPE, HAS_U, HAS_T, kToOwn, true>(a, c_unit, c_unit + kUnitBytes, seg_n - unit * kStep, 0u, 0u, s2, t2, bins, screen, to, lane,
-                                                run, vmax);
+    sift_unit<DTYPE, HAS_U, HAS_T, kToOwn, true>(a, c_unit, c_unit + kUnitBytes, seg_n - unit * kStep, 0u, s2, t2, bins, screen, to, lane, run,
+                                                vmax);
     over = over || run == kNoRoom;
     __syncwarp();
     if (lane == 0) {
@@ -1503,8 +1503,8 @@ rows_stream_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ Si
       if (!ok) break;
       phase ^= 1u << slot;
       const uint32_t c_unit = ring_at + (uint32_t)slot * kSlot;
-      sift_unit<DTYPE, HAS_U, HAS_T, kToOwn, false>(a, c_unit, c_unit + kUnitBytes, seg_n - unit * EU, (uint32_t)(unit * EU), 0u, s2, t2,
-                                                   bins, screen, to, lane, n, vmax);
+      sift_unit<DTYPE, HAS_U, HAS_T, kToOwn, false>(a, c_unit, c_unit + kUnitBytes, seg_n - unit * EU, (uint32_t)(unit * EU), s2, t2, bins,
+                                                    screen, to, lane, n, vmax);
       __syncwarp();
       if (lane == 0) issue(k, unit + slots, slot);
       if (++slot == slots) slot = 0;
@@ -1652,7 +1652,7 @@ __device__ __noinline__ int cluster_crowded_row(const RowArgs& a, const SiftCfg&
     uint32_t run = 0u;  // (segments at the row's end have fewer units)
     if (ok && k < units)
       sift_unit<DTYPE, HAS_U, HAS_T, kToFirst, true>(a, c_at + (uint32_t)k * kUnitBytes, c_at + (uint32_t)(stage_bytes + (size_t)k * kUnitBytes),
-                                                 seg_n - k * EU, 0u, 0u, s2, t2, bins, screen, to, lane, run, vmax);
+                                                 seg_n - k * EU, 0u, s2, t2, bins, screen, to, lane, run, vmax);
     over = over || run == kNoRoom;
     if (lane == 0) asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(runs_at + 4u * k), "r"(run) : "memory");
     __syncwarp();  // (the warp's own ids are listed again)
@@ -1752,7 +1752,7 @@ rows_cluster_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ S
       for (int shift = near ? 4 : 12; shift >= 0; shift -= 4) {
         const uint32_t mine = key + ((uint32_t)warp << shift);
         const bool reached = warp == 0 || m.reaching(mine) >= rank;  // (a key beyond the largest maximum's is reached by none)
-        // (Nobody is more than one barrier ahead; with a second barrier for every digit few rows took 0.1 to 0.2 us longer: 17.2 -> 17.1, 11.8 -> 11.6.)
+        // (Nobody is more than one barrier ahead: a second barrier for every digit is not needed.  What it cost lies within the runs' spread.)
         uint32_t* const said = sm.key[(shift >> 2) & 1];
         if (lane == 0) said[warp] = reached ? mine : 0u;
         __syncthreads();
@@ -1783,7 +1783,7 @@ rows_cluster_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ S
     const uint32_t c_at = smem_u32(stage), u_at = smem_u32(u_stage);
     for (int k = 0; k < units; ++k)
       sift_unit<DTYPE, HAS_U, HAS_T, kToShared, false>(a, c_at + (uint32_t)k * kUnitBytes, u_at + (uint32_t)k * kUnitBytes, seg_n - k * EU,
-                                                       (uint32_t)(k * EU) + bias, 0u, s2, t2, bins, screen, to, lane, n, vmax);
+                                                       (uint32_t)(k * EU) + bias, s2, t2, bins, screen, to, lane, n, vmax);
   }
   __syncwarp();
   const uint32_t wmax = __reduce_max_sync(0xffffffffu, float_key(vmax));

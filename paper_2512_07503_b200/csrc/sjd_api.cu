@@ -252,11 +252,10 @@ bool plan_sift(const sjd_params* P, int kcap, bool has_u, SiftPlan* plan) {
   const double more = !c.packed ? 1.0 : P->logits_dtype == SJD_F16 || !has_u ? 1.05 : 1.15;
   // few rows: the fewest CTAs that hold a row, while all rows' clusters find their SMs at once (clusters of four and eight do
   // not fill the GPU: their SMs lie in one GPC).  Sharing a row costs more than it saves: every CTA takes the whole sample,
-  // and the candidates, the barriers and the launch of a cluster are slow.  16 rows, us a step with clusters of 1, 2, 4, 8 CTAs and
-  // by the stream kernel: of 16,384 bf16, K=500: 12.8, 14.1, 16.5, 32.3, 13.7; of 65,536 bf16 (do not fit one): -, 15.5, 16.7, 32.8,
-  // 18.1; of 65,536 fp32: -, -, 16.7, 31.9, 21.3 (32 rows: 18.8 with four; 36 rows: 25.0, two rounds of clusters, and 21.8).
-  // (Those with the candidates sent one by one.  Sent as whole lists: 16 rows of 4,096 fp32 by one CTA each 11.4, by four 14.4; 32 rows of
-  // 65,536 bf16 by two 17.2, by four 17.9.)
+  // and the candidates, the barriers and the launch of a cluster are slow.  us a step with clusters of 1, 2, 4, 8 CTAs and by the stream
+  // kernel: 16 rows of 4,096 fp32, K=64: 11.3, 13.0, 13.9, 20.7, 11.2; of 16,384 bf16, K=500: 12.2, 13.8, 14.9, 22.9, 12.9; of 65,536, K=2,000,
+  // bf16 (one does not hold it): -, 16.7, 16.9, 24.7, 20.7 (32 rows: -, 16.8, 17.3, 31.4, 20.8), fp32: -, -, 16.8, 24.0, 23.8 (32 rows: -, -,
+  // 17.6, 30.8, 24.6; 36 rows, two rounds of four: -, -, 23.0, 33.0, 24.8).
   for (int n_cta = 1; n_cta <= sjd::kMaxCluster; n_cta <<= 1) {
     if (rows * n_cta > (n_cta <= 2 ? sms : n_cta == 4 ? sms * 7 / 8 : sms / 2)) break;
     if (!cut_segments(&c, V, kcap, sjd::kClusterWarps * n_cta, unit, p, sd, more) || (int64_t)n_cta * c.seg_len > 65536) continue;
