@@ -356,7 +356,8 @@ cudaError_t launch_verify_of(const sjd::VerifyArgs& va, cudaStream_t st, bool de
   // 300 x 1: 16.8, 15.3; 1,024 x 1: 39.2, 33.1; 1,024, 64, 2,048 x 1: 98.0, 85.6; 65,536, 2,000, 200 x 4: 64.6, 63.2; 4,096, 2,100, 1,024 x 1: 68.0, 52.6;
   // 65,536, 8,192, 200 x 4: 129.4, 124.1.  A few more than one to an SM end about as early the one way as the other: 4,096, 64, 149 x 1: 13.7, 13.8;
   // 524,288, 2,000, 150 x 1: 133.1, 135.0.
-  return va.B > sm_count() + sm_count() / 8 ? launch_verify_as<LONG, LOOK, true>(va, st, dependent) : launch_verify_as<LONG, LOOK, false>(va, st, dependent);
+  const int sms = sm_count();
+  return va.B > sms + sms / 8 ? launch_verify_as<LONG, LOOK, true>(va, st, dependent) : launch_verify_as<LONG, LOOK, false>(va, st, dependent);
 }
 cudaError_t launch_verify(const sjd::VerifyArgs& va, cudaStream_t st, bool dependent) {
   const bool is_long = va.kcap > sjd::kVerifyShort;
